@@ -1,0 +1,814 @@
+// The general operator's backward on samples sorted by key cell: see dsa3d_cells.cuh.
+//
+//   cells_bin_kernel     sorts the samples of a query tile by key block; 18 bytes per sample
+//   cells_dots_kernel    per block: samples by cell, 16 at a time  q . K_corner  and  dO . V_corner  (tensor cores), the
+//                        trilinear value and derivatives of both per sample: eight numbers
+//   cells_query_kernel   per query: alpha, delta, dS, dOffsets, the two coefficients per sample, dQ (a gather of K rows)
+//   cells_sums_kernel    per block: samples by cell, 16 at a time their contributions to the eight corner rows of dK or dV
+//                        (tensor cores), reduced into the fp32 accumulators
+//   cells_far_kernel     what falls beyond the bins (more than 12 positions from the query's tile), row by row
+#include <cuda_bf16.h>
+
+#include "dsa3d_cells.cuh"
+#include "dsa3d_kernels.h"
+
+namespace dsa3d {
+namespace {
+
+using namespace cells;
+using bf16 = __nv_bfloat16;
+
+// ------------------------------------------------------------------------------------------------ binning
+constexpr int kBinThreads = 512, kBinWarps = kBinThreads / 32, kCopies = 8;
+
+__global__ void __launch_bounds__(kBinThreads, 2)
+cells_bin_kernel(const float* __restrict__ offsets, const Problem pr, const Slab sl, unsigned inv_p) {
+    extern __shared__ __align__(16) unsigned char raw[];
+    uint32_t* counters = reinterpret_cast<uint32_t*>(raw);                 // [kBins + 1][kCopies]: lanes of a warp mostly hit the same bin
+    uint32_t* words = counters + (kBins + 1) * kCopies;                     // [128 * P]: bin (9 bits), cell (6), rank in its counter (16)
+    __shared__ uint32_t scan[kBinWarps];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const long long tile = blockIdx.x;
+    int r = static_cast<int>(tile % (sl.tiles_t * sl.tiles_y * sl.tiles_x));
+    const int m = sl.m0 + static_cast<int>(tile / (sl.tiles_t * sl.tiles_y * sl.tiles_x));
+    const int x0 = (r % sl.tiles_x) * 8; r /= sl.tiles_x;
+    const int y0 = (r % sl.tiles_y) * 4, t0 = sl.f0 + (r / sl.tiles_y) * 4;
+    const int samples = kRows * pr.P;
+    for (int i = tid; i < (kBins + 1) * kCopies / 4; i += kBinThreads) reinterpret_cast<uint4*>(counters)[i] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    auto row_of = [&](int s) { return static_cast<int>((static_cast<unsigned long long>(static_cast<unsigned>(s)) * inv_p) >> 24); };
+    auto cell_of = [&](int s, int& n) -> Cell {
+        const int row = row_of(s), p = s - row * pr.P;
+        const int t = t0 + (row >> 5), y = y0 + ((row >> 3) & 3), x = x0 + (row & 7);
+        n = (t * pr.H + y) * pr.W + x;
+        if (t >= sl.f1 || y >= pr.H || x >= pr.W) { Cell c; c.it = c.iy = c.ix = 0; c.mask = 0u; c.ft = c.fy = c.fx = 0.0f; return c; }
+        return make_cell(pr, t, y, x, p, offsets + ((static_cast<long long>(n) * pr.heads + m) * pr.P + p) * 3);
+    };
+    for (int base = 0; base < samples; base += 4 * kBinThreads) {
+        uint32_t w[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {                  // four samples per thread at a time: their offsets load together
+            const int s = base + i * kBinThreads + tid;
+            w[i] = 0xffffffffu;
+            if (s >= samples) continue;
+            int n;
+            const Cell c = cell_of(s, n);
+            if (c.mask == 0u) continue;
+            const int rt = c.it - t0 + kReach, ry = c.iy - y0 + kReach, rx = c.ix - x0 + kReach;
+            uint32_t bin = kBins, cell = 0u;
+            if (static_cast<unsigned>(rt) < 4u * kBinsT && static_cast<unsigned>(ry) < 4u * kBinsY && static_cast<unsigned>(rx) < 4u * kBinsX) {
+                bin = static_cast<uint32_t>(((rt >> 2) * kBinsY + (ry >> 2)) * kBinsX + (rx >> 2));
+                cell = static_cast<uint32_t>(((rt & 3) << 4) | ((ry & 3) << 2) | (rx & 3));
+            }
+            w[i] = bin | (cell << 9);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int s = base + i * kBinThreads + tid;
+            if (s >= samples) continue;
+            if (w[i] != 0xffffffffu) w[i] |= atomicAdd(&counters[(w[i] & 511u) * kCopies + (lane & (kCopies - 1))], 1u) << 15;
+            words[s] = w[i];
+        }
+    }
+    __syncthreads();
+    uint32_t c[kCopies], total = 0u;
+    if (tid <= kBins) {
+#pragma unroll
+        for (int i = 0; i < kCopies; i += 4) {
+            const uint4 v = *reinterpret_cast<const uint4*>(&counters[tid * kCopies + i]);
+            c[i] = v.x; c[i + 1] = v.y; c[i + 2] = v.z; c[i + 3] = v.w;
+        }
+#pragma unroll
+        for (int i = 0; i < kCopies; ++i) total += c[i];
+    }
+    uint32_t incl = total;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t up = __shfl_up_sync(kFullMask, incl, o);
+        if (lane >= o) incl += up;
+    }
+    if (lane == 31) scan[warp] = incl;
+    __syncthreads();
+    uint32_t start = incl - total;
+#pragma unroll
+    for (int i = 0; i < kBinWarps; ++i) if (i < warp) start += scan[i];
+    if (tid <= kBins) {
+        sl.seg[tile * (kBins + 1) + tid] = start | (total << 16);
+#pragma unroll
+        for (int i = 0; i < kCopies; ++i) {
+            const uint32_t n = c[i];
+            c[i] = start;
+            start += n;
+        }
+#pragma unroll
+        for (int i = 0; i < kCopies; i += 4) *reinterpret_cast<uint4*>(&counters[tid * kCopies + i]) = make_uint4(c[i], c[i + 1], c[i + 2], c[i + 3]);
+    }
+    __syncthreads();
+    uint4* geo = sl.geo + tile * samples;
+    uint16_t* meta = sl.meta + tile * samples;
+    for (int s = tid; s < samples; s += kBinThreads) {
+        const uint32_t w = words[s];
+        if (w == 0xffffffffu) continue;
+        int n;
+        const Cell cl = cell_of(s, n);                 // once more from the offsets, in L1 or L2 by now
+        const uint32_t at = counters[(w & 511u) * kCopies + (lane & (kCopies - 1))] + (w >> 15);
+        geo[at] = make_uint4(static_cast<uint32_t>(n), __float_as_uint(cl.ft), __float_as_uint(cl.fy), __float_as_uint(cl.fx));
+        meta[at] = static_cast<uint16_t>(static_cast<uint32_t>(s - row_of(s) * pr.P) | (((w >> 9) & 63u) << 8));
+    }
+}
+
+// ------------------------------------------------------------------------------------------------ a block's samples
+struct BlockPos { int m, t, y, x; };               // head, first cell along t, y, x
+
+__device__ __forceinline__ BlockPos block_pos(const Slab& sl, long long id) {
+    BlockPos b;
+    b.x = (static_cast<int>(id % sl.blocks_x) - 1) * 4; id /= sl.blocks_x;
+    b.y = (static_cast<int>(id % sl.blocks_y) - 1) * 4; id /= sl.blocks_y;
+    b.t = sl.f0 + (static_cast<int>(id % sl.blocks_t) + sl.bt0) * 4;
+    b.m = sl.m0 + static_cast<int>(id / sl.blocks_t);
+    return b;
+}
+
+struct Segments {
+    uint32_t first[kSegs + 1];                      // samples before the segment
+    uint32_t start[kSegs];                          // its place in its tile's list
+    int tile[kSegs];
+    uint32_t scan[8];
+};
+
+// Finds the segments of a block (at least 224 threads, all of the CTA); returns how many samples they hold.
+__device__ __forceinline__ uint32_t find_segments(const Slab& sl, const BlockPos& b, Segments& sg) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint32_t count = 0u, start = 0u;
+    int tile = 0;
+    if (tid < kSegs) {
+        const int bt = tid / (kBinsY * (kBinsX / 2)), by = (tid / (kBinsX / 2)) % kBinsY;
+        const int Bt = (b.t - sl.f0) >> 2, By = b.y >> 2, Bx = b.x >> 2;            // arithmetic: -4 >> 2 = -1
+        const int bx = ((Bx + 3) & 1) + 2 * (tid % (kBinsX / 2));
+        const int tt = Bt + 3 - bt, ty = By + 3 - by, tx = (Bx + 3 - bx) / 2;
+        if (static_cast<unsigned>(tt) < static_cast<unsigned>(sl.tiles_t) && static_cast<unsigned>(ty) < static_cast<unsigned>(sl.tiles_y) &&
+            Bx + 3 - bx >= 0 && tx < sl.tiles_x) {
+            tile = (((b.m - sl.m0) * sl.tiles_t + tt) * sl.tiles_y + ty) * sl.tiles_x + tx;
+            const uint32_t w = __ldg(sl.seg + static_cast<long long>(tile) * (kBins + 1) + (bt * kBinsY + by) * kBinsX + bx);
+            start = w & 0xffffu;
+            count = w >> 16;
+        }
+    }
+    uint32_t incl = count;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t up = __shfl_up_sync(kFullMask, incl, o);
+        if (lane >= o) incl += up;
+    }
+    if (warp < 7 && lane == 31) sg.scan[warp] = incl;
+    __syncthreads();
+    uint32_t before = 0u, total = 0u;
+#pragma unroll
+    for (int i = 0; i < 7; ++i) {
+        const uint32_t v = sg.scan[i];
+        if (i < warp) before += v;
+        total += v;
+    }
+    if (tid < kSegs) {
+        sg.first[tid] = before + incl - count;
+        sg.start[tid] = start;
+        sg.tile[tid] = tile;
+        if (tid == kSegs - 1) sg.first[kSegs] = total;
+    }
+    __syncthreads();
+    return total;
+}
+
+// Index, in the slab's sample lists, of the block's i-th sample.
+__device__ __forceinline__ long long sample_of(const Segments& sg, uint32_t i, int samples_per_tile) {
+    int lo = 0, hi = kSegs;                         // first[lo] <= i < first[hi]
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const int mid = (lo + hi) >> 1;
+        if (sg.first[mid] <= i) lo = mid; else hi = mid;
+    }
+    return static_cast<long long>(sg.tile[lo]) * samples_per_tile + sg.start[lo] + (i - sg.first[lo]);
+}
+
+// Byte of 16-byte chunk `chunk` of box row `row` in shared memory: rows of 128 bytes and more have their chunks permuted by
+// the row's parity, so that the four chunks a quarter-warp reads of two neighbouring rows lie in different banks.
+template <int D> __device__ __forceinline__ int box_byte(int row, int chunk) {
+    return row * (D * 2) + ((D >= 64 ? (chunk ^ ((row & 1) << 2)) : chunk) << 4);
+}
+
+// The rows of a block's box of one tensor into shared memory, zeros outside the grid.
+template <int D, int NT>
+__device__ __forceinline__ void load_box(unsigned char* dst, const bf16* __restrict__ src, const BlockPos& b, const Problem& pr) {
+    constexpr int CH = D / 8;
+    for (int i = threadIdx.x; i < kBox * CH; i += NT) {
+        const int row = i / CH, chunk = i - row * CH;
+        const int t = b.t + row / 25, y = b.y + (row / 5) % 5, x = b.x + row % 5;
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (static_cast<unsigned>(t) < static_cast<unsigned>(pr.T) && static_cast<unsigned>(y) < static_cast<unsigned>(pr.H) && static_cast<unsigned>(x) < static_cast<unsigned>(pr.W))
+            v = __ldg(reinterpret_cast<const uint4*>(src + (((static_cast<long long>(t) * pr.H + y) * pr.W + x) * pr.heads + b.m) * D) + chunk);
+        *reinterpret_cast<uint4*>(dst + box_byte<D>(row, chunk)) = v;
+    }
+}
+
+// ------------------------------------------------------------------------------------------------ dot products
+constexpr int kDotThreads = 512, kDotCap = 2048;
+
+template <int D> struct DotSmem {
+    unsigned char box[2][kBox * D * 2];
+    float4 geo[kDotCap];                            // ft, fy, fx, token (bits); sorted by cell
+    uint32_t dest[kDotCap];                         // where the sample's results go
+    uint32_t group[kDotCap / 16 + kCells];          // cell | first sample << 8 | samples - 1 << 20
+    uint32_t count[kCells], first[kCells + 1], gfirst[kCells + 1];
+    Segments sg;
+};
+
+// Value and derivatives of the trilinear interpolant of eight corner numbers, two corners (2j, 2j + 1: x pair of (ct, cy) =
+// (j >> 1, j & 1)) on each of four lanes: lane j returns number j of (value, d/dt, d/dy, d/dx).  Corners whose
+// weight and weight derivatives are all zero do not enter (they may hold anything).
+__device__ __forceinline__ float trilerp_lanes(float s0, float s1, int j, float ft, float fy, float fx) {
+    const float wt = (j & 2) ? ft : 1.0f - ft, wy = (j & 1) ? fy : 1.0f - fy;
+    const bool at = wt != 0.0f, ay = wy != 0.0f, ax = fx != 0.0f;
+    if (!(at || ay)) s0 = 0.0f;
+    if (!((at && ay) || (ax && (at || ay)))) s1 = 0.0f;
+    const float X = s1 - s0, L = fmaf(fx, X, s0), wty = wt * wy;
+    const float v0 = wty * L, v1 = (j & 2) ? wy * L : -wy * L, v2 = (j & 1) ? wt * L : -wt * L, v3 = wty * X;
+    const bool up = (j & 2) != 0;
+    const float keep0 = up ? v2 : v0, keep1 = up ? v3 : v1, send0 = up ? v0 : v2, send1 = up ? v1 : v3;
+    const float r0 = keep0 + __shfl_xor_sync(kFullMask, send0, 2), r1 = keep1 + __shfl_xor_sync(kFullMask, send1, 2);
+    const bool odd = (j & 1) != 0;
+    return (odd ? r1 : r0) + __shfl_xor_sync(kFullMask, odd ? r0 : r1, 1);
+}
+
+// q . K and dO . V with derivatives, eight numbers per sample into stats; even warps take q . K, odd ones dO . V.
+template <int D>
+__global__ void __launch_bounds__(kDotThreads, 2)
+cells_dots_kernel(const bf16* __restrict__ q, const bf16* __restrict__ k, const bf16* __restrict__ v, const bf16* __restrict__ dout,
+                  const Problem pr, const Slab sl) {
+    constexpr int I = D / 32, W = kDotThreads / 64, PER = kDotCap / kDotThreads;
+    extern __shared__ __align__(16) unsigned char raw[];
+    DotSmem<D>& s = *reinterpret_cast<DotSmem<D>*>(raw);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g8 = lane >> 2, j = lane & 3;
+    const int tensor = warp & 1;
+    const BlockPos b = block_pos(sl, blockIdx.x);
+    const uint32_t total = find_segments(sl, b, s.sg);
+    if (total == 0u) return;
+    load_box<D, kDotThreads>(s.box[0], k, b, pr);
+    load_box<D, kDotThreads>(s.box[1], v, b, pr);
+    const bf16* src = (tensor ? dout : q) + static_cast<long long>(b.m) * D + j * 8;
+    const unsigned char* box = s.box[tensor];
+    const long long tok = static_cast<long long>(pr.heads) * D;
+    for (uint32_t b0 = 0; b0 < total; b0 += kDotCap) {
+        const int nb = static_cast<int>(min(static_cast<uint32_t>(kDotCap), total - b0));
+        if (tid < kCells) s.count[tid] = 0u;
+        __syncthreads();
+        uint4 u[PER];
+        uint32_t rank[PER], dest[PER];              // rank: cell | rank in the cell << 8
+#pragma unroll
+        for (int e = 0; e < PER; ++e) {
+            const int i = e * kDotThreads + tid;
+            rank[e] = 0xffffffffu;
+            if (i >= nb) continue;
+            const long long at = sample_of(s.sg, b0 + static_cast<uint32_t>(i), kRows * pr.P);
+            u[e] = __ldg(sl.geo + at);
+            rank[e] = __ldg(sl.meta + at);
+        }
+#pragma unroll
+        for (int e = 0; e < PER; ++e) {
+            if (rank[e] == 0xffffffffu) continue;
+            dest[e] = static_cast<uint32_t>(sample_at(sl, pr, b.m, static_cast<int>(u[e].x), static_cast<int>(rank[e] & 255u)));
+            rank[e] = (rank[e] >> 8) | (atomicAdd(&s.count[rank[e] >> 8], 1u) << 8);
+        }
+        __syncthreads();
+        if (warp == 0) {                            // exclusive sums over the cells: samples and groups of 16
+            const uint32_t c0 = s.count[2 * lane], c1 = s.count[2 * lane + 1];
+            const uint32_t n0 = (c0 + 15u) >> 4, n1 = (c1 + 15u) >> 4;
+            uint32_t inc = c0 + c1, ginc = n0 + n1;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t up = __shfl_up_sync(kFullMask, inc, o), gup = __shfl_up_sync(kFullMask, ginc, o);
+                if (lane >= o) { inc += up; ginc += gup; }
+            }
+            s.first[2 * lane] = inc - c0 - c1; s.first[2 * lane + 1] = inc - c1;
+            s.gfirst[2 * lane] = ginc - n0 - n1; s.gfirst[2 * lane + 1] = ginc - n1;
+            if (lane == 31) { s.first[kCells] = inc; s.gfirst[kCells] = ginc; }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < PER; ++e)
+            if (rank[e] != 0xffffffffu) {
+                const uint32_t at = s.first[rank[e] & 63u] + (rank[e] >> 8);
+                s.geo[at] = make_float4(__uint_as_float(u[e].y), __uint_as_float(u[e].z), __uint_as_float(u[e].w), __uint_as_float(u[e].x));
+                s.dest[at] = dest[e];
+            }
+        if (tid < kCells) {
+            const uint32_t c = s.count[tid], f = s.first[tid], gf = s.gfirst[tid];
+            for (uint32_t i = 0; i * 16u < c; ++i) s.group[gf + i] = static_cast<uint32_t>(tid) | ((f + i * 16u) << 8) | ((min(16u, c - i * 16u) - 1u) << 20);
+        }
+        __syncthreads();
+        const int groups = static_cast<int>(s.gfirst[kCells]);
+        for (int g = warp >> 1; g < groups; g += W) {
+            const uint32_t gw = s.group[g];
+            const int row = box_row(static_cast<int>(gw & 63u)) + box_step(g8);
+            const int f = static_cast<int>((gw >> 8) & 0xfffu), last = static_cast<int>(gw >> 20);
+            const int ia = f + min(g8, last), ib = f + min(g8 + 8, last);       // a missing sample repeats the last one
+            const float4 ga = s.geo[ia], gb = s.geo[ib];
+            const uint4* pa = reinterpret_cast<const uint4*>(src + __float_as_int(ga.w) * tok);
+            const uint4* pb = reinterpret_cast<const uint4*>(src + __float_as_int(gb.w) * tok);
+            // The order of the channels inside a product is free: lane j takes chunk j of every 64 bytes, whole
+            // 16-byte pieces on both sides.
+            uint4 ra[I], rb[I];
+#pragma unroll
+            for (int i = 0; i < I; ++i) {
+                ra[i] = __ldg(pa + 4 * i);
+                rb[i] = __ldg(pb + 4 * i);
+            }
+            float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+            for (int i = 0; i < I; ++i) {
+                const uint4 kb = *reinterpret_cast<const uint4*>(box + box_byte<D>(row, 4 * i + j));
+                mma_bf16(c, ra[i].x, rb[i].x, ra[i].y, rb[i].y, kb.x, kb.y);
+                mma_bf16(c, ra[i].z, rb[i].z, ra[i].w, rb[i].w, kb.z, kb.w);
+            }
+            const float xa = trilerp_lanes(c[0], c[1], j, ga.x, ga.y, ga.z), xb = trilerp_lanes(c[2], c[3], j, gb.x, gb.y, gb.z);
+            float* d = sl.stats + tensor * 4 + j;
+            if (g8 <= last) d[static_cast<size_t>(s.dest[ia]) * 8] = xa;
+            if (g8 + 8 <= last) d[static_cast<size_t>(s.dest[ib]) * 8] = xb;
+        }
+        __syncthreads();                            // the batch's places are free for the next one
+    }
+}
+
+// ------------------------------------------------------------------------------------------------ per query
+constexpr int kQueryThreads = 256;
+
+// alpha from the saved lse, delta, dS, dOffsets, the two coefficients per sample (ck = scale dS, cv = alpha), and
+// dQ = sum_p ck_p sum_c w_c K_c: a group of D / 8 lanes per (query, head), 16 bytes of a row per lane.  A sample with
+// anything that is not finite (its rows of q, dO, K or V, or its coefficients) is marked by the sign of cv: its
+// contributions to dK and dV are formed one by one, so that they reach only the corners with a weight.
+template <int D>
+__global__ void __launch_bounds__(kQueryThreads, 4)
+cells_query_kernel(const bf16* __restrict__ k, const float* __restrict__ offsets, const float* __restrict__ lse, bf16* __restrict__ dq,
+                   float* __restrict__ doffsets, const Problem pr, const Slab sl) {
+    using E = Elt<bf16, 1>;
+    using Row = typename E::Row;
+    constexpr int LPR = D / 8;
+    const int lane = threadIdx.x & 31, gl = lane & (LPR - 1);
+    const long long per_head = static_cast<long long>(pr.H) * pr.W * (sl.f1 - sl.f0), items = per_head * sl.heads;
+    long long item = (static_cast<long long>(blockIdx.x) * kQueryThreads + threadIdx.x) / LPR;
+    const long long warp_first = (static_cast<long long>(blockIdx.x) * kQueryThreads + (threadIdx.x & ~31)) / LPR;
+    if (warp_first >= items) return;
+    const bool active = item < items;               // a trailing group repeats the last item, stores off
+    if (!active) item = items - 1;
+    const int m = sl.m0 + static_cast<int>(item / per_head);
+    const int n = static_cast<int>(static_cast<long long>(pr.H) * pr.W * sl.f0 + item % per_head);
+    const int x = n % pr.W, y = (n / pr.W) % pr.H, t = n / (pr.W * pr.H);
+    const long long row = static_cast<long long>(n) * pr.heads + m;
+    const float scale = rsqrtf(static_cast<float>(D)), lse2 = __ldg(lse + row) * kLog2e;
+    const float* off_row = offsets + row * pr.P * 3;
+    const float* st_row = sl.stats + item * pr.P * 8;
+    const long long tok = static_cast<long long>(pr.heads) * D;
+    const long long sy = static_cast<long long>(pr.W) * tok, st = static_cast<long long>(pr.H) * sy;
+    const bf16* kh = k + static_cast<long long>(m) * D + gl * 8;
+    [[maybe_unused]] const long long kv_extent = pr.N * pr.heads * D;
+
+    float delta = 0.0f;
+    for (int p = gl; p < pr.P; p += LPR) {
+        const Cell c = make_cell(pr, t, y, x, p, off_row + p * 3);
+        if (c.mask == 0u) continue;                 // a dead sample has g = 0
+        const float sv = __ldg(st_row + p * 8), g = __ldg(st_row + p * 8 + 4);
+        delta = fmaf(exp2f(fmaf(sv, scale * kLog2e, -lse2)), g, delta);
+    }
+    delta = group_sum<LPR>(delta, kFullMask);
+    float acc[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) acc[e] = 0.0f;
+    for (int pb = 0; pb < pr.P; pb += LPR) {
+        Sample mine;
+        mine.base = 0; mine.mask = 0u; mine.ft = mine.fy = mine.fx = 0.0f;
+        float my_ck = 0.0f;
+        if (pb + gl < pr.P) {
+            const int p = pb + gl;
+            mine = to_sample(pr, make_cell(pr, t, y, x, p, off_row + p * 3));
+            float d0 = 0.0f, d1 = 0.0f, d2 = 0.0f;
+            if (mine.mask != 0u) {
+                const float4 a = __ldg(reinterpret_cast<const float4*>(st_row + p * 8)), b = __ldg(reinterpret_cast<const float4*>(st_row + p * 8) + 1);
+                const float alpha = exp2f(fmaf(a.x, scale * kLog2e, -lse2));
+                my_ck = scale * (alpha * (b.x - delta));
+                d0 = fmaf(my_ck, a.y, alpha * b.y);
+                d1 = fmaf(my_ck, a.z, alpha * b.z);
+                d2 = fmaf(my_ck, a.w, alpha * b.w);
+                const bool odd = !(fabsf(a.x) < INFINITY) || !(fabsf(b.x) < INFINITY) || !(fabsf(my_ck) < INFINITY) || !(alpha < INFINITY);
+                if (active) sl.coef[item * pr.P + p] = make_float2(my_ck, __uint_as_float(__float_as_uint(alpha) | (odd ? 0x80000000u : 0u)));
+            }
+            if (active) {
+                float* d = doffsets + (row * pr.P + p) * 3;
+                d[0] = d0; d[1] = d1; d[2] = d2;
+            }
+        }
+        const int cnt = min(LPR, pr.P - pb);
+        for (int j = 0; j < cnt; ++j) {
+            const Sample s = group_bcast<LPR>(mine, j, kFullMask);
+            const float ck = __shfl_sync(kFullMask, my_ck, j, LPR);
+            const float wt[2] = {1.0f - s.ft, s.ft}, wy[2] = {1.0f - s.fy, s.fy}, wx[2] = {1.0f - s.fx, s.fx};
+            const bf16* kp4[4];
+            kp4[0] = kh + s.base * tok;
+            kp4[1] = kp4[0] + sy;
+            kp4[2] = kp4[0] + st;
+            kp4[3] = kp4[2] + sy;
+            if (s.mask == 0xffu && s.ft != 0.0f && s.fy != 0.0f && s.fx != 0.0f) {
+                Row kk[8];
+#pragma unroll
+                for (int c = 0; c < 8; ++c) kk[c] = DSA3D_IN_RANGE(pr, kp4[c >> 1] + (c & 1) * tok - k, kv_extent, 4) ? E::load(kp4[c >> 1] + (c & 1) * tok) : E::zero();
+#pragma unroll
+                for (int c = 0; c < 8; ++c) E::axpy_paired(ck * (wt[c >> 2] * wy[(c >> 1) & 1] * wx[c & 1]), kk[c], acc);
+            } else {
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    const float w = wt[c >> 2] * wy[(c >> 1) & 1] * wx[c & 1];
+                    if (((s.mask >> c) & 1u) && w != 0.0f && DSA3D_IN_RANGE(pr, kp4[c >> 1] + (c & 1) * tok - k, kv_extent, 6))
+                        E::axpy_paired(ck * w, E::load(kp4[c >> 1] + (c & 1) * tok), acc);
+                }
+            }
+        }
+    }
+    if (active) E::store(dq + row * D + gl * 8, acc);
+}
+
+// ------------------------------------------------------------------------------------------------ dK, dV
+constexpr int kSumThreads = 256;
+
+template <int D> struct SumSmem {
+    static constexpr int CAP = 1792, PER = CAP / kSumThreads;     // samples at a time: two CTAs per SM fit
+    static constexpr int STAGES = D == 128 ? 2 : 3;
+    float4 geo[CAP];                                // ft, fy, fx, ck; sorted by cell, as everything below
+    unsigned char stage[kSumThreads / 32][STAGES][16 * D * 2];    // a warp's ring of 16 query rows
+    float cv[CAP];
+    uint32_t token[CAP];
+    uint32_t count[kCells], first[kCells + 1];
+    Segments sg;
+};
+
+__device__ __forceinline__ void red_add_v2(float* addr, float a, float b) {
+    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(addr), "f"(a), "f"(b) : "memory");
+}
+
+// Contributions of one sample to dK and dV, corner by corner (those with a weight), by one thread.
+template <int D>
+__device__ __noinline__ void add_sample(const bf16* q, const bf16* dout, float* acc_dk, float* acc_dv, const Problem& pr, int m, int n, int t0, int y0,
+                                        int x0, float ft, float fy, float fx, float ck, float cv) {
+    const bf16 *qr = q + (static_cast<long long>(n) * pr.heads + m) * D, *dr = dout + (static_cast<long long>(n) * pr.heads + m) * D;
+    for (int c = 0; c < 8; ++c) {
+        const int t = t0 + (c >> 2), y = y0 + ((c >> 1) & 1), x = x0 + (c & 1);
+        const float w = ((c & 4) ? ft : 1.0f - ft) * ((c & 2) ? fy : 1.0f - fy) * ((c & 1) ? fx : 1.0f - fx);
+        if (w == 0.0f || static_cast<unsigned>(t) >= static_cast<unsigned>(pr.T) || static_cast<unsigned>(y) >= static_cast<unsigned>(pr.H) ||
+            static_cast<unsigned>(x) >= static_cast<unsigned>(pr.W)) continue;
+        const long long o = (((static_cast<long long>(t) * pr.H + y) * pr.W + x) * pr.heads + m) * D;
+        for (int ch = 0; ch < D; ++ch) {
+            atomicAdd(acc_dk + o + ch, w * ck * __bfloat162float(qr[ch]));
+            atomicAdd(acc_dv + o + ch, w * cv * __bfloat162float(dr[ch]));
+        }
+    }
+}
+
+// A warp works on one tensor and runs of four cells along x.  Cell by cell the products of 16 samples at a time
+// accumulate in registers, a corner on each of eight lane groups.  The groups of a cell's right corners are those of the next
+// cell's left corners (the two sides swap places from cell to cell), so a row of the accumulators is reduced
+// once per run of cells.  The query rows come by cp.async a group (or two) ahead, across cells and runs.
+template <int D>
+__global__ void __launch_bounds__(kSumThreads, 2)
+cells_sums_kernel(const bf16* __restrict__ q, const bf16* __restrict__ dout, float* __restrict__ acc_dk, float* __restrict__ acc_dv,
+                  const Problem pr, const Slab sl) {
+    using S = SumSmem<D>;
+    constexpr int PER = S::PER, RUNS = 4;           // the four warps of a tensor take the 16 runs in turn
+    constexpr int CPR = D / 8;                      // 16-byte chunks of a staged row
+    constexpr int LD = 16 * CPR / 32;               // chunks a lane fetches per 16 rows
+    constexpr int SWZ = CPR < 8 ? CPR - 1 : 7;
+    extern __shared__ __align__(16) unsigned char raw[];
+    S& s = *reinterpret_cast<S*>(raw);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g8 = lane >> 2, j = lane & 3;
+    const BlockPos b = block_pos(sl, blockIdx.x);
+    const uint32_t total = find_segments(sl, b, s.sg);
+    if (total == 0u) return;
+    const long long tok = static_cast<long long>(pr.heads) * D;
+    [[maybe_unused]] const long long kv_extent = pr.N * pr.heads * D;
+    const int tensor = warp & 1, run0 = warp >> 1;
+    const bf16* src = (tensor ? dout : q) + static_cast<long long>(b.m) * D + (lane % CPR) * 8;
+    float* acc = (tensor ? acc_dv : acc_dk) + static_cast<long long>(b.m) * D + 2 * j;
+    const float st = (g8 & 4) ? 1.0f : -1.0f, ot = (g8 & 4) ? 0.0f : 1.0f, sy = (g8 & 2) ? 1.0f : -1.0f, oy = (g8 & 2) ? 0.0f : 1.0f;
+    for (uint32_t b0 = 0; b0 < total; b0 += S::CAP) {
+        const int nb = static_cast<int>(min(static_cast<uint32_t>(S::CAP), total - b0));
+        if (tid < kCells) s.count[tid] = 0u;
+        __syncthreads();
+        uint4 u[PER];
+        float2 cf[PER];
+        uint32_t rank[PER];                         // cell | rank in the cell << 8
+#pragma unroll
+        for (int e = 0; e < PER; ++e) {
+            const int i = e * kSumThreads + tid;
+            rank[e] = 0xffffffffu;
+            if (i >= nb) continue;
+            const long long at = sample_of(s.sg, b0 + static_cast<uint32_t>(i), kRows * pr.P);
+            u[e] = __ldg(sl.geo + at);
+            rank[e] = __ldg(sl.meta + at);
+        }
+#pragma unroll
+        for (int e = 0; e < PER; ++e)
+            if (rank[e] != 0xffffffffu) cf[e] = __ldg(sl.coef + sample_at(sl, pr, b.m, static_cast<int>(u[e].x), static_cast<int>(rank[e] & 255u)));
+#pragma unroll
+        for (int e = 0; e < PER; ++e) {
+            if (rank[e] == 0xffffffffu) continue;
+            const uint32_t cell = rank[e] >> 8;
+            if (__float_as_uint(cf[e].y) >> 31) {
+                add_sample<D>(q, dout, acc_dk, acc_dv, pr, b.m, static_cast<int>(u[e].x), b.t + static_cast<int>(cell >> 4), b.y + static_cast<int>((cell >> 2) & 3u),
+                              b.x + static_cast<int>(cell & 3u), __uint_as_float(u[e].y), __uint_as_float(u[e].z), __uint_as_float(u[e].w), cf[e].x, fabsf(cf[e].y));
+                rank[e] = 0xffffffffu;
+            } else {
+                rank[e] = cell | (atomicAdd(&s.count[cell], 1u) << 8);
+            }
+        }
+        __syncthreads();
+        if (warp == 0) {
+            const uint32_t c0 = s.count[2 * lane], c1 = s.count[2 * lane + 1];
+            uint32_t inc = c0 + c1;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t up = __shfl_up_sync(kFullMask, inc, o);
+                if (lane >= o) inc += up;
+            }
+            s.first[2 * lane] = inc - c0 - c1; s.first[2 * lane + 1] = inc - c1;
+            if (lane == 31) s.first[kCells] = inc;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < PER; ++e)
+            if (rank[e] != 0xffffffffu) {
+                const uint32_t at = s.first[rank[e] & 63u] + (rank[e] >> 8);
+                s.geo[at] = make_float4(__uint_as_float(u[e].y), __uint_as_float(u[e].z), __uint_as_float(u[e].w), cf[e].x);
+                s.cv[at] = cf[e].y;
+                s.token[at] = u[e].x;
+            }
+        __syncthreads();
+        // The groups of the warp's cells in order: cell k of its runs, samples `ff` on.
+        constexpr int KC = 16 / RUNS * 4;
+        auto cell_at = [&](int k) { return 4 * (run0 + RUNS * (k >> 2)) + (k & 3); };
+        int fk = -1, ff = 0, fstop = 0, fslot = 0;
+        auto fetch_next = [&]() {
+            while (ff >= fstop && fk < KC - 1) {
+                ++fk;
+                ff = static_cast<int>(s.first[cell_at(fk)]);
+                fstop = static_cast<int>(s.first[cell_at(fk) + 1]);
+            }
+            if (ff < fstop) {
+                unsigned char* to = s.stage[warp][fslot];
+#pragma unroll
+                for (int i = 0; i < LD; ++i) {      // beyond the cell its last sample again (the weight is zero)
+                    const int r = i * (32 / CPR) + lane / CPR;
+                    const bf16* from = src + s.token[min(ff + r, fstop - 1)] * tok;
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(to + r * (D * 2) + (((lane % CPR) ^ (r & SWZ)) << 4)))), "l"(from) : "memory");
+                }
+                ff += 16;
+                fslot = fslot == S::STAGES - 1 ? 0 : fslot + 1;
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+#pragma unroll
+        for (int i = 0; i < S::STAGES - 1; ++i) fetch_next();
+        int slot = 0;
+        for (int rk = 0; rk < 16 / RUNS; ++rk) {
+            const int run = run0 + RUNS * rk;
+            if (s.first[4 * run] == s.first[4 * run + 4]) continue;
+            // the lane's corner row of dK / dV: (ct, cy) = (g8 >> 2, (g8 >> 1) & 1)
+            const int rt = b.t + (run >> 2) + (g8 >> 2), ry = b.y + (run & 3) + ((g8 >> 1) & 1);
+            const bool row_in = static_cast<unsigned>(rt) < static_cast<unsigned>(pr.T) && static_cast<unsigned>(ry) < static_cast<unsigned>(pr.H);
+            float* acc_row = acc + ((static_cast<long long>(rt) * pr.H + ry) * pr.W + b.x) * tok;
+            float c[D / 8][4];
+#pragma unroll
+            for (int i = 0; i < D / 8; ++i) c[i][0] = c[i][1] = c[i][2] = c[i][3] = 0.0f;
+            auto flush = [&](int xi) {                 // the left corners of cell xi are complete: heads and remainders together, out
+                if ((g8 ^ xi) & 1) return;
+                if (row_in && static_cast<unsigned>(b.x + xi) < static_cast<unsigned>(pr.W)) {
+                    float* to = acc_row + xi * tok;
+                    if (DSA3D_IN_RANGE(pr, to - (tensor ? acc_dv : acc_dk), kv_extent, 10))
+#pragma unroll
+                        for (int i = 0; i < D / 8; ++i) red_add_v2(to + 8 * i, c[i][0] + c[i][2], c[i][1] + c[i][3]);
+                }
+#pragma unroll
+                for (int i = 0; i < D / 8; ++i) c[i][0] = c[i][1] = c[i][2] = c[i][3] = 0.0f;
+            };
+            bool carry = false;                        // the sums hold something
+            for (int xi = 0; xi < 4; ++xi) {
+                int f = static_cast<int>(s.first[4 * run + xi]);
+                const int stop = static_cast<int>(s.first[4 * run + xi + 1]);
+                const bool any = f < stop;
+                const float sx = ((g8 ^ xi) & 1) ? 1.0f : -1.0f, ox = ((g8 ^ xi) & 1) ? 0.0f : 1.0f;
+                for (; f < stop; f += 16) {
+                    asm volatile("cp.async.wait_group %0;" ::"n"(S::STAGES - 2) : "memory");
+                    __syncwarp();
+                    const unsigned char* stage = s.stage[warp][slot];
+                    slot = slot == S::STAGES - 1 ? 0 : slot + 1;
+                    fetch_next();                      // into the slot that the group before this one was read from
+                    // weights of the lane's corner for samples 2j, 2j + 1, 2j + 8, 2j + 9: rows 0 - 7 of A the heads, rows 8 - 15
+                    // the remainders
+                    uint32_t a[4];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        float w2[2];
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            const int k = f + 2 * j + e + 8 * h, i = min(k, stop - 1);
+                            const float4 ge = s.geo[i];
+                            const float co = k < stop ? (tensor ? s.cv[i] : ge.w) : 0.0f;
+                            w2[e] = fmaf(ge.x, st, ot) * fmaf(ge.y, sy, oy) * fmaf(ge.z, sx, ox) * co;
+                        }
+                        const __nv_bfloat162 hd = __floats2bfloat162_rn(w2[0], w2[1]);
+                        const uint32_t hw = *reinterpret_cast<const uint32_t*>(&hd);
+                        const __nv_bfloat162 rs = __floats2bfloat162_rn(w2[0] - __uint_as_float(hw << 16), w2[1] - __uint_as_float(hw & 0xffff0000u));
+                        a[2 * h] = hw;
+                        a[2 * h + 1] = *reinterpret_cast<const uint32_t*>(&rs);
+                    }
+                    const int mr = lane & 15;
+#pragma unroll
+                    for (int i = 0; i < D / 16; ++i) {
+                        uint32_t b0r, b1r, b2r, b3r;
+                        const uint32_t addr = static_cast<uint32_t>(__cvta_generic_to_shared(stage + mr * (D * 2) + (((2 * i + (lane >> 4)) ^ (mr & SWZ)) << 4)));
+                        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(b0r), "=r"(b1r), "=r"(b2r), "=r"(b3r) : "r"(addr));
+                        mma_bf16(c[2 * i], a[0], a[1], a[2], a[3], b0r, b1r);
+                        mma_bf16(c[2 * i + 1], a[0], a[1], a[2], a[3], b2r, b3r);
+                    }
+                }
+                if (any || carry) flush(xi);
+                carry = any;
+            }
+            if (carry) flush(4);
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+    }
+}
+
+// ------------------------------------------------------------------------------------------------ beyond the bins
+// The samples in bin kBins of every tile, a warp per sample, row by row.  kScatter: their contributions to dK and dV; otherwise
+// what cells_dots_kernel leaves for the others.
+template <int D, bool kScatter>
+__global__ void __launch_bounds__(256)
+cells_far_kernel(const bf16* __restrict__ q, const bf16* __restrict__ k, const bf16* __restrict__ v, const bf16* __restrict__ dout,
+                 const float* __restrict__ offsets, float* __restrict__ acc_dk, float* __restrict__ acc_dv, const Problem pr, const Slab sl,
+                 int tiles) {
+    constexpr int V = D / 32;                       // channels per lane
+    const int lane = threadIdx.x & 31, warps = gridDim.x * 8;
+    const long long tok = static_cast<long long>(pr.heads) * D;
+    const int per_head = sl.tiles_t * sl.tiles_y * sl.tiles_x;
+    [[maybe_unused]] const long long kv_extent = pr.N * pr.heads * D;
+    for (int base = (static_cast<int>(blockIdx.x) * 8 + static_cast<int>(threadIdx.x >> 5)) * 32; base < tiles; base += warps * 32) {
+        uint32_t mine = 0u;
+        if (base + lane < tiles) mine = __ldg(sl.seg + static_cast<long long>(base + lane) * (kBins + 1) + kBins);
+        unsigned todo = __ballot_sync(kFullMask, (mine >> 16) != 0u);
+        while (todo) {
+            const int src = __ffs(static_cast<int>(todo)) - 1;
+            todo &= todo - 1u;
+            const uint32_t w = __shfl_sync(kFullMask, mine, src);
+            const long long tile = base + src;
+            const int m = sl.m0 + static_cast<int>(tile / per_head);
+            for (uint32_t i = 0; i < (w >> 16); ++i) {
+                const long long at = tile * (kRows * pr.P) + (w & 0xffffu) + i;
+                const int n = static_cast<int>(__ldg(sl.geo + at).x), p = static_cast<int>(__ldg(sl.meta + at) & 255u);
+                const int x = n % pr.W, y = (n / pr.W) % pr.H, t = n / (pr.W * pr.H);
+                const long long row = static_cast<long long>(n) * pr.heads + m;
+                const Sample smp = to_sample(pr, make_cell(pr, t, y, x, p, offsets + (row * pr.P + p) * 3));
+                const long long o0 = static_cast<long long>(m) * D + smp.base * tok + lane * V;
+                float qv[V], dv[V];
+#pragma unroll
+                for (int z = 0; z < V; ++z) {
+                    qv[z] = __bfloat162float(q[row * D + lane * V + z]);
+                    dv[z] = __bfloat162float(dout[row * D + lane * V + z]);
+                }
+                const float wt[2] = {1.0f - smp.ft, smp.ft}, wy[2] = {1.0f - smp.fy, smp.fy}, wx[2] = {1.0f - smp.fx, smp.fx};
+                const long long sy = static_cast<long long>(pr.W) * tok, st = static_cast<long long>(pr.H) * sy;
+                const long long sidx = sample_at(sl, pr, m, n, p);
+                if constexpr (kScatter) {
+                    const float2 cf = sl.coef[sidx];
+                    for (int j = 0; j < 8; ++j) {
+                        const float wj = wt[j >> 2] * wy[(j >> 1) & 1] * wx[j & 1];
+                        const long long o = o0 + (j >> 2) * st + ((j >> 1) & 1) * sy + (j & 1) * tok;
+                        if (!((smp.mask >> j) & 1u) || wj == 0.0f || !DSA3D_IN_RANGE(pr, o, kv_extent, 7)) continue;
+#pragma unroll
+                        for (int z = 0; z < V; ++z) {
+                            atomicAdd(acc_dk + o + z, wj * cf.x * qv[z]);
+                            atomicAdd(acc_dv + o + z, wj * fabsf(cf.y) * dv[z]);
+                        }
+                    }
+                } else {
+                    float a[8], bb[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const int ct = j >> 2, cy = (j >> 1) & 1, cx = j & 1;
+                        const bool needed = wt[ct] * wy[cy] * wx[cx] != 0.0f || wy[cy] * wx[cx] != 0.0f || wt[ct] * wx[cx] != 0.0f || wt[ct] * wy[cy] != 0.0f;
+                        const long long o = o0 + ct * st + cy * sy + cx * tok;
+                        a[j] = bb[j] = 0.0f;
+                        if (!((smp.mask >> j) & 1u) || !needed || !DSA3D_IN_RANGE(pr, o, kv_extent, 5)) continue;
+#pragma unroll
+                        for (int z = 0; z < V; ++z) {
+                            a[j] = fmaf(qv[z], __bfloat162float(k[o + z]), a[j]);
+                            bb[j] = fmaf(dv[z], __bfloat162float(v[o + z]), bb[j]);
+                        }
+                    }
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        a[j] = group_sum<32>(a[j], kFullMask);
+                        bb[j] = group_sum<32>(bb[j], kFullMask);
+                    }
+                    float r[8];
+                    trilerp_grad(a, smp.ft, smp.fy, smp.fx, r[0], r[1], r[2], r[3]);
+                    trilerp_grad(bb, smp.ft, smp.fy, smp.fx, r[4], r[5], r[6], r[7]);
+                    if (lane == 0) {
+#pragma unroll
+                        for (int z = 0; z < 8; ++z) sl.stats[sidx * 8 + z] = r[z];
+                    }
+                }
+            }
+        }
+    }
+}
+
+// ------------------------------------------------------------------------------------------------ host
+int floor_div4(int a) { return a >= 0 ? a / 4 : -((-a + 3) / 4); }
+
+size_t round256(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
+
+// Lays a slab's buffers out at `base` (may be NULL); returns their bytes.
+size_t lay_out(const Problem& pr, int m0, int heads, int f0, int f1, char* base, Slab& s) {
+    s.m0 = m0; s.heads = heads; s.f0 = f0; s.f1 = f1;
+    s.tiles_t = (f1 - f0 + 3) / 4; s.tiles_y = (pr.H + 3) / 4; s.tiles_x = (pr.W + 7) / 8;
+    const int lo = floor_div4(-1 - f0), hi = floor_div4(pr.T - 1 - f0);
+    s.bt0 = lo < -3 ? -3 : lo;
+    const int top = s.tiles_t - 1 + 3 < hi ? s.tiles_t - 1 + 3 : hi;
+    s.blocks_t = top - s.bt0 + 1;
+    s.blocks_y = (pr.H - 1) / 4 + 2;
+    s.blocks_x = (pr.W - 1) / 4 + 2;
+    const size_t tiles = static_cast<size_t>(heads) * s.tiles_t * s.tiles_y * s.tiles_x, samples = tiles * kRows * pr.P;
+    const size_t live = static_cast<size_t>(heads) * (f1 - f0) * pr.H * pr.W * pr.P;
+    size_t at = 0;
+    s.geo = reinterpret_cast<uint4*>(base + at); at += round256(samples * sizeof(uint4));
+    s.meta = reinterpret_cast<uint16_t*>(base + at); at += round256(samples * sizeof(uint16_t));
+    s.seg = reinterpret_cast<uint32_t*>(base + at); at += round256(tiles * (kBins + 1) * sizeof(uint32_t));
+    s.stats = reinterpret_cast<float*>(base + at); at += round256(live * 8 * sizeof(float));
+    s.coef = reinterpret_cast<float2*>(base + at); at += round256(live * sizeof(float2));
+    return at;
+}
+
+template <int D>
+cudaError_t launch_slab(const void* q_, const void* k_, const void* v_, const float* offsets, const float* lse, const void* dout_, void* dq_,
+                        float* acc_dk, float* acc_dv, float* doffsets, const Problem& pr, const Slab& s, cudaStream_t stream) {
+    const bf16 *q = static_cast<const bf16*>(q_), *k = static_cast<const bf16*>(k_), *v = static_cast<const bf16*>(v_), *dout = static_cast<const bf16*>(dout_);
+    const int tiles = s.heads * s.tiles_t * s.tiles_y * s.tiles_x, blocks = s.heads * s.blocks_t * s.blocks_y * s.blocks_x;
+    const unsigned inv_p = ((1u << 24) + static_cast<unsigned>(pr.P) - 1u) / static_cast<unsigned>(pr.P);
+    const size_t bin_smem = static_cast<size_t>((kBins + 1) * kCopies + kRows * pr.P) * sizeof(uint32_t);
+    cudaError_t e = cudaFuncSetAttribute(cells_bin_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bin_smem));
+    if (e != cudaSuccess) return e;
+    cells_bin_kernel<<<static_cast<unsigned>(tiles), kBinThreads, bin_smem, stream>>>(offsets, pr, s, inv_p);
+    const size_t dot_smem = sizeof(DotSmem<D>), sum_smem = sizeof(SumSmem<D>);
+    e = cudaFuncSetAttribute(cells_dots_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(dot_smem));
+    if (e != cudaSuccess) return e;
+    cells_dots_kernel<D><<<static_cast<unsigned>(blocks), kDotThreads, dot_smem, stream>>>(q, k, v, dout, pr, s);
+    const unsigned far_grid = static_cast<unsigned>(tiles / 256 + 1 < 148 * 8 ? tiles / 256 + 1 : 148 * 8);
+    cells_far_kernel<D, false><<<far_grid, 256, 0, stream>>>(q, k, v, dout, offsets, acc_dk, acc_dv, pr, s, tiles);
+    const long long items = static_cast<long long>(s.heads) * (s.f1 - s.f0) * pr.H * pr.W;
+    constexpr int per_block = kQueryThreads / (D / 8);
+    cells_query_kernel<D><<<static_cast<unsigned>((items + per_block - 1) / per_block), kQueryThreads, 0, stream>>>(k, offsets, lse, static_cast<bf16*>(dq_), doffsets, pr, s);
+    e = cudaFuncSetAttribute(cells_sums_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sum_smem));
+    if (e != cudaSuccess) return e;
+    cells_sums_kernel<D><<<static_cast<unsigned>(blocks), kSumThreads, sum_smem, stream>>>(q, dout, acc_dk, acc_dv, pr, s);
+    cells_far_kernel<D, true><<<far_grid, 256, 0, stream>>>(q, k, v, dout, offsets, acc_dk, acc_dv, pr, s, tiles);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+// Splits the queries of `pr` (whole frames) into passes whose buffers fit `bytes`: by heads first (they share nothing),
+// then by frames.
+bool try_cells_backward(const void* q, const void* k, const void* v, const float* offsets, const float* lse, const void* dout, void* dq,
+                        float* acc_dk, float* acc_dv, float* doffsets, void* scratch, size_t bytes, const Problem& pr, cudaStream_t stream,
+                        cudaError_t* err) {
+    *err = cudaSuccess;
+    const long long frame = static_cast<long long>(pr.H) * pr.W;
+    const int f_begin = static_cast<int>(pr.q_begin / frame), f_end = f_begin + static_cast<int>(pr.q_count / frame);
+    int heads = pr.heads, frames = f_end - f_begin;
+    Slab s;
+    while (lay_out(pr, 0, heads, f_begin, f_begin + frames, nullptr, s) > bytes) {
+        if (heads > 1) heads = (heads + 1) / 2;
+        else if (frames > 4) frames = ((frames + 1) / 2 + 3) / 4 * 4;
+        else return false;
+    }
+    for (int f = f_begin; f < f_end; f += frames)
+        for (int m = 0; m < pr.heads; m += heads) {
+            const int f1 = f + frames < f_end ? f + frames : f_end, mh = m + heads < pr.heads ? heads : pr.heads - m;
+            lay_out(pr, m, mh, f, f1, static_cast<char*>(scratch), s);
+            *err = pr.d == 128 ? launch_slab<128>(q, k, v, offsets, lse, dout, dq, acc_dk, acc_dv, doffsets, pr, s, stream)
+                 : pr.d == 64  ? launch_slab<64>(q, k, v, offsets, lse, dout, dq, acc_dk, acc_dv, doffsets, pr, s, stream)
+                               : launch_slab<32>(q, k, v, offsets, lse, dout, dq, acc_dk, acc_dv, doffsets, pr, s, stream);
+            if (*err != cudaSuccess) return true;
+        }
+    return true;
+}
+
+}  // namespace dsa3d

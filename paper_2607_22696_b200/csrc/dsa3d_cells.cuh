@@ -1,0 +1,57 @@
+// Cell-sorted sampling (bf16 storage): pieces shared by the kernels of dsa3d_cells.cu.
+//
+// A sample reads (and its gradient writes) the eight corner rows of the grid cell it falls into.  All samples of a cell,
+// whichever query they belong to, share those eight rows.  So the samples are first sorted by key cell: then the dot
+// products of 16 samples with their eight corners are one m16n8k16 product chain (16 query rows x 8 key rows), the
+// dK / dV contributions of 16 samples another (8 corners, head and remainder of the weights, x 16 query rows), and the
+// row traffic per sample falls from eight key rows to one query row.  Nothing depends on how far the offsets reach.
+// (The groups are 16 samples of one cell, so the warp-level product is the one that fits: a tcgen05 tile would hold
+// 128 rows of which a cell fills 27.)
+//
+// Queries come in tiles of 4 x 4 x 8 (t, y, x) of one head, cells in blocks of 4 x 4 x 4 whose rows are a box of
+// 5 x 5 x 5 positions.  cells_bin_kernel sorts the samples of a tile by the block they fall into, relative to
+// the tile (bins); a block then finds its samples as one segment per (tile, bin).
+#pragma once
+#include "dsa3d_common.cuh"
+
+namespace dsa3d {
+namespace cells {
+
+constexpr int kRows = 128;                        // queries per tile: 4 x 4 x 8
+constexpr int kReach = 12;                        // bins reach this far below and above the tile on every axis
+constexpr int kBinsT = 7, kBinsY = 7, kBinsX = 8; // blocks of the bin grid
+constexpr int kBins = kBinsT * kBinsY * kBinsX;   // 392; bin 392 takes the samples beyond them
+constexpr int kSegs = kBinsT * kBinsY * (kBinsX / 2);   // tiles whose bins can hold a given block: 196
+constexpr int kBox = 125;                         // rows of a box
+constexpr int kCells = 64;                        // cells of a block
+
+// The part of a problem one pass takes: heads [m0, m0 + heads), frames [f0, f1) of queries.  Tiles are numbered
+// ((head * tiles_t + tt) * tiles_y + ty) * tiles_x + tx, tile tt starts at frame f0 + 4 tt.
+struct Slab {
+    int m0, heads, f0, f1;
+    int tiles_t, tiles_y, tiles_x;
+    int blocks_t, blocks_y, blocks_x;             // blocks that samples of these queries can fall into: block b starts at cell
+    int bt0;                                      // f0 + 4 (b + bt0) along t and 4 (b - 1) along y and x
+    uint4* geo;                                   // [tile][128 * P]: {token, ft, fy, fx}
+    uint16_t* meta;                               // [tile][128 * P]: sample | cell in its block << 8
+    uint32_t* seg;                                // [tile][kBins + 1]: start | count << 16
+    float* stats;                                 // [head][frame of the slab][y][x][P][8]
+    float2* coef;                                 // [head][...][P]: scale dS, alpha (sign bit: not for the products, see cells_query_kernel)
+};
+
+// Place of sample p of token n in stats / coef (in samples).
+__device__ __forceinline__ long long sample_at(const Slab& s, const Problem& pr, int m, int n, int p) {
+    const long long frame = static_cast<long long>(pr.H) * pr.W;
+    return ((m - s.m0) * (frame * (s.f1 - s.f0)) + (n - frame * s.f0)) * pr.P + p;
+}
+
+__device__ __forceinline__ int box_row(int cell) { return (cell >> 4) * 25 + ((cell >> 2) & 3) * 5 + (cell & 3); }
+__device__ __forceinline__ int box_step(int corner) { return (corner >> 2) * 25 + ((corner >> 1) & 1) * 5 + (corner & 1); }
+
+__device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+}  // namespace cells
+}  // namespace dsa3d

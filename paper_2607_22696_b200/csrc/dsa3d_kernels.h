@@ -33,6 +33,13 @@ cudaError_t launch_scatter_tiles(const void* q, const void* dout, const float* o
                                  float* acc_dk, float* acc_dv, void* scratch, int ctas,
                                  long long entries_per_cta, const Problem& pr, cudaStream_t stream);
 
+// The whole backward of the bf16 queries of `pr` (whole frames) on samples sorted by key cell (dsa3d_cells.cu): dq, doffsets, and
+// the contributions to the fp32 accumulators.  `scratch`: `bytes` of device memory, worked through in as many passes as
+// it takes; false: not even the smallest pass fits, nothing launched.
+bool try_cells_backward(const void* q, const void* k, const void* v, const float* offsets, const float* lse, const void* dout, void* dq,
+                        float* acc_dk, float* acc_dv, float* doffsets, void* scratch, size_t bytes, const Problem& pr, cudaStream_t stream,
+                        cudaError_t* err);
+
 // Dynamic shared memory of the tile kernel for this problem's tiling.
 size_t tile_smem_bytes(const Problem& pr);
 
