@@ -25,29 +25,30 @@ __global__ void __launch_bounds__(kBinThreads, 2)
 cells_bin_kernel(const float* __restrict__ offsets, const Problem pr, const Slab sl, unsigned inv_p) {
     extern __shared__ __align__(16) unsigned char raw[];
     uint32_t* counters = reinterpret_cast<uint32_t*>(raw);                 // [kBins + 1][kCopies]: lanes of a warp mostly hit the same bin
-    uint32_t* words = counters + (kBins + 1) * kCopies;                     // [128 * P]: bin (9 bits), cell (6), rank in its counter (16)
+    uint32_t* words = counters + (kBins + 1) * kCopies;                     // [kRows * P]: bin (9 bits), cell (6), rank in its counter (16)
     __shared__ uint32_t scan[kBinWarps];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const long long tile = blockIdx.x;
     int r = static_cast<int>(tile % (sl.tiles_t * sl.tiles_y * sl.tiles_x));
     const int m = sl.m0 + static_cast<int>(tile / (sl.tiles_t * sl.tiles_y * sl.tiles_x));
-    const int x0 = (r % sl.tiles_x) * 8; r /= sl.tiles_x;
+    const int x0 = (r % sl.tiles_x) * kTileX; r /= sl.tiles_x;
     const int y0 = (r % sl.tiles_y) * 4, t0 = sl.f0 + (r / sl.tiles_y) * 4;
     const int samples = kRows * pr.P;
+    if (blockIdx.x == 0 && tid == 0) *sl.marked = 0;
     for (int i = tid; i < (kBins + 1) * kCopies / 4; i += kBinThreads) reinterpret_cast<uint4*>(counters)[i] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
     auto row_of = [&](int s) { return static_cast<int>((static_cast<unsigned long long>(static_cast<unsigned>(s)) * inv_p) >> 24); };
     auto cell_of = [&](int s, int& n) -> Cell {
         const int row = row_of(s), p = s - row * pr.P;
-        const int t = t0 + (row >> 5), y = y0 + ((row >> 3) & 3), x = x0 + (row & 7);
+        const int ty = row / kTileX, t = t0 + (ty >> 2), y = y0 + (ty & 3), x = x0 + row - ty * kTileX;
         n = (t * pr.H + y) * pr.W + x;
         if (t >= sl.f1 || y >= pr.H || x >= pr.W) { Cell c; c.it = c.iy = c.ix = 0; c.mask = 0u; c.ft = c.fy = c.fx = 0.0f; return c; }
         return make_cell(pr, t, y, x, p, offsets + ((static_cast<long long>(n) * pr.heads + m) * pr.P + p) * 3);
     };
-    for (int base = 0; base < samples; base += 4 * kBinThreads) {
-        uint32_t w[4];
+    for (int base = 0; base < samples; base += 3 * kBinThreads) {
+        uint32_t w[3];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {                  // four samples per thread at a time: their offsets load together
+        for (int i = 0; i < 3; ++i) {                  // three samples per thread at a time: their offsets load together
             const int s = base + i * kBinThreads + tid;
             w[i] = 0xffffffffu;
             if (s >= samples) continue;
@@ -56,14 +57,15 @@ cells_bin_kernel(const float* __restrict__ offsets, const Problem pr, const Slab
             if (c.mask == 0u) continue;
             const int rt = c.it - t0 + kReach, ry = c.iy - y0 + kReach, rx = c.ix - x0 + kReach;
             uint32_t bin = kBins, cell = 0u;
-            if (static_cast<unsigned>(rt) < 4u * kBinsT && static_cast<unsigned>(ry) < 4u * kBinsY && static_cast<unsigned>(rx) < 4u * kBinsX) {
-                bin = static_cast<uint32_t>(((rt >> 2) * kBinsY + (ry >> 2)) * kBinsX + (rx >> 2));
-                cell = static_cast<uint32_t>(((rt & 3) << 4) | ((ry & 3) << 2) | (rx & 3));
+            if (static_cast<unsigned>(rt) < 4u * kBinsT && static_cast<unsigned>(ry) < 4u * kBinsY && static_cast<unsigned>(rx) < 3u * kBinsX) {
+                const int bx = rx / kBlockX;
+                bin = static_cast<uint32_t>(((rt >> 2) * kBinsY + (ry >> 2)) * kBinsX + bx);
+                cell = static_cast<uint32_t>(((rt & 3) * 4 + (ry & 3)) * kBlockX + rx - bx * kBlockX);
             }
             w[i] = bin | (cell << 9);
         }
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < 3; ++i) {
             const int s = base + i * kBinThreads + tid;
             if (s >= samples) continue;
             if (w[i] != 0xffffffffu) w[i] |= atomicAdd(&counters[(w[i] & 511u) * kCopies + (lane & (kCopies - 1))], 1u) << 15;
@@ -118,14 +120,17 @@ cells_bin_kernel(const float* __restrict__ offsets, const Problem pr, const Slab
 }
 
 // ------------------------------------------------------------------------------------------------ a block's samples
-struct BlockPos { int m, t, y, x; };               // head, first cell along t, y, x
+struct BlockPos { int m, t, y, x, bt, by, bx; };   // head, first cell along t, y, x; block numbers (bt from the slab's first frame)
 
 __device__ __forceinline__ BlockPos block_pos(const Slab& sl, long long id) {
     BlockPos b;
-    b.x = (static_cast<int>(id % sl.blocks_x) - 1) * 4; id /= sl.blocks_x;
-    b.y = (static_cast<int>(id % sl.blocks_y) - 1) * 4; id /= sl.blocks_y;
-    b.t = sl.f0 + (static_cast<int>(id % sl.blocks_t) + sl.bt0) * 4;
+    b.bx = static_cast<int>(id % sl.blocks_x) - 1; id /= sl.blocks_x;
+    b.by = static_cast<int>(id % sl.blocks_y) - 1; id /= sl.blocks_y;
+    b.bt = static_cast<int>(id % sl.blocks_t) + sl.bt0;
     b.m = sl.m0 + static_cast<int>(id / sl.blocks_t);
+    b.t = sl.f0 + 4 * b.bt;
+    b.y = 4 * b.by;
+    b.x = kBlockX * b.bx;
     return b;
 }
 
@@ -136,18 +141,17 @@ struct Segments {
     uint32_t scan[8];
 };
 
-// Finds the segments of a block (at least 224 threads, all of the CTA); returns how many samples they hold.
+// Finds the segments of a block (at least 256 threads, all of the CTA); returns how many samples they hold.
 __device__ __forceinline__ uint32_t find_segments(const Slab& sl, const BlockPos& b, Segments& sg) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint32_t count = 0u, start = 0u;
     int tile = 0;
     if (tid < kSegs) {
-        const int bt = tid / (kBinsY * (kBinsX / 2)), by = (tid / (kBinsX / 2)) % kBinsY;
-        const int Bt = (b.t - sl.f0) >> 2, By = b.y >> 2, Bx = b.x >> 2;            // arithmetic: -4 >> 2 = -1
-        const int bx = ((Bx + 3) & 1) + 2 * (tid % (kBinsX / 2));
-        const int tt = Bt + 3 - bt, ty = By + 3 - by, tx = (Bx + 3 - bx) / 2;
+        const int bt = tid / (kBinsY * kSegsX), by = (tid / kSegsX) % kBinsY;
+        const int bx = (b.bx & 1) + 2 * (tid % kSegsX);             // kReach is an even number of blocks: same parity as b.bx
+        const int tt = b.bt + kReach / 4 - bt, ty = b.by + kReach / 4 - by, dx = b.bx + kReach / kBlockX - bx, tx = dx / 2;
         if (static_cast<unsigned>(tt) < static_cast<unsigned>(sl.tiles_t) && static_cast<unsigned>(ty) < static_cast<unsigned>(sl.tiles_y) &&
-            Bx + 3 - bx >= 0 && tx < sl.tiles_x) {
+            dx >= 0 && tx < sl.tiles_x) {
             tile = (((b.m - sl.m0) * sl.tiles_t + tt) * sl.tiles_y + ty) * sl.tiles_x + tx;
             const uint32_t w = __ldg(sl.seg + static_cast<long long>(tile) * (kBins + 1) + (bt * kBinsY + by) * kBinsX + bx);
             start = w & 0xffffu;
@@ -160,11 +164,11 @@ __device__ __forceinline__ uint32_t find_segments(const Slab& sl, const BlockPos
         const uint32_t up = __shfl_up_sync(kFullMask, incl, o);
         if (lane >= o) incl += up;
     }
-    if (warp < 7 && lane == 31) sg.scan[warp] = incl;
+    if (warp < 8 && lane == 31) sg.scan[warp] = incl;
     __syncthreads();
     uint32_t before = 0u, total = 0u;
 #pragma unroll
-    for (int i = 0; i < 7; ++i) {
+    for (int i = 0; i < 8; ++i) {
         const uint32_t v = sg.scan[i];
         if (i < warp) before += v;
         total += v;
@@ -202,7 +206,7 @@ __device__ __forceinline__ void load_box(unsigned char* dst, const bf16* __restr
     constexpr int CH = D / 8;
     for (int i = threadIdx.x; i < kBox * CH; i += NT) {
         const int row = i / CH, chunk = i - row * CH;
-        const int t = b.t + row / 25, y = b.y + (row / 5) % 5, x = b.x + row % 5;
+        const int t = b.t + row / 20, y = b.y + (row / 4) % 5, x = b.x + row % 4;
         uint4 v = make_uint4(0u, 0u, 0u, 0u);
         if (static_cast<unsigned>(t) < static_cast<unsigned>(pr.T) && static_cast<unsigned>(y) < static_cast<unsigned>(pr.H) && static_cast<unsigned>(x) < static_cast<unsigned>(pr.W))
             v = __ldg(reinterpret_cast<const uint4*>(src + (((static_cast<long long>(t) * pr.H + y) * pr.W + x) * pr.heads + b.m) * D) + chunk);
@@ -211,7 +215,7 @@ __device__ __forceinline__ void load_box(unsigned char* dst, const bf16* __restr
 }
 
 // ------------------------------------------------------------------------------------------------ dot products
-constexpr int kDotThreads = 512, kDotCap = 2048;
+constexpr int kDotThreads = 512, kDotCap = 1536;
 
 template <int D> struct DotSmem {
     unsigned char box[2][kBox * D * 2];
@@ -280,7 +284,7 @@ cells_dots_kernel(const bf16* __restrict__ q, const bf16* __restrict__ k, const 
         }
         __syncthreads();
         if (warp == 0) {                            // exclusive sums over the cells: samples and groups of 16
-            const uint32_t c0 = s.count[2 * lane], c1 = s.count[2 * lane + 1];
+            const uint32_t c0 = lane < kCells / 2 ? s.count[2 * lane] : 0u, c1 = lane < kCells / 2 ? s.count[2 * lane + 1] : 0u;
             const uint32_t n0 = (c0 + 15u) >> 4, n1 = (c1 + 15u) >> 4;
             uint32_t inc = c0 + c1, ginc = n0 + n1;
 #pragma unroll
@@ -288,8 +292,10 @@ cells_dots_kernel(const bf16* __restrict__ q, const bf16* __restrict__ k, const 
                 const uint32_t up = __shfl_up_sync(kFullMask, inc, o), gup = __shfl_up_sync(kFullMask, ginc, o);
                 if (lane >= o) { inc += up; ginc += gup; }
             }
-            s.first[2 * lane] = inc - c0 - c1; s.first[2 * lane + 1] = inc - c1;
-            s.gfirst[2 * lane] = ginc - n0 - n1; s.gfirst[2 * lane + 1] = ginc - n1;
+            if (lane < kCells / 2) {
+                s.first[2 * lane] = inc - c0 - c1; s.first[2 * lane + 1] = inc - c1;
+                s.gfirst[2 * lane] = ginc - n0 - n1; s.gfirst[2 * lane + 1] = ginc - n1;
+            }
             if (lane == 31) { s.first[kCells] = inc; s.gfirst[kCells] = ginc; }
         }
         __syncthreads();
@@ -398,6 +404,7 @@ cells_query_kernel(const bf16* __restrict__ k, const float* __restrict__ offsets
                 d1 = fmaf(my_ck, a.z, alpha * b.z);
                 d2 = fmaf(my_ck, a.w, alpha * b.w);
                 const bool odd = !(fabsf(a.x) < INFINITY) || !(fabsf(b.x) < INFINITY) || !(fabsf(my_ck) < INFINITY) || !(alpha < INFINITY);
+                if (odd) *sl.marked = 1;
                 if (active) sl.coef[item * pr.P + p] = make_float2(my_ck, __uint_as_float(__float_as_uint(alpha) | (odd ? 0x80000000u : 0u)));
             }
             if (active) {
@@ -438,12 +445,11 @@ cells_query_kernel(const bf16* __restrict__ k, const float* __restrict__ offsets
 constexpr int kSumThreads = 256;
 
 template <int D> struct SumSmem {
-    static constexpr int CAP = 1792, PER = CAP / kSumThreads;     // samples at a time: two CTAs per SM fit
-    static constexpr int STAGES = D == 128 ? 2 : 3;
-    float4 geo[CAP];                                // ft, fy, fx, ck; sorted by cell, as everything below
-    unsigned char stage[kSumThreads / 32][STAGES][16 * D * 2];    // a warp's ring of 16 query rows
-    float cv[CAP];
-    uint32_t token[CAP];
+    static constexpr int CAP = 1536, PER = CAP / kSumThreads;     // samples at a time: two CTAs per SM fit
+    static constexpr int STAGES = D == 128 ? 2 : 3, GROUP = 16 * D * 2;
+    unsigned char stage[kSumThreads / 32][STAGES][GROUP];         // a warp's ring of 16 query rows
+    float4 geo[CAP];                                // ft, fy, fx, token (bits); sorted by cell, as ck and cv
+    float ck[CAP + 1], cv[CAP + 1];                 // the last one is zero: what a group beyond its run's samples takes
     uint32_t count[kCells], first[kCells + 1];
     Segments sg;
 };
@@ -452,49 +458,41 @@ __device__ __forceinline__ void red_add_v2(float* addr, float a, float b) {
     asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(addr), "f"(a), "f"(b) : "memory");
 }
 
-// Contributions of one sample to dK and dV, corner by corner (those with a weight), by one thread.
-template <int D>
-__device__ __noinline__ void add_sample(const bf16* q, const bf16* dout, float* acc_dk, float* acc_dv, const Problem& pr, int m, int n, int t0, int y0,
-                                        int x0, float ft, float fy, float fx, float ck, float cv) {
-    const bf16 *qr = q + (static_cast<long long>(n) * pr.heads + m) * D, *dr = dout + (static_cast<long long>(n) * pr.heads + m) * D;
-    for (int c = 0; c < 8; ++c) {
-        const int t = t0 + (c >> 2), y = y0 + ((c >> 1) & 1), x = x0 + (c & 1);
-        const float w = ((c & 4) ? ft : 1.0f - ft) * ((c & 2) ? fy : 1.0f - fy) * ((c & 1) ? fx : 1.0f - fx);
-        if (w == 0.0f || static_cast<unsigned>(t) >= static_cast<unsigned>(pr.T) || static_cast<unsigned>(y) >= static_cast<unsigned>(pr.H) ||
-            static_cast<unsigned>(x) >= static_cast<unsigned>(pr.W)) continue;
-        const long long o = (((static_cast<long long>(t) * pr.H + y) * pr.W + x) * pr.heads + m) * D;
-        for (int ch = 0; ch < D; ++ch) {
-            atomicAdd(acc_dk + o + ch, w * ck * __bfloat162float(qr[ch]));
-            atomicAdd(acc_dv + o + ch, w * cv * __bfloat162float(dr[ch]));
-        }
-    }
-}
-
-// A warp works on one tensor and runs of four cells along x.  Cell by cell the products of 16 samples at a time
-// accumulate in registers, a corner on each of eight lane groups.  The groups of a cell's right corners are those of the next
-// cell's left corners (the two sides swap places from cell to cell), so a row of the accumulators is reduced
-// once per run of cells.  The query rows come by cp.async a group (or two) ahead, across cells and runs.
+// A warp works on one tensor and runs of three cells along x: the corners of a run are 4 columns x 4 (t, y) rows of the
+// accumulators, the 16 rows of the product tile, and 16 of the run's samples at a time are its depth.  A lane forms
+// the weights of its (t, y) in columns g8 / 4 and g8 / 4 + 2: a sample has a weight in exactly one of the two, which goes in
+// as bf16 head and remainder, two products into the same sums.  The query rows come by cp.async a group (or two)
+// ahead, across runs.
 template <int D>
 __global__ void __launch_bounds__(kSumThreads, 2)
 cells_sums_kernel(const bf16* __restrict__ q, const bf16* __restrict__ dout, float* __restrict__ acc_dk, float* __restrict__ acc_dv,
                   const Problem pr, const Slab sl) {
     using S = SumSmem<D>;
-    constexpr int PER = S::PER, RUNS = 4;           // the four warps of a tensor take the 16 runs in turn
-    constexpr int CPR = D / 8;                      // 16-byte chunks of a staged row
-    constexpr int LD = 16 * CPR / 32;               // chunks a lane fetches per 16 rows
+    constexpr int PER = S::PER, STRIDE = 4;         // the four warps of a tensor take the runs in turn
+    constexpr int CPR = D / 8;                      // 16-byte chunks of a staged row, permuted by the row (SWZ)
+    constexpr int LD = 16 * CPR / 32, RPI = 32 / CPR;      // fetches per lane for 16 rows; rows per fetch of the warp
     constexpr int SWZ = CPR < 8 ? CPR - 1 : 7;
     extern __shared__ __align__(16) unsigned char raw[];
-    S& s = *reinterpret_cast<S*>(raw);
+    S& s = *reinterpret_cast<S*>((reinterpret_cast<uintptr_t>(raw) + 255) & ~uintptr_t(255));
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g8 = lane >> 2, j = lane & 3;
     const BlockPos b = block_pos(sl, blockIdx.x);
     const uint32_t total = find_segments(sl, b, s.sg);
     if (total == 0u) return;
     const long long tok = static_cast<long long>(pr.heads) * D;
+    const uint32_t tok_bytes = static_cast<uint32_t>(tok) * 2u;
     [[maybe_unused]] const long long kv_extent = pr.N * pr.heads * D;
     const int tensor = warp & 1, run0 = warp >> 1;
-    const bf16* src = (tensor ? dout : q) + static_cast<long long>(b.m) * D + (lane % CPR) * 8;
+    const char* src = reinterpret_cast<const char*>((tensor ? dout : q) + static_cast<long long>(b.m) * D + (lane % CPR) * 8);
     float* acc = (tensor ? acc_dv : acc_dk) + static_cast<long long>(b.m) * D + 2 * j;
-    const float st = (g8 & 4) ? 1.0f : -1.0f, ot = (g8 & 4) ? 0.0f : 1.0f, sy = (g8 & 2) ? 1.0f : -1.0f, oy = (g8 & 2) ? 0.0f : 1.0f;
+    const float* co = tensor ? s.cv : s.ck;
+    const float st = (g8 & 2) ? 1.0f : -1.0f, ot = (g8 & 2) ? 0.0f : 1.0f, sy = (g8 & 1) ? 1.0f : -1.0f, oy = (g8 & 1) ? 0.0f : 1.0f;
+    const int col = g8 >> 2;
+    const uint32_t stage0 = static_cast<uint32_t>(__cvta_generic_to_shared(s.stage[warp][0]));
+    // where the lane's chunk of row i * RPI + lane / CPR goes, and where its row pointer of an ldmatrix points: the
+    // chunk's permutation is an exclusive or within 256 aligned bytes
+    const uint32_t put = static_cast<uint32_t>((lane / CPR) * (D * 2) + (((lane % CPR) ^ ((lane / CPR) & SWZ)) << 4));
+    const uint32_t get = static_cast<uint32_t>((lane & 15) * (D * 2) + (((lane >> 4) ^ (lane & SWZ)) << 4));
+    if (tid == 0) { s.ck[S::CAP] = s.cv[S::CAP] = 0.0f; }
     for (uint32_t b0 = 0; b0 < total; b0 += S::CAP) {
         const int nb = static_cast<int>(min(static_cast<uint32_t>(S::CAP), total - b0));
         if (tid < kCells) s.count[tid] = 0u;
@@ -517,25 +515,19 @@ cells_sums_kernel(const bf16* __restrict__ q, const bf16* __restrict__ dout, flo
 #pragma unroll
         for (int e = 0; e < PER; ++e) {
             if (rank[e] == 0xffffffffu) continue;
-            const uint32_t cell = rank[e] >> 8;
-            if (__float_as_uint(cf[e].y) >> 31) {
-                add_sample<D>(q, dout, acc_dk, acc_dv, pr, b.m, static_cast<int>(u[e].x), b.t + static_cast<int>(cell >> 4), b.y + static_cast<int>((cell >> 2) & 3u),
-                              b.x + static_cast<int>(cell & 3u), __uint_as_float(u[e].y), __uint_as_float(u[e].z), __uint_as_float(u[e].w), cf[e].x, fabsf(cf[e].y));
-                rank[e] = 0xffffffffu;
-            } else {
-                rank[e] = cell | (atomicAdd(&s.count[cell], 1u) << 8);
-            }
+            if (__float_as_uint(cf[e].y) >> 31) rank[e] = 0xffffffffu;       // marked: cells_far_kernel takes it
+            else rank[e] = (rank[e] >> 8) | (atomicAdd(&s.count[rank[e] >> 8], 1u) << 8);
         }
         __syncthreads();
         if (warp == 0) {
-            const uint32_t c0 = s.count[2 * lane], c1 = s.count[2 * lane + 1];
+            const uint32_t c0 = lane < kCells / 2 ? s.count[2 * lane] : 0u, c1 = lane < kCells / 2 ? s.count[2 * lane + 1] : 0u;
             uint32_t inc = c0 + c1;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const uint32_t up = __shfl_up_sync(kFullMask, inc, o);
                 if (lane >= o) inc += up;
             }
-            s.first[2 * lane] = inc - c0 - c1; s.first[2 * lane + 1] = inc - c1;
+            if (lane < kCells / 2) { s.first[2 * lane] = inc - c0 - c1; s.first[2 * lane + 1] = inc - c1; }
             if (lane == 31) s.first[kCells] = inc;
         }
         __syncthreads();
@@ -543,103 +535,96 @@ cells_sums_kernel(const bf16* __restrict__ q, const bf16* __restrict__ dout, flo
         for (int e = 0; e < PER; ++e)
             if (rank[e] != 0xffffffffu) {
                 const uint32_t at = s.first[rank[e] & 63u] + (rank[e] >> 8);
-                s.geo[at] = make_float4(__uint_as_float(u[e].y), __uint_as_float(u[e].z), __uint_as_float(u[e].w), cf[e].x);
+                s.geo[at] = make_float4(__uint_as_float(u[e].y), __uint_as_float(u[e].z), __uint_as_float(u[e].w), __uint_as_float(u[e].x));
+                s.ck[at] = cf[e].x;
                 s.cv[at] = cf[e].y;
-                s.token[at] = u[e].x;
             }
         __syncthreads();
-        // The groups of the warp's cells in order: cell k of its runs, samples `ff` on.
-        constexpr int KC = 16 / RUNS * 4;
-        auto cell_at = [&](int k) { return 4 * (run0 + RUNS * (k >> 2)) + (k & 3); };
-        int fk = -1, ff = 0, fstop = 0, fslot = 0;
+        // The groups of the warp's runs in order: run fr, samples `ff` on.
+        int fr = run0 - STRIDE, ff = 0, fstop = 0;
+        uint32_t fstage = stage0;
         auto fetch_next = [&]() {
-            while (ff >= fstop && fk < KC - 1) {
-                ++fk;
-                ff = static_cast<int>(s.first[cell_at(fk)]);
-                fstop = static_cast<int>(s.first[cell_at(fk) + 1]);
+            while (ff >= fstop && fr < kRuns - STRIDE) {
+                fr += STRIDE;
+                ff = static_cast<int>(s.first[kBlockX * fr]);
+                fstop = static_cast<int>(s.first[kBlockX * fr + kBlockX]);
             }
             if (ff < fstop) {
-                unsigned char* to = s.stage[warp][fslot];
 #pragma unroll
-                for (int i = 0; i < LD; ++i) {      // beyond the cell its last sample again (the weight is zero)
-                    const int r = i * (32 / CPR) + lane / CPR;
-                    const bf16* from = src + s.token[min(ff + r, fstop - 1)] * tok;
-                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(to + r * (D * 2) + (((lane % CPR) ^ (r & SWZ)) << 4)))), "l"(from) : "memory");
+                for (int i = 0; i < LD; ++i) {      // beyond the run its last sample again (the weight is zero)
+                    const uint32_t token = __float_as_uint(s.geo[min(ff + i * RPI + lane / CPR, fstop - 1)].w);
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
+                                 ::"r"(fstage + ((put ^ (((i * RPI) & SWZ) << 4)) + i * RPI * (D * 2))), "l"(src + static_cast<uint64_t>(token) * tok_bytes) : "memory");
                 }
                 ff += 16;
-                fslot = fslot == S::STAGES - 1 ? 0 : fslot + 1;
+                fstage = fstage == stage0 + (S::STAGES - 1) * S::GROUP ? stage0 : fstage + S::GROUP;
             }
             asm volatile("cp.async.commit_group;" ::: "memory");
         };
 #pragma unroll
         for (int i = 0; i < S::STAGES - 1; ++i) fetch_next();
-        int slot = 0;
-        for (int rk = 0; rk < 16 / RUNS; ++rk) {
-            const int run = run0 + RUNS * rk;
-            if (s.first[4 * run] == s.first[4 * run + 4]) continue;
-            // the lane's corner row of dK / dV: (ct, cy) = (g8 >> 2, (g8 >> 1) & 1)
-            const int rt = b.t + (run >> 2) + (g8 >> 2), ry = b.y + (run & 3) + ((g8 >> 1) & 1);
-            const bool row_in = static_cast<unsigned>(rt) < static_cast<unsigned>(pr.T) && static_cast<unsigned>(ry) < static_cast<unsigned>(pr.H);
-            float* acc_row = acc + ((static_cast<long long>(rt) * pr.H + ry) * pr.W + b.x) * tok;
+        uint32_t at_stage = stage0;
+#pragma unroll 1
+        for (int run = run0; run < kRuns; run += STRIDE) {
+            int f = static_cast<int>(s.first[kBlockX * run]);
+            const int stop = static_cast<int>(s.first[kBlockX * run + kBlockX]);
+            if (f == stop) continue;
+            const int from1 = static_cast<int>(s.first[kBlockX * run + 1]), from2 = static_cast<int>(s.first[kBlockX * run + 2]);
             float c[D / 8][4];
 #pragma unroll
             for (int i = 0; i < D / 8; ++i) c[i][0] = c[i][1] = c[i][2] = c[i][3] = 0.0f;
-            auto flush = [&](int xi) {                 // the left corners of cell xi are complete: heads and remainders together, out
-                if ((g8 ^ xi) & 1) return;
-                if (row_in && static_cast<unsigned>(b.x + xi) < static_cast<unsigned>(pr.W)) {
-                    float* to = acc_row + xi * tok;
-                    if (DSA3D_IN_RANGE(pr, to - (tensor ? acc_dv : acc_dk), kv_extent, 10))
+#pragma unroll 1
+            for (; f < stop; f += 16) {
+                asm volatile("cp.async.wait_group %0;" ::"n"(S::STAGES - 2) : "memory");
+                __syncwarp();
+                const uint32_t from = at_stage + get;
+                at_stage = at_stage == stage0 + (S::STAGES - 1) * S::GROUP ? stage0 : at_stage + S::GROUP;
+                fetch_next();                          // into the slot that the group before this one was read from
+                // weights for samples 2j, 2j + 1, 2j + 8, 2j + 9; `first`: those that belong to column `col`, the others to col + 2
+                uint32_t head[2], rest[2], first[2];
 #pragma unroll
-                        for (int i = 0; i < D / 8; ++i) red_add_v2(to + 8 * i, c[i][0] + c[i][2], c[i][1] + c[i][3]);
-                }
+                for (int h = 0; h < 2; ++h) {
+                    float w2[2];
+                    first[h] = 0u;
 #pragma unroll
-                for (int i = 0; i < D / 8; ++i) c[i][0] = c[i][1] = c[i][2] = c[i][3] = 0.0f;
-            };
-            bool carry = false;                        // the sums hold something
-            for (int xi = 0; xi < 4; ++xi) {
-                int f = static_cast<int>(s.first[4 * run + xi]);
-                const int stop = static_cast<int>(s.first[4 * run + xi + 1]);
-                const bool any = f < stop;
-                const float sx = ((g8 ^ xi) & 1) ? 1.0f : -1.0f, ox = ((g8 ^ xi) & 1) ? 0.0f : 1.0f;
-                for (; f < stop; f += 16) {
-                    asm volatile("cp.async.wait_group %0;" ::"n"(S::STAGES - 2) : "memory");
-                    __syncwarp();
-                    const unsigned char* stage = s.stage[warp][slot];
-                    slot = slot == S::STAGES - 1 ? 0 : slot + 1;
-                    fetch_next();                      // into the slot that the group before this one was read from
-                    // weights of the lane's corner for samples 2j, 2j + 1, 2j + 8, 2j + 9: rows 0 - 7 of A the heads, rows 8 - 15
-                    // the remainders
-                    uint32_t a[4];
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        float w2[2];
-#pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            const int k = f + 2 * j + e + 8 * h, i = min(k, stop - 1);
-                            const float4 ge = s.geo[i];
-                            const float co = k < stop ? (tensor ? s.cv[i] : ge.w) : 0.0f;
-                            w2[e] = fmaf(ge.x, st, ot) * fmaf(ge.y, sy, oy) * fmaf(ge.z, sx, ox) * co;
-                        }
-                        const __nv_bfloat162 hd = __floats2bfloat162_rn(w2[0], w2[1]);
-                        const uint32_t hw = *reinterpret_cast<const uint32_t*>(&hd);
-                        const __nv_bfloat162 rs = __floats2bfloat162_rn(w2[0] - __uint_as_float(hw << 16), w2[1] - __uint_as_float(hw & 0xffff0000u));
-                        a[2 * h] = hw;
-                        a[2 * h + 1] = *reinterpret_cast<const uint32_t*>(&rs);
+                    for (int e = 0; e < 2; ++e) {
+                        const int k = f + 2 * j + e + 8 * h;
+                        const float4 ge = s.geo[min(k, stop - 1)];
+                        const int d = col - (k >= from1 ? 1 : 0) - (k >= from2 ? 1 : 0);     // column - cell: -2, 0 left, -1, 1 right
+                        w2[e] = fmaf(ge.x, st, ot) * fmaf(ge.y, sy, oy) * ((d & 1) ? ge.z : 1.0f - ge.z) * co[k < stop ? k : S::CAP];
+                        if (d >= 0) first[h] |= 0xffffu << (16 * e);
                     }
-                    const int mr = lane & 15;
-#pragma unroll
-                    for (int i = 0; i < D / 16; ++i) {
-                        uint32_t b0r, b1r, b2r, b3r;
-                        const uint32_t addr = static_cast<uint32_t>(__cvta_generic_to_shared(stage + mr * (D * 2) + (((2 * i + (lane >> 4)) ^ (mr & SWZ)) << 4)));
-                        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(b0r), "=r"(b1r), "=r"(b2r), "=r"(b3r) : "r"(addr));
-                        mma_bf16(c[2 * i], a[0], a[1], a[2], a[3], b0r, b1r);
-                        mma_bf16(c[2 * i + 1], a[0], a[1], a[2], a[3], b2r, b3r);
-                    }
+                    const __nv_bfloat162 hd = __floats2bfloat162_rn(w2[0], w2[1]);
+                    head[h] = *reinterpret_cast<const uint32_t*>(&hd);
+                    const __nv_bfloat162 rs = __floats2bfloat162_rn(w2[0] - __uint_as_float(head[h] << 16), w2[1] - __uint_as_float(head[h] & 0xffff0000u));
+                    rest[h] = *reinterpret_cast<const uint32_t*>(&rs);
                 }
-                if (any || carry) flush(xi);
-                carry = any;
+                const uint32_t a0 = head[0] & first[0], a1 = head[0] & ~first[0], a2 = head[1] & first[1], a3 = head[1] & ~first[1];
+                const uint32_t r0 = rest[0] & first[0], r1 = rest[0] & ~first[0], r2 = rest[1] & first[1], r3 = rest[1] & ~first[1];
+#pragma unroll
+                for (int i = 0; i < D / 16; ++i) {
+                    uint32_t b0r, b1r, b2r, b3r;
+                    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(b0r), "=r"(b1r), "=r"(b2r), "=r"(b3r) : "r"(from ^ (i << 5)));
+                    mma_bf16(c[2 * i], a0, a1, a2, a3, b0r, b1r);
+                    mma_bf16(c[2 * i + 1], a0, a1, a2, a3, b2r, b3r);
+                    mma_bf16(c[2 * i], r0, r1, r2, r3, b0r, b1r);
+                    mma_bf16(c[2 * i + 1], r0, r1, r2, r3, b2r, b3r);
+                }
             }
-            if (carry) flush(4);
+            const int rt = b.t + (run >> 2) + ((g8 >> 1) & 1), ry = b.y + (run & 3) + (g8 & 1), rx = b.x + col;
+            if (static_cast<unsigned>(rt) < static_cast<unsigned>(pr.T) && static_cast<unsigned>(ry) < static_cast<unsigned>(pr.H)) {
+                float* to = acc + ((static_cast<long long>(rt) * pr.H + ry) * pr.W + rx) * tok;
+                if (static_cast<unsigned>(rx) < static_cast<unsigned>(pr.W) && DSA3D_IN_RANGE(pr, to - (tensor ? acc_dv : acc_dk), kv_extent, 10)) {
+#pragma unroll
+                    for (int i = 0; i < D / 8; ++i) red_add_v2(to + 8 * i, c[i][0], c[i][1]);
+                }
+                to += 2 * tok;
+                if (static_cast<unsigned>(rx + 2) < static_cast<unsigned>(pr.W) && DSA3D_IN_RANGE(pr, to - (tensor ? acc_dv : acc_dk), kv_extent, 10)) {
+#pragma unroll
+                    for (int i = 0; i < D / 8; ++i) red_add_v2(to + 8 * i, c[i][2], c[i][3]);
+                }
+            }
+            __syncwarp();
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
@@ -647,8 +632,8 @@ cells_sums_kernel(const bf16* __restrict__ q, const bf16* __restrict__ dout, flo
 }
 
 // ------------------------------------------------------------------------------------------------ beyond the bins
-// The samples in bin kBins of every tile, a warp per sample, row by row.  kScatter: their contributions to dK and dV; otherwise
-// what cells_dots_kernel leaves for the others.
+// The samples in bin kBins of every tile, a warp per sample, row by row.  kScatter: their contributions to dK and dV, and those
+// of marked samples of the other bins; otherwise what cells_dots_kernel leaves for the others.
 template <int D, bool kScatter>
 __global__ void __launch_bounds__(256)
 cells_far_kernel(const bf16* __restrict__ q, const bf16* __restrict__ k, const bf16* __restrict__ v, const bf16* __restrict__ dout,
@@ -662,6 +647,8 @@ cells_far_kernel(const bf16* __restrict__ q, const bf16* __restrict__ k, const b
     for (int base = (static_cast<int>(blockIdx.x) * 8 + static_cast<int>(threadIdx.x >> 5)) * 32; base < tiles; base += warps * 32) {
         uint32_t mine = 0u;
         if (base + lane < tiles) mine = __ldg(sl.seg + static_cast<long long>(base + lane) * (kBins + 1) + kBins);
+        const bool marked = kScatter && *sl.marked != 0;
+        if (marked) mine = ((mine & 0xffffu) + (mine >> 16)) << 16;        // all samples of the tile: those beyond the bins are its last
         unsigned todo = __ballot_sync(kFullMask, (mine >> 16) != 0u);
         while (todo) {
             const int src = __ffs(static_cast<int>(todo)) - 1;
@@ -669,6 +656,7 @@ cells_far_kernel(const bf16* __restrict__ q, const bf16* __restrict__ k, const b
             const uint32_t w = __shfl_sync(kFullMask, mine, src);
             const long long tile = base + src;
             const int m = sl.m0 + static_cast<int>(tile / per_head);
+            const uint32_t far_from = marked ? __ldg(sl.seg + tile * (kBins + 1) + kBins) & 0xffffu : 0u;
             for (uint32_t i = 0; i < (w >> 16); ++i) {
                 const long long at = tile * (kRows * pr.P) + (w & 0xffffu) + i;
                 const int n = static_cast<int>(__ldg(sl.geo + at).x), p = static_cast<int>(__ldg(sl.meta + at) & 255u);
@@ -687,6 +675,7 @@ cells_far_kernel(const bf16* __restrict__ q, const bf16* __restrict__ k, const b
                 const long long sidx = sample_at(sl, pr, m, n, p);
                 if constexpr (kScatter) {
                     const float2 cf = sl.coef[sidx];
+                    if (marked && i < far_from && !(__float_as_uint(cf.y) >> 31)) continue;
                     for (int j = 0; j < 8; ++j) {
                         const float wj = wt[j >> 2] * wy[(j >> 1) & 1] * wx[j & 1];
                         const long long o = o0 + (j >> 2) * st + ((j >> 1) & 1) * sy + (j & 1) * tok;
@@ -738,13 +727,13 @@ size_t round256(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
 // Lays a slab's buffers out at `base` (may be NULL); returns their bytes.
 size_t lay_out(const Problem& pr, int m0, int heads, int f0, int f1, char* base, Slab& s) {
     s.m0 = m0; s.heads = heads; s.f0 = f0; s.f1 = f1;
-    s.tiles_t = (f1 - f0 + 3) / 4; s.tiles_y = (pr.H + 3) / 4; s.tiles_x = (pr.W + 7) / 8;
+    s.tiles_t = (f1 - f0 + 3) / 4; s.tiles_y = (pr.H + 3) / 4; s.tiles_x = (pr.W + kTileX - 1) / kTileX;
     const int lo = floor_div4(-1 - f0), hi = floor_div4(pr.T - 1 - f0);
     s.bt0 = lo < -3 ? -3 : lo;
     const int top = s.tiles_t - 1 + 3 < hi ? s.tiles_t - 1 + 3 : hi;
     s.blocks_t = top - s.bt0 + 1;
     s.blocks_y = (pr.H - 1) / 4 + 2;
-    s.blocks_x = (pr.W - 1) / 4 + 2;
+    s.blocks_x = (pr.W - 1) / kBlockX + 2;
     const size_t tiles = static_cast<size_t>(heads) * s.tiles_t * s.tiles_y * s.tiles_x, samples = tiles * kRows * pr.P;
     const size_t live = static_cast<size_t>(heads) * (f1 - f0) * pr.H * pr.W * pr.P;
     size_t at = 0;
@@ -753,6 +742,7 @@ size_t lay_out(const Problem& pr, int m0, int heads, int f0, int f1, char* base,
     s.seg = reinterpret_cast<uint32_t*>(base + at); at += round256(tiles * (kBins + 1) * sizeof(uint32_t));
     s.stats = reinterpret_cast<float*>(base + at); at += round256(live * 8 * sizeof(float));
     s.coef = reinterpret_cast<float2*>(base + at); at += round256(live * sizeof(float2));
+    s.marked = reinterpret_cast<int*>(base + at); at += 256;
     return at;
 }
 
@@ -766,7 +756,7 @@ cudaError_t launch_slab(const void* q_, const void* k_, const void* v_, const fl
     cudaError_t e = cudaFuncSetAttribute(cells_bin_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bin_smem));
     if (e != cudaSuccess) return e;
     cells_bin_kernel<<<static_cast<unsigned>(tiles), kBinThreads, bin_smem, stream>>>(offsets, pr, s, inv_p);
-    const size_t dot_smem = sizeof(DotSmem<D>), sum_smem = sizeof(SumSmem<D>);
+    const size_t dot_smem = sizeof(DotSmem<D>), sum_smem = sizeof(SumSmem<D>) + 256;
     e = cudaFuncSetAttribute(cells_dots_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(dot_smem));
     if (e != cudaSuccess) return e;
     cells_dots_kernel<D><<<static_cast<unsigned>(blocks), kDotThreads, dot_smem, stream>>>(q, k, v, dout, pr, s);
