@@ -1,6 +1,7 @@
 // The general operator's backward on samples sorted by key cell: see dsa3d_cells.cuh.
 //
 //   cells_bin_kernel     sorts the samples of a query tile by key block; 18 bytes per sample
+//   cells_sort_kernel    per block: its samples in the order of their cells
 //   cells_dots_kernel    per block: samples by cell, 16 at a time  q . K_corner  and  dO . V_corner  (tensor cores), the
 //                        trilinear value and derivatives of both per sample: eight numbers
 //   cells_query_kernel   per query: alpha, delta, dS, dOffsets, the two coefficients per sample, dQ (a gather of K rows)
@@ -34,7 +35,7 @@ cells_bin_kernel(const float* __restrict__ offsets, const Problem pr, const Slab
     const int x0 = (r % sl.tiles_x) * kTileX; r /= sl.tiles_x;
     const int y0 = (r % sl.tiles_y) * 4, t0 = sl.f0 + (r / sl.tiles_y) * 4;
     const int samples = kRows * pr.P;
-    if (blockIdx.x == 0 && tid == 0) *sl.marked = 0;
+    if (blockIdx.x == 0 && tid == 0) { *sl.marked = 0; *sl.used = 0u; }
     for (int i = tid; i < (kBins + 1) * kCopies / 4; i += kBinThreads) reinterpret_cast<uint4*>(counters)[i] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
     auto row_of = [&](int s) { return static_cast<int>((static_cast<unsigned long long>(static_cast<unsigned>(s)) * inv_p) >> 24); };
@@ -194,6 +195,55 @@ __device__ __forceinline__ long long sample_of(const Segments& sg, uint32_t i, i
     return static_cast<long long>(sg.tile[lo]) * samples_per_tile + sg.start[lo] + (i - sg.first[lo]);
 }
 
+// A block's samples in the order of their cells.  (A kernel of its own: it is a chain of dependent loads - segment,
+// sample, place - which wants many small CTAs per SM, and both block kernels read what it leaves in one stream.)
+constexpr int kSortThreads = 256, kSortKeep = 2048;
+__global__ void __launch_bounds__(kSortThreads)
+cells_sort_kernel(const Problem pr, const Slab sl) {
+    __shared__ Segments sg;
+    __shared__ uint32_t count[kCells], cursor[kCells], base;
+    __shared__ uint32_t kept[kSortKeep];                    // place in its tile's list of the first samples
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const BlockPos b = block_pos(sl, blockIdx.x);
+    if (tid < kCells) count[tid] = 0u;
+    const uint32_t total = find_segments(sl, b, sg);
+    uint32_t* first = sl.first + static_cast<long long>(blockIdx.x) * (kCells + 1);
+    if (total == 0u) {
+        if (tid <= kCells) first[tid] = 0u;
+        return;
+    }
+    for (uint32_t i = tid; i < total; i += kSortThreads) {
+        const uint32_t at = static_cast<uint32_t>(sample_of(sg, i, kRows * pr.P));
+        if (i < kSortKeep) kept[i] = at;
+        atomicAdd(&count[__ldg(sl.meta + at) >> 8], 1u);
+    }
+    if (tid == 0) base = atomicAdd(sl.used, total);
+    __syncthreads();
+    if (warp == 0) {
+        const uint32_t c0 = lane < kCells / 2 ? count[2 * lane] : 0u, c1 = lane < kCells / 2 ? count[2 * lane + 1] : 0u;
+        uint32_t inc = c0 + c1;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t up = __shfl_up_sync(kFullMask, inc, o);
+            if (lane >= o) inc += up;
+        }
+        if (lane < kCells / 2) {
+            cursor[2 * lane] = first[2 * lane] = base + inc - c0 - c1;
+            cursor[2 * lane + 1] = first[2 * lane + 1] = base + inc - c1;
+        }
+        if (lane == 31) first[kCells] = base + inc;
+    }
+    __syncthreads();
+    for (uint32_t i = tid; i < total; i += kSortThreads) {
+        const uint32_t at = i < kSortKeep ? kept[i] : static_cast<uint32_t>(sample_of(sg, i, kRows * pr.P));
+        const uint32_t mt = __ldg(sl.meta + at);
+        const uint4 u = __ldg(sl.geo + at);
+        const uint32_t to = atomicAdd(&cursor[mt >> 8], 1u);
+        sl.sorted[to] = make_float4(__uint_as_float(u.y), __uint_as_float(u.z), __uint_as_float(u.w), __uint_as_float(u.x));
+        sl.place[to] = static_cast<uint32_t>(sample_at(sl, pr, b.m, static_cast<int>(u.x), static_cast<int>(mt & 255u)));
+    }
+}
+
 // Byte of 16-byte chunk `chunk` of box row `row` in shared memory: rows of 128 bytes and more have their chunks permuted by
 // the row's parity, so that the four chunks a quarter-warp reads of two neighbouring rows lie in different banks.
 template <int D> __device__ __forceinline__ int box_byte(int row, int chunk) {
@@ -215,15 +265,11 @@ __device__ __forceinline__ void load_box(unsigned char* dst, const bf16* __restr
 }
 
 // ------------------------------------------------------------------------------------------------ dot products
-constexpr int kDotThreads = 512, kDotCap = 1536;
+constexpr int kDotThreads = 256;
 
 template <int D> struct DotSmem {
     unsigned char box[2][kBox * D * 2];
-    float4 geo[kDotCap];                            // ft, fy, fx, token (bits); sorted by cell
-    uint32_t dest[kDotCap];                         // where the sample's results go
-    uint32_t group[kDotCap / 16 + kCells];          // cell | first sample << 8 | samples - 1 << 20
-    uint32_t count[kCells], first[kCells + 1], gfirst[kCells + 1];
-    Segments sg;
+    uint32_t first[kCells + 1], groups[64];         // groups: of 16 samples, before the cell (the rest of the 64 never reached)
 };
 
 // Value and derivatives of the trilinear interpolant of eight corner numbers, two corners (2j, 2j + 1: x pair of (ct, cy) =
@@ -245,102 +291,85 @@ __device__ __forceinline__ float trilerp_lanes(float s0, float s1, int j, float 
 
 // q . K and dO . V with derivatives, eight numbers per sample into stats; even warps take q . K, odd ones dO . V.
 template <int D>
-__global__ void __launch_bounds__(kDotThreads, 2)
+__global__ void __launch_bounds__(kDotThreads, D == 128 ? 3 : 4)
 cells_dots_kernel(const bf16* __restrict__ q, const bf16* __restrict__ k, const bf16* __restrict__ v, const bf16* __restrict__ dout,
                   const Problem pr, const Slab sl) {
-    constexpr int I = D / 32, W = kDotThreads / 64, PER = kDotCap / kDotThreads;
+    constexpr int I = D / 32, W = kDotThreads / 64;
     extern __shared__ __align__(16) unsigned char raw[];
     DotSmem<D>& s = *reinterpret_cast<DotSmem<D>*>(raw);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g8 = lane >> 2, j = lane & 3;
     const int tensor = warp & 1;
+    const uint32_t* first = sl.first + static_cast<long long>(blockIdx.x) * (kCells + 1);
+    if (__ldg(first) == __ldg(first + kCells)) return;
     const BlockPos b = block_pos(sl, blockIdx.x);
-    const uint32_t total = find_segments(sl, b, s.sg);
-    if (total == 0u) return;
+    if (warp == 0) {
+        const uint32_t f0 = __ldg(first + min(2 * lane, kCells)), f1 = __ldg(first + min(2 * lane + 1, kCells)), f2 = __ldg(first + min(2 * lane + 2, kCells));
+        const uint32_t n0 = (f1 - f0 + 15u) >> 4, n1 = (f2 - f1 + 15u) >> 4;
+        uint32_t inc = n0 + n1;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t up = __shfl_up_sync(kFullMask, inc, o);
+            if (lane >= o) inc += up;
+        }
+        if (lane <= kCells / 2) s.first[2 * lane] = f0;
+        if (lane < kCells / 2) s.first[2 * lane + 1] = f1;
+        s.groups[2 * lane] = inc - n0 - n1;
+        s.groups[2 * lane + 1] = inc - n1;
+    }
     load_box<D, kDotThreads>(s.box[0], k, b, pr);
     load_box<D, kDotThreads>(s.box[1], v, b, pr);
+    __syncthreads();
     const bf16* src = (tensor ? dout : q) + static_cast<long long>(b.m) * D + j * 8;
     const unsigned char* box = s.box[tensor];
     const long long tok = static_cast<long long>(pr.heads) * D;
-    for (uint32_t b0 = 0; b0 < total; b0 += kDotCap) {
-        const int nb = static_cast<int>(min(static_cast<uint32_t>(kDotCap), total - b0));
-        if (tid < kCells) s.count[tid] = 0u;
-        __syncthreads();
-        uint4 u[PER];
-        uint32_t rank[PER], dest[PER];              // rank: cell | rank in the cell << 8
+    const int groups = static_cast<int>(s.groups[kCells]);
+    float* out = sl.stats + tensor * 4 + j;
+    // what the lane needs of a group: its cell, its samples (rows g8 and g8 + 8 of the tile)
+    int cell = 0;
+    bool live_a = false, live_b = false;
+    float4 ga = make_float4(0.0f, 0.0f, 0.0f, 0.0f), gb = ga;
+    uint32_t pa = 0u, pb = 0u;
+    auto fetch = [&](int g) {
+        const uint32_t ug = static_cast<uint32_t>(g);
+        // cells 1 .. 47 whose groups begin at or before this one
+        cell = __popc(__ballot_sync(kFullMask, s.groups[lane + 1] <= ug)) + __popc(__ballot_sync(kFullMask, lane < kCells - 33 && s.groups[min(lane + 33, 63)] <= ug));
+        const uint32_t f = s.first[cell] + 16u * (ug - s.groups[cell]), end = s.first[cell + 1];
+        const uint32_t ia = min(f + static_cast<uint32_t>(g8), end - 1u), ib = min(f + static_cast<uint32_t>(g8) + 8u, end - 1u);   // a missing sample repeats the last one
+        live_a = f + static_cast<uint32_t>(g8) < end;
+        live_b = f + static_cast<uint32_t>(g8) + 8u < end;
+        ga = __ldg(sl.sorted + ia);
+        gb = __ldg(sl.sorted + ib);
+        pa = __ldg(sl.place + ia);
+        pb = __ldg(sl.place + ib);
+    };
+    int g = warp >> 1;
+    if (g < groups) fetch(g);
+    for (; g < groups; g += W) {
+        const int row = box_row(cell) + box_step(g8);
+        const uint4* ra_p = reinterpret_cast<const uint4*>(src + __float_as_int(ga.w) * tok);
+        const uint4* rb_p = reinterpret_cast<const uint4*>(src + __float_as_int(gb.w) * tok);
+        // The order of the channels inside a product is free: lane j takes chunk j of every 64 bytes, whole
+        // 16-byte pieces on both sides.
+        uint4 ra[I], rb[I];
 #pragma unroll
-        for (int e = 0; e < PER; ++e) {
-            const int i = e * kDotThreads + tid;
-            rank[e] = 0xffffffffu;
-            if (i >= nb) continue;
-            const long long at = sample_of(s.sg, b0 + static_cast<uint32_t>(i), kRows * pr.P);
-            u[e] = __ldg(sl.geo + at);
-            rank[e] = __ldg(sl.meta + at);
+        for (int i = 0; i < I; ++i) {
+            ra[i] = __ldg(ra_p + 4 * i);
+            rb[i] = __ldg(rb_p + 4 * i);
         }
+        const float fa0 = ga.x, fa1 = ga.y, fa2 = ga.z, fb0 = gb.x, fb1 = gb.y, fb2 = gb.z;
+        float* da = live_a ? out + static_cast<size_t>(pa) * 8 : nullptr;
+        float* db = live_b ? out + static_cast<size_t>(pb) * 8 : nullptr;
+        if (g + W < groups) fetch(g + W);           // the next group's samples, a group ahead of its rows
+        float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-        for (int e = 0; e < PER; ++e) {
-            if (rank[e] == 0xffffffffu) continue;
-            dest[e] = static_cast<uint32_t>(sample_at(sl, pr, b.m, static_cast<int>(u[e].x), static_cast<int>(rank[e] & 255u)));
-            rank[e] = (rank[e] >> 8) | (atomicAdd(&s.count[rank[e] >> 8], 1u) << 8);
+        for (int i = 0; i < I; ++i) {
+            const uint4 kb = *reinterpret_cast<const uint4*>(box + box_byte<D>(row, 4 * i + j));
+            mma_bf16(c, ra[i].x, rb[i].x, ra[i].y, rb[i].y, kb.x, kb.y);
+            mma_bf16(c, ra[i].z, rb[i].z, ra[i].w, rb[i].w, kb.z, kb.w);
         }
-        __syncthreads();
-        if (warp == 0) {                            // exclusive sums over the cells: samples and groups of 16
-            const uint32_t c0 = lane < kCells / 2 ? s.count[2 * lane] : 0u, c1 = lane < kCells / 2 ? s.count[2 * lane + 1] : 0u;
-            const uint32_t n0 = (c0 + 15u) >> 4, n1 = (c1 + 15u) >> 4;
-            uint32_t inc = c0 + c1, ginc = n0 + n1;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t up = __shfl_up_sync(kFullMask, inc, o), gup = __shfl_up_sync(kFullMask, ginc, o);
-                if (lane >= o) { inc += up; ginc += gup; }
-            }
-            if (lane < kCells / 2) {
-                s.first[2 * lane] = inc - c0 - c1; s.first[2 * lane + 1] = inc - c1;
-                s.gfirst[2 * lane] = ginc - n0 - n1; s.gfirst[2 * lane + 1] = ginc - n1;
-            }
-            if (lane == 31) { s.first[kCells] = inc; s.gfirst[kCells] = ginc; }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int e = 0; e < PER; ++e)
-            if (rank[e] != 0xffffffffu) {
-                const uint32_t at = s.first[rank[e] & 63u] + (rank[e] >> 8);
-                s.geo[at] = make_float4(__uint_as_float(u[e].y), __uint_as_float(u[e].z), __uint_as_float(u[e].w), __uint_as_float(u[e].x));
-                s.dest[at] = dest[e];
-            }
-        if (tid < kCells) {
-            const uint32_t c = s.count[tid], f = s.first[tid], gf = s.gfirst[tid];
-            for (uint32_t i = 0; i * 16u < c; ++i) s.group[gf + i] = static_cast<uint32_t>(tid) | ((f + i * 16u) << 8) | ((min(16u, c - i * 16u) - 1u) << 20);
-        }
-        __syncthreads();
-        const int groups = static_cast<int>(s.gfirst[kCells]);
-        for (int g = warp >> 1; g < groups; g += W) {
-            const uint32_t gw = s.group[g];
-            const int row = box_row(static_cast<int>(gw & 63u)) + box_step(g8);
-            const int f = static_cast<int>((gw >> 8) & 0xfffu), last = static_cast<int>(gw >> 20);
-            const int ia = f + min(g8, last), ib = f + min(g8 + 8, last);       // a missing sample repeats the last one
-            const float4 ga = s.geo[ia], gb = s.geo[ib];
-            const uint4* pa = reinterpret_cast<const uint4*>(src + __float_as_int(ga.w) * tok);
-            const uint4* pb = reinterpret_cast<const uint4*>(src + __float_as_int(gb.w) * tok);
-            // The order of the channels inside a product is free: lane j takes chunk j of every 64 bytes, whole
-            // 16-byte pieces on both sides.
-            uint4 ra[I], rb[I];
-#pragma unroll
-            for (int i = 0; i < I; ++i) {
-                ra[i] = __ldg(pa + 4 * i);
-                rb[i] = __ldg(pb + 4 * i);
-            }
-            float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-            for (int i = 0; i < I; ++i) {
-                const uint4 kb = *reinterpret_cast<const uint4*>(box + box_byte<D>(row, 4 * i + j));
-                mma_bf16(c, ra[i].x, rb[i].x, ra[i].y, rb[i].y, kb.x, kb.y);
-                mma_bf16(c, ra[i].z, rb[i].z, ra[i].w, rb[i].w, kb.z, kb.w);
-            }
-            const float xa = trilerp_lanes(c[0], c[1], j, ga.x, ga.y, ga.z), xb = trilerp_lanes(c[2], c[3], j, gb.x, gb.y, gb.z);
-            float* d = sl.stats + tensor * 4 + j;
-            if (g8 <= last) d[static_cast<size_t>(s.dest[ia]) * 8] = xa;
-            if (g8 + 8 <= last) d[static_cast<size_t>(s.dest[ib]) * 8] = xb;
-        }
-        __syncthreads();                            // the batch's places are free for the next one
+        const float xa = trilerp_lanes(c[0], c[1], j, fa0, fa1, fa2), xb = trilerp_lanes(c[2], c[3], j, fb0, fb1, fb2);
+        if (da) *da = xa;
+        if (db) *db = xb;
     }
 }
 
@@ -445,13 +474,10 @@ cells_query_kernel(const bf16* __restrict__ k, const float* __restrict__ offsets
 constexpr int kSumThreads = 256;
 
 template <int D> struct SumSmem {
-    static constexpr int CAP = 1536, PER = CAP / kSumThreads;     // samples at a time: two CTAs per SM fit
-    static constexpr int STAGES = D == 128 ? 2 : 3, GROUP = 16 * D * 2;
+    static constexpr int STAGES = 2, GROUP = 16 * D * 2;
     unsigned char stage[kSumThreads / 32][STAGES][GROUP];         // a warp's ring of 16 query rows
-    float4 geo[CAP];                                // ft, fy, fx, token (bits); sorted by cell, as ck and cv
-    float ck[CAP + 1], cv[CAP + 1];                 // the last one is zero: what a group beyond its run's samples takes
-    uint32_t count[kCells], first[kCells + 1];
-    Segments sg;
+    float4 geo[kSumThreads / 32][2][16];                          // ft, fy, fx, coefficient of a group's samples
+    uint32_t first[kCells + 1];
 };
 
 __device__ __forceinline__ void red_add_v2(float* addr, float a, float b) {
@@ -461,30 +487,32 @@ __device__ __forceinline__ void red_add_v2(float* addr, float a, float b) {
 // A warp works on one tensor and runs of three cells along x: the corners of a run are 4 columns x 4 (t, y) rows of the
 // accumulators, the 16 rows of the product tile, and 16 of the run's samples at a time are its depth.  A lane forms
 // the weights of its (t, y) in columns g8 / 4 and g8 / 4 + 2: a sample has a weight in exactly one of the two, which goes in
-// as bf16 head and remainder, two products into the same sums.  The query rows come by cp.async a group (or two)
-// ahead, across runs.
+// as bf16 head and remainder, two products into the same sums.  Nothing is shared between warps: each walks through its
+// groups in three steps that overlap - samples (two groups ahead), coefficients and query rows (one ahead), products.
 template <int D>
-__global__ void __launch_bounds__(kSumThreads, 2)
+__global__ void __launch_bounds__(kSumThreads, D == 32 ? 3 : 2)
 cells_sums_kernel(const bf16* __restrict__ q, const bf16* __restrict__ dout, float* __restrict__ acc_dk, float* __restrict__ acc_dv,
                   const Problem pr, const Slab sl) {
     using S = SumSmem<D>;
-    constexpr int PER = S::PER, STRIDE = 4;         // the four warps of a tensor take the runs in turn
+    constexpr int STRIDE = 4;                       // the four warps of a tensor take the runs in turn
     constexpr int CPR = D / 8;                      // 16-byte chunks of a staged row, permuted by the row (SWZ)
     constexpr int LD = 16 * CPR / 32, RPI = 32 / CPR;      // fetches per lane for 16 rows; rows per fetch of the warp
     constexpr int SWZ = CPR < 8 ? CPR - 1 : 7;
     extern __shared__ __align__(16) unsigned char raw[];
     S& s = *reinterpret_cast<S*>((reinterpret_cast<uintptr_t>(raw) + 255) & ~uintptr_t(255));
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g8 = lane >> 2, j = lane & 3;
+    const uint32_t* first = sl.first + static_cast<long long>(blockIdx.x) * (kCells + 1);
+    if (__ldg(first) == __ldg(first + kCells)) return;
     const BlockPos b = block_pos(sl, blockIdx.x);
-    const uint32_t total = find_segments(sl, b, s.sg);
-    if (total == 0u) return;
+    if (tid <= kCells) s.first[tid] = __ldg(first + tid);
+    __syncthreads();
     const long long tok = static_cast<long long>(pr.heads) * D;
     const uint32_t tok_bytes = static_cast<uint32_t>(tok) * 2u;
     [[maybe_unused]] const long long kv_extent = pr.N * pr.heads * D;
     const int tensor = warp & 1, run0 = warp >> 1;
     const char* src = reinterpret_cast<const char*>((tensor ? dout : q) + static_cast<long long>(b.m) * D + (lane % CPR) * 8);
     float* acc = (tensor ? acc_dv : acc_dk) + static_cast<long long>(b.m) * D + 2 * j;
-    const float* co = tensor ? s.cv : s.ck;
+    const float* coef = reinterpret_cast<const float*>(sl.coef) + tensor;
     const float st = (g8 & 2) ? 1.0f : -1.0f, ot = (g8 & 2) ? 0.0f : 1.0f, sy = (g8 & 1) ? 1.0f : -1.0f, oy = (g8 & 1) ? 0.0f : 1.0f;
     const int col = g8 >> 2;
     const uint32_t stage0 = static_cast<uint32_t>(__cvta_generic_to_shared(s.stage[warp][0]));
@@ -492,125 +520,113 @@ cells_sums_kernel(const bf16* __restrict__ q, const bf16* __restrict__ dout, flo
     // chunk's permutation is an exclusive or within 256 aligned bytes
     const uint32_t put = static_cast<uint32_t>((lane / CPR) * (D * 2) + (((lane % CPR) ^ ((lane / CPR) & SWZ)) << 4));
     const uint32_t get = static_cast<uint32_t>((lane & 15) * (D * 2) + (((lane >> 4) ^ (lane & SWZ)) << 4));
-    if (tid == 0) { s.ck[S::CAP] = s.cv[S::CAP] = 0.0f; }
-    for (uint32_t b0 = 0; b0 < total; b0 += S::CAP) {
-        const int nb = static_cast<int>(min(static_cast<uint32_t>(S::CAP), total - b0));
-        if (tid < kCells) s.count[tid] = 0u;
-        __syncthreads();
-        uint4 u[PER];
-        float2 cf[PER];
-        uint32_t rank[PER];                         // cell | rank in the cell << 8
-#pragma unroll
-        for (int e = 0; e < PER; ++e) {
-            const int i = e * kSumThreads + tid;
-            rank[e] = 0xffffffffu;
-            if (i >= nb) continue;
-            const long long at = sample_of(s.sg, b0 + static_cast<uint32_t>(i), kRows * pr.P);
-            u[e] = __ldg(sl.geo + at);
-            rank[e] = __ldg(sl.meta + at);
+
+    // step 1: a group's samples, lane l sample l % 16 (beyond the run its last one again)
+    int run1 = run0 - STRIDE;
+    uint32_t f1 = 0u, stop1 = 0u;
+    float4 geo1 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    uint32_t place1 = 0u;
+    bool any1 = false;
+    auto samples = [&]() {                          // the group at f1, or the next run's first
+        while (f1 >= stop1 && run1 < kRuns - STRIDE) {
+            run1 += STRIDE;
+            f1 = s.first[kBlockX * run1];
+            stop1 = s.first[kBlockX * run1 + kBlockX];
         }
-#pragma unroll
-        for (int e = 0; e < PER; ++e)
-            if (rank[e] != 0xffffffffu) cf[e] = __ldg(sl.coef + sample_at(sl, pr, b.m, static_cast<int>(u[e].x), static_cast<int>(rank[e] & 255u)));
-#pragma unroll
-        for (int e = 0; e < PER; ++e) {
-            if (rank[e] == 0xffffffffu) continue;
-            if (__float_as_uint(cf[e].y) >> 31) rank[e] = 0xffffffffu;       // marked: cells_far_kernel takes it
-            else rank[e] = (rank[e] >> 8) | (atomicAdd(&s.count[rank[e] >> 8], 1u) << 8);
+        any1 = f1 < stop1;
+        if (any1) {
+            const uint32_t i = min(f1 + static_cast<uint32_t>(lane & 15), stop1 - 1u);
+            geo1 = __ldg(sl.sorted + i);
+            place1 = __ldg(sl.place + i);
         }
-        __syncthreads();
-        if (warp == 0) {
-            const uint32_t c0 = lane < kCells / 2 ? s.count[2 * lane] : 0u, c1 = lane < kCells / 2 ? s.count[2 * lane + 1] : 0u;
-            uint32_t inc = c0 + c1;
+    };
+    // step 2: their coefficients and query rows
+    int run2 = 0;
+    uint32_t f2 = 0u, stop2 = 0u;
+    float4 geo2 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    float coef2 = 0.0f, mark2 = 0.0f;
+    bool any2 = false;
+    uint32_t stage2 = stage0;
+    auto rows = [&]() {
+        any2 = any1;
+        if (any1) {
+            run2 = run1; f2 = f1; stop2 = stop1; geo2 = geo1;
+            coef2 = __ldg(coef + static_cast<size_t>(place1) * 2);
+            mark2 = tensor ? coef2 : __ldg(coef + static_cast<size_t>(place1) * 2 + 1);
+            const uint32_t token = __float_as_uint(geo1.w);
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t up = __shfl_up_sync(kFullMask, inc, o);
-                if (lane >= o) inc += up;
+            for (int i = 0; i < LD; ++i) {
+                const uint32_t t = __shfl_sync(kFullMask, token, i * RPI + lane / CPR);
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
+                             ::"r"(stage2 + ((put ^ (((i * RPI) & SWZ) << 4)) + i * RPI * (D * 2))), "l"(src + static_cast<uint64_t>(t) * tok_bytes) : "memory");
             }
-            if (lane < kCells / 2) { s.first[2 * lane] = inc - c0 - c1; s.first[2 * lane + 1] = inc - c1; }
-            if (lane == 31) s.first[kCells] = inc;
+            stage2 = stage2 == stage0 + (S::STAGES - 1) * S::GROUP ? stage0 : stage2 + S::GROUP;
+            f1 += 16u;
         }
-        __syncthreads();
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    samples();
+    rows();
+    samples();
+    uint32_t stage3 = stage0;
+    int slot = 0;
+    float c[D / 8][4];
 #pragma unroll
-        for (int e = 0; e < PER; ++e)
-            if (rank[e] != 0xffffffffu) {
-                const uint32_t at = s.first[rank[e] & 63u] + (rank[e] >> 8);
-                s.geo[at] = make_float4(__uint_as_float(u[e].y), __uint_as_float(u[e].z), __uint_as_float(u[e].w), __uint_as_float(u[e].x));
-                s.ck[at] = cf[e].x;
-                s.cv[at] = cf[e].y;
-            }
-        __syncthreads();
-        // The groups of the warp's runs in order: run fr, samples `ff` on.
-        int fr = run0 - STRIDE, ff = 0, fstop = 0;
-        uint32_t fstage = stage0;
-        auto fetch_next = [&]() {
-            while (ff >= fstop && fr < kRuns - STRIDE) {
-                fr += STRIDE;
-                ff = static_cast<int>(s.first[kBlockX * fr]);
-                fstop = static_cast<int>(s.first[kBlockX * fr + kBlockX]);
-            }
-            if (ff < fstop) {
-#pragma unroll
-                for (int i = 0; i < LD; ++i) {      // beyond the run its last sample again (the weight is zero)
-                    const uint32_t token = __float_as_uint(s.geo[min(ff + i * RPI + lane / CPR, fstop - 1)].w);
-                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
-                                 ::"r"(fstage + ((put ^ (((i * RPI) & SWZ) << 4)) + i * RPI * (D * 2))), "l"(src + static_cast<uint64_t>(token) * tok_bytes) : "memory");
-                }
-                ff += 16;
-                fstage = fstage == stage0 + (S::STAGES - 1) * S::GROUP ? stage0 : fstage + S::GROUP;
-            }
-            asm volatile("cp.async.commit_group;" ::: "memory");
-        };
-#pragma unroll
-        for (int i = 0; i < S::STAGES - 1; ++i) fetch_next();
-        uint32_t at_stage = stage0;
+    for (int i = 0; i < D / 8; ++i) c[i][0] = c[i][1] = c[i][2] = c[i][3] = 0.0f;
 #pragma unroll 1
-        for (int run = run0; run < kRuns; run += STRIDE) {
-            int f = static_cast<int>(s.first[kBlockX * run]);
-            const int stop = static_cast<int>(s.first[kBlockX * run + kBlockX]);
-            if (f == stop) continue;
-            const int from1 = static_cast<int>(s.first[kBlockX * run + 1]), from2 = static_cast<int>(s.first[kBlockX * run + 2]);
-            float c[D / 8][4];
+    while (any2) {
+        // step 3: the products of the group whose rows are on their way
+        const int run = run2;
+        const uint32_t f = f2, stop = stop2, from1 = s.first[kBlockX * run + 1], from2 = s.first[kBlockX * run + 2];
+        const bool odd = __float_as_uint(mark2) >> 31;             // marked: cells_far_kernel takes it
+        const unsigned odds = __ballot_sync(kFullMask, odd);
+        if (lane < 16) s.geo[warp][slot][lane] = make_float4(geo2.x, geo2.y, geo2.z, (odd || f + lane >= stop) ? 0.0f : coef2);
+        const uint32_t from = stage3;
+        stage3 = stage3 == stage0 + (S::STAGES - 1) * S::GROUP ? stage0 : stage3 + S::GROUP;
+        __syncwarp();                                  // also: everybody has read the slot that the next rows go to
+        rows();
+        samples();
+        // weights for samples 2j, 2j + 1, 2j + 8, 2j + 9; `mine`: those that belong to column `col`, the others to col + 2
+        uint32_t head[2], rest[2], mine[2];
 #pragma unroll
-            for (int i = 0; i < D / 8; ++i) c[i][0] = c[i][1] = c[i][2] = c[i][3] = 0.0f;
-#pragma unroll 1
-            for (; f < stop; f += 16) {
-                asm volatile("cp.async.wait_group %0;" ::"n"(S::STAGES - 2) : "memory");
-                __syncwarp();
-                const uint32_t from = at_stage + get;
-                at_stage = at_stage == stage0 + (S::STAGES - 1) * S::GROUP ? stage0 : at_stage + S::GROUP;
-                fetch_next();                          // into the slot that the group before this one was read from
-                // weights for samples 2j, 2j + 1, 2j + 8, 2j + 9; `first`: those that belong to column `col`, the others to col + 2
-                uint32_t head[2], rest[2], first[2];
+        for (int h = 0; h < 2; ++h) {
+            float w2[2];
+            mine[h] = 0u;
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    float w2[2];
-                    first[h] = 0u;
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const int k = f + 2 * j + e + 8 * h;
-                        const float4 ge = s.geo[min(k, stop - 1)];
-                        const int d = col - (k >= from1 ? 1 : 0) - (k >= from2 ? 1 : 0);     // column - cell: -2, 0 left, -1, 1 right
-                        w2[e] = fmaf(ge.x, st, ot) * fmaf(ge.y, sy, oy) * ((d & 1) ? ge.z : 1.0f - ge.z) * co[k < stop ? k : S::CAP];
-                        if (d >= 0) first[h] |= 0xffffu << (16 * e);
-                    }
-                    const __nv_bfloat162 hd = __floats2bfloat162_rn(w2[0], w2[1]);
-                    head[h] = *reinterpret_cast<const uint32_t*>(&hd);
-                    const __nv_bfloat162 rs = __floats2bfloat162_rn(w2[0] - __uint_as_float(head[h] << 16), w2[1] - __uint_as_float(head[h] & 0xffff0000u));
-                    rest[h] = *reinterpret_cast<const uint32_t*>(&rs);
-                }
-                const uint32_t a0 = head[0] & first[0], a1 = head[0] & ~first[0], a2 = head[1] & first[1], a3 = head[1] & ~first[1];
-                const uint32_t r0 = rest[0] & first[0], r1 = rest[0] & ~first[0], r2 = rest[1] & first[1], r3 = rest[1] & ~first[1];
-#pragma unroll
-                for (int i = 0; i < D / 16; ++i) {
-                    uint32_t b0r, b1r, b2r, b3r;
-                    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(b0r), "=r"(b1r), "=r"(b2r), "=r"(b3r) : "r"(from ^ (i << 5)));
-                    mma_bf16(c[2 * i], a0, a1, a2, a3, b0r, b1r);
-                    mma_bf16(c[2 * i + 1], a0, a1, a2, a3, b2r, b3r);
-                    mma_bf16(c[2 * i], r0, r1, r2, r3, b0r, b1r);
-                    mma_bf16(c[2 * i + 1], r0, r1, r2, r3, b2r, b3r);
-                }
+            for (int e = 0; e < 2; ++e) {
+                const int i = 2 * j + e + 8 * h;
+                const float4 ge = s.geo[warp][slot][i];
+                const uint32_t k = f + static_cast<uint32_t>(i);
+                const int d = col - (k >= from1 ? 1 : 0) - (k >= from2 ? 1 : 0);     // column - cell: -2, 0 left, -1, 1 right
+                w2[e] = fmaf(ge.x, st, ot) * fmaf(ge.y, sy, oy) * ((d & 1) ? ge.z : 1.0f - ge.z) * ge.w;
+                if (d >= 0) mine[h] |= 0xffffu << (16 * e);
             }
+            const __nv_bfloat162 hd = __floats2bfloat162_rn(w2[0], w2[1]);
+            head[h] = *reinterpret_cast<const uint32_t*>(&hd);
+            const __nv_bfloat162 rs = __floats2bfloat162_rn(w2[0] - __uint_as_float(head[h] << 16), w2[1] - __uint_as_float(head[h] & 0xffff0000u));
+            rest[h] = *reinterpret_cast<const uint32_t*>(&rs);
+        }
+        slot ^= 1;
+        const uint32_t a0 = head[0] & mine[0], a1 = head[0] & ~mine[0], a2 = head[1] & mine[1], a3 = head[1] & ~mine[1];
+        const uint32_t r0 = rest[0] & mine[0], r1 = rest[0] & ~mine[0], r2 = rest[1] & mine[1], r3 = rest[1] & ~mine[1];
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncwarp();
+        if (odds) {                                    // rows of marked samples may hold anything
+            for (int r = 0; r < 16; ++r)
+                if ((odds >> r) & 1u)
+                    for (int i = lane; i < CPR; i += 32) asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(from + r * (D * 2) + i * 16), "r"(0) : "memory");
+            __syncwarp();
+        }
+#pragma unroll
+        for (int i = 0; i < D / 16; ++i) {
+            uint32_t b0r, b1r, b2r, b3r;
+            asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(b0r), "=r"(b1r), "=r"(b2r), "=r"(b3r) : "r"((from + get) ^ (i << 5)));
+            mma_bf16(c[2 * i], a0, a1, a2, a3, b0r, b1r);
+            mma_bf16(c[2 * i + 1], a0, a1, a2, a3, b2r, b3r);
+            mma_bf16(c[2 * i], r0, r1, r2, r3, b0r, b1r);
+            mma_bf16(c[2 * i + 1], r0, r1, r2, r3, b2r, b3r);
+        }
+        if (f + 16u >= stop) {                         // the run is complete
             const int rt = b.t + (run >> 2) + ((g8 >> 1) & 1), ry = b.y + (run & 3) + (g8 & 1), rx = b.x + col;
             if (static_cast<unsigned>(rt) < static_cast<unsigned>(pr.T) && static_cast<unsigned>(ry) < static_cast<unsigned>(pr.H)) {
                 float* to = acc + ((static_cast<long long>(rt) * pr.H + ry) * pr.W + rx) * tok;
@@ -625,10 +641,11 @@ cells_sums_kernel(const bf16* __restrict__ q, const bf16* __restrict__ dout, flo
                 }
             }
             __syncwarp();
+#pragma unroll
+            for (int i = 0; i < D / 8; ++i) c[i][0] = c[i][1] = c[i][2] = c[i][3] = 0.0f;
         }
-        asm volatile("cp.async.wait_all;" ::: "memory");
-        __syncthreads();
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
 // ------------------------------------------------------------------------------------------------ beyond the bins
@@ -736,13 +753,19 @@ size_t lay_out(const Problem& pr, int m0, int heads, int f0, int f1, char* base,
     s.blocks_x = (pr.W - 1) / kBlockX + 2;
     const size_t tiles = static_cast<size_t>(heads) * s.tiles_t * s.tiles_y * s.tiles_x, samples = tiles * kRows * pr.P;
     const size_t live = static_cast<size_t>(heads) * (f1 - f0) * pr.H * pr.W * pr.P;
+    if (samples >> 32) return ~static_cast<size_t>(0);          // places are 32-bit
     size_t at = 0;
     s.geo = reinterpret_cast<uint4*>(base + at); at += round256(samples * sizeof(uint4));
     s.meta = reinterpret_cast<uint16_t*>(base + at); at += round256(samples * sizeof(uint16_t));
     s.seg = reinterpret_cast<uint32_t*>(base + at); at += round256(tiles * (kBins + 1) * sizeof(uint32_t));
+    const size_t blocks = static_cast<size_t>(heads) * s.blocks_t * s.blocks_y * s.blocks_x;
+    s.sorted = reinterpret_cast<float4*>(base + at); at += round256(live * sizeof(float4));
+    s.place = reinterpret_cast<uint32_t*>(base + at); at += round256(live * sizeof(uint32_t));
+    s.first = reinterpret_cast<uint32_t*>(base + at); at += round256(blocks * (kCells + 1) * sizeof(uint32_t));
     s.stats = reinterpret_cast<float*>(base + at); at += round256(live * 8 * sizeof(float));
     s.coef = reinterpret_cast<float2*>(base + at); at += round256(live * sizeof(float2));
-    s.marked = reinterpret_cast<int*>(base + at); at += 256;
+    s.marked = reinterpret_cast<int*>(base + at);
+    s.used = reinterpret_cast<uint32_t*>(base + at + 128); at += 256;
     return at;
 }
 
@@ -756,6 +779,7 @@ cudaError_t launch_slab(const void* q_, const void* k_, const void* v_, const fl
     cudaError_t e = cudaFuncSetAttribute(cells_bin_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bin_smem));
     if (e != cudaSuccess) return e;
     cells_bin_kernel<<<static_cast<unsigned>(tiles), kBinThreads, bin_smem, stream>>>(offsets, pr, s, inv_p);
+    cells_sort_kernel<<<static_cast<unsigned>(blocks), kSortThreads, 0, stream>>>(pr, s);
     const size_t dot_smem = sizeof(DotSmem<D>), sum_smem = sizeof(SumSmem<D>) + 256;
     e = cudaFuncSetAttribute(cells_dots_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(dot_smem));
     if (e != cudaSuccess) return e;

@@ -11,7 +11,7 @@
 // Queries come in tiles of 4 x 4 x 6 (t, y, x) of one head, cells in blocks of 4 x 4 x 3 whose rows are a box of
 // 5 x 5 x 4 positions.  Three cells along x: their corners are 4 x 4 rows, the sixteen rows of one product tile of
 // the dK / dV sums.  cells_bin_kernel sorts the samples of a tile by the block they fall into, relative to the tile
-// (bins); a block then finds its samples as one segment per (tile, bin).
+// (bins); a block finds its samples as one segment per (tile, bin), and cells_sort_kernel lays them down cell after cell.
 #pragma once
 #include "dsa3d_common.cuh"
 
@@ -37,6 +37,10 @@ struct Slab {
     uint4* geo;                                   // [tile][kRows * P]: {token, ft, fy, fx}
     uint16_t* meta;                               // [tile][kRows * P]: sample | cell in its block << 8
     uint32_t* seg;                                // [tile][kBins + 1]: start | count << 16
+    float4* sorted;                               // samples in the order of (block, cell): {ft, fy, fx, token (bits)}
+    uint32_t* place;                              // of the same sample in stats and coef
+    uint32_t* first;                              // [block][kCells + 1]: where the samples of a cell begin in `sorted`
+    uint32_t* used;                               // samples laid down so far
     float* stats;                                 // [head][frame of the slab][y][x][P][8]
     float2* coef;                                 // [head][...][P]: scale dS, alpha (sign bit: marked, see cells_query_kernel)
     int* marked;                                  // is any sample marked
