@@ -374,100 +374,86 @@ cells_dots_kernel(const bf16* __restrict__ q, const bf16* __restrict__ k, const 
 }
 
 // ------------------------------------------------------------------------------------------------ per query
-constexpr int kQueryThreads = 256;
+constexpr int kQueryWarps = 2;
 
 // alpha from the saved lse, delta, dS, dOffsets, the two coefficients per sample (ck = scale dS, cv = alpha), and
-// dQ = sum_p ck_p sum_c w_c K_c: a group of D / 8 lanes per (query, head), 16 bytes of a row per lane.  A sample with
-// anything that is not finite (its rows of q, dO, K or V, or its coefficients) is marked by the sign of cv: its
-// contributions to dK and dV are formed one by one, so that they reach only the corners with a weight.
+// dQ = sum_p ck_p sum_c w_c K_c: a warp per (query, head), 32 samples at a time, a sample per lane; the K rows are summed as
+// in the forward (dsa3d_gather.cuh).  A sample with anything that is not finite (its rows of q, dO, K or V, or its
+// coefficients) is marked by the sign of cv: its contributions to dK and dV are formed one by one, so that they reach only
+// the corners with a weight.
 template <int D>
-__global__ void __launch_bounds__(kQueryThreads, 4)
+__global__ void __launch_bounds__(kQueryWarps * 32, 16)
 cells_query_kernel(const bf16* __restrict__ k, const float* __restrict__ offsets, const float* __restrict__ lse, bf16* __restrict__ dq,
-                   float* __restrict__ doffsets, const Problem pr, const Slab sl) {
-    using E = Elt<bf16, 1>;
-    using Row = typename E::Row;
-    constexpr int LPR = D / 8;
-    const int lane = threadIdx.x & 31, gl = lane & (LPR - 1);
-    const long long per_head = static_cast<long long>(pr.H) * pr.W * (sl.f1 - sl.f0), items = per_head * sl.heads;
-    long long item = (static_cast<long long>(blockIdx.x) * kQueryThreads + threadIdx.x) / LPR;
-    const long long warp_first = (static_cast<long long>(blockIdx.x) * kQueryThreads + (threadIdx.x & ~31)) / LPR;
-    if (warp_first >= items) return;
-    const bool active = item < items;               // a trailing group repeats the last item, stores off
-    if (!active) item = items - 1;
-    const int m = sl.m0 + static_cast<int>(item / per_head);
-    const int n = static_cast<int>(static_cast<long long>(pr.H) * pr.W * sl.f0 + item % per_head);
-    const int x = n % pr.W, y = (n / pr.W) % pr.H, t = n / (pr.W * pr.H);
-    const long long row = static_cast<long long>(n) * pr.heads + m;
+                   float* __restrict__ doffsets, const __grid_constant__ Problem pr, const __grid_constant__ Slab sl, unsigned blocks_per_head) {
+    __shared__ GatherList lists[kQueryWarps];
+    constexpr int step = GatherStep<D>::N;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    GatherList& gl = lists[warp];
+    const int frame = pr.H * pr.W, mh = static_cast<int>(blockIdx.x / blocks_per_head), per_head = frame * (sl.f1 - sl.f0);
+    const int local = static_cast<int>(blockIdx.x - static_cast<unsigned>(mh) * blocks_per_head) * kQueryWarps + warp;
+    if (local >= per_head) return;
+    const int m = sl.m0 + mh, n = frame * sl.f0 + local;
+    const int x = n % pr.W, ty = n / pr.W, y = ty % pr.H, t = ty / pr.H;
+    const long long row = static_cast<long long>(n) * pr.heads + m, item = static_cast<long long>(mh) * per_head + local;
     const float scale = rsqrtf(static_cast<float>(D)), lse2 = __ldg(lse + row) * kLog2e;
     const float* off_row = offsets + row * pr.P * 3;
     const float* st_row = sl.stats + item * pr.P * 8;
-    const long long tok = static_cast<long long>(pr.heads) * D;
-    const long long sy = static_cast<long long>(pr.W) * tok, st = static_cast<long long>(pr.H) * sy;
-    const bf16* kh = k + static_cast<long long>(m) * D + gl * 8;
-    [[maybe_unused]] const long long kv_extent = pr.N * pr.heads * D;
-
-    float delta = 0.0f;
-    for (int p = gl; p < pr.P; p += LPR) {
-        const Cell c = make_cell(pr, t, y, x, p, off_row + p * 3);
-        if (c.mask == 0u) continue;                 // a dead sample has g = 0
-        const float sv = __ldg(st_row + p * 8), g = __ldg(st_row + p * 8 + 4);
-        delta = fmaf(exp2f(fmaf(sv, scale * kLog2e, -lse2)), g, delta);
+    const uint32_t tok_bytes = static_cast<uint32_t>(pr.heads) * (D * 2);
+    const bf16* kh = k + static_cast<long long>(m) * D;
+    auto sample = [&](int p, Sample& s, float4& a, float4& b) {
+        s.base = 0; s.mask = 0u; s.ft = s.fy = s.fx = 0.0f;
+        a = b = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (p >= pr.P) return;
+        s = to_sample(pr, make_cell(pr, t, y, x, p, off_row + p * 3));
+        if (s.mask == 0u) return;                   // a dead sample has g = 0
+        a = __ldg(reinterpret_cast<const float4*>(st_row + p * 8));
+        b = __ldg(reinterpret_cast<const float4*>(st_row + p * 8) + 1);
+    };
+    auto weight = [&](float sv) { return exp2f(fmaf(sv, scale * kLog2e, -lse2)); };
+    Sample s;
+    float4 a, b;
+    sample(lane, s, a, b);
+    float delta = s.mask ? weight(a.x) * b.x : 0.0f;
+    for (int p = lane + 32; p < pr.P; p += 32) {
+        Sample s2;
+        float4 a2, b2;
+        sample(p, s2, a2, b2);
+        if (s2.mask) delta = fmaf(weight(a2.x), b2.x, delta);
     }
-    delta = group_sum<LPR>(delta, kFullMask);
+    delta = group_sum<32>(delta, kFullMask);
     float acc[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) acc[e] = 0.0f;
-    for (int pb = 0; pb < pr.P; pb += LPR) {
-        Sample mine;
-        mine.base = 0; mine.mask = 0u; mine.ft = mine.fy = mine.fx = 0.0f;
-        float my_ck = 0.0f;
-        if (pb + gl < pr.P) {
-            const int p = pb + gl;
-            mine = to_sample(pr, make_cell(pr, t, y, x, p, off_row + p * 3));
-            float d0 = 0.0f, d1 = 0.0f, d2 = 0.0f;
-            if (mine.mask != 0u) {
-                const float4 a = __ldg(reinterpret_cast<const float4*>(st_row + p * 8)), b = __ldg(reinterpret_cast<const float4*>(st_row + p * 8) + 1);
-                const float alpha = exp2f(fmaf(a.x, scale * kLog2e, -lse2));
-                my_ck = scale * (alpha * (b.x - delta));
-                d0 = fmaf(my_ck, a.y, alpha * b.y);
-                d1 = fmaf(my_ck, a.z, alpha * b.z);
-                d2 = fmaf(my_ck, a.w, alpha * b.w);
-                const bool odd = !(fabsf(a.x) < INFINITY) || !(fabsf(b.x) < INFINITY) || !(fabsf(my_ck) < INFINITY) || !(alpha < INFINITY);
-                if (odd) *sl.marked = 1;
-                if (active) sl.coef[item * pr.P + p] = make_float2(my_ck, __uint_as_float(__float_as_uint(alpha) | (odd ? 0x80000000u : 0u)));
-            }
-            if (active) {
-                float* d = doffsets + (row * pr.P + p) * 3;
-                d[0] = d0; d[1] = d1; d[2] = d2;
-            }
+    for (int pb = 0; pb < pr.P; pb += 32) {
+        const int p = pb + lane;
+        if (pb > 0) sample(p, s, a, b);
+        float ck = 0.0f, d0 = 0.0f, d1 = 0.0f, d2 = 0.0f;
+        if (s.mask != 0u) {
+            const float alpha = weight(a.x);
+            ck = scale * (alpha * (b.x - delta));
+            d0 = fmaf(ck, a.y, alpha * b.y);
+            d1 = fmaf(ck, a.z, alpha * b.z);
+            d2 = fmaf(ck, a.w, alpha * b.w);
+            const bool odd = !(fabsf(a.x) < INFINITY) || !(fabsf(b.x) < INFINITY) || !(fabsf(ck) < INFINITY) || !(alpha < INFINITY);
+            if (odd) *sl.marked = 1;
+            sl.coef[item * pr.P + p] = make_float2(ck, __uint_as_float(__float_as_uint(alpha) | (odd ? 0x80000000u : 0u)));
         }
-        const int cnt = min(LPR, pr.P - pb);
-        for (int j = 0; j < cnt; ++j) {
-            const Sample s = group_bcast<LPR>(mine, j, kFullMask);
-            const float ck = __shfl_sync(kFullMask, my_ck, j, LPR);
-            const float wt[2] = {1.0f - s.ft, s.ft}, wy[2] = {1.0f - s.fy, s.fy}, wx[2] = {1.0f - s.fx, s.fx};
-            const bf16* kp4[4];
-            kp4[0] = kh + s.base * tok;
-            kp4[1] = kp4[0] + sy;
-            kp4[2] = kp4[0] + st;
-            kp4[3] = kp4[2] + sy;
-            if (s.mask == 0xffu && s.ft != 0.0f && s.fy != 0.0f && s.fx != 0.0f) {
-                Row kk[8];
-#pragma unroll
-                for (int c = 0; c < 8; ++c) kk[c] = DSA3D_IN_RANGE(pr, kp4[c >> 1] + (c & 1) * tok - k, kv_extent, 4) ? E::load(kp4[c >> 1] + (c & 1) * tok) : E::zero();
-#pragma unroll
-                for (int c = 0; c < 8; ++c) E::axpy_paired(ck * (wt[c >> 2] * wy[(c >> 1) & 1] * wx[c & 1]), kk[c], acc);
-            } else {
-#pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    const float w = wt[c >> 2] * wy[(c >> 1) & 1] * wx[c & 1];
-                    if (((s.mask >> c) & 1u) && w != 0.0f && DSA3D_IN_RANGE(pr, kp4[c >> 1] + (c & 1) * tok - k, kv_extent, 6))
-                        E::axpy_paired(ck * w, E::load(kp4[c >> 1] + (c & 1) * tok), acc);
-                }
-            }
+        if (p < pr.P) {
+            float* d = doffsets + (row * pr.P + p) * 3;
+            d[0] = d0; d[1] = d1; d[2] = d2;
         }
+        const GatherPart part = gather_list(gl, checked_corners(pr, weighted_corners(s.mask, s.ft, s.fy, s.fx), s.base, 4), s.base, pr, step);
+        const float wt[2] = {1.0f - s.ft, s.ft}, wy[2] = {1.0f - s.fy, s.fy}, wx[2] = {1.0f - s.fx, s.fx};
+        float w[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) w[c] = wt[c >> 2] * wy[(c >> 1) & 1] * wx[c & 1];
+        gather_weights(gl, part, ck, w, step);
+        __syncwarp();
+        gather_sum<D>(gl, part.total, kh, tok_bytes, acc);
+        __syncwarp();
     }
-    if (active) E::store(dq + row * D + gl * 8, acc);
+    gather_finish<D>(acc);
+    if (lane < D / 8) Elt<bf16, 1>::store(dq + row * D + lane * 8, acc);
 }
 
 // ------------------------------------------------------------------------------------------------ dK, dV
@@ -786,9 +772,8 @@ cudaError_t launch_slab(const void* q_, const void* k_, const void* v_, const fl
     cells_dots_kernel<D><<<static_cast<unsigned>(blocks), kDotThreads, dot_smem, stream>>>(q, k, v, dout, pr, s);
     const unsigned far_grid = static_cast<unsigned>(tiles / 256 + 1 < 148 * 8 ? tiles / 256 + 1 : 148 * 8);
     cells_far_kernel<D, false><<<far_grid, 256, 0, stream>>>(q, k, v, dout, offsets, acc_dk, acc_dv, pr, s, tiles);
-    const long long items = static_cast<long long>(s.heads) * (s.f1 - s.f0) * pr.H * pr.W;
-    constexpr int per_block = kQueryThreads / (D / 8);
-    cells_query_kernel<D><<<static_cast<unsigned>((items + per_block - 1) / per_block), kQueryThreads, 0, stream>>>(k, offsets, lse, static_cast<bf16*>(dq_), doffsets, pr, s);
+    const unsigned per_head = static_cast<unsigned>((static_cast<long long>(s.f1 - s.f0) * pr.H * pr.W + kQueryWarps - 1) / kQueryWarps);
+    cells_query_kernel<D><<<per_head * static_cast<unsigned>(s.heads), kQueryWarps * 32, 0, stream>>>(k, offsets, lse, static_cast<bf16*>(dq_), doffsets, pr, s, per_head);
     e = cudaFuncSetAttribute(cells_sums_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sum_smem));
     if (e != cudaSuccess) return e;
     cells_sums_kernel<D><<<static_cast<unsigned>(blocks), kSumThreads, sum_smem, stream>>>(q, dout, acc_dk, acc_dv, pr, s);

@@ -14,6 +14,7 @@
 // (bins); a block finds its samples as one segment per (tile, bin), and cells_sort_kernel lays them down cell after cell.
 #pragma once
 #include "dsa3d_common.cuh"
+#include "dsa3d_gather.cuh"
 
 namespace dsa3d {
 namespace cells {
@@ -58,11 +59,6 @@ __device__ __forceinline__ int cell_y(int cell) { return (cell / 3) & 3; }
 __device__ __forceinline__ int cell_x(int cell) { return cell % 3; }
 __device__ __forceinline__ int box_row(int cell) { return cell_t(cell) * 20 + cell_y(cell) * 4 + cell_x(cell); }
 __device__ __forceinline__ int box_step(int corner) { return (corner >> 2) * 20 + ((corner >> 1) & 1) * 4 + (corner & 1); }
-
-__device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
 
 }  // namespace cells
 }  // namespace dsa3d

@@ -1,23 +1,160 @@
-// Forward of 3D Deformable Slide Attention (Eq. 1 second term and the softmax under it).
+// Forward of 3D Deformable Slide Attention (Eq. 1 second term and the softmax under it).  Two kernels, both with an online
+// softmax in fp32; nothing of size N*P is written.  Work items are ordered head-major, neighbours along x in one
+// CTA, so that the CTAs in flight gather from one head's K / V over a few frames: L2, and L1 within a CTA, serve most rows.
 //
-// One group of LPR = d / VEC lanes owns one (token, head) item; each lane holds VEC
-// consecutive channels (16 bytes) of every row it touches.  Work items are ordered
-// head-major (item = head * N + token) so that the CTAs in flight at any time gather from
-// one head's K/V over a few neighbouring frames, which is what keeps the corner gathers in
-// L2.  Per sample: the 8 corner rows of K and of V are loaded with 16-byte loads, the
-// logit is the weighted sum of the corner dot products, and the output is accumulated with
-// an online softmax in fp32 registers; nothing of size N*P is written.
+// gather_forward_kernel (bf16, windows of more than 16 samples): a warp owns one (token, head) item and takes its samples
+// 32 at a time, one per lane.  The corner rows with a weight are listed in shared memory; q . K_corner of 16 rows is one chain
+// of m16n8k16 products, a lane adds the trilinear combination of its sample's corners to a logit, the softmax runs over
+// the lanes, and the V rows are summed with fp32 FMAs (dsa3d_gather.cuh).  What bounds it: the L1 data pipe (83 % busy on
+// 12 x 45 x 80, 8 heads of 128: 110 KB of rows per item, 5.6 cycles per 512 bytes with the misses, 4 without).
+// 32 x 45 x 80, 16 heads of 128, window (3,3,3), offsets N(0, 1.5): 11.4 -> 10.5 ms; N(0, 3): 11.7 -> 9.8; window (3,7,7) on
+// 4 x 68 x 120: 18.5 -> 9.8 ms.
 //
-// A sample whose 8 corners are all inside the grid with non-zero weights (the usual case
-// for real-valued offsets) takes a branch-free path that issues its 16 row loads back to
-// back; border samples and samples on integer positions take a per-corner path that skips
+// forward_kernel (the rest): one group of LPR = d / VEC lanes owns one item; each lane holds VEC consecutive channels
+// (16 bytes) of every row it touches.  Per sample: the 8 corner rows of K and of V are loaded with 16-byte loads, the
+// logit is the weighted sum of the corner dot products, and the output is accumulated in fp32 registers.  A sample whose 8
+// corners are all inside the grid with non-zero weights (the usual case for real-valued offsets) takes a branch-free path
+// that issues its 16 row loads back to back; border samples and samples on integer positions take a per-corner path that skips
 // corners outside the grid and corners of weight zero.
 #include "dsa3d_common.cuh"
+#include "dsa3d_gather.cuh"
 #include "dsa3d_kernels.h"
 
 namespace dsa3d {
 
 __device__ const float kZeroOffset[3] = {0.0f, 0.0f, 0.0f};     // stands in for a NULL offsets tensor
+
+// Two warps per CTA: a warp's slot is free again as soon as it is done (CTAs of 8 warps: 11.2 against 10.5 ms on 32 x 45 x 80,
+// 16 heads of 128, offsets N(0, 1.5)).
+constexpr int kFwdWarps = 2;
+
+// One item by a warp, row by row: taken when a result is not finite, so that NaN and infinity reach exactly the
+// results whose definition they enter (a product with a zero weight makes NaN of infinity).
+template <int D>
+__device__ __noinline__ void forward_item_plain(const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v, const float* offsets,
+                                                const __nv_bfloat16* addend, __nv_bfloat16* out, float* lse, const Problem& pr, int m, int t, int y, int x) {
+    constexpr int V = D / 32;
+    const int lane = threadIdx.x & 31;
+    const long long row = ((static_cast<long long>(t) * pr.H + y) * pr.W + x) * pr.heads + m, tok = static_cast<long long>(pr.heads) * D;
+    const long long sy = static_cast<long long>(pr.W) * tok, st = static_cast<long long>(pr.H) * sy;
+    float acc[V], qv[V], m_run = -INFINITY, l_run = 0.0f;
+    for (int i = 0; i < V; ++i) { acc[i] = 0.0f; qv[i] = __bfloat162float(q[row * D + lane * V + i]); }
+    for (int p = 0; p < pr.P; ++p) {
+        const Sample s = to_sample(pr, make_cell(pr, t, y, x, p, offsets ? offsets + (row * pr.P + p) * 3 : kZeroOffset));
+        const unsigned mask = weighted_corners(s.mask, s.ft, s.fy, s.fx);
+        const long long o0 = static_cast<long long>(m) * D + s.base * tok + lane * V;
+        float sdot = 0.0f;
+        for (int c = 0; c < 8; ++c) {
+            if (!((mask >> c) & 1u)) continue;
+            const float w = ((c & 4) ? s.ft : 1.0f - s.ft) * ((c & 2) ? s.fy : 1.0f - s.fy) * ((c & 1) ? s.fx : 1.0f - s.fx);
+            float dot = 0.0f;
+            for (int i = 0; i < V; ++i) dot = fmaf(qv[i], __bfloat162float(k[o0 + (c >> 2) * st + ((c >> 1) & 1) * sy + (c & 1) * tok + i]), dot);
+            sdot = fmaf(w, group_sum<32>(dot, kFullMask), sdot);
+        }
+        const float sp = sdot * rsqrtf(static_cast<float>(D)) * kLog2e;
+        if (sp > m_run) {
+            const float corr = exp2f(m_run - sp);
+            l_run *= corr;
+            for (int i = 0; i < V; ++i) acc[i] *= corr;
+            m_run = sp;
+        }
+        const float pe = exp2f(sp - m_run);
+        l_run += pe;
+        for (int c = 0; c < 8; ++c) {
+            if (!((mask >> c) & 1u)) continue;
+            const float w = pe * (((c & 4) ? s.ft : 1.0f - s.ft) * ((c & 2) ? s.fy : 1.0f - s.fy) * ((c & 1) ? s.fx : 1.0f - s.fx));
+            for (int i = 0; i < V; ++i) acc[i] = fmaf(w, __bfloat162float(v[o0 + (c >> 2) * st + ((c >> 1) & 1) * sy + (c & 1) * tok + i]), acc[i]);
+        }
+    }
+    for (int i = 0; i < V; ++i)
+        out[row * D + lane * V + i] = __float2bfloat16_rn(acc[i] / l_run + (addend ? __bfloat162float(addend[row * D + lane * V + i]) : 0.0f));
+    if (lane == 0) lse[row] = (m_run + log2f(l_run)) * kLn2;
+}
+
+template <int D, bool kAdd>
+__global__ void __launch_bounds__(kFwdWarps * 32, 16)
+gather_forward_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v,
+                      const float* __restrict__ offsets, const __nv_bfloat16* addend, __nv_bfloat16* out, float* __restrict__ lse,
+                      const __grid_constant__ Problem pr, unsigned blocks_per_head, const int* __restrict__ gate) {
+    if (gate && *gate == 0) return;                      // another kernel takes this call (see launch_forward)
+    __shared__ GatherList lists[kFwdWarps];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    GatherList& gl = lists[warp];
+    const int m = static_cast<int>(blockIdx.x / blocks_per_head);
+    const long long local = static_cast<long long>(blockIdx.x - static_cast<unsigned>(m) * blocks_per_head) * kFwdWarps + warp;
+    if (local >= pr.q_count) return;
+    const int n = static_cast<int>(pr.q_begin + local);
+    const int x = n % pr.W, ty = n / pr.W, y = ty % pr.H, t = ty / pr.H;
+    const long long row = static_cast<long long>(n) * pr.heads + m;
+    const uint32_t tok_bytes = static_cast<uint32_t>(pr.heads) * (D * 2);
+    const __nv_bfloat16 *kh = k + static_cast<long long>(m) * D, *vh = v + static_cast<long long>(m) * D;
+    const float lscale = rsqrtf(static_cast<float>(D)) * kLog2e;    // logits in log2 units
+    constexpr int step = GatherStep<D>::N;
+    float acc[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) acc[e] = 0.0f;
+    float m_run = -INFINITY, l_run = 0.0f;               // l_run: the lane's part
+    for (int pb = 0; pb < pr.P; pb += 32) {
+        const bool have = pb + lane < pr.P;
+        Sample s;
+        GatherQuery<D> qr;                               // on its way while the samples are listed
+        gather_query<D>(qr, q + row * D);
+        s.base = 0; s.mask = 0u; s.ft = s.fy = s.fx = 0.0f;
+        if (have) s = to_sample(pr, make_cell(pr, t, y, x, pb + lane, offsets ? offsets + (row * pr.P + pb + lane) * 3 : kZeroOffset));
+        const unsigned mask = checked_corners(pr, weighted_corners(s.mask, s.ft, s.fy, s.fx), s.base, 2);
+        const GatherPart part = gather_list(gl, mask, s.base, pr, step);
+        __syncwarp();
+        gather_dots<D>(gl, part.total, qr, kh, tok_bytes);
+        __syncwarp();
+        const float wt[2] = {1.0f - s.ft, s.ft}, wy[2] = {1.0f - s.fy, s.fy}, wx[2] = {1.0f - s.fx, s.fx};
+        float w[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) w[c] = wt[c >> 2] * wy[(c >> 1) & 1] * wx[c & 1];
+        float sp = gather_combine(gl, part, w);
+        sp = have ? sp * lscale : -INFINITY;             // a dead sample stays in the softmax with logit 0
+        float mx = sp;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(kFullMask, mx, o));
+        if (mx > m_run) {
+            const float corr = exp2f(m_run - mx);
+            l_run *= corr;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) acc[e] *= corr;
+            m_run = mx;
+        }
+        const float pe = have ? exp2f(sp - m_run) : 0.0f;
+        l_run += pe;
+        __syncwarp();
+        gather_weights(gl, part, pe, w, step);
+        __syncwarp();
+        gather_sum<D>(gl, part.total, vh, tok_bytes, acc);
+        __syncwarp();
+    }
+    l_run = group_sum<32>(l_run, kFullMask);
+    const float inv = 1.0f / l_run;
+    bool bad = !(l_run < INFINITY);
+    gather_finish<D>(acc);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        acc[e] *= inv;
+        bad = bad || !(fabsf(acc[e]) < INFINITY);
+    }
+    if (__any_sync(kFullMask, bad)) {
+        forward_item_plain<D>(q, k, v, offsets, kAdd ? addend : nullptr, out, lse, pr, m, t, y, x);
+        return;
+    }
+    if (lane < D / 8) {
+        using E = Elt<__nv_bfloat16, 1>;
+        if constexpr (kAdd) {                            // first term of Eq. 1, added before the rounding
+            float add[8];
+            E::to_float(E::load(addend + row * D + lane * 8), add);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) acc[e] += add[e];
+        }
+        E::store(out + row * D + lane * 8, acc);
+    }
+    if (lane == 0) lse[row] = (m_run + log2f(l_run)) * kLn2;
+}
 
 #ifndef DSA3D_FWD_MINBLOCKS
 #define DSA3D_FWD_MINBLOCKS 3
@@ -202,6 +339,23 @@ forward_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __rest
 template <typename T, int D> struct FwdLaneWidth { static constexpr int NV = 1; };
 template <> struct FwdLaneWidth<__nv_bfloat16, 128> { static constexpr int NV = DSA3D_FWD_BF16_NV; };
 
+template <int D>
+static cudaError_t launch_gather_forward(const void* q, const void* k, const void* v, const float* offsets, const void* addend, void* out,
+                                         float* lse, const Problem& pr, cudaStream_t stream, const int* gate) {
+    using T = __nv_bfloat16;
+    const long long per_head = (pr.q_count + kFwdWarps - 1) / kFwdWarps;
+    const unsigned blocks = static_cast<unsigned>(per_head * pr.heads);
+    if (addend)
+        gather_forward_kernel<D, true><<<blocks, kFwdWarps * 32, 0, stream>>>(
+            static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v), offsets, static_cast<const T*>(addend),
+            static_cast<T*>(out), lse, pr, static_cast<unsigned>(per_head), gate);
+    else
+        gather_forward_kernel<D, false><<<blocks, kFwdWarps * 32, 0, stream>>>(
+            static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v), offsets, nullptr, static_cast<T*>(out), lse, pr,
+            static_cast<unsigned>(per_head), gate);
+    return cudaGetLastError();
+}
+
 template <typename T, int D>
 static cudaError_t launch_forward_t(const void* q, const void* k, const void* v, const float* offsets,
                                     const void* addend, void* out, float* lse, const Problem& pr,
@@ -224,10 +378,16 @@ static cudaError_t launch_forward_t(const void* q, const void* k, const void* v,
 
 cudaError_t launch_forward(const void* q, const void* k, const void* v, const float* offsets, const void* addend,
                            void* out, float* lse, const Problem& pr, bool bf16, cudaStream_t stream, const int* gate) {
+    // A warp of gather_forward_kernel takes 32 samples of one item at a time: with 16 samples or fewer half its lanes are idle, and
+    // at 32 channels with 32 samples or fewer its fixed cost per item is as much as the row traffic it saves.  Measured against
+    // the other kernel: window (2,2,2) 0.5 - 0.9x, (3,3,3) 1.02 - 1.22x at 128 channels, 1.08 - 1.11x at 64, 0.96x at 32,
+    // (3,7,7) 1.9x; grids of a few hundred tokens 1.5x.
+    const bool warp_per_item = bf16 && pr.P > (pr.d == 32 ? 32 : 16);
 #define DSA3D_CASE(DD)                                                                                    \
     case DD:                                                                                              \
-        return bf16 ? launch_forward_t<__nv_bfloat16, DD>(q, k, v, offsets, addend, out, lse, pr, stream, gate)   \
-                    : launch_forward_t<float, DD>(q, k, v, offsets, addend, out, lse, pr, stream, gate);
+        return warp_per_item ? launch_gather_forward<DD>(q, k, v, offsets, addend, out, lse, pr, stream, gate)    \
+               : bf16 ? launch_forward_t<__nv_bfloat16, DD>(q, k, v, offsets, addend, out, lse, pr, stream, gate) \
+                      : launch_forward_t<float, DD>(q, k, v, offsets, addend, out, lse, pr, stream, gate);
     switch (pr.d) {
         DSA3D_CASE(32)
         DSA3D_CASE(64)
