@@ -245,9 +245,9 @@ cells_sort_kernel(const Problem pr, const Slab sl) {
 }
 
 // Byte of 16-byte chunk `chunk` of box row `row` in shared memory: rows of 128 bytes and more have their chunks permuted by
-// the row's parity, so that the four chunks a quarter-warp reads of two neighbouring rows lie in different banks.
+// the row's parity, so that the four even (or odd) chunks a quarter-warp reads of two neighbouring rows lie in different banks.
 template <int D> __device__ __forceinline__ int box_byte(int row, int chunk) {
-    return row * (D * 2) + ((D >= 64 ? (chunk ^ ((row & 1) << 2)) : chunk) << 4);
+    return row * (D * 2) + ((D >= 64 ? (chunk ^ (row & 1)) : chunk) << 4);
 }
 
 // The rows of a block's box of one tensor into shared memory, zeros outside the grid.
@@ -289,8 +289,20 @@ __device__ __forceinline__ float trilerp_lanes(float s0, float s1, int j, float 
     return (odd ? r1 : r0) + __shfl_xor_sync(kFullMask, odd ? r0 : r1, 1);
 }
 
+// 32 bytes of a row (16 where I = 1).  One 32-byte load where the tensor's alignment allows: a quarter-warp then reads whole 128-byte
+// lines, while two 16-byte loads meet in the same banks (8 data-pipe cycles per 512 bytes against 4).
+template <bool kWide, int I> __device__ __forceinline__ void load_piece(const uint4* p, uint4* r) {
+    if constexpr (kWide && I > 1) {
+        asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=r"(r[0].x), "=r"(r[0].y), "=r"(r[0].z), "=r"(r[0].w), "=r"(r[1].x), "=r"(r[1].y), "=r"(r[1].z), "=r"(r[1].w) : "l"(p));
+    } else {
+        r[0] = __ldg(p);
+        if constexpr (I > 1) r[1] = __ldg(p + 1);
+    }
+}
+
 // q . K and dO . V with derivatives, eight numbers per sample into stats; even warps take q . K, odd ones dO . V.
-template <int D>
+template <int D, bool kWide>
 __global__ void __launch_bounds__(kDotThreads, D == 128 ? 3 : 4)
 cells_dots_kernel(const bf16* __restrict__ q, const bf16* __restrict__ k, const bf16* __restrict__ v, const bf16* __restrict__ dout,
                   const Problem pr, const Slab sl) {
@@ -319,7 +331,7 @@ cells_dots_kernel(const bf16* __restrict__ q, const bf16* __restrict__ k, const 
     load_box<D, kDotThreads>(s.box[0], k, b, pr);
     load_box<D, kDotThreads>(s.box[1], v, b, pr);
     __syncthreads();
-    const bf16* src = (tensor ? dout : q) + static_cast<long long>(b.m) * D + j * 8;
+    const bf16* src = (tensor ? dout : q) + static_cast<long long>(b.m) * D + j * (I > 1 ? 16 : 8);
     const unsigned char* box = s.box[tensor];
     const long long tok = static_cast<long long>(pr.heads) * D;
     const int groups = static_cast<int>(s.groups[kCells]);
@@ -348,13 +360,13 @@ cells_dots_kernel(const bf16* __restrict__ q, const bf16* __restrict__ k, const 
         const int row = box_row(cell) + box_step(g8);
         const uint4* ra_p = reinterpret_cast<const uint4*>(src + __float_as_int(ga.w) * tok);
         const uint4* rb_p = reinterpret_cast<const uint4*>(src + __float_as_int(gb.w) * tok);
-        // The order of the channels inside a product is free: lane j takes chunk j of every 64 bytes, whole
-        // 16-byte pieces on both sides.
+        // The order of the channels inside a product is free: lane j takes bytes 32 j .. of every 128 (chunk j of
+        // the 64 of a 32-channel row), whole pieces on both sides.
         uint4 ra[I], rb[I];
 #pragma unroll
-        for (int i = 0; i < I; ++i) {
-            ra[i] = __ldg(ra_p + 4 * i);
-            rb[i] = __ldg(rb_p + 4 * i);
+        for (int i = 0; i < I; i += 2) {
+            load_piece<kWide, I>(ra_p + (I > 1 ? 4 * i : 0), ra + i);
+            load_piece<kWide, I>(rb_p + (I > 1 ? 4 * i : 0), rb + i);
         }
         const float fa0 = ga.x, fa1 = ga.y, fa2 = ga.z, fb0 = gb.x, fb1 = gb.y, fb2 = gb.z;
         float* da = live_a ? out + static_cast<size_t>(pa) * 8 : nullptr;
@@ -363,7 +375,7 @@ cells_dots_kernel(const bf16* __restrict__ q, const bf16* __restrict__ k, const 
         float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
         for (int i = 0; i < I; ++i) {
-            const uint4 kb = *reinterpret_cast<const uint4*>(box + box_byte<D>(row, 4 * i + j));
+            const uint4 kb = *reinterpret_cast<const uint4*>(box + box_byte<D>(row, I > 1 ? (i >> 1) * 8 + 2 * j + (i & 1) : j));
             mma_bf16(c, ra[i].x, rb[i].x, ra[i].y, rb[i].y, kb.x, kb.y);
             mma_bf16(c, ra[i].z, rb[i].z, ra[i].w, rb[i].w, kb.z, kb.w);
         }
@@ -556,6 +568,7 @@ cells_sums_kernel(const bf16* __restrict__ q, const bf16* __restrict__ dout, flo
     samples();
     uint32_t stage3 = stage0;
     int slot = 0;
+    uint32_t used_a = 0u, used_b = 0u;                 // weights the lane has put into its two rows of the run
     float c[D / 8][4];
 #pragma unroll
     for (int i = 0; i < D / 8; ++i) c[i][0] = c[i][1] = c[i][2] = c[i][3] = 0.0f;
@@ -593,6 +606,8 @@ cells_sums_kernel(const bf16* __restrict__ q, const bf16* __restrict__ dout, flo
             rest[h] = *reinterpret_cast<const uint32_t*>(&rs);
         }
         slot ^= 1;
+        used_a |= (head[0] & mine[0]) | (head[1] & mine[1]);
+        used_b |= (head[0] & ~mine[0]) | (head[1] & ~mine[1]);
         const uint32_t a0 = head[0] & mine[0], a1 = head[0] & ~mine[0], a2 = head[1] & mine[1], a3 = head[1] & ~mine[1];
         const uint32_t r0 = rest[0] & mine[0], r1 = rest[0] & ~mine[0], r2 = rest[1] & mine[1], r3 = rest[1] & ~mine[1];
         asm volatile("cp.async.wait_group 1;" ::: "memory");
@@ -614,14 +629,17 @@ cells_sums_kernel(const bf16* __restrict__ q, const bf16* __restrict__ dout, flo
         }
         if (f + 16u >= stop) {                         // the run is complete
             const int rt = b.t + (run >> 2) + ((g8 >> 1) & 1), ry = b.y + (run & 3) + (g8 & 1), rx = b.x + col;
+            // rows that no sample has a weight for (most of them when offsets are integers) are left alone
+            const unsigned any_a = __ballot_sync(kFullMask, used_a != 0u) >> (lane & 28), any_b = __ballot_sync(kFullMask, used_b != 0u) >> (lane & 28);
+            used_a = used_b = 0u;
             if (static_cast<unsigned>(rt) < static_cast<unsigned>(pr.T) && static_cast<unsigned>(ry) < static_cast<unsigned>(pr.H)) {
                 float* to = acc + ((static_cast<long long>(rt) * pr.H + ry) * pr.W + rx) * tok;
-                if (static_cast<unsigned>(rx) < static_cast<unsigned>(pr.W) && DSA3D_IN_RANGE(pr, to - (tensor ? acc_dv : acc_dk), kv_extent, 10)) {
+                if ((any_a & 15u) && static_cast<unsigned>(rx) < static_cast<unsigned>(pr.W) && DSA3D_IN_RANGE(pr, to - (tensor ? acc_dv : acc_dk), kv_extent, 10)) {
 #pragma unroll
                     for (int i = 0; i < D / 8; ++i) red_add_v2(to + 8 * i, c[i][0], c[i][1]);
                 }
                 to += 2 * tok;
-                if (static_cast<unsigned>(rx + 2) < static_cast<unsigned>(pr.W) && DSA3D_IN_RANGE(pr, to - (tensor ? acc_dv : acc_dk), kv_extent, 10)) {
+                if ((any_b & 15u) && static_cast<unsigned>(rx + 2) < static_cast<unsigned>(pr.W) && DSA3D_IN_RANGE(pr, to - (tensor ? acc_dv : acc_dk), kv_extent, 10)) {
 #pragma unroll
                     for (int i = 0; i < D / 8; ++i) red_add_v2(to + 8 * i, c[i][2], c[i][3]);
                 }
@@ -767,9 +785,11 @@ cudaError_t launch_slab(const void* q_, const void* k_, const void* v_, const fl
     cells_bin_kernel<<<static_cast<unsigned>(tiles), kBinThreads, bin_smem, stream>>>(offsets, pr, s, inv_p);
     cells_sort_kernel<<<static_cast<unsigned>(blocks), kSortThreads, 0, stream>>>(pr, s);
     const size_t dot_smem = sizeof(DotSmem<D>), sum_smem = sizeof(SumSmem<D>) + 256;
-    e = cudaFuncSetAttribute(cells_dots_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(dot_smem));
+    const bool wide = ((reinterpret_cast<uintptr_t>(q) | reinterpret_cast<uintptr_t>(dout)) & 31u) == 0;
+    auto dots = wide ? cells_dots_kernel<D, true> : cells_dots_kernel<D, false>;
+    e = cudaFuncSetAttribute(dots, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(dot_smem));
     if (e != cudaSuccess) return e;
-    cells_dots_kernel<D><<<static_cast<unsigned>(blocks), kDotThreads, dot_smem, stream>>>(q, k, v, dout, pr, s);
+    dots<<<static_cast<unsigned>(blocks), kDotThreads, dot_smem, stream>>>(q, k, v, dout, pr, s);
     const unsigned far_grid = static_cast<unsigned>(tiles / 256 + 1 < 148 * 8 ? tiles / 256 + 1 : 148 * 8);
     cells_far_kernel<D, false><<<far_grid, 256, 0, stream>>>(q, k, v, dout, offsets, acc_dk, acc_dv, pr, s, tiles);
     const unsigned per_head = static_cast<unsigned>((static_cast<long long>(s.f1 - s.f0) * pr.H * pr.W + kQueryWarps - 1) / kQueryWarps);
