@@ -392,18 +392,22 @@ constexpr int kQueryWarps = 2;
 // dQ = sum_p ck_p sum_c w_c K_c: a warp per (query, head), 32 samples at a time, a sample per lane; the K rows are summed as
 // in the forward (dsa3d_gather.cuh).  A sample with anything that is not finite (its rows of q, dO, K or V, or its
 // coefficients) is marked by the sign of cv: its contributions to dK and dV are formed one by one, so that they reach only
-// the corners with a weight.
-template <int D>
+// the corners with a weight.  Windows of at most 8 (16) samples: G = 4 (2) neighbouring queries share a warp.
+template <int D, int G>
 __global__ void __launch_bounds__(kQueryWarps * 32, 16)
 cells_query_kernel(const bf16* __restrict__ k, const float* __restrict__ offsets, const float* __restrict__ lse, bf16* __restrict__ dq,
                    float* __restrict__ doffsets, const __grid_constant__ Problem pr, const __grid_constant__ Slab sl, unsigned blocks_per_head) {
     __shared__ GatherList lists[kQueryWarps];
-    constexpr int step = GatherStep<D>::N;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int L = 32 / G;                       // lanes per query
+    constexpr int U = GatherStep<D>::U, PER = U > G ? U / G : 1, ITEMS = G > U ? G / U : 1;      // subgroups per query, queries per subgroup
+    constexpr int step = G == 1 ? GatherStep<D>::N : 4 * PER;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gl_lane = lane & (L - 1);
     GatherList& gl = lists[warp];
     const int frame = pr.H * pr.W, mh = static_cast<int>(blockIdx.x / blocks_per_head), per_head = frame * (sl.f1 - sl.f0);
-    const int local = static_cast<int>(blockIdx.x - static_cast<unsigned>(mh) * blocks_per_head) * kQueryWarps + warp;
-    if (local >= per_head) return;
+    const int warp_first = (static_cast<int>(blockIdx.x - static_cast<unsigned>(mh) * blocks_per_head) * kQueryWarps + warp) * G;
+    if (warp_first >= per_head) return;
+    const bool active = warp_first + lane / L < per_head;        // a query past the end repeats the last one, stores off
+    const int local = active ? warp_first + lane / L : per_head - 1;
     const int m = sl.m0 + mh, n = frame * sl.f0 + local;
     const int x = n % pr.W, ty = n / pr.W, y = ty % pr.H, t = ty / pr.H;
     const long long row = static_cast<long long>(n) * pr.heads + m, item = static_cast<long long>(mh) * per_head + local;
@@ -424,20 +428,20 @@ cells_query_kernel(const bf16* __restrict__ k, const float* __restrict__ offsets
     auto weight = [&](float sv) { return exp2f(fmaf(sv, scale * kLog2e, -lse2)); };
     Sample s;
     float4 a, b;
-    sample(lane, s, a, b);
+    sample(gl_lane, s, a, b);
     float delta = s.mask ? weight(a.x) * b.x : 0.0f;
-    for (int p = lane + 32; p < pr.P; p += 32) {
+    for (int p = gl_lane + L; p < pr.P; p += L) {   // (one sample per lane when G > 1)
         Sample s2;
         float4 a2, b2;
         sample(p, s2, a2, b2);
         if (s2.mask) delta = fmaf(weight(a2.x), b2.x, delta);
     }
-    delta = group_sum<32>(delta, kFullMask);
+    delta = group_sum<L>(delta, kFullMask);
     float acc[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) acc[e] = 0.0f;
-    for (int pb = 0; pb < pr.P; pb += 32) {
-        const int p = pb + lane;
+    for (int pb = 0; pb < pr.P; pb += L) {
+        const int p = pb + gl_lane;
         if (pb > 0) sample(p, s, a, b);
         float ck = 0.0f, d0 = 0.0f, d1 = 0.0f, d2 = 0.0f;
         if (s.mask != 0u) {
@@ -448,24 +452,45 @@ cells_query_kernel(const bf16* __restrict__ k, const float* __restrict__ offsets
             d2 = fmaf(ck, a.w, alpha * b.w);
             const bool odd = !(fabsf(a.x) < INFINITY) || !(fabsf(b.x) < INFINITY) || !(fabsf(ck) < INFINITY) || !(alpha < INFINITY);
             if (odd) *sl.marked = 1;
-            sl.coef[item * pr.P + p] = make_float2(ck, __uint_as_float(__float_as_uint(alpha) | (odd ? 0x80000000u : 0u)));
+            if (active) sl.coef[item * pr.P + p] = make_float2(ck, __uint_as_float(__float_as_uint(alpha) | (odd ? 0x80000000u : 0u)));
         }
-        if (p < pr.P) {
+        if (active && p < pr.P) {
             float* d = doffsets + (row * pr.P + p) * 3;
             d[0] = d0; d[1] = d1; d[2] = d2;
         }
-        const GatherPart part = gather_list(gl, checked_corners(pr, weighted_corners(s.mask, s.ft, s.fy, s.fx), s.base, 4), s.base, pr, step);
+        const GatherPart part = gather_list<G>(gl, checked_corners(pr, weighted_corners(s.mask, s.ft, s.fy, s.fx), s.base, 4), s.base, pr, step);
         const float wt[2] = {1.0f - s.ft, s.ft}, wy[2] = {1.0f - s.fy, s.fy}, wx[2] = {1.0f - s.fx, s.fx};
         float w[8];
 #pragma unroll
         for (int c = 0; c < 8; ++c) w[c] = wt[c >> 2] * wy[(c >> 1) & 1] * wx[c & 1];
-        gather_weights(gl, part, ck, w, step);
+        gather_weights<G>(gl, part, ck, w, step);
         __syncwarp();
-        gather_sum<D>(gl, part.total, kh, tok_bytes, acc);
+        if constexpr (G == 1) {
+            gather_sum<D>(gl, part.total, kh, tok_bytes, acc);
+        } else {
+            constexpr int LPR = GatherStep<D>::LPR;
+#pragma unroll
+            for (int i = 0; i < ITEMS; ++i) {
+                const int u = lane / LPR, it = PER > 1 ? u / PER : u * ITEMS + i;
+                const int total = __shfl_sync(kFullMask, part.total, it * L);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) acc[e] = 0.0f;
+                gather_sum_item<D, PER>(gl, it * (kGatherRows / G), total, PER > 1 ? u % PER : 0, kh, tok_bytes, acc);
+                __syncwarp();
+#pragma unroll
+                for (int o = LPR; o < LPR * PER; o <<= 1)
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) acc[e] += __shfl_xor_sync(kFullMask, acc[e], o);
+                if (warp_first + it < per_head && (PER == 1 || u % PER == 0))
+                    Elt<bf16, 1>::store(dq + (static_cast<long long>(frame * sl.f0 + warp_first + it) * pr.heads + m) * D + (lane % LPR) * 8, acc);
+            }
+        }
         __syncwarp();
     }
-    gather_finish<D>(acc);
-    if (lane < D / 8) Elt<bf16, 1>::store(dq + row * D + lane * 8, acc);
+    if constexpr (G == 1) {
+        gather_finish<D>(acc);
+        if (lane < D / 8) Elt<bf16, 1>::store(dq + row * D + lane * 8, acc);
+    }
 }
 
 // ------------------------------------------------------------------------------------------------ dK, dV
@@ -792,8 +817,11 @@ cudaError_t launch_slab(const void* q_, const void* k_, const void* v_, const fl
     dots<<<static_cast<unsigned>(blocks), kDotThreads, dot_smem, stream>>>(q, k, v, dout, pr, s);
     const unsigned far_grid = static_cast<unsigned>(tiles / 256 + 1 < 148 * 8 ? tiles / 256 + 1 : 148 * 8);
     cells_far_kernel<D, false><<<far_grid, 256, 0, stream>>>(q, k, v, dout, offsets, acc_dk, acc_dv, pr, s, tiles);
-    const unsigned per_head = static_cast<unsigned>((static_cast<long long>(s.f1 - s.f0) * pr.H * pr.W + kQueryWarps - 1) / kQueryWarps);
-    cells_query_kernel<D><<<per_head * static_cast<unsigned>(s.heads), kQueryWarps * 32, 0, stream>>>(k, offsets, lse, static_cast<bf16*>(dq_), doffsets, pr, s, per_head);
+    // As many queries per warp as have a lane for every sample.
+    const int share = pr.P <= 8 ? 4 : pr.P <= 16 ? 2 : 1, per_block = kQueryWarps * share;
+    const unsigned per_head = static_cast<unsigned>((static_cast<long long>(s.f1 - s.f0) * pr.H * pr.W + per_block - 1) / per_block);
+    auto query = share == 4 ? cells_query_kernel<D, 4> : share == 2 ? cells_query_kernel<D, 2> : cells_query_kernel<D, 1>;
+    query<<<per_head * static_cast<unsigned>(s.heads), kQueryWarps * 32, 0, stream>>>(k, offsets, lse, static_cast<bf16*>(dq_), doffsets, pr, s, per_head);
     e = cudaFuncSetAttribute(cells_sums_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sum_smem));
     if (e != cudaSuccess) return e;
     cells_sums_kernel<D><<<static_cast<unsigned>(blocks), kSumThreads, sum_smem, stream>>>(q, dout, acc_dk, acc_dv, pr, s);

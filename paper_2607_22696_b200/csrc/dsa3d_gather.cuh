@@ -49,16 +49,21 @@ __device__ __forceinline__ unsigned checked_corners(const Problem& pr, unsigned 
 // two aligned 16-byte pieces.
 struct GatherPart { int first, total; unsigned mask; bool whole; };
 
-// Lists the corners `mask` of every lane's sample (corner (0,0,0) at linear index `base`), padded to a multiple of `step` with the last row.
+// G items of 32 / G samples share a warp: item i has entries i * kGatherRows / G on.  Lists the corners `mask` of every lane's sample
+// (corner (0,0,0) at linear index `base`), each item's padded to a multiple of `step` (<= 32 / G) with its last row;
+// `total`: entries of the lane's item.
+template <int G = 1>
 __device__ __forceinline__ GatherPart gather_list(GatherList& gl, unsigned mask, int base, const Problem& pr, int step) {
+    constexpr int L = 32 / G;
     const int lane = threadIdx.x & 31, n = __popc(mask), sy = pr.W, st = pr.H * pr.W;
+    const int lane0 = lane & ~(L - 1), region = (lane / L) * (kGatherRows / G);
     GatherPart part;
     part.mask = mask;
     part.whole = __all_sync(kFullMask, n == 8 || n == 0);
-    const unsigned have = __ballot_sync(kFullMask, n > 0);
+    const unsigned have = (__ballot_sync(kFullMask, n > 0) >> lane0) & (L == 32 ? 0xffffffffu : (1u << L) - 1u);
     int last = 0;
     if (part.whole) {
-        part.first = 8 * __popc(have & ((1u << lane) - 1u));
+        part.first = region + 8 * __popc(have & ((1u << (lane - lane0)) - 1u));
         part.total = 8 * __popc(have);
         last = base + st + sy + 1;
         if (n) {
@@ -69,12 +74,12 @@ __device__ __forceinline__ GatherPart gather_list(GatherList& gl, unsigned mask,
     } else {
         int incl = n;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int up = __shfl_up_sync(kFullMask, incl, o);
-            if (lane >= o) incl += up;
+        for (int o = 1; o < L; o <<= 1) {
+            const int up = __shfl_up_sync(kFullMask, incl, o, L);
+            if (lane - lane0 >= o) incl += up;
         }
-        part.total = __shfl_sync(kFullMask, incl, 31);
-        part.first = incl - n;
+        part.total = __shfl_sync(kFullMask, incl, L - 1, L);
+        part.first = region + incl - n;
         int at = part.first;
 #pragma unroll
         for (int c = 0; c < 8; ++c)
@@ -83,9 +88,9 @@ __device__ __forceinline__ GatherPart gather_list(GatherList& gl, unsigned mask,
                 gl.token[at++] = static_cast<uint32_t>(last);
             }
     }
-    last = __shfl_sync(kFullMask, last, have ? 31 - __clz(static_cast<int>(have)) : 0);
-    const int pad = part.total + lane;
-    if (lane < step && pad < (part.total + step - 1) / step * step) gl.token[pad] = static_cast<uint32_t>(last);
+    last = __shfl_sync(kFullMask, last, have ? 31 - __clz(static_cast<int>(have)) : 0, L);
+    const int pad = part.total + lane - lane0;
+    if (pad < (part.total + step - 1) / step * step) gl.token[region + pad] = static_cast<uint32_t>(last);
     return part;
 }
 
@@ -105,6 +110,7 @@ __device__ __forceinline__ float gather_combine(const GatherList& gl, const Gath
     }
     return sum;
 }
+template <int G = 1>
 __device__ __forceinline__ void gather_weights(GatherList& gl, const GatherPart& part, float s, const float (&w)[8], int step) {
     if (part.whole) {
         if (part.mask) {
@@ -118,8 +124,9 @@ __device__ __forceinline__ void gather_weights(GatherList& gl, const GatherPart&
         for (int c = 0; c < 8; ++c)
             if ((part.mask >> c) & 1u) gl.value[at++] = s * w[c];
     }
-    const int lane = threadIdx.x & 31, pad = part.total + lane;
-    if (lane < step && pad < (part.total + step - 1) / step * step) gl.value[pad] = 0.0f;
+    constexpr int L = 32 / G;
+    const int lane = threadIdx.x & 31, pad = part.total + (lane & (L - 1));
+    if (pad < (part.total + step - 1) / step * step) gl.value[(lane / L) * (kGatherRows / G) + pad] = 0.0f;
 }
 
 // 16 rows: those of entries s + g (a) and s + 8 + g (b).
@@ -197,6 +204,27 @@ _Pragma("unroll 1")
             E::axpy_paired(w.z, r[4 * b + 2], acc);
             E::axpy_paired(w.w, r[4 * b + 3], acc);
         }
+    }
+}
+
+// The same for the item whose entries start at `region` by PER neighbouring subgroups of the warp (`sub`: which of them this is); the
+// list is padded to a multiple of 4 * PER.
+template <int D, int PER>
+__device__ __forceinline__ void gather_sum_item(const GatherList& gl, int region, int total, int sub, const __nv_bfloat16* __restrict__ rows, uint32_t tok_bytes,
+                                                float (&acc)[8]) {
+    using E = Elt<__nv_bfloat16, 1>;
+    const char* src = reinterpret_cast<const char*>(rows) + ((threadIdx.x & 31) % GatherStep<D>::LPR) * 16;
+    for (int s = region + sub * 4; s < region + total; s += 4 * PER) {
+        const uint4 t = *reinterpret_cast<const uint4*>(gl.token + s);
+        const uint32_t tk[4] = {t.x, t.y, t.z, t.w};
+        E::Row r[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) r[i] = E::load(reinterpret_cast<const __nv_bfloat16*>(src + static_cast<uint64_t>(tk[i]) * tok_bytes));
+        const float4 w = *reinterpret_cast<const float4*>(gl.value + s);
+        E::axpy_paired(w.x, r[0], acc);
+        E::axpy_paired(w.y, r[1], acc);
+        E::axpy_paired(w.z, r[2], acc);
+        E::axpy_paired(w.w, r[3], acc);
     }
 }
 
