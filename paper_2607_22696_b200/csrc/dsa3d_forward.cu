@@ -2,7 +2,7 @@
 // softmax in fp32; nothing of size N*P is written.  Work items are ordered head-major, neighbours along x in one
 // CTA, so that the CTAs in flight gather from one head's K / V over a few frames: L2, and L1 within a CTA, serve most rows.
 //
-// gather_forward_kernel (bf16, windows of more than 16 samples): a warp owns one (token, head) item and takes its samples
+// gather_forward_kernel (bf16): a warp owns one (token, head) item and takes its samples
 // 32 at a time, one per lane.  The corner rows with a weight are listed in shared memory; q . K_corner of 16 rows is one chain
 // of m16n8k16 products, a lane adds the trilinear combination of its sample's corners to a logit, the softmax runs over
 // the lanes, and the V rows are summed with fp32 FMAs (dsa3d_gather.cuh).  What bounds it: the L1 data pipe (83 % busy on
@@ -10,7 +10,10 @@
 // 32 x 45 x 80, 16 heads of 128, window (3,3,3), offsets N(0, 1.5): 11.4 -> 10.5 ms; N(0, 3): 11.7 -> 9.8; window (3,7,7) on
 // 4 x 68 x 120: 18.5 -> 9.8 ms.
 //
-// forward_kernel (the rest): one group of LPR = d / VEC lanes owns one item; each lane holds VEC consecutive channels
+// (gather_forward_small_kernel: the same for two or four items per warp where the window is small: 32 x 45 x 80, 16 heads of 128, window
+// (2,2,2): 3.83 -> 3.24 ms, integer offsets 1.25 -> 0.94 ms.)
+//
+// forward_kernel (fp32; bf16 with 32 channels and few samples): one group of LPR = d / VEC lanes owns one item; each lane holds VEC consecutive channels
 // (16 bytes) of every row it touches.  Per sample: the 8 corner rows of K and of V are loaded with 16-byte loads, the
 // logit is the weighted sum of the corner dot products, and the output is accumulated in fp32 registers.  A sample whose 8
 // corners are all inside the grid with non-zero weights (the usual case for real-valued offsets) takes a branch-free path
@@ -154,6 +157,105 @@ gather_forward_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* 
         E::store(out + row * D + lane * 8, acc);
     }
     if (lane == 0) lse[row] = (m_run + log2f(l_run)) * kLn2;
+}
+
+// Windows of at most 8 (G = 4) or 16 (G = 2) samples: G neighbouring items share a warp, 32 / G lanes each, so that one trip
+// through list, products and softmax serves them all.
+template <int D, int G, bool kAdd>
+__global__ void __launch_bounds__(kFwdWarps * 32, 16)
+gather_forward_small_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v,
+                            const float* __restrict__ offsets, const __nv_bfloat16* addend, __nv_bfloat16* out, float* __restrict__ lse,
+                            const __grid_constant__ Problem pr, unsigned blocks_per_head, const int* __restrict__ gate) {
+    if (gate && *gate == 0) return;
+    using E = Elt<__nv_bfloat16, 1>;
+    constexpr int L = 32 / G, LPR = GatherStep<D>::LPR, U = GatherStep<D>::U;
+    constexpr int PER = U > G ? U / G : 1, ITEMS = G > U ? G / U : 1;        // subgroups per item, items per subgroup
+    constexpr int step = 4 * PER > 8 ? 4 * PER : 8, region = kGatherRows / G;
+    static_assert(step <= L, "a lane per padding entry");
+    __shared__ GatherList lists[kFwdWarps];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, p = lane & (L - 1);
+    GatherList& gl = lists[warp];
+    const int m = static_cast<int>(blockIdx.x / blocks_per_head);
+    const long long warp_first = (static_cast<long long>(blockIdx.x - static_cast<unsigned>(m) * blocks_per_head) * kFwdWarps + warp) * G;
+    if (warp_first >= pr.q_count) return;
+    const int items = static_cast<int>(min(static_cast<long long>(G), pr.q_count - warp_first));      // an item past the end repeats the last one, stores off
+    const int mine = min(lane / L, items - 1), n0 = static_cast<int>(pr.q_begin + warp_first), n = n0 + mine;
+    const int x = n % pr.W, ty = n / pr.W, y = ty % pr.H, t = ty / pr.H;
+    const long long row = static_cast<long long>(n) * pr.heads + m, row0 = static_cast<long long>(n0) * pr.heads + m;
+    const uint32_t tok_bytes = static_cast<uint32_t>(pr.heads) * (D * 2);
+    const __nv_bfloat16 *kh = k + static_cast<long long>(m) * D, *vh = v + static_cast<long long>(m) * D;
+    const bool have = p < pr.P;
+    Sample s;
+    s.base = 0; s.mask = 0u; s.ft = s.fy = s.fx = 0.0f;
+    if (have) s = to_sample(pr, make_cell(pr, t, y, x, p, offsets ? offsets + (row * pr.P + p) * 3 : kZeroOffset));
+    const GatherPart part = gather_list<G>(gl, checked_corners(pr, weighted_corners(s.mask, s.ft, s.fy, s.fx), s.base, 2), s.base, pr, step);
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < G; i += 2) {
+        const int ta = __shfl_sync(kFullMask, part.total, i * L), tb = __shfl_sync(kFullMask, part.total, (i + 1) * L);
+        gather_dots_pair<D>(gl, i * region, ta, (i + 1) * region, tb, q + (row0 + static_cast<long long>(min(i, items - 1)) * pr.heads) * D,
+                            q + (row0 + static_cast<long long>(min(i + 1, items - 1)) * pr.heads) * D, kh, tok_bytes);
+    }
+    __syncwarp();
+    const float wt[2] = {1.0f - s.ft, s.ft}, wy[2] = {1.0f - s.fy, s.fy}, wx[2] = {1.0f - s.fx, s.fx};
+    float w[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) w[c] = wt[c >> 2] * wy[(c >> 1) & 1] * wx[c & 1];
+    const float sp = have ? gather_combine(gl, part, w) * (rsqrtf(static_cast<float>(D)) * kLog2e) : -INFINITY;
+    float mx = sp;
+#pragma unroll
+    for (int o = L / 2; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(kFullMask, mx, o));
+    const float pe = have ? exp2f(sp - mx) : 0.0f, l = group_sum<L>(pe, kFullMask), inv = 1.0f / l;
+    __syncwarp();
+    gather_weights<G>(gl, part, pe * inv, w, step);
+    if (p == 0 && lane / L < items) lse[row] = (mx + log2f(l)) * kLn2;
+    bool bad = !(l < INFINITY);
+    const unsigned bad_l = __ballot_sync(kFullMask, bad && p == 0);
+    unsigned redo = 0u;                                  // items with something that is not finite
+#pragma unroll
+    for (int i = 0; i < G; ++i) redo |= ((bad_l >> (i * L)) & 1u) << i;
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+        const int u = lane / LPR, it = PER > 1 ? u / PER : u * ITEMS + i;
+        const int total = __shfl_sync(kFullMask, part.total, it * L);
+        float acc[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) acc[e] = 0.0f;
+        gather_sum_item<D, PER>(gl, it * region, total, PER > 1 ? u % PER : 0, vh, tok_bytes, acc);
+        __syncwarp();
+#pragma unroll
+        for (int o = LPR; o < LPR * PER; o <<= 1)
+#pragma unroll
+            for (int e = 0; e < 8; ++e) acc[e] += __shfl_xor_sync(kFullMask, acc[e], o);
+        bad = false;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) bad = bad || !(fabsf(acc[e]) < INFINITY);
+#pragma unroll
+        for (int z = 0; z < G; ++z)
+            if (__any_sync(kFullMask, bad && it == z)) redo |= 1u << z;
+        if (it < items && (PER == 1 || u % PER == 0)) {
+            const long long at = (row0 + static_cast<long long>(it) * pr.heads) * D + (lane % LPR) * 8;
+            if constexpr (kAdd) {                        // first term of Eq. 1, added before the rounding
+                if (!((redo >> it) & 1u)) {              // (out may be the addend: the plain path below reads it)
+                    float add[8];
+                    E::to_float(E::load(addend + at), add);
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) acc[e] += add[e];
+                    E::store(out + at, acc);
+                }
+            } else {
+                E::store(out + at, acc);
+            }
+        }
+    }
+    while (redo) {
+        const int it = __ffs(static_cast<int>(redo)) - 1;
+        redo &= redo - 1u;
+        if (it >= items) break;
+        const int n2 = n0 + it;
+        forward_item_plain<D>(q, k, v, offsets, kAdd ? addend : nullptr, out, lse, pr, m, n2 / pr.W / pr.H, n2 / pr.W % pr.H, n2 % pr.W);
+    }
 }
 
 #ifndef DSA3D_FWD_MINBLOCKS
@@ -343,8 +445,17 @@ template <int D>
 static cudaError_t launch_gather_forward(const void* q, const void* k, const void* v, const float* offsets, const void* addend, void* out,
                                          float* lse, const Problem& pr, cudaStream_t stream, const int* gate) {
     using T = __nv_bfloat16;
-    const long long per_head = (pr.q_count + kFwdWarps - 1) / kFwdWarps;
+    // as many items per warp as have a lane for every sample
+    const int share = pr.P <= 8 ? 4 : pr.P <= 16 ? 2 : 1;
+    const long long per_head = (pr.q_count + kFwdWarps * share - 1) / (kFwdWarps * share);
     const unsigned blocks = static_cast<unsigned>(per_head * pr.heads);
+    if (share > 1) {
+        auto kern = share == 4 ? (addend ? gather_forward_small_kernel<D, 4, true> : gather_forward_small_kernel<D, 4, false>)
+                               : (addend ? gather_forward_small_kernel<D, 2, true> : gather_forward_small_kernel<D, 2, false>);
+        kern<<<blocks, kFwdWarps * 32, 0, stream>>>(static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v), offsets,
+                                                    static_cast<const T*>(addend), static_cast<T*>(out), lse, pr, static_cast<unsigned>(per_head), gate);
+        return cudaGetLastError();
+    }
     if (addend)
         gather_forward_kernel<D, true><<<blocks, kFwdWarps * 32, 0, stream>>>(
             static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v), offsets, static_cast<const T*>(addend),
@@ -378,11 +489,10 @@ static cudaError_t launch_forward_t(const void* q, const void* k, const void* v,
 
 cudaError_t launch_forward(const void* q, const void* k, const void* v, const float* offsets, const void* addend,
                            void* out, float* lse, const Problem& pr, bool bf16, cudaStream_t stream, const int* gate) {
-    // A warp of gather_forward_kernel takes 32 samples of one item at a time: with 16 samples or fewer half its lanes are idle, and
-    // at 32 channels with 32 samples or fewer its fixed cost per item is as much as the row traffic it saves.  Measured against
-    // the other kernel: window (2,2,2) 0.5 - 0.9x, (3,3,3) 1.02 - 1.22x at 128 channels, 1.08 - 1.11x at 64, 0.96x at 32,
-    // (3,7,7) 1.9x; grids of a few hundred tokens 1.5x.
-    const bool warp_per_item = bf16 && pr.P > (pr.d == 32 ? 32 : 16);
+    // At 32 channels and up to 32 samples the row traffic is too small to pay for the list: 0.94 - 0.97x of the other kernel.
+    // Elsewhere (32 x 45 x 80, 16 heads of 128): window (2,2,2) 1.18x (integer offsets 1.34x), (3,3,3) 1.02 - 1.20x, 64 channels 1.08 -
+    // 1.14x; (3,7,7) 1.9x; grids of a few hundred tokens 1.7x.
+    const bool warp_per_item = bf16 && !(pr.d == 32 && pr.P <= 32);
 #define DSA3D_CASE(DD)                                                                                    \
     case DD:                                                                                              \
         return warp_per_item ? launch_gather_forward<DD>(q, k, v, offsets, addend, out, lse, pr, stream, gate)    \

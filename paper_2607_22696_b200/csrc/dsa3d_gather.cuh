@@ -176,6 +176,38 @@ __device__ __forceinline__ void gather_dots(GatherList& gl, int total, const Gat
     }
 }
 
+// The same for two items that share the warp: rows of the entries from `ra` on against query `qa`, from `rb` on against `qb`, eight
+// of each at a time (lists padded to a multiple of 8).
+template <int D>
+__device__ __forceinline__ void gather_dots_pair(GatherList& gl, int ra, int ta, int rb, int tb, const __nv_bfloat16* __restrict__ qa,
+                                                 const __nv_bfloat16* __restrict__ qb, const __nv_bfloat16* __restrict__ rows, uint32_t tok_bytes) {
+    constexpr int I = D / 32;
+    const int lane = threadIdx.x & 31, g = lane >> 2, j = lane & 3;
+    GatherQuery<D> qr;                                 // columns 0, 1 (4, 5) the first query, 2, 3 the second
+    gather_query<D>(qr, (g & 2) ? qb : qa);
+    const char* src = reinterpret_cast<const char*>(rows) + j * 16;
+    const uint32_t odd = I > 1 ? (g & 1) * 64u : 0u;
+    const int other = I > 1 ? ((g & 1) ? -64 : 64) : 0;
+    for (int s = 0; s < max(ta, tb); s += 8) {
+        const char* pa = src + static_cast<uint64_t>(gl.token[(s < ta ? ra : rb) + s + g]) * tok_bytes + odd;     // a list that is at its end repeats the other's rows
+        const char* pb = src + static_cast<uint64_t>(gl.token[(s < tb ? rb : ra) + s + g]) * tok_bytes + odd;
+        uint4 a[I], b[I];
+#pragma unroll
+        for (int i = 0; i < I; ++i) {
+            a[i] = __ldg(reinterpret_cast<const uint4*>(pa + (i >> 1) * 128 + ((i & 1) ? other : 0)));
+            b[i] = __ldg(reinterpret_cast<const uint4*>(pb + (i >> 1) * 128 + ((i & 1) ? other : 0)));
+        }
+        float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+        for (int i = 0; i < I; ++i) {
+            mma_bf16(c, a[i].x, b[i].x, a[i].y, b[i].y, qr.v[i].x, qr.v[i].y);
+            mma_bf16(c, a[i].z, b[i].z, a[i].w, b[i].w, qr.v[i].z, qr.v[i].w);
+        }
+        if (j == 0 && s < ta) gl.value[ra + s + g] = (g & 1) ? c[1] : c[0];
+        if (j == 1 && s < tb) gl.value[rb + s + g] = (g & 1) ? c[3] : c[2];
+    }
+}
+
 // acc += sum of value[i] * row i: D / 8 lanes per row, 8 channels per lane; the subgroups of a warp take four rows each in turn and
 // their sums are added up by gather_finish.  The list is padded to a multiple of kGatherStep.
 template <int D> struct GatherStep { static constexpr int LPR = D / 8, U = 32 / LPR, N = D == 128 ? 16 : 4 * U; };
