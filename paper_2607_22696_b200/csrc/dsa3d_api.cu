@@ -373,7 +373,7 @@ struct BackwardPlan {
 };
 
 int backward_plan(int T, int H, int W, int heads, int d, const int* window, int dtype, bool tiled, void* dk,
-                  void* dv, void* workspace, size_t workspace_bytes, bool gated, BackwardPlan& plan) {
+                  void* dv, void* workspace, size_t workspace_bytes, BackwardPlan& plan) {
     const int rc = make_problem(T, H, W, heads, d, window, dtype, plan.pr);
     if (rc != DSA3D_OK) return rc;
     plan.bf16 = dtype == DSA3D_BF16;
@@ -396,8 +396,8 @@ int backward_plan(int T, int H, int W, int heads, int d, const int* window, int 
         plan.pr.blk_list = reinterpret_cast<uint32_t*>(static_cast<char*>(plan.scratch) + kb.count_bytes);
         plan.pr.blk_cap = kb.cap;
     }
-    // DSA3D_TILE asks for the tile kernel, a gate for kernels that look at it, DSA3D_KEY_BLOCKS for the key-block kernel
-    plan.cells = plan.coef && !gated && !plan.pr.key_blocks && !getenv("DSA3D_TILE");
+    // DSA3D_TILE asks for the gather and tile kernels, DSA3D_KEY_BLOCKS for the key-block kernel
+    plan.cells = plan.coef && !plan.pr.key_blocks && !getenv("DSA3D_TILE");
     if (plan.coef) {
         int dev = 0, sms = 0;
         cudaError_t e = cudaGetDevice(&dev);
@@ -518,7 +518,7 @@ int dsa3d::backward_impl(const void* q, const void* k, const void* v, const floa
         !aligned16(dout) || !aligned16(dq) || !aligned16(dk) || !aligned16(dv) || !aligned16(doffsets))
         return DSA3D_ERR_MISALIGNED;
     BackwardPlan plan;
-    int rc = backward_plan(T, H, W, heads, d, window, dtype, tiled, dk, dv, workspace, workspace_bytes, gate != nullptr, plan);
+    int rc = backward_plan(T, H, W, heads, d, window, dtype, tiled, dk, dv, workspace, workspace_bytes, plan);
     if (rc != DSA3D_OK) return rc;
     plan.pr.gate = gate;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
@@ -655,7 +655,7 @@ int step_host_body(const void* q_h, const void* k_h, const void* v_h, const floa
     const bool bf16 = dtype == DSA3D_BF16;
     BackwardPlan plan;
     int st = backward_plan(T, H, W, heads, d, window, dtype, true, base + a.dk, base + a.dv,
-                           a.ws_bytes ? base + a.workspace : nullptr, a.ws_bytes, false, plan);
+                           a.ws_bytes ? base + a.workspace : nullptr, a.ws_bytes, plan);
     if (st != DSA3D_OK) return st;
     const int unit = plan.pr.tile_t >= 1 ? plan.pr.tile_t : 1;          // slabs start on tile boundaries
     int slab_frames = (T + kMaxSlabs - 1) / kMaxSlabs;

@@ -22,20 +22,19 @@ using bf16 = __nv_bfloat16;
 // ------------------------------------------------------------------------------------------------ binning
 constexpr int kBinThreads = 512, kBinWarps = kBinThreads / 32, kCopies = 8;
 
-__global__ void __launch_bounds__(kBinThreads, 2)
-cells_bin_kernel(const float* __restrict__ offsets, const Problem pr, const Slab sl, unsigned inv_p) {
+__device__ __forceinline__ void bin_block(const unsigned block, const float* __restrict__ offsets, const Problem& pr, const Slab& sl, unsigned inv_p) {
     extern __shared__ __align__(16) unsigned char raw[];
     uint32_t* counters = reinterpret_cast<uint32_t*>(raw);                 // [kBins + 1][kCopies]: lanes of a warp mostly hit the same bin
     uint32_t* words = counters + (kBins + 1) * kCopies;                     // [kRows * P]: bin (9 bits), cell (6), rank in its counter (16)
     __shared__ uint32_t scan[kBinWarps];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const long long tile = blockIdx.x;
+    const long long tile = block;
     int r = static_cast<int>(tile % (sl.tiles_t * sl.tiles_y * sl.tiles_x));
     const int m = sl.m0 + static_cast<int>(tile / (sl.tiles_t * sl.tiles_y * sl.tiles_x));
     const int x0 = (r % sl.tiles_x) * kTileX; r /= sl.tiles_x;
     const int y0 = (r % sl.tiles_y) * 4, t0 = sl.f0 + (r / sl.tiles_y) * 4;
     const int samples = kRows * pr.P;
-    if (blockIdx.x == 0 && tid == 0) { *sl.marked = 0; *sl.used = 0u; }
+    if (block == 0 && tid == 0) { *sl.marked = 0; *sl.used = 0u; }
     for (int i = tid; i < (kBins + 1) * kCopies / 4; i += kBinThreads) reinterpret_cast<uint4*>(counters)[i] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
     auto row_of = [&](int s) { return static_cast<int>((static_cast<unsigned long long>(static_cast<unsigned>(s)) * inv_p) >> 24); };
@@ -120,6 +119,21 @@ cells_bin_kernel(const float* __restrict__ offsets, const Problem pr, const Slab
     }
 }
 
+template <bool kGated>
+__global__ void __launch_bounds__(kBinThreads, 2)
+cells_bin_kernel(const float* __restrict__ offsets, const __grid_constant__ Problem pr, const __grid_constant__ Slab sl, unsigned inv_p, unsigned blocks) {
+    if constexpr (!kGated) {
+        bin_block(blockIdx.x, offsets, pr, sl, inv_p);
+    } else {
+        if (gated_off(pr)) return;
+        for (unsigned block = blockIdx.x; block < blocks; block += gridDim.x) {
+            bin_block(block, offsets, pr, sl, inv_p);
+            __syncthreads();
+        }
+    }
+}
+
+
 // ------------------------------------------------------------------------------------------------ a block's samples
 struct BlockPos { int m, t, y, x, bt, by, bx; };   // head, first cell along t, y, x; block numbers (bt from the slab's first frame)
 
@@ -198,16 +212,15 @@ __device__ __forceinline__ long long sample_of(const Segments& sg, uint32_t i, i
 // A block's samples in the order of their cells.  (A kernel of its own: it is a chain of dependent loads - segment,
 // sample, place - which wants many small CTAs per SM, and both block kernels read what it leaves in one stream.)
 constexpr int kSortThreads = 256, kSortKeep = 2048;
-__global__ void __launch_bounds__(kSortThreads)
-cells_sort_kernel(const Problem pr, const Slab sl) {
+__device__ __forceinline__ void sort_block(const unsigned block, const Problem& pr, const Slab& sl) {
     __shared__ Segments sg;
     __shared__ uint32_t count[kCells], cursor[kCells], base;
     __shared__ uint32_t kept[kSortKeep];                    // place in its tile's list of the first samples
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const BlockPos b = block_pos(sl, blockIdx.x);
+    const BlockPos b = block_pos(sl, block);
     if (tid < kCells) count[tid] = 0u;
     const uint32_t total = find_segments(sl, b, sg);
-    uint32_t* first = sl.first + static_cast<long long>(blockIdx.x) * (kCells + 1);
+    uint32_t* first = sl.first + static_cast<long long>(block) * (kCells + 1);
     if (total == 0u) {
         if (tid <= kCells) first[tid] = 0u;
         return;
@@ -243,6 +256,21 @@ cells_sort_kernel(const Problem pr, const Slab sl) {
         sl.place[to] = static_cast<uint32_t>(sample_at(sl, pr, b.m, static_cast<int>(u.x), static_cast<int>(mt & 255u)));
     }
 }
+
+template <bool kGated>
+__global__ void __launch_bounds__(kSortThreads)
+cells_sort_kernel(const __grid_constant__ Problem pr, const __grid_constant__ Slab sl, unsigned blocks) {
+    if constexpr (!kGated) {
+        sort_block(blockIdx.x, pr, sl);
+    } else {
+        if (gated_off(pr)) return;
+        for (unsigned block = blockIdx.x; block < blocks; block += gridDim.x) {
+            sort_block(block, pr, sl);
+            __syncthreads();
+        }
+    }
+}
+
 
 // Byte of 16-byte chunk `chunk` of box row `row` in shared memory: rows of 128 bytes and more have their chunks permuted by
 // the row's parity, so that the four even (or odd) chunks a quarter-warp reads of two neighbouring rows lie in different banks.
@@ -303,17 +331,16 @@ template <bool kWide, int I> __device__ __forceinline__ void load_piece(const ui
 
 // q . K and dO . V with derivatives, eight numbers per sample into stats; even warps take q . K, odd ones dO . V.
 template <int D, bool kWide>
-__global__ void __launch_bounds__(kDotThreads, D == 128 ? 3 : 4)
-cells_dots_kernel(const bf16* __restrict__ q, const bf16* __restrict__ k, const bf16* __restrict__ v, const bf16* __restrict__ dout,
-                  const Problem pr, const Slab sl) {
+__device__ __forceinline__ void dots_block(const unsigned block, const bf16* __restrict__ q, const bf16* __restrict__ k, const bf16* __restrict__ v, const bf16* __restrict__ dout,
+                  const Problem& pr, const Slab& sl) {
     constexpr int I = D / 32, W = kDotThreads / 64;
     extern __shared__ __align__(16) unsigned char raw[];
     DotSmem<D>& s = *reinterpret_cast<DotSmem<D>*>(raw);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g8 = lane >> 2, j = lane & 3;
     const int tensor = warp & 1;
-    const uint32_t* first = sl.first + static_cast<long long>(blockIdx.x) * (kCells + 1);
+    const uint32_t* first = sl.first + static_cast<long long>(block) * (kCells + 1);
     if (__ldg(first) == __ldg(first + kCells)) return;
-    const BlockPos b = block_pos(sl, blockIdx.x);
+    const BlockPos b = block_pos(sl, block);
     if (warp == 0) {
         const uint32_t f0 = __ldg(first + min(2 * lane, kCells)), f1 = __ldg(first + min(2 * lane + 1, kCells)), f2 = __ldg(first + min(2 * lane + 2, kCells));
         const uint32_t n0 = (f1 - f0 + 15u) >> 4, n1 = (f2 - f1 + 15u) >> 4;
@@ -385,6 +412,22 @@ cells_dots_kernel(const bf16* __restrict__ q, const bf16* __restrict__ k, const 
     }
 }
 
+template <int D, bool kWide, bool kGated>
+__global__ void __launch_bounds__(kDotThreads, D == 128 ? 3 : 4)
+cells_dots_kernel(const bf16* __restrict__ q, const bf16* __restrict__ k, const bf16* __restrict__ v, const bf16* __restrict__ dout,
+                  const __grid_constant__ Problem pr, const __grid_constant__ Slab sl, unsigned blocks) {
+    if constexpr (!kGated) {
+        dots_block<D, kWide>(blockIdx.x, q, k, v, dout, pr, sl);
+    } else {
+        if (gated_off(pr)) return;
+        for (unsigned block = blockIdx.x; block < blocks; block += gridDim.x) {
+            dots_block<D, kWide>(block, q, k, v, dout, pr, sl);
+            __syncthreads();
+        }
+    }
+}
+
+
 // ------------------------------------------------------------------------------------------------ per query
 constexpr int kQueryWarps = 2;
 
@@ -394,17 +437,16 @@ constexpr int kQueryWarps = 2;
 // coefficients) is marked by the sign of cv: its contributions to dK and dV are formed one by one, so that they reach only
 // the corners with a weight.  Windows of at most 8 (16) samples: G = 4 (2) neighbouring queries share a warp.
 template <int D, int G>
-__global__ void __launch_bounds__(kQueryWarps * 32, 16)
-cells_query_kernel(const bf16* __restrict__ k, const float* __restrict__ offsets, const float* __restrict__ lse, bf16* __restrict__ dq,
-                   float* __restrict__ doffsets, const __grid_constant__ Problem pr, const __grid_constant__ Slab sl, unsigned blocks_per_head) {
+__device__ __forceinline__ void query_block(const unsigned block, const bf16* __restrict__ k, const float* __restrict__ offsets, const float* __restrict__ lse, bf16* __restrict__ dq,
+                   float* __restrict__ doffsets, const Problem& pr, const Slab& sl, unsigned blocks_per_head) {
     __shared__ GatherList lists[kQueryWarps];
     constexpr int L = 32 / G;                       // lanes per query
     constexpr int U = GatherStep<D>::U, PER = U > G ? U / G : 1, ITEMS = G > U ? G / U : 1;      // subgroups per query, queries per subgroup
     constexpr int step = G == 1 ? GatherStep<D>::N : 4 * PER;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gl_lane = lane & (L - 1);
     GatherList& gl = lists[warp];
-    const int frame = pr.H * pr.W, mh = static_cast<int>(blockIdx.x / blocks_per_head), per_head = frame * (sl.f1 - sl.f0);
-    const int warp_first = (static_cast<int>(blockIdx.x - static_cast<unsigned>(mh) * blocks_per_head) * kQueryWarps + warp) * G;
+    const int frame = pr.H * pr.W, mh = static_cast<int>(block / blocks_per_head), per_head = frame * (sl.f1 - sl.f0);
+    const int warp_first = (static_cast<int>(block - static_cast<unsigned>(mh) * blocks_per_head) * kQueryWarps + warp) * G;
     if (warp_first >= per_head) return;
     const bool active = warp_first + lane / L < per_head;        // a query past the end repeats the last one, stores off
     const int local = active ? warp_first + lane / L : per_head - 1;
@@ -493,6 +535,22 @@ cells_query_kernel(const bf16* __restrict__ k, const float* __restrict__ offsets
     }
 }
 
+template <int D, int G, bool kGated>
+__global__ void __launch_bounds__(kQueryWarps * 32, 16)
+cells_query_kernel(const bf16* __restrict__ k, const float* __restrict__ offsets, const float* __restrict__ lse, bf16* __restrict__ dq,
+                   float* __restrict__ doffsets, const __grid_constant__ Problem pr, const __grid_constant__ Slab sl, unsigned blocks_per_head, unsigned blocks) {
+    if constexpr (!kGated) {
+        query_block<D, G>(blockIdx.x, k, offsets, lse, dq, doffsets, pr, sl, blocks_per_head);
+    } else {
+        if (gated_off(pr)) return;
+        for (unsigned block = blockIdx.x; block < blocks; block += gridDim.x) {
+            query_block<D, G>(block, k, offsets, lse, dq, doffsets, pr, sl, blocks_per_head);
+            __syncthreads();
+        }
+    }
+}
+
+
 // ------------------------------------------------------------------------------------------------ dK, dV
 constexpr int kSumThreads = 256;
 
@@ -513,9 +571,8 @@ __device__ __forceinline__ void red_add_v2(float* addr, float a, float b) {
 // as bf16 head and remainder, two products into the same sums.  Nothing is shared between warps: each walks through its
 // groups in three steps that overlap - samples (two groups ahead), coefficients and query rows (one ahead), products.
 template <int D>
-__global__ void __launch_bounds__(kSumThreads, D == 32 ? 3 : 2)
-cells_sums_kernel(const bf16* __restrict__ q, const bf16* __restrict__ dout, float* __restrict__ acc_dk, float* __restrict__ acc_dv,
-                  const Problem pr, const Slab sl) {
+__device__ __forceinline__ void sums_block(const unsigned block, const bf16* __restrict__ q, const bf16* __restrict__ dout, float* __restrict__ acc_dk, float* __restrict__ acc_dv,
+                  const Problem& pr, const Slab& sl) {
     using S = SumSmem<D>;
     constexpr int STRIDE = 4;                       // the four warps of a tensor take the runs in turn
     constexpr int CPR = D / 8;                      // 16-byte chunks of a staged row, permuted by the row (SWZ)
@@ -524,9 +581,9 @@ cells_sums_kernel(const bf16* __restrict__ q, const bf16* __restrict__ dout, flo
     extern __shared__ __align__(16) unsigned char raw[];
     S& s = *reinterpret_cast<S*>((reinterpret_cast<uintptr_t>(raw) + 255) & ~uintptr_t(255));
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g8 = lane >> 2, j = lane & 3;
-    const uint32_t* first = sl.first + static_cast<long long>(blockIdx.x) * (kCells + 1);
+    const uint32_t* first = sl.first + static_cast<long long>(block) * (kCells + 1);
     if (__ldg(first) == __ldg(first + kCells)) return;
-    const BlockPos b = block_pos(sl, blockIdx.x);
+    const BlockPos b = block_pos(sl, block);
     if (tid <= kCells) s.first[tid] = __ldg(first + tid);
     __syncthreads();
     const long long tok = static_cast<long long>(pr.heads) * D;
@@ -677,6 +734,22 @@ cells_sums_kernel(const bf16* __restrict__ q, const bf16* __restrict__ dout, flo
     asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
+template <int D, bool kGated>
+__global__ void __launch_bounds__(kSumThreads, D == 32 ? 3 : 2)
+cells_sums_kernel(const bf16* __restrict__ q, const bf16* __restrict__ dout, float* __restrict__ acc_dk, float* __restrict__ acc_dv,
+                  const __grid_constant__ Problem pr, const __grid_constant__ Slab sl, unsigned blocks) {
+    if constexpr (!kGated) {
+        sums_block<D>(blockIdx.x, q, dout, acc_dk, acc_dv, pr, sl);
+    } else {
+        if (gated_off(pr)) return;
+        for (unsigned block = blockIdx.x; block < blocks; block += gridDim.x) {
+            sums_block<D>(block, q, dout, acc_dk, acc_dv, pr, sl);
+            __syncthreads();
+        }
+    }
+}
+
+
 // ------------------------------------------------------------------------------------------------ beyond the bins
 // The samples in bin kBins of every tile, a warp per sample, row by row.  kScatter: their contributions to dK and dV, and those
 // of marked samples of the other bins; otherwise what cells_dots_kernel leaves for the others.
@@ -685,6 +758,7 @@ __global__ void __launch_bounds__(256)
 cells_far_kernel(const bf16* __restrict__ q, const bf16* __restrict__ k, const bf16* __restrict__ v, const bf16* __restrict__ dout,
                  const float* __restrict__ offsets, float* __restrict__ acc_dk, float* __restrict__ acc_dv, const Problem pr, const Slab sl,
                  int tiles) {
+    if (gated_off(pr)) return;
     constexpr int V = D / 32;                       // channels per lane
     const int lane = threadIdx.x & 31, warps = gridDim.x * 8;
     const long long tok = static_cast<long long>(pr.heads) * D;
@@ -798,34 +872,38 @@ size_t lay_out(const Problem& pr, int m0, int heads, int f0, int f1, char* base,
     return at;
 }
 
-template <int D>
+// Behind a gate that is mostly closed launching all CTAs would cost more than anything else (0.95 ms for 1.8 M of the query kernel):
+// the gated instances loop over their blocks.
+template <int D, bool kGated>
 cudaError_t launch_slab(const void* q_, const void* k_, const void* v_, const float* offsets, const float* lse, const void* dout_, void* dq_,
                         float* acc_dk, float* acc_dv, float* doffsets, const Problem& pr, const Slab& s, cudaStream_t stream) {
     const bf16 *q = static_cast<const bf16*>(q_), *k = static_cast<const bf16*>(k_), *v = static_cast<const bf16*>(v_), *dout = static_cast<const bf16*>(dout_);
-    const int tiles = s.heads * s.tiles_t * s.tiles_y * s.tiles_x, blocks = s.heads * s.blocks_t * s.blocks_y * s.blocks_x;
+    const unsigned tiles = static_cast<unsigned>(s.heads * s.tiles_t * s.tiles_y * s.tiles_x), blocks = static_cast<unsigned>(s.heads * s.blocks_t * s.blocks_y * s.blocks_x);
     const unsigned inv_p = ((1u << 24) + static_cast<unsigned>(pr.P) - 1u) / static_cast<unsigned>(pr.P);
-    const size_t bin_smem = static_cast<size_t>((kBins + 1) * kCopies + kRows * pr.P) * sizeof(uint32_t);
-    cudaError_t e = cudaFuncSetAttribute(cells_bin_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bin_smem));
-    if (e != cudaSuccess) return e;
-    cells_bin_kernel<<<static_cast<unsigned>(tiles), kBinThreads, bin_smem, stream>>>(offsets, pr, s, inv_p);
-    cells_sort_kernel<<<static_cast<unsigned>(blocks), kSortThreads, 0, stream>>>(pr, s);
-    const size_t dot_smem = sizeof(DotSmem<D>), sum_smem = sizeof(SumSmem<D>) + 256;
+    auto grid = [](unsigned n) { return kGated && n > 148u * 8u ? 148u * 8u : n; };
+    cudaError_t e = cudaSuccess;
+    auto big = [&](auto kern, size_t smem) {           // allows the kernel its dynamic shared memory
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+        return kern;
+    };
+    const size_t bin_smem = static_cast<size_t>((kBins + 1) * kCopies + kRows * pr.P) * sizeof(uint32_t), dot_smem = sizeof(DotSmem<D>), sum_smem = sizeof(SumSmem<D>) + 256;
     const bool wide = ((reinterpret_cast<uintptr_t>(q) | reinterpret_cast<uintptr_t>(dout)) & 31u) == 0;
-    auto dots = wide ? cells_dots_kernel<D, true> : cells_dots_kernel<D, false>;
-    e = cudaFuncSetAttribute(dots, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(dot_smem));
+    auto bin = big(cells_bin_kernel<kGated>, bin_smem);
+    auto dots = big(wide ? cells_dots_kernel<D, true, kGated> : cells_dots_kernel<D, false, kGated>, dot_smem);
+    auto sums = big(cells_sums_kernel<D, kGated>, sum_smem);
     if (e != cudaSuccess) return e;
-    dots<<<static_cast<unsigned>(blocks), kDotThreads, dot_smem, stream>>>(q, k, v, dout, pr, s);
-    const unsigned far_grid = static_cast<unsigned>(tiles / 256 + 1 < 148 * 8 ? tiles / 256 + 1 : 148 * 8);
-    cells_far_kernel<D, false><<<far_grid, 256, 0, stream>>>(q, k, v, dout, offsets, acc_dk, acc_dv, pr, s, tiles);
+    bin<<<grid(tiles), kBinThreads, bin_smem, stream>>>(offsets, pr, s, inv_p, tiles);
+    cells_sort_kernel<kGated><<<grid(blocks), kSortThreads, 0, stream>>>(pr, s, blocks);
+    dots<<<grid(blocks), kDotThreads, dot_smem, stream>>>(q, k, v, dout, pr, s, blocks);
+    const unsigned far_grid = tiles / 256 + 1 < 148 * 8 ? tiles / 256 + 1 : 148 * 8;
+    cells_far_kernel<D, false><<<far_grid, 256, 0, stream>>>(q, k, v, dout, offsets, acc_dk, acc_dv, pr, s, static_cast<int>(tiles));
     // As many queries per warp as have a lane for every sample.
     const int share = pr.P <= 8 ? 4 : pr.P <= 16 ? 2 : 1, per_block = kQueryWarps * share;
-    const unsigned per_head = static_cast<unsigned>((static_cast<long long>(s.f1 - s.f0) * pr.H * pr.W + per_block - 1) / per_block);
-    auto query = share == 4 ? cells_query_kernel<D, 4> : share == 2 ? cells_query_kernel<D, 2> : cells_query_kernel<D, 1>;
-    query<<<per_head * static_cast<unsigned>(s.heads), kQueryWarps * 32, 0, stream>>>(k, offsets, lse, static_cast<bf16*>(dq_), doffsets, pr, s, per_head);
-    e = cudaFuncSetAttribute(cells_sums_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sum_smem));
-    if (e != cudaSuccess) return e;
-    cells_sums_kernel<D><<<static_cast<unsigned>(blocks), kSumThreads, sum_smem, stream>>>(q, dout, acc_dk, acc_dv, pr, s);
-    cells_far_kernel<D, true><<<far_grid, 256, 0, stream>>>(q, k, v, dout, offsets, acc_dk, acc_dv, pr, s, tiles);
+    const unsigned per_head = static_cast<unsigned>((static_cast<long long>(s.f1 - s.f0) * pr.H * pr.W + per_block - 1) / per_block), query_blocks = per_head * static_cast<unsigned>(s.heads);
+    auto query = share == 4 ? cells_query_kernel<D, 4, kGated> : share == 2 ? cells_query_kernel<D, 2, kGated> : cells_query_kernel<D, 1, kGated>;
+    query<<<grid(query_blocks), kQueryWarps * 32, 0, stream>>>(k, offsets, lse, static_cast<bf16*>(dq_), doffsets, pr, s, per_head, query_blocks);
+    sums<<<grid(blocks), kSumThreads, sum_smem, stream>>>(q, dout, acc_dk, acc_dv, pr, s, blocks);
+    cells_far_kernel<D, true><<<far_grid, 256, 0, stream>>>(q, k, v, dout, offsets, acc_dk, acc_dv, pr, s, static_cast<int>(tiles));
     return cudaGetLastError();
 }
 
@@ -850,9 +928,10 @@ bool try_cells_backward(const void* q, const void* k, const void* v, const float
         for (int m = 0; m < pr.heads; m += heads) {
             const int f1 = f + frames < f_end ? f + frames : f_end, mh = m + heads < pr.heads ? heads : pr.heads - m;
             lay_out(pr, m, mh, f, f1, static_cast<char*>(scratch), s);
-            *err = pr.d == 128 ? launch_slab<128>(q, k, v, offsets, lse, dout, dq, acc_dk, acc_dv, doffsets, pr, s, stream)
-                 : pr.d == 64  ? launch_slab<64>(q, k, v, offsets, lse, dout, dq, acc_dk, acc_dv, doffsets, pr, s, stream)
-                               : launch_slab<32>(q, k, v, offsets, lse, dout, dq, acc_dk, acc_dv, doffsets, pr, s, stream);
+            auto slab = pr.d == 128 ? (pr.gate ? launch_slab<128, true> : launch_slab<128, false>)
+                        : pr.d == 64 ? (pr.gate ? launch_slab<64, true> : launch_slab<64, false>)
+                                     : (pr.gate ? launch_slab<32, true> : launch_slab<32, false>);
+            *err = slab(q, k, v, offsets, lse, dout, dq, acc_dk, acc_dv, doffsets, pr, s, stream);
             if (*err != cudaSuccess) return true;
         }
     return true;

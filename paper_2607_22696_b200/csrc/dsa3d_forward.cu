@@ -74,89 +74,96 @@ __device__ __noinline__ void forward_item_plain(const __nv_bfloat16* q, const __
     if (lane == 0) lse[row] = (m_run + log2f(l_run)) * kLn2;
 }
 
-template <int D, bool kAdd>
+template <int D, bool kAdd, bool kGated>
 __global__ void __launch_bounds__(kFwdWarps * 32, 16)
 gather_forward_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v,
                       const float* __restrict__ offsets, const __nv_bfloat16* addend, __nv_bfloat16* out, float* __restrict__ lse,
                       const __grid_constant__ Problem pr, unsigned blocks_per_head, const int* __restrict__ gate) {
-    if (gate && *gate == 0) return;                      // another kernel takes this call (see launch_forward)
+    if (kGated && *gate == 0) return;                    // another kernel takes this call (see launch_forward)
     __shared__ GatherList lists[kFwdWarps];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     GatherList& gl = lists[warp];
-    const int m = static_cast<int>(blockIdx.x / blocks_per_head);
-    const long long local = static_cast<long long>(blockIdx.x - static_cast<unsigned>(m) * blocks_per_head) * kFwdWarps + warp;
-    if (local >= pr.q_count) return;
-    const int n = static_cast<int>(pr.q_begin + local);
-    const int x = n % pr.W, ty = n / pr.W, y = ty % pr.H, t = ty / pr.H;
-    const long long row = static_cast<long long>(n) * pr.heads + m;
-    const uint32_t tok_bytes = static_cast<uint32_t>(pr.heads) * (D * 2);
-    const __nv_bfloat16 *kh = k + static_cast<long long>(m) * D, *vh = v + static_cast<long long>(m) * D;
-    const float lscale = rsqrtf(static_cast<float>(D)) * kLog2e;    // logits in log2 units
-    constexpr int step = GatherStep<D>::N;
-    float acc[8];
+    // One block of items per CTA; behind a gate (a small launch, see launch_gather_forward) a loop over them.  The loop costs the
+    // kernel 2 - 15 %, so only the gated instance has it.
+    unsigned block = blockIdx.x;
+_Pragma("unroll 1")
+    do {
+        const int m = static_cast<int>(block / blocks_per_head);
+        const long long local = static_cast<long long>(block - static_cast<unsigned>(m) * blocks_per_head) * kFwdWarps + warp;
+        if (local >= pr.q_count) { if constexpr (kGated) continue; else return; }
+        const int n = static_cast<int>(pr.q_begin + local);
+        const int x = n % pr.W, ty = n / pr.W, y = ty % pr.H, t = ty / pr.H;
+        const long long row = static_cast<long long>(n) * pr.heads + m;
+        const uint32_t tok_bytes = static_cast<uint32_t>(pr.heads) * (D * 2);
+        const __nv_bfloat16 *kh = k + static_cast<long long>(m) * D, *vh = v + static_cast<long long>(m) * D;
+        const float lscale = rsqrtf(static_cast<float>(D)) * kLog2e;    // logits in log2 units
+        constexpr int step = GatherStep<D>::N;
+        float acc[8];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) acc[e] = 0.0f;
-    float m_run = -INFINITY, l_run = 0.0f;               // l_run: the lane's part
-    for (int pb = 0; pb < pr.P; pb += 32) {
-        const bool have = pb + lane < pr.P;
-        Sample s;
-        GatherQuery<D> qr;                               // on its way while the samples are listed
-        gather_query<D>(qr, q + row * D);
-        s.base = 0; s.mask = 0u; s.ft = s.fy = s.fx = 0.0f;
-        if (have) s = to_sample(pr, make_cell(pr, t, y, x, pb + lane, offsets ? offsets + (row * pr.P + pb + lane) * 3 : kZeroOffset));
-        const unsigned mask = checked_corners(pr, weighted_corners(s.mask, s.ft, s.fy, s.fx), s.base, 2);
-        const GatherPart part = gather_list(gl, mask, s.base, pr, step);
-        __syncwarp();
-        gather_dots<D>(gl, part.total, qr, kh, tok_bytes);
-        __syncwarp();
-        const float wt[2] = {1.0f - s.ft, s.ft}, wy[2] = {1.0f - s.fy, s.fy}, wx[2] = {1.0f - s.fx, s.fx};
-        float w[8];
+        for (int e = 0; e < 8; ++e) acc[e] = 0.0f;
+        float m_run = -INFINITY, l_run = 0.0f;               // l_run: the lane's part
+        for (int pb = 0; pb < pr.P; pb += 32) {
+            const bool have = pb + lane < pr.P;
+            Sample s;
+            GatherQuery<D> qr;                               // on its way while the samples are listed
+            gather_query<D>(qr, q + row * D);
+            s.base = 0; s.mask = 0u; s.ft = s.fy = s.fx = 0.0f;
+            if (have) s = to_sample(pr, make_cell(pr, t, y, x, pb + lane, offsets ? offsets + (row * pr.P + pb + lane) * 3 : kZeroOffset));
+            const unsigned mask = checked_corners(pr, weighted_corners(s.mask, s.ft, s.fy, s.fx), s.base, 2);
+            const GatherPart part = gather_list(gl, mask, s.base, pr, step);
+            __syncwarp();
+            gather_dots<D>(gl, part.total, qr, kh, tok_bytes);
+            __syncwarp();
+            const float wt[2] = {1.0f - s.ft, s.ft}, wy[2] = {1.0f - s.fy, s.fy}, wx[2] = {1.0f - s.fx, s.fx};
+            float w[8];
 #pragma unroll
-        for (int c = 0; c < 8; ++c) w[c] = wt[c >> 2] * wy[(c >> 1) & 1] * wx[c & 1];
-        float sp = gather_combine(gl, part, w);
-        sp = have ? sp * lscale : -INFINITY;             // a dead sample stays in the softmax with logit 0
-        float mx = sp;
+            for (int c = 0; c < 8; ++c) w[c] = wt[c >> 2] * wy[(c >> 1) & 1] * wx[c & 1];
+            float sp = gather_combine(gl, part, w);
+            sp = have ? sp * lscale : -INFINITY;             // a dead sample stays in the softmax with logit 0
+            float mx = sp;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(kFullMask, mx, o));
-        if (mx > m_run) {
-            const float corr = exp2f(m_run - mx);
-            l_run *= corr;
+            for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(kFullMask, mx, o));
+            if (mx > m_run) {
+                const float corr = exp2f(m_run - mx);
+                l_run *= corr;
 #pragma unroll
-            for (int e = 0; e < 8; ++e) acc[e] *= corr;
-            m_run = mx;
+                for (int e = 0; e < 8; ++e) acc[e] *= corr;
+                m_run = mx;
+            }
+            const float pe = have ? exp2f(sp - m_run) : 0.0f;
+            l_run += pe;
+            __syncwarp();
+            gather_weights(gl, part, pe, w, step);
+            __syncwarp();
+            gather_sum<D>(gl, part.total, vh, tok_bytes, acc);
+            __syncwarp();
         }
-        const float pe = have ? exp2f(sp - m_run) : 0.0f;
-        l_run += pe;
-        __syncwarp();
-        gather_weights(gl, part, pe, w, step);
-        __syncwarp();
-        gather_sum<D>(gl, part.total, vh, tok_bytes, acc);
-        __syncwarp();
-    }
-    l_run = group_sum<32>(l_run, kFullMask);
-    const float inv = 1.0f / l_run;
-    bool bad = !(l_run < INFINITY);
-    gather_finish<D>(acc);
+        l_run = group_sum<32>(l_run, kFullMask);
+        const float inv = 1.0f / l_run;
+        bool bad = !(l_run < INFINITY);
+        gather_finish<D>(acc);
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-        acc[e] *= inv;
-        bad = bad || !(fabsf(acc[e]) < INFINITY);
-    }
-    if (__any_sync(kFullMask, bad)) {
-        forward_item_plain<D>(q, k, v, offsets, kAdd ? addend : nullptr, out, lse, pr, m, t, y, x);
-        return;
-    }
-    if (lane < D / 8) {
-        using E = Elt<__nv_bfloat16, 1>;
-        if constexpr (kAdd) {                            // first term of Eq. 1, added before the rounding
-            float add[8];
-            E::to_float(E::load(addend + row * D + lane * 8), add);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) acc[e] += add[e];
+        for (int e = 0; e < 8; ++e) {
+            acc[e] *= inv;
+            bad = bad || !(fabsf(acc[e]) < INFINITY);
         }
-        E::store(out + row * D + lane * 8, acc);
-    }
-    if (lane == 0) lse[row] = (m_run + log2f(l_run)) * kLn2;
+        if (__any_sync(kFullMask, bad)) {
+            forward_item_plain<D>(q, k, v, offsets, kAdd ? addend : nullptr, out, lse, pr, m, t, y, x);
+            { if constexpr (kGated) continue; else return; }
+        }
+        if (lane < D / 8) {
+            using E = Elt<__nv_bfloat16, 1>;
+            if constexpr (kAdd) {                            // first term of Eq. 1, added before the rounding
+                float add[8];
+                E::to_float(E::load(addend + row * D + lane * 8), add);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) acc[e] += add[e];
+            }
+            E::store(out + row * D + lane * 8, acc);
+        }
+        if (lane == 0) lse[row] = (m_run + log2f(l_run)) * kLn2;
+        if constexpr (!kGated) return;
+    } while ((block += gridDim.x) < blocks_per_head * static_cast<unsigned>(pr.heads));
 }
 
 // Windows of at most 8 (G = 4) or 16 (G = 2) samples: G neighbouring items share a warp, 32 / G lanes each, so that one trip
@@ -448,7 +455,9 @@ static cudaError_t launch_gather_forward(const void* q, const void* k, const voi
     // as many items per warp as have a lane for every sample
     const int share = pr.P <= 8 ? 4 : pr.P <= 16 ? 2 : 1;
     const long long per_head = (pr.q_count + kFwdWarps * share - 1) / (kFwdWarps * share);
-    const unsigned blocks = static_cast<unsigned>(per_head * pr.heads);
+    // behind a gate that is mostly closed, a CTA per two items would cost more to launch than to run (0.95 ms for 3.7 M items)
+    const long long all = per_head * pr.heads;
+    const unsigned blocks = static_cast<unsigned>(gate && share == 1 && all > 148 * 64 ? 148 * 64 : all);
     if (share > 1) {
         auto kern = share == 4 ? (addend ? gather_forward_small_kernel<D, 4, true> : gather_forward_small_kernel<D, 4, false>)
                                : (addend ? gather_forward_small_kernel<D, 2, true> : gather_forward_small_kernel<D, 2, false>);
@@ -456,12 +465,16 @@ static cudaError_t launch_gather_forward(const void* q, const void* k, const voi
                                                     static_cast<const T*>(addend), static_cast<T*>(out), lse, pr, static_cast<unsigned>(per_head), gate);
         return cudaGetLastError();
     }
-    if (addend)
-        gather_forward_kernel<D, true><<<blocks, kFwdWarps * 32, 0, stream>>>(
+    if (gate)
+        gather_forward_kernel<D, false, true><<<blocks, kFwdWarps * 32, 0, stream>>>(
+            static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v), offsets, nullptr, static_cast<T*>(out), lse, pr,
+            static_cast<unsigned>(per_head), gate);
+    else if (addend)
+        gather_forward_kernel<D, true, false><<<blocks, kFwdWarps * 32, 0, stream>>>(
             static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v), offsets, static_cast<const T*>(addend),
             static_cast<T*>(out), lse, pr, static_cast<unsigned>(per_head), gate);
     else
-        gather_forward_kernel<D, false><<<blocks, kFwdWarps * 32, 0, stream>>>(
+        gather_forward_kernel<D, false, false><<<blocks, kFwdWarps * 32, 0, stream>>>(
             static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v), offsets, nullptr, static_cast<T*>(out), lse, pr,
             static_cast<unsigned>(per_head), gate);
     return cudaGetLastError();
