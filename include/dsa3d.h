@@ -50,16 +50,10 @@
  * Experiment switches.  A few environment variables, read on each call, select an alternative
  * kernel for the same result (they exist to measure one variant against another; none changes
  * what is computed beyond fp32 summation order):
- *   DSA3D_TILE="tt,ty,tx,halo"     query tiling of the dK/dV pre-reduction of dsa3d_backward
- *                                  (default 4,8,8,6; "0" = no tiling, every contribution is an
- *                                  atomic add); also changes dsa3d_backward_workspace_bytes
- *   DSA3D_KEY_BLOCKS=1             dsa3d_backward (bf16, d = 64 or 128) forms dK/dV per
- *                                  block of 4 x 8 x 8 keys as tensor-core products (coefficient matrix of the
- *                                  block against chunks of 32 queries, tcgen05 in tf32: the coefficients lose
- *                                  the bits below 2^-10 relative, q and dO none) instead of the tile kernel's
- *                                  binning (the gather kernel then lists every sample per key block); slower
- *                                  so far; also changes dsa3d_backward_workspace_bytes; a
- *                                  non-finite q or dO row then reaches every key whose block it lies near
+ *   DSA3D_TILE="tt,ty,tx,halo"     dsa3d_backward (bf16) by the gather kernel and a tile kernel that pre-reduces dK/dV per
+ *                                  tile of queries ("0" = no tiling, every contribution is an atomic add)
+ *                                  instead of on samples sorted by key cell; also changes
+ *                                  dsa3d_backward_workspace_bytes
  *   DSA3D_NO_TENSOR_FIXED_WINDOW   dsa3d_forward_fixed_window and dsa3d_forward_bounded_offsets use the general
  *                                  kernel, dsa3d_backward_bounded_offsets the kernels of dsa3d_backward;
  *                                  dsa3d_backward_fixed_window uses its per-row CUDA-core kernels only
@@ -425,8 +419,8 @@ int dsa3d_forward_bounded_offsets(const void* q, const void* k, const void* v, c
  * asynchronous.  dk and dv of the tile route are written once in `dtype` (no atomics, bitwise deterministic).
  * `workspace`: dsa3d_backward_bounded_offsets_workspace_bytes(...) bytes (for the tile route 2.7 KB per
  * (token, head): the tables and the coefficient boxes), 16-byte aligned, contents undefined afterwards.
- * Other shapes and dtypes, grids of 2^31 / (125 heads) tokens or more, and the switches
- * DSA3D_NO_TENSOR_FIXED_WINDOW and DSA3D_KEY_BLOCKS=1, make it dsa3d_backward.  Bounded waits as in dsa3d_offsets_linear_forward (dsa3d_device_timeout_flag).
+ * Other shapes and dtypes, grids of 2^31 / (125 heads) tokens or more, and the switch
+ * DSA3D_NO_TENSOR_FIXED_WINDOW make it dsa3d_backward.  Bounded waits as in dsa3d_offsets_linear_forward (dsa3d_device_timeout_flag).
  */
 int dsa3d_backward_bounded_offsets(const void* q, const void* k, const void* v, const float* offsets, const float* lse,
                                    const void* dout, int T, int H, int W, int heads, int d, const int window[3], void* dq,

@@ -61,10 +61,6 @@ int make_problem(int T, int H, int W, int heads, int d, const int* window, int d
     pr.halo = 0;
     pr.tiles_t = pr.tiles_y = pr.tiles_x = 0;
     pr.tt_begin = pr.tt_count = 0;
-    pr.key_blocks = 0;
-    pr.blk_count = nullptr;
-    pr.blk_list = nullptr;
-    pr.blk_cap = 0;
     pr.gate = nullptr;
     pr.debug_word = debug_word_address();
     return DSA3D_OK;
@@ -94,10 +90,6 @@ void set_tiling(dsa3d::Problem& pr) {
     pr.tiles_x = (pr.W + tx - 1) / tx;
     pr.tt_begin = 0;
     pr.tt_count = pr.tiles_t;
-    // DSA3D_KEY_BLOCKS=1 replaces the tile kernel by the tensor-core key-block kernel where that covers the
-    // shape (and no tiling was asked for explicitly): correct and tested, but slower so far.
-    const char* kb = getenv("DSA3D_KEY_BLOCKS");
-    pr.key_blocks = (kb && kb[0] == '1' && !getenv("DSA3D_TILE") && dsa3d::key_blocks_shape_covered(pr)) ? 1 : 0;
 }
 
 struct BackwardWorkspace {
@@ -112,14 +104,8 @@ BackwardWorkspace backward_workspace(const dsa3d::Problem& pr, int dtype, bool t
     if (tiled && pr.tile_t >= 1) {
         // rounded up so that the 16-byte bin entries behind it stay 16-byte aligned
         w.coef_bytes = (static_cast<size_t>(pr.items) * pr.P * sizeof(float2) + 255) & ~static_cast<size_t>(255);
-        if (pr.key_blocks) {
-            // per-block counters and sample lists, sorted records of the resident CTAs, in place of the bin entries
-            const dsa3d::KeyBlockLayout kb = dsa3d::key_block_layout(pr);
-            w.scratch_bytes = kb.count_bytes + kb.list_bytes + kb.sorted_bytes;
-        } else {
-            w.entries_per_cta = static_cast<long long>(pr.tile_t) * pr.tile_y * pr.tile_x * pr.P * 8;
-            w.scratch_bytes = static_cast<size_t>(kTileSlots) * w.entries_per_cta * sizeof(dsa3d::TileEntry);
-        }
+        w.entries_per_cta = static_cast<long long>(pr.tile_t) * pr.tile_y * pr.tile_x * pr.P * 8;
+        w.scratch_bytes = static_cast<size_t>(kTileSlots) * w.entries_per_cta * sizeof(dsa3d::TileEntry);
     }
     w.total = w.acc_bytes + w.coef_bytes + w.scratch_bytes;
     return w;
@@ -228,9 +214,7 @@ int dsa3d_forward_bounded_offsets(const void* q, const void* k, const void* v, c
 
 namespace {
 bool bounded_backward_tiled(const dsa3d::Problem& pr, int dtype) {
-    const char* kb = std::getenv("DSA3D_KEY_BLOCKS");
-    return dtype == DSA3D_BF16 && dsa3d::bounded_offsets_backward_covers(pr, true) &&
-           !std::getenv("DSA3D_NO_TENSOR_FIXED_WINDOW") && !(kb && kb[0] == '1');
+    return dtype == DSA3D_BF16 && dsa3d::bounded_offsets_backward_covers(pr, true) && !std::getenv("DSA3D_NO_TENSOR_FIXED_WINDOW");
 }
 }  // namespace
 
@@ -368,7 +352,8 @@ struct BackwardPlan {
     float2* coef = nullptr;
     void* scratch = nullptr;
     void* workspace = nullptr;
-    bool cells = false;               // samples sorted by key cell instead of the gather and tile kernels
+    void* cells = nullptr;            // scratch of the cell-sorted route; NULL: the gather and tile kernels
+    size_t cells_bytes = 0;
     int ctas = 0;                     // resident CTAs of the tile kernel
 };
 
@@ -390,14 +375,11 @@ int backward_plan(int T, int H, int W, int heads, int d, const int* window, int 
     plan.acc_dv = plan.bf16 ? reinterpret_cast<float*>(wsp) + plan.count : static_cast<float*>(dv);
     plan.coef = plan.ws.coef_bytes ? reinterpret_cast<float2*>(wsp + plan.ws.acc_bytes) : nullptr;
     plan.scratch = plan.ws.scratch_bytes ? wsp + plan.ws.acc_bytes + plan.ws.coef_bytes : nullptr;
-    if (plan.pr.key_blocks) {
-        const dsa3d::KeyBlockLayout kb = dsa3d::key_block_layout(plan.pr);
-        plan.pr.blk_count = static_cast<uint32_t*>(plan.scratch);
-        plan.pr.blk_list = reinterpret_cast<uint32_t*>(static_cast<char*>(plan.scratch) + kb.count_bytes);
-        plan.pr.blk_cap = kb.cap;
+    // Everything behind the accumulators, unless DSA3D_TILE asks for the gather and tile kernels.
+    if (plan.bf16 && !getenv("DSA3D_TILE")) {
+        plan.cells = wsp + plan.ws.acc_bytes;
+        plan.cells_bytes = workspace_bytes - plan.ws.acc_bytes;
     }
-    // DSA3D_TILE asks for the gather and tile kernels, DSA3D_KEY_BLOCKS for the key-block kernel
-    plan.cells = plan.coef && !plan.pr.key_blocks && !getenv("DSA3D_TILE");
     if (plan.coef) {
         int dev = 0, sms = 0;
         cudaError_t e = cudaGetDevice(&dev);
@@ -448,12 +430,8 @@ int backward_frames(const BackwardPlan& plan, const void* q, const void* k, cons
     const dsa3d::Problem pr = frames_of(plan.pr, f0, f1);
     cudaError_t e = record(2, stream);
     if (e != cudaSuccess) return cuda_failed(e);
-    if (pr.key_blocks) {                 // the sample lists of the key blocks start empty for every launch
-        e = cudaMemsetAsync(pr.blk_count, 0, dsa3d::key_block_layout(pr).count_bytes, stream);
-        if (e != cudaSuccess) return cuda_failed(e);
-    }
-    if (plan.cells && dsa3d::try_cells_backward(q, k, v, offsets, lse, dout, dq, plan.acc_dk, plan.acc_dv, doffsets, plan.coef,
-                                                plan.ws.coef_bytes + plan.ws.scratch_bytes, pr, stream, &e)) {
+    if (plan.cells && dsa3d::try_cells_backward(q, k, v, offsets, lse, dout, dq, plan.acc_dk, plan.acc_dv, doffsets, plan.cells,
+                                                plan.cells_bytes, pr, stream, &e)) {
         if (e != cudaSuccess) return cuda_failed(e);
         e = record(3, stream);
         if (e != cudaSuccess) return cuda_failed(e);
@@ -475,9 +453,8 @@ int backward_frames(const BackwardPlan& plan, const void* q, const void* k, cons
     if (plan.coef) {
         e = record(4, stream);
         if (e != cudaSuccess) return cuda_failed(e);
-        e = pr.key_blocks ? dsa3d::launch_dkdv_blocks(q, dout, offsets, plan.coef, plan.acc_dk, plan.acc_dv, pr, stream)
-                          : dsa3d::launch_scatter_tiles(q, dout, offsets, plan.coef, plan.acc_dk, plan.acc_dv, plan.scratch,
-                                                        plan.ctas, plan.ws.entries_per_cta, pr, stream);
+        e = dsa3d::launch_scatter_tiles(q, dout, offsets, plan.coef, plan.acc_dk, plan.acc_dv, plan.scratch, plan.ctas,
+                                        plan.ws.entries_per_cta, pr, stream);
         if (e != cudaSuccess) return cuda_failed(e);
         e = record(5, stream);
         if (e != cudaSuccess) return cuda_failed(e);

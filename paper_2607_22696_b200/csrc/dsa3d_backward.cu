@@ -250,9 +250,7 @@ backward_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __res
             const int p = pb + gl;
             const Cell cell = make_cell(pr, t, y, x, p, off_row + p * 3);
             mine = to_sample(pr, cell);
-            // corners the tile kernel (or the key-block kernel) does not take
-            if (pr.key_blocks) mine.mask = active ? block_lists_append(pr, cell, t, y, x, m, p) : 0u;
-            else mine.mask = cell.mask & ~halo_corner_mask(pr, cell, t, y, x);
+            mine.mask = cell.mask & ~halo_corner_mask(pr, cell, t, y, x);       // corners the tile kernel does not take
             if (!active) mine.mask = 0u;
             const float* sts = stats + p * kStats;
             const float alpha = sts[0];

@@ -78,8 +78,9 @@ int dsa3d_backward_noalloc(const void* q, const void* k, const void* v, const fl
     const int rc = scratch_for_current_device(&scratch);
     if (rc != DSA3D_OK) return rc;
     // The shared implementation validates the rest, clears the accumulators (the array keeps
-    // whatever the previous call left) and scatters every dK/dV contribution straight into
-    // them: the tile pre-reduction of dsa3d_backward needs far more scratch than this array.
+    // whatever the previous call left) and takes what the array has left behind them as the scratch of the
+    // cell-sorted kernels, in as many passes as that needs.  Where it is too little for the smallest pass, every dK/dV
+    // contribution is scattered straight into the accumulators.
     return dsa3d::backward_impl(q, k, v, offsets, lse, dout, T, H, W, heads, d, window, dq, dk, dv, doffsets,
                                 scratch, 2 * kMaxElements * sizeof(float), dtype, stream, false);
 }
