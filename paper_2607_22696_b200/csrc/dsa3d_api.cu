@@ -303,7 +303,8 @@ int dsa3d_backward_fixed_window(const void* q, const void* k, const void* v, con
     if (dsa3d::fixed_window_table_floats(pr, dtype == DSA3D_BF16) > 0 && !std::getenv("DSA3D_NO_TENSOR_FIXED_WINDOW")) {
         const size_t coef_bytes = (static_cast<size_t>(pr.items) * pr.P * sizeof(float2) + 255) & ~static_cast<size_t>(255);
         float* tab = reinterpret_cast<float*>(static_cast<char*>(workspace) + coef_bytes);
-        if (dsa3d::try_fixed_window_tables(q, k, v, dout, tab, pr, st, &e)) {
+        if (dsa3d::try_fixed_window_tables(q, k, v, dout, tab, pr,
+                                           dsa3d::fixed_window_table_narrow(pr, doffsets != nullptr), st, &e)) {
             if (e != cudaSuccess) return cuda_failed(e);
             table = tab;
         }

@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(256, TABLE ? DSA3D_FWB_TABLE_BLOCKS : 1)
 fixed_window_backward_query_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
                                    const float* __restrict__ lse, const T* __restrict__ dout, T* __restrict__ dq,
                                    float* __restrict__ doffsets, float2* __restrict__ coef,
-                                   const float* __restrict__ table, const bool coef_planes, const Problem pr) {
+                                   const float* __restrict__ table, const bool narrow, const bool coef_planes, const Problem pr) {
     using E = Elt<T, 1>;
     using Row = typename E::Row;
     constexpr int VEC = E::VEC;
@@ -63,9 +63,10 @@ fixed_window_backward_query_kernel(const T* __restrict__ q, const T* __restrict_
     if (!active) item = pr.items - 1;
 
     const bool want_doff = doffsets != nullptr;
-    // with a table the box always has the +1 neighbours (that is how the table is laid out)
-    const bool wide = want_doff || TABLE;
-    const int BT = win_t + (wide ? 1 : 0), BY = win_y + (wide ? 1 : 0), BX = win_x + (wide ? 1 : 0);
+    // a table has the +1 neighbours, or (narrow) box rows padded to whole 16-byte pieces: the box is read as it is laid out
+    const bool wide = want_doff || (TABLE && !narrow);
+    const int BT = win_t + (wide ? 1 : 0), BY = win_y + (wide ? 1 : 0);
+    const int BX = TABLE && narrow ? (win_x + 3) / 4 * 4 : win_x + (wide ? 1 : 0);
     const int NB = BT * BY * BX;
     const int NB8 = (NB + 7) & ~7;
     // per block: box_tab[NB8] = displacement of box position idx from the box origin and whether
@@ -300,8 +301,10 @@ template <typename T, int D>
 cudaError_t launch_t(const void* q, const void* k, const void* v, const float* lse, const void* dout, void* dq,
                      void* dk, void* dv, float* doffsets, float2* coef, const float* table, const Problem& pr,
                      bool tile_grad, cudaStream_t stream) {
+    const bool narrow = table && fixed_window_table_narrow(pr, doffsets != nullptr);
     constexpr int LPR = D / Elt<T, 1>::VEC;
-    const int box = (doffsets || table) ? (pr.kt + 1) * (pr.kh + 1) * (pr.kw + 1) : pr.P;
+    const int box = narrow ? pr.kt * pr.kh * ((pr.kw + 3) / 4 * 4)
+                           : (doffsets || table) ? (pr.kt + 1) * (pr.kh + 1) * (pr.kw + 1) : pr.P;
     const size_t box8 = static_cast<size_t>((box + 7) & ~7);
     const size_t per_group = (2 * box8 + 2 * pr.P) * sizeof(float);
     const size_t tables = box8 * sizeof(int4) + static_cast<size_t>((pr.P + 3) & ~3) * sizeof(int);
@@ -327,7 +330,7 @@ cudaError_t launch_t(const void* q, const void* k, const void* v, const float* l
     const bool tiled = planes || (std::is_same<T, __nv_bfloat16>::value && tile_grad && fixed_window_tile_grad_covers(pr, true));
     qk<<<static_cast<unsigned>(blocks), threads, smem, stream>>>(
         static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v), lse, static_cast<const T*>(dout),
-        tiled ? nullptr : static_cast<T*>(dq), doffsets, coef, table, planes, pr);
+        tiled ? nullptr : static_cast<T*>(dq), doffsets, coef, table, narrow, planes, pr);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (tiled) {
@@ -338,7 +341,7 @@ cudaError_t launch_t(const void* q, const void* k, const void* v, const float* l
         // coefficients in the order the key kernel reads them)
         qk<<<static_cast<unsigned>(blocks), threads, smem, stream>>>(
             static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v), lse, static_cast<const T*>(dout),
-            static_cast<T*>(dq), doffsets, coef, table, false, pr);
+            static_cast<T*>(dq), doffsets, coef, table, narrow, false, pr);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }

@@ -8,7 +8,8 @@
 // tile's region (tile + box - 1 per axis), which this kernel forms by tcgen05.mma one region
 // plane at a time (fp32 accumulators in TMEM) and from which every thread copies the box of its
 // query into a table in global memory:  table[item][0][cell] = a,  table[item][1][cell] = b  with
-// item = token * heads + head and cell = (u * (kh+1) + v) * (kw+1) + w.  Positions outside the grid
+// item = token * heads + head and cell = (u * (kh+1) + v) * (kw+1) + w (without the neighbours, when nobody reads
+// them: see fixed_window_table_narrow).  Positions outside the grid
 // read as zero rows (TMA fill), i.e. a = b = 0, which is what the gather kernel would have used.
 // fixed_window_backward_query_kernel then takes its dot products from the table instead of
 // gathering K and V rows.
@@ -33,11 +34,14 @@ constexpr int kTbWorkers = 128 * kTbSplit, kTbThreads = kTbWorkers + 96;      //
 constexpr int kTbSlots = 4;                                                   // plane buffers, at most
 constexpr int kTbScoreBufs = 4;                                               // score planes in flight in TMEM, at most
 
-template <int D, int KT, int KH, int KW>
+// PAD: rows of the box padded to whole 16-byte pieces in the table, so that a row of an odd length is written in
+// whole pieces (and whole 32-byte sectors for rows of 5 to 8) instead of float by float.
+template <int D, int KT, int KH, int KW, bool PAD = false>
 struct TableShape {
     static constexpr int NH = D / 64;
     static constexpr int BT = KT + 1, BY = KH + 1, BX = KW + 1;     // the box of a query
-    static constexpr int CELLS = BT * BY * BX, CELLS8 = (CELLS + 7) / 8 * 8;
+    static constexpr int BXP = PAD ? (BX + 3) / 4 * 4 : BX;         // floats of a box row in the table
+    static constexpr int CELLS = BT * BY * BXP, CELLS8 = (CELLS + 7) / 8 * 8;
     static constexpr int RT = kTbTT + BT - 1, RY = kTbTY + BY - 1, RX = kTbTX + BX - 1;
     static constexpr int PS = RY * RX, PSP = (PS + 15) / 16 * 16;
     static constexpr int PIECES = (PS + 31) / 32;
@@ -57,9 +61,9 @@ struct TableShape {
     static_assert(SLOT_HALF % 1024 == 0 || PSP % 8 == 0, "");
 };
 
-template <int D, int KT, int KH, int KW>
+template <int D, int KT, int KH, int KW, bool PAD>
 struct __align__(1024) TbSmem {
-    using S = TableShape<D, KT, KH, KW>;
+    using S = TableShape<D, KT, KH, KW, PAD>;
     unsigned char a[2][S::A_BYTES];                                 // Q, dO: 64-channel halves, swizzled 128-byte rows
     unsigned char slot[S::NS][S::NH][(S::SLOT_HALF + 1023) / 1024 * 1024];
     unsigned char stage[S::STAGE_BYTES];                            // a score plane as [column][query] floats
@@ -71,21 +75,21 @@ struct __align__(1024) TbSmem {
 // the warps that share a TMEM quadrant
 __device__ __forceinline__ void pair_barrier(int id) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(32 * kTbSplit) : "memory"); }
 
-template <int D, int KT, int KH, int KW>
+template <int D, int KT, int KH, int KW, bool PAD>
 __global__ void __launch_bounds__(kTbThreads, 1)
 fixed_window_tables_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_do,
                            const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                            float* __restrict__ table, int T, int H, int W, int heads, int tiles_x, int tiles_y, int total,
                            int* timeout_flag, const int* __restrict__ gate) {
-    using S = TableShape<D, KT, KH, KW>;
+    using S = TableShape<D, KT, KH, KW, PAD>;
     constexpr int NH = S::NH, RT = S::RT, RX = S::RX, PS = S::PS, PSP = S::PSP, VH = S::VH, NS = S::NS;
-    constexpr int BT = S::BT, BY = S::BY, BX = S::BX;
+    constexpr int BT = S::BT, BY = S::BY, BX = S::BX, BXP = S::BXP;
     constexpr int JOBS = 2 * RT;                                      // per tile: RT planes of K (against Q), RT of V (against dO)
     constexpr int NB = S::NB;
     constexpr int TMEM_COLS = NB * S::SBUF <= 128 ? 128 : (NB * S::SBUF <= 256 ? 256 : 512);
     extern __shared__ unsigned char raw[];
-    TbSmem<D, KT, KH, KW>& s =
-        *reinterpret_cast<TbSmem<D, KT, KH, KW>*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
+    TbSmem<D, KT, KH, KW, PAD>& s =
+        *reinterpret_cast<TbSmem<D, KT, KH, KW, PAD>*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     if (tid == 0) {
@@ -236,10 +240,10 @@ fixed_window_tables_kernel(const __grid_constant__ CUtensorMap map_q, const __gr
                         // this thread's rows of the box plane are neighbours (vv = half * VH ...), so its cells
                         // are one contiguous run of the table: written as 16-byte pieces when BX = 4 (a warp's
                         // stores then fill whole 32-byte sectors instead of touching each one eight times)
-                        float* dst = my_table + which * S::CELLS8 + u_rt * (BY * BX) + half * VH * BX;
-                        float cells[VH * BX];
+                        float* dst = my_table + which * S::CELLS8 + u_rt * (BY * BXP) + half * VH * BXP;
+                        float cells[VH * BXP];
 #pragma unroll
-                        for (int i = 0; i < VH * BX; ++i) cells[i] = 0.0f;
+                        for (int i = 0; i < VH * BXP; ++i) cells[i] = 0.0f;
 #pragma unroll
                         for (int sub = 0; sub < S::SUBS; ++sub) {
                             constexpr int PPS = S::PPS;
@@ -257,7 +261,7 @@ fixed_window_tables_kernel(const __grid_constant__ CUtensorMap map_q, const __gr
                                     for (int ww = 0; ww < BX; ++ww) {
                                         const int vv = vi + half * VH;
                                         const int col = (ly + vv) * RX + lx + ww - sub * PPS * 32;
-                                        if (vv < BY && (S::SUBS == 1 || (col >= 0 && col < PPS * 32))) cells[vi * BX + ww] = stage[col * kTbQ + r];
+                                        if (vv < BY && (S::SUBS == 1 || (col >= 0 && col < PPS * 32))) cells[vi * BXP + ww] = stage[col * kTbQ + r];
                                     }
                             }
                             pair_barrier(1 + lt);                     // both have copied: the staging rows may be refilled
@@ -266,7 +270,13 @@ fixed_window_tables_kernel(const __grid_constant__ CUtensorMap map_q, const __gr
                             // the run of VH * BX floats, in the widest pieces its alignment allows
                             constexpr int RUN = VH * BX;
                             constexpr bool whole = BY % kTbSplit == 0;     // every thread of the group has all VH rows
-                            if constexpr (whole && RUN % 4 == 0 && (BY * BX) % 4 == 0 && S::CELLS8 % 4 == 0) {
+                            if constexpr (PAD) {
+#pragma unroll
+                                for (int i = 0; i < VH * BXP / 4; ++i)
+                                    if (4 * i / BXP + half * VH < BY)
+                                        reinterpret_cast<float4*>(dst)[i] =
+                                            make_float4(cells[4 * i], cells[4 * i + 1], cells[4 * i + 2], cells[4 * i + 3]);
+                            } else if constexpr (whole && RUN % 4 == 0 && (BY * BX) % 4 == 0 && S::CELLS8 % 4 == 0) {
 #pragma unroll
                                 for (int i = 0; i < RUN / 4; ++i)
                                     reinterpret_cast<float4*>(dst)[i] = make_float4(cells[4 * i], cells[4 * i + 1], cells[4 * i + 2], cells[4 * i + 3]);
@@ -317,10 +327,10 @@ fixed_window_tables_kernel(const __grid_constant__ CUtensorMap map_q, const __gr
     if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS));
 }
 
-template <int D, int KT, int KH, int KW>
+template <int D, int KT, int KH, int KW, bool PAD = false>
 cudaError_t launch_tables(const void* q, const void* k, const void* v, const void* dout, float* table, const Problem& pr,
                           int* flag, cudaStream_t stream, bool* unsupported, const int* gate = nullptr) {
-    using S = TableShape<D, KT, KH, KW>;
+    using S = TableShape<D, KT, KH, KW, PAD>;
     const unsigned long long d = static_cast<unsigned long long>(pr.d), hd = static_cast<unsigned long long>(pr.heads);
     const unsigned long long dims[5] = {d, hd, static_cast<unsigned long long>(pr.W), static_cast<unsigned long long>(pr.H),
                                         static_cast<unsigned long long>(pr.T)};
@@ -343,8 +353,8 @@ cudaError_t launch_tables(const void* q, const void* k, const void* v, const voi
         *unsupported = true;
         return cudaSuccess;
     }
-    const size_t smem = sizeof(TbSmem<D, KT, KH, KW>) + 1024;
-    auto kern = fixed_window_tables_kernel<D, KT, KH, KW>;
+    const size_t smem = sizeof(TbSmem<D, KT, KH, KW, PAD>) + 1024;
+    auto kern = fixed_window_tables_kernel<D, KT, KH, KW, PAD>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0;
@@ -388,24 +398,30 @@ int fixed_window_table_floats(const Problem& pr, bool bf16) {
     return 0;
 }
 
+// Without dOffsets nobody reads the +1 neighbours: for a window of odd lengths the box is then the window itself, which
+// is the table of the window one smaller per axis (that table's box starts at the same position: odd / 2 == (odd - 1) / 2).
+// Per item 40, 120 or 168 floats instead of 64, 144 or 256 for (3,3,3), (3,5,5), (3,7,7), and smaller region planes.
+bool fixed_window_table_narrow(const Problem& pr, bool want_doffsets) {
+    return !want_doffsets && (pr.kt & 1) && (pr.kh & 1) && (pr.kw & 1);
+}
+
 bool try_fixed_window_tables(const void* q, const void* k, const void* v, const void* dout, float* table,
-                             const Problem& pr, cudaStream_t stream, cudaError_t* err) {
+                             const Problem& pr, bool narrow, cudaStream_t stream, cudaError_t* err) {
     *err = cudaSuccess;
     if (fixed_window_table_floats(pr, true) == 0) return false;
     int* flag = timeout_flag_device_address();
     if (!flag) return false;
     bool unsupported = false;
-    const bool w333 = pr.kt == 3 && pr.kh == 3, w355 = pr.kt == 3 && pr.kh == 5, w377 = pr.kt == 3 && pr.kh == 7;
-    if (pr.d == 128)
-        *err = w333 ? launch_tables<128, 3, 3, 3>(q, k, v, dout, table, pr, flag, stream, &unsupported)
-             : w355 ? launch_tables<128, 3, 5, 5>(q, k, v, dout, table, pr, flag, stream, &unsupported)
-             : w377 ? launch_tables<128, 3, 7, 7>(q, k, v, dout, table, pr, flag, stream, &unsupported)
-                    : launch_tables<128, 2, 2, 2>(q, k, v, dout, table, pr, flag, stream, &unsupported);
-    else
-        *err = w333 ? launch_tables<64, 3, 3, 3>(q, k, v, dout, table, pr, flag, stream, &unsupported)
-             : w355 ? launch_tables<64, 3, 5, 5>(q, k, v, dout, table, pr, flag, stream, &unsupported)
-             : w377 ? launch_tables<64, 3, 7, 7>(q, k, v, dout, table, pr, flag, stream, &unsupported)
-                    : launch_tables<64, 2, 2, 2>(q, k, v, dout, table, pr, flag, stream, &unsupported);
+#define DSA3D_TABLES(DD)                                                                                            \
+    (narrow ? (pr.kh == 3   ? launch_tables<DD, 2, 2, 2, true>(q, k, v, dout, table, pr, flag, stream, &unsupported)  \
+               : pr.kh == 5 ? launch_tables<DD, 2, 4, 4, true>(q, k, v, dout, table, pr, flag, stream, &unsupported)  \
+                            : launch_tables<DD, 2, 6, 6, true>(q, k, v, dout, table, pr, flag, stream, &unsupported)) \
+            : (pr.kh == 3   ? launch_tables<DD, 3, 3, 3>(q, k, v, dout, table, pr, flag, stream, &unsupported)        \
+               : pr.kh == 2 ? launch_tables<DD, 2, 2, 2>(q, k, v, dout, table, pr, flag, stream, &unsupported)        \
+               : pr.kh == 5 ? launch_tables<DD, 3, 5, 5>(q, k, v, dout, table, pr, flag, stream, &unsupported)        \
+                            : launch_tables<DD, 3, 7, 7>(q, k, v, dout, table, pr, flag, stream, &unsupported)))
+    *err = pr.d == 128 ? DSA3D_TABLES(128) : DSA3D_TABLES(64);
+#undef DSA3D_TABLES
     return !unsupported;
 }
 

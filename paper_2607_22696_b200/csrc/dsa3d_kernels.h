@@ -70,7 +70,10 @@ cudaError_t launch_fixed_window_backward(const void* q, const void* k, const voi
 // Dot-product tables of the fixed-window backward on the tensor cores (dsa3d_fixed_window_tables.cu).
 // fixed_window_table_floats: floats per (token, head) item, 0 when the shape is not covered.
 // try_fixed_window_tables: false when the shape is not covered (nothing launched).
+// fixed_window_table_narrow: whether the box is the window without its +1 neighbours, rows of kw padded to whole
+// 16-byte pieces (odd windows, dOffsets not asked for).
 int fixed_window_table_floats(const Problem& pr, bool bf16);
+bool fixed_window_table_narrow(const Problem& pr, bool want_doffsets);
 
 // The three weighted row sums of the fixed-window backward (dQ over the K region, dK over the q region, dV over
 // the dO region) per tile of 4 x 4 x 8 outputs with the region in shared memory (dsa3d_fixed_window_tile_grad.cu),
@@ -106,7 +109,7 @@ bool fixed_window_planes_grad_covers(const Problem& pr, bool bf16);
 bool try_fixed_window_planes_grad(const void* q, const void* k, const void* dout, const float* coef_planes, void* dq, void* dk,
                                   void* dv, const Problem& pr, cudaStream_t stream, cudaError_t* err);
 bool try_fixed_window_tables(const void* q, const void* k, const void* v, const void* dout, float* table,
-                             const Problem& pr, cudaStream_t stream, cudaError_t* err);
+                             const Problem& pr, bool narrow, cudaStream_t stream, cudaError_t* err);
 
 // Host side of the TMA kernels (dsa3d_producer.cu).  encode_tensor_map_bf16: a tiled map over
 // a bf16 tensor of `rank` dimensions (innermost first; strides_bytes has rank-1 entries, the
