@@ -245,6 +245,169 @@ fixed_window_backward_query_kernel(const T* __restrict__ q, const T* __restrict_
     if (active) E::store(dq + row * D + ch, dqv);
 }
 
+// The coefficients alone, from the table - all the tile kernels need when dOffsets is not wanted: a thread per item,
+// a warp per 32 consecutive tokens of a head (two warps that share the samples for the larger windows, whose 43 KB of
+// table rows leave room for five blocks).  The table rows come into shared memory asynchronously, in rows 4 floats
+// longer (an odd number of 16-byte pieces: the threads' 16-byte reads of their own rows meet no bank twice);
+// softmax, delta and dS are then the thread's own serial sums, without a reduction across lanes, and a warp's stores of
+// one sample's coefficients are 32 neighbours.  What bounds it is the table's trip from memory (1.3 KB in, 1.2 KB out
+// per item for (3,7,7)) and the instructions of two walks over the samples.  fixed_window_backward_query_kernel, 16
+// lanes per item, spends its time in the latency of many short phases: 32x45x80x16, d 128, on a B200, (3,3,3)
+// 1.48 -> 0.30 ms, (3,7,7) 4.02 -> 1.48 ms.
+template <int KT, int KH, int KW>
+struct CoefShape {
+    static constexpr bool NARROW = (KT & 1) && (KH & 1) && (KW & 1);         // as fixed_window_table_narrow without dOffsets
+    static constexpr bool PLANES = KT * KH * KW > 32;                        // written as the plane-by-plane tile kernel reads them
+    static constexpr int P = KT * KH * KW, WARPS = PLANES ? 2 : 1;
+    static constexpr int BT = NARROW ? KT : KT + 1, BY = NARROW ? KH : KH + 1, BX = NARROW ? (KW + 3) / 4 * 4 : KW + 1;
+    static constexpr int NB8 = (BT * BY * BX + 7) / 8 * 8;
+    static constexpr int PITCH = 2 * NB8 + 4;                                // floats
+    static_assert((PITCH / 4) % 2 == 1 && P <= NB8, "");
+};
+
+template <int D, int KT, int KH, int KW>
+__global__ void __launch_bounds__(32 * CoefShape<KT, KH, KW>::WARPS)
+fixed_window_coefficients_kernel(const float* __restrict__ lse, const float* __restrict__ table, float2* __restrict__ coef,
+                                 const Problem pr) {
+    using S = CoefShape<KT, KH, KW>;
+    constexpr int LPR = D / Elt<__nv_bfloat16, 1>::VEC;                      // lanes of an item in the query kernel
+    extern __shared__ __align__(16) float rows[];                            // [32][PITCH]
+    __shared__ float part_other[S::WARPS][LPR / 2][32];
+    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
+    const int m = static_cast<int>(blockIdx.x % static_cast<unsigned>(pr.heads));
+    const long long n0 = static_cast<long long>(blockIdx.x / static_cast<unsigned>(pr.heads)) * 32;
+    const int here = pr.N - n0 < 32 ? static_cast<int>(pr.N - n0) : 32;      // tokens of this block
+    constexpr int PIECES = 2 * S::NB8 / 4;                                   // 16-byte pieces of a table row
+    const float* src = table + (n0 * pr.heads + m) * (2 * S::NB8);
+    const long long src_step = static_cast<long long>(pr.heads) * (2 * S::NB8);
+    const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(rows));
+#pragma unroll 4
+    for (int c = threadIdx.x; c < here * PIECES; c += 32 * S::WARPS) {
+        const int i = c / PIECES, j = c - i * PIECES;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + (i * S::PITCH + 4 * j) * 4), "l"(src + i * src_step + 4 * j) : "memory");
+    }
+    const bool active = lane < here;
+    const long long row = (n0 + (active ? lane : 0)) * pr.heads + m;
+    const float lse2 = __ldg(lse + row) * kLog2e;
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+
+    const float scale = rsqrtf(static_cast<float>(D));
+    float* a = rows + lane * S::PITCH;                                       // a thread without a token works on what lies there, stores off
+    float* b = a + S::NB8;
+    // the samples of window row uv = (u, v): KW neighbouring cells
+    auto cell = [](int uv) { return ((uv / KH) * S::BY + uv % KH) * S::BX; };
+    auto load_row = [](const float* p, float (&x)[KW]) {
+        if constexpr (S::BX % 4 == 0) {
+#pragma unroll
+            for (int i = 0; i < S::BX; i += 4) {
+                const float4 w = *reinterpret_cast<const float4*>(p + i);
+                x[i] = w.x;
+                if (i + 1 < KW) x[i + 1] = w.y;
+                if (i + 2 < KW) x[i + 2] = w.z;
+                if (i + 3 < KW) x[i + 3] = w.w;
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < KW; ++i) x[i] = p[i];
+        }
+    };
+    // ---- alpha (over the dot products a), and delta: in the order of the query kernel's lanes and of its sum across
+    //      them, so that asking for dOffsets, which takes that kernel, changes no bit of the other gradients.  Of two
+    //      warps one takes the samples of the lower half of those lanes, the other those of the upper half.
+    float part[LPR];
+#pragma unroll
+    for (int i = 0; i < LPR; ++i) part[i] = 0.0f;
+    auto walk = [&](auto which) {                                            // -1: every sample
+        constexpr int kHalf = decltype(which)::value;
+#pragma unroll
+        for (int uv = 0; uv < KT * KH; ++uv) {
+            float al[KW], bb[KW];
+            load_row(a + cell(uv), al);
+            load_row(b + cell(uv), bb);
+#pragma unroll
+            for (int i = 0; i < KW; ++i) {
+                const int cls = (uv * KW + i) % LPR;
+                if (kHalf >= 0 && cls / (LPR / 2) != kHalf) continue;
+                const float alpha = exp2f(fmaf(al[i], scale * kLog2e, -lse2));            // a position outside the grid: logit 0
+                a[cell(uv) + i] = alpha;
+                part[cls] = fmaf(alpha, bb[i], part[cls]);
+            }
+        }
+    };
+    if constexpr (S::WARPS == 1) {
+        walk(std::integral_constant<int, -1>{});
+#pragma unroll
+        for (int i = 0; i < LPR / 2; ++i) part[i] += part[i + LPR / 2];
+    } else {
+        if (wi == 0) {
+            walk(std::integral_constant<int, 0>{});
+#pragma unroll
+            for (int i = 0; i < LPR / 2; ++i) part_other[0][i][lane] = part[i];
+        } else {
+            walk(std::integral_constant<int, 1>{});
+#pragma unroll
+            for (int i = 0; i < LPR / 2; ++i) part_other[1][i][lane] = part[i + LPR / 2];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < LPR / 2; ++i) part[i] = part_other[0][i][lane] + part_other[1][i][lane];
+    }
+#pragma unroll
+    for (int o = LPR / 4; o > 0; o >>= 1)
+#pragma unroll
+        for (int i = 0; i < o; ++i) part[i] += part[i + o];
+    const float delta = part[0];
+
+    // ---- the coefficients
+    if constexpr (S::PLANES) {
+        uint32_t* ck = reinterpret_cast<uint32_t*>(coef) + static_cast<long long>(m) * S::P * pr.N + n0 + lane;
+        const long long to_cv = pr.N * pr.heads * S::P;
+#pragma unroll 3
+        for (int uv = wi; uv < KT * KH; uv += S::WARPS) {
+            float al[KW], bb[KW];
+            load_row(a + cell(uv), al);
+            load_row(b + cell(uv), bb);
+            if (active) {
+                uint32_t* to = ck + static_cast<long long>(uv * KW) * pr.N;
+#pragma unroll
+                for (int i = 0; i < KW; ++i, to += pr.N) {
+                    *to = split_bf16_pair(scale * al[i] * (bb[i] - delta));
+                    to[to_cv] = split_bf16_pair(al[i]);
+                }
+            }
+        }
+    } else {
+        // pairs [item][sample], written out by the warp as a run of P pairs per item by way of the thread's row
+        float2 mine[S::P];
+#pragma unroll
+        for (int uv = 0; uv < KT * KH; ++uv) {
+            float al[KW], bb[KW];
+            load_row(a + cell(uv), al);
+            load_row(b + cell(uv), bb);
+#pragma unroll
+            for (int i = 0; i < KW; ++i) mine[uv * KW + i] = make_float2(scale * al[i] * (bb[i] - delta), al[i]);
+        }
+#pragma unroll
+        for (int p = 0; p < S::P; ++p) *reinterpret_cast<float2*>(a + 2 * p) = mine[p];
+        __syncwarp();
+        for (int c = lane; c < here * S::P; c += 32) {
+            const int i = c / S::P, p = c - i * S::P;
+            coef[((n0 + i) * pr.heads + m) * S::P + p] = *reinterpret_cast<const float2*>(rows + i * S::PITCH + 2 * p);
+        }
+    }
+}
+
+template <int D, int KT, int KH, int KW>
+cudaError_t launch_coefficients(const float* lse, const float* table, float2* coef, const Problem& pr, cudaStream_t stream) {
+    using S = CoefShape<KT, KH, KW>;
+    constexpr int smem = 32 * S::PITCH * static_cast<int>(sizeof(float));
+    static_assert(smem + 2 * 8 * 32 * 4 <= 48 * 1024, "");
+    const long long blocks = (pr.N + 31) / 32 * pr.heads;
+    fixed_window_coefficients_kernel<D, KT, KH, KW><<<static_cast<unsigned>(blocks), 32 * S::WARPS, smem, stream>>>(lse, table, coef, pr);
+    return cudaGetLastError();
+}
+
 template <typename T, int D>
 __global__ void __launch_bounds__(256)
 fixed_window_backward_key_kernel(const T* __restrict__ q, const T* __restrict__ dout, const float2* __restrict__ coef,
@@ -328,10 +491,23 @@ cudaError_t launch_t(const void* q, const void* k, const void* v, const float* l
     // small windows, as plane-by-plane products on the tensor cores for the larger ones
     const bool planes = std::is_same<T, __nv_bfloat16>::value && tile_grad && fixed_window_planes_grad_covers(pr, true);
     const bool tiled = planes || (std::is_same<T, __nv_bfloat16>::value && tile_grad && fixed_window_tile_grad_covers(pr, true));
-    qk<<<static_cast<unsigned>(blocks), threads, smem, stream>>>(
-        static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v), lse, static_cast<const T*>(dout),
-        tiled ? nullptr : static_cast<T*>(dq), doffsets, coef, table, narrow, planes, pr);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = cudaSuccess;
+    bool by_item = false;
+    if constexpr (std::is_same<T, __nv_bfloat16>::value && D >= 64) {
+        if (tiled && table && !doffsets) {                    // nothing but the coefficients is left to form here
+            by_item = true;
+            e = pr.kh == 7   ? launch_coefficients<D, 3, 7, 7>(lse, table, coef, pr, stream)
+                : pr.kh == 5 ? launch_coefficients<D, 3, 5, 5>(lse, table, coef, pr, stream)
+                : pr.kh == 3 ? launch_coefficients<D, 3, 3, 3>(lse, table, coef, pr, stream)
+                             : launch_coefficients<D, 2, 2, 2>(lse, table, coef, pr, stream);
+        }
+    }
+    if (!by_item) {
+        qk<<<static_cast<unsigned>(blocks), threads, smem, stream>>>(
+            static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v), lse, static_cast<const T*>(dout),
+            tiled ? nullptr : static_cast<T*>(dq), doffsets, coef, table, narrow, planes, pr);
+        e = cudaGetLastError();
+    }
     if (e != cudaSuccess) return e;
     if (tiled) {
         if (planes ? try_fixed_window_planes_grad(q, k, dout, reinterpret_cast<const float*>(coef), dq, dk, dv, pr, stream, &e)
