@@ -13,9 +13,30 @@ is the incoming one).  The log-sum-exp saved by the forward is not differentiabl
 """
 from __future__ import annotations
 
+import importlib.util
+import os
+
 import torch
 
 from . import binding
+
+_native_module = None
+
+
+def _native():
+    """The compiled forms of the functions below (csrc/dsa3d_autograd.cpp): same calls, without the interpreter.
+    They return None for arguments that have to be converted or refused first; the Python function does that."""
+    global _native_module
+    if _native_module is None:
+        binding.load()
+        path = os.path.join(os.path.dirname(binding.LIB_PATH), "_autograd_native.so")
+        if not os.path.exists(path):
+            raise RuntimeError(f"{path} is missing: build it with `python -m paper_2607_22696_b200.build`")
+        spec = importlib.util.spec_from_file_location("_autograd_native", path)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        _native_module = module
+    return _native_module
 
 
 def _dims(q):
@@ -145,9 +166,19 @@ def offsets_linear(u, w, bias):
 
 def dsa3d(q, k, v, offsets, window, residual=None):
     """3D deformable slide attention (Eq. 1, second term; plus `residual` if given)."""
-    return _Dsa3d.apply(q, k, v, offsets, residual, tuple(window))
+    window = tuple(int(s) for s in window)
+    if len(window) == 3:
+        out = _native().dsa3d(q, k, v, offsets, residual, *window)
+        if out is not None:
+            return out
+    return _Dsa3d.apply(q, k, v, offsets, residual, window)
 
 
 def dsa3d_fixed_window(q, k, v, window):
     """The operator with all offsets zero (no offsets tensor, no offset gradient)."""
-    return _Dsa3dFixedWindow.apply(q, k, v, tuple(window))
+    window = tuple(int(s) for s in window)
+    if len(window) == 3:
+        out = _native().dsa3d_fixed_window(q, k, v, *window)
+        if out is not None:
+            return out
+    return _Dsa3dFixedWindow.apply(q, k, v, window)
