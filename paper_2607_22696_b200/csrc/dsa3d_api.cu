@@ -424,15 +424,15 @@ dsa3d::Problem frames_of(const dsa3d::Problem& pr, int f0, int f1) {
     return s;
 }
 
-// dQ, dOffsets of the queries of frames [f0, f1) and their contributions to dK/dV.
+// dQ, dOffsets of the queries of frames [f0, f1) and their contributions to dK/dV; `clear`: zero the accumulators first.
 int backward_frames(const BackwardPlan& plan, const void* q, const void* k, const void* v, const float* offsets,
                     const float* lse, const void* dout, void* dq, float* doffsets, int f0, int f1,
-                    cudaStream_t stream, cudaEvent_t after_gather) {
+                    bool clear, cudaStream_t stream, cudaEvent_t after_gather) {
     const dsa3d::Problem pr = frames_of(plan.pr, f0, f1);
     cudaError_t e = record(2, stream);
     if (e != cudaSuccess) return cuda_failed(e);
     if (plan.cells && dsa3d::try_cells_backward(q, k, v, offsets, lse, dout, dq, plan.acc_dk, plan.acc_dv, doffsets, plan.cells,
-                                                plan.cells_bytes, pr, stream, &e)) {
+                                                plan.cells_bytes, plan.workspace, clear ? plan.ws.acc_bytes : 0, pr, stream, &e)) {
         if (e != cudaSuccess) return cuda_failed(e);
         e = record(3, stream);
         if (e != cudaSuccess) return cuda_failed(e);
@@ -441,6 +441,10 @@ int backward_frames(const BackwardPlan& plan, const void* q, const void* k, cons
             if (e != cudaSuccess) return cuda_failed(e);
         }
         return DSA3D_OK;
+    }
+    if (clear) {
+        const int rc = backward_clear(plan, stream);
+        if (rc != DSA3D_OK) return rc;
     }
     e = dsa3d::launch_backward(q, k, v, offsets, lse, dout, dq, plan.acc_dk, plan.acc_dv, doffsets, plan.coef, pr,
                                plan.bf16, stream);
@@ -466,11 +470,8 @@ int backward_frames(const BackwardPlan& plan, const void* q, const void* k, cons
 // Accumulators -> dk, dv (bf16 storage only; fp32 storage accumulated in place).
 int backward_finish(const BackwardPlan& plan, void* dk, void* dv, cudaStream_t stream) {
     if (!plan.bf16) return DSA3D_OK;
-    cudaError_t e = dsa3d::launch_convert_bf16(plan.acc_dk, dk, static_cast<long long>(plan.count), stream, plan.pr.gate);
-    if (e != cudaSuccess) return cuda_failed(e);
-    e = dsa3d::launch_convert_bf16(plan.acc_dv, dv, static_cast<long long>(plan.count), stream, plan.pr.gate);
-    if (e != cudaSuccess) return cuda_failed(e);
-    return DSA3D_OK;
+    const cudaError_t e = dsa3d::launch_convert_bf16(plan.acc_dk, dk, dv, static_cast<long long>(plan.count), stream, plan.pr.gate);
+    return e == cudaSuccess ? DSA3D_OK : cuda_failed(e);
 }
 
 int forward_frames(const dsa3d::Problem& full, const void* q, const void* k, const void* v, const float* offsets,
@@ -500,9 +501,7 @@ int dsa3d::backward_impl(const void* q, const void* k, const void* v, const floa
     if (rc != DSA3D_OK) return rc;
     plan.pr.gate = gate;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-    rc = backward_clear(plan, stream);
-    if (rc != DSA3D_OK) return rc;
-    rc = backward_frames(plan, q, k, v, offsets, lse, dout, dq, doffsets, 0, T, stream, nullptr);
+    rc = backward_frames(plan, q, k, v, offsets, lse, dout, dq, doffsets, 0, T, true, stream, nullptr);
     if (rc != DSA3D_OK) return rc;
     return backward_finish(plan, dk, dv, stream);
 }
@@ -693,8 +692,6 @@ int step_host_body(const void* q_h, const void* k_h, const void* v_h, const floa
     // fp32 storage accumulates dk/dv in place: the previous call's download of them comes first.
     // (bf16 accumulates in the workspace; its dk/dv are only written by backward_finish below.)
     if (!bf16) DSA3D_TRY(cudaStreamWaitEvent(stream, hs->dkdv_dl_done, 0));
-    st = backward_clear(plan, stream);
-    if (st != DSA3D_OK) return st;
     DSA3D_TRY(cudaStreamWaitEvent(stream, hs->kv_ready, 0));
     const float* off_d = reinterpret_cast<const float*>(base + a.offsets);
     float* lse_d = reinterpret_cast<float*>(base + a.lse);
@@ -717,7 +714,7 @@ int step_host_body(const void* q_h, const void* k_h, const void* v_h, const floa
 
         DSA3D_TRY(cudaStreamWaitEvent(stream, hs->dout_ready[s], 0));
         st = backward_frames(plan, base + a.q, k_d, v_d, off_d, lse_d, base + a.dout, base + a.dq,
-                             doff_d, f0, f1, stream, hs->gather_done[s]);
+                             doff_d, f0, f1, s == 0, stream, hs->gather_done[s]);
         if (st != DSA3D_OK) return st;
         DSA3D_TRY(cudaEventRecord(hs->slab_in_free[s], stream));
         DSA3D_TRY(cudaStreamWaitEvent(hs->out, hs->gather_done[s], 0));

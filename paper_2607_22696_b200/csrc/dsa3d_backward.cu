@@ -596,9 +596,11 @@ cudaError_t launch_scatter_tiles(const void* q, const void* dout, const float* o
 }
 
 __global__ void __launch_bounds__(256)
-convert_bf16_kernel(const float4* __restrict__ acc, uint2* __restrict__ dst, long long count4, const int* __restrict__ gate) {
+convert_bf16_kernel(const float4* __restrict__ acc, uint2* __restrict__ dk, uint2* __restrict__ dv, long long count4, const int* __restrict__ gate) {
     if (gate != nullptr && *gate == 0) return;      // the tile kernels of a bounded-offsets backward wrote dk and dv
     const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
+    uint2* dst = blockIdx.y ? dv : dk;
+    if (blockIdx.y) acc += count4;
     for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < count4; i += stride) {
         const float4 a = acc[i];
         const __nv_bfloat162 lo = __floats2bfloat162_rn(a.x, a.y);
@@ -626,13 +628,13 @@ cudaError_t launch_gated_clear(void* dst, size_t bytes, const int* gate, cudaStr
     return cudaGetLastError();
 }
 
-cudaError_t launch_convert_bf16(const float* acc, void* dst, long long count, cudaStream_t stream, const int* gate) {
+cudaError_t launch_convert_bf16(const float* acc, void* dk, void* dv, long long count, cudaStream_t stream, const int* gate) {
     const long long count4 = count / 4;      // d is a multiple of 32, so count is a multiple of 4
     long long blocks = (count4 + 255) / 256;
-    if (blocks > 148LL * 16) blocks = 148LL * 16;
+    if (blocks > 148LL * 8) blocks = 148LL * 8;
     if (blocks < 1) blocks = 1;
-    convert_bf16_kernel<<<static_cast<unsigned>(blocks), 256, 0, stream>>>(
-        reinterpret_cast<const float4*>(acc), reinterpret_cast<uint2*>(dst), count4, gate);
+    convert_bf16_kernel<<<dim3(static_cast<unsigned>(blocks), 2), 256, 0, stream>>>(
+        reinterpret_cast<const float4*>(acc), reinterpret_cast<uint2*>(dk), reinterpret_cast<uint2*>(dv), count4, gate);
     return cudaGetLastError();
 }
 

@@ -7,7 +7,8 @@
 //   cells_query_kernel   per query: alpha, delta, dS, dOffsets, the two coefficients per sample, dQ (a gather of K rows)
 //   cells_sums_kernel    per block: samples by cell, 16 at a time their contributions to the eight corner rows of dK or dV
 //                        (tensor cores), reduced into the fp32 accumulators
-//   cells_far_kernel     what falls beyond the bins (more than 12 positions from the query's tile), row by row
+//   far_part             what falls beyond the bins (more than 12 positions from the query's tile), row by row, in
+//                        CTAs of the last two block kernels
 #include <cuda_bf16.h>
 
 #include "dsa3d_cells.cuh"
@@ -22,7 +23,8 @@ using bf16 = __nv_bfloat16;
 // ------------------------------------------------------------------------------------------------ binning
 constexpr int kBinThreads = 512, kBinWarps = kBinThreads / 32, kCopies = 8;
 
-__device__ __forceinline__ void bin_block(const unsigned block, const float* __restrict__ offsets, const Problem& pr, const Slab& sl, unsigned inv_p) {
+__device__ __forceinline__ void bin_block(const unsigned block, const float* __restrict__ offsets, const Problem& pr, const Slab& sl, unsigned inv_p,
+                                          uint4* __restrict__ clear, long long clear_each, long long clear_all) {
     extern __shared__ __align__(16) unsigned char raw[];
     uint32_t* counters = reinterpret_cast<uint32_t*>(raw);                 // [kBins + 1][kCopies]: lanes of a warp mostly hit the same bin
     uint32_t* words = counters + (kBins + 1) * kCopies;                     // [kRows * P]: bin (9 bits), cell (6), rank in its counter (16)
@@ -35,6 +37,9 @@ __device__ __forceinline__ void bin_block(const unsigned block, const float* __r
     const int y0 = (r % sl.tiles_y) * 4, t0 = sl.f0 + (r / sl.tiles_y) * 4;
     const int samples = kRows * pr.P;
     if (block == 0 && tid == 0) { *sl.marked = 0; *sl.used = 0u; }
+    // the block's part of the accumulators: stores in the shadow of a kernel that waits for its offsets
+    const long long clear_to = min(clear_all, (block + 1ll) * clear_each);
+    for (long long i = block * clear_each + tid; i < clear_to; i += kBinThreads) clear[i] = make_uint4(0u, 0u, 0u, 0u);
     for (int i = tid; i < (kBins + 1) * kCopies / 4; i += kBinThreads) reinterpret_cast<uint4*>(counters)[i] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
     auto row_of = [&](int s) { return static_cast<int>((static_cast<unsigned long long>(static_cast<unsigned>(s)) * inv_p) >> 24); };
@@ -121,13 +126,14 @@ __device__ __forceinline__ void bin_block(const unsigned block, const float* __r
 
 template <bool kGated>
 __global__ void __launch_bounds__(kBinThreads, 2)
-cells_bin_kernel(const float* __restrict__ offsets, const __grid_constant__ Problem pr, const __grid_constant__ Slab sl, unsigned inv_p, unsigned blocks) {
+cells_bin_kernel(const float* __restrict__ offsets, const __grid_constant__ Problem pr, const __grid_constant__ Slab sl, unsigned inv_p, unsigned blocks,
+                 uint4* __restrict__ clear, long long clear_each, long long clear_all) {
     if constexpr (!kGated) {
-        bin_block(blockIdx.x, offsets, pr, sl, inv_p);
+        bin_block(blockIdx.x, offsets, pr, sl, inv_p, clear, clear_each, clear_all);
     } else {
         if (gated_off(pr)) return;
         for (unsigned block = blockIdx.x; block < blocks; block += gridDim.x) {
-            bin_block(block, offsets, pr, sl, inv_p);
+            bin_block(block, offsets, pr, sl, inv_p, clear, clear_each, clear_all);
             __syncthreads();
         }
     }
@@ -292,6 +298,96 @@ __device__ __forceinline__ void load_box(unsigned char* dst, const bf16* __restr
     }
 }
 
+// ------------------------------------------------------------------------------------------------ beyond the bins
+// The samples in bin kBins of every tile, a warp per sample, row by row: part `part` of `parts` (256 threads each).
+// kScatter: their contributions to dK and dV, and those of marked samples of the other bins; otherwise what the
+// products of cells_dots_kernel leave for the others.  There are none in nearly every call: the work rides in CTAs
+// behind those of the block kernels instead of two launches of its own.
+template <int D, bool kScatter>
+__device__ __noinline__ void far_part(const unsigned part, const unsigned parts, const bf16* __restrict__ q, const bf16* __restrict__ k, const bf16* __restrict__ v,
+                                      const bf16* __restrict__ dout, const float* __restrict__ offsets, float* __restrict__ acc_dk, float* __restrict__ acc_dv,
+                                      const Problem& pr, const Slab& sl) {
+    const int tiles = sl.heads * sl.tiles_t * sl.tiles_y * sl.tiles_x;
+    constexpr int V = D / 32;                       // channels per lane
+    const int lane = threadIdx.x & 31, warps = static_cast<int>(parts) * 8;
+    const long long tok = static_cast<long long>(pr.heads) * D;
+    const int per_head = sl.tiles_t * sl.tiles_y * sl.tiles_x;
+    [[maybe_unused]] const long long kv_extent = pr.N * pr.heads * D;
+    for (int base = (static_cast<int>(part) * 8 + static_cast<int>(threadIdx.x >> 5)) * 32; base < tiles; base += warps * 32) {
+        uint32_t mine = 0u;
+        if (base + lane < tiles) mine = __ldg(sl.seg + static_cast<long long>(base + lane) * (kBins + 1) + kBins);
+        const bool marked = kScatter && *sl.marked != 0;
+        if (marked) mine = ((mine & 0xffffu) + (mine >> 16)) << 16;        // all samples of the tile: those beyond the bins are its last
+        unsigned todo = __ballot_sync(kFullMask, (mine >> 16) != 0u);
+        while (todo) {
+            const int src = __ffs(static_cast<int>(todo)) - 1;
+            todo &= todo - 1u;
+            const uint32_t w = __shfl_sync(kFullMask, mine, src);
+            const long long tile = base + src;
+            const int m = sl.m0 + static_cast<int>(tile / per_head);
+            const uint32_t far_from = marked ? __ldg(sl.seg + tile * (kBins + 1) + kBins) & 0xffffu : 0u;
+            for (uint32_t i = 0; i < (w >> 16); ++i) {
+                const long long at = tile * (kRows * pr.P) + (w & 0xffffu) + i;
+                const int n = static_cast<int>(__ldg(sl.geo + at).x), p = static_cast<int>(__ldg(sl.meta + at) & 255u);
+                const int x = n % pr.W, y = (n / pr.W) % pr.H, t = n / (pr.W * pr.H);
+                const long long row = static_cast<long long>(n) * pr.heads + m;
+                const Sample smp = to_sample(pr, make_cell(pr, t, y, x, p, offsets + (row * pr.P + p) * 3));
+                const long long o0 = static_cast<long long>(m) * D + smp.base * tok + lane * V;
+                float qv[V], dv[V];
+#pragma unroll
+                for (int z = 0; z < V; ++z) {
+                    qv[z] = __bfloat162float(q[row * D + lane * V + z]);
+                    dv[z] = __bfloat162float(dout[row * D + lane * V + z]);
+                }
+                const float wt[2] = {1.0f - smp.ft, smp.ft}, wy[2] = {1.0f - smp.fy, smp.fy}, wx[2] = {1.0f - smp.fx, smp.fx};
+                const long long sy = static_cast<long long>(pr.W) * tok, st = static_cast<long long>(pr.H) * sy;
+                const long long sidx = sample_at(sl, pr, m, n, p);
+                if constexpr (kScatter) {
+                    const float2 cf = sl.coef[sidx];
+                    if (marked && i < far_from && !(__float_as_uint(cf.y) >> 31)) continue;
+                    for (int j = 0; j < 8; ++j) {
+                        const float wj = wt[j >> 2] * wy[(j >> 1) & 1] * wx[j & 1];
+                        const long long o = o0 + (j >> 2) * st + ((j >> 1) & 1) * sy + (j & 1) * tok;
+                        if (!((smp.mask >> j) & 1u) || wj == 0.0f || !DSA3D_IN_RANGE(pr, o, kv_extent, 7)) continue;
+#pragma unroll
+                        for (int z = 0; z < V; ++z) {
+                            atomicAdd(acc_dk + o + z, wj * cf.x * qv[z]);
+                            atomicAdd(acc_dv + o + z, wj * fabsf(cf.y) * dv[z]);
+                        }
+                    }
+                } else {
+                    float a[8], bb[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const int ct = j >> 2, cy = (j >> 1) & 1, cx = j & 1;
+                        const bool needed = wt[ct] * wy[cy] * wx[cx] != 0.0f || wy[cy] * wx[cx] != 0.0f || wt[ct] * wx[cx] != 0.0f || wt[ct] * wy[cy] != 0.0f;
+                        const long long o = o0 + ct * st + cy * sy + cx * tok;
+                        a[j] = bb[j] = 0.0f;
+                        if (!((smp.mask >> j) & 1u) || !needed || !DSA3D_IN_RANGE(pr, o, kv_extent, 5)) continue;
+#pragma unroll
+                        for (int z = 0; z < V; ++z) {
+                            a[j] = fmaf(qv[z], __bfloat162float(k[o + z]), a[j]);
+                            bb[j] = fmaf(dv[z], __bfloat162float(v[o + z]), bb[j]);
+                        }
+                    }
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        a[j] = group_sum<32>(a[j], kFullMask);
+                        bb[j] = group_sum<32>(bb[j], kFullMask);
+                    }
+                    float r[8];
+                    trilerp_grad(a, smp.ft, smp.fy, smp.fx, r[0], r[1], r[2], r[3]);
+                    trilerp_grad(bb, smp.ft, smp.fy, smp.fx, r[4], r[5], r[6], r[7]);
+                    if (lane == 0) {
+#pragma unroll
+                        for (int z = 0; z < 8; ++z) sl.stats[sidx * 8 + z] = r[z];
+                    }
+                }
+            }
+        }
+    }
+}
+
 // ------------------------------------------------------------------------------------------------ dot products
 constexpr int kDotThreads = 256;
 
@@ -415,15 +511,17 @@ __device__ __forceinline__ void dots_block(const unsigned block, const bf16* __r
 template <int D, bool kWide, bool kGated>
 __global__ void __launch_bounds__(kDotThreads, D == 128 ? 3 : 4)
 cells_dots_kernel(const bf16* __restrict__ q, const bf16* __restrict__ k, const bf16* __restrict__ v, const bf16* __restrict__ dout,
-                  const __grid_constant__ Problem pr, const __grid_constant__ Slab sl, unsigned blocks) {
+                  const float* __restrict__ offsets, const __grid_constant__ Problem pr, const __grid_constant__ Slab sl, unsigned blocks) {
     if constexpr (!kGated) {
-        dots_block<D, kWide>(blockIdx.x, q, k, v, dout, pr, sl);
+        if (blockIdx.x < blocks) dots_block<D, kWide>(blockIdx.x, q, k, v, dout, pr, sl);
+        else far_part<D, false>(blockIdx.x - blocks, gridDim.x - blocks, q, k, v, dout, offsets, nullptr, nullptr, pr, sl);
     } else {
         if (gated_off(pr)) return;
         for (unsigned block = blockIdx.x; block < blocks; block += gridDim.x) {
             dots_block<D, kWide>(block, q, k, v, dout, pr, sl);
             __syncthreads();
         }
+        far_part<D, false>(blockIdx.x, gridDim.x, q, k, v, dout, offsets, nullptr, nullptr, pr, sl);
     }
 }
 
@@ -659,7 +757,7 @@ __device__ __forceinline__ void sums_block(const unsigned block, const bf16* __r
         // step 3: the products of the group whose rows are on their way
         const int run = run2;
         const uint32_t f = f2, stop = stop2, from1 = s.first[kBlockX * run + 1], from2 = s.first[kBlockX * run + 2];
-        const bool odd = __float_as_uint(mark2) >> 31;             // marked: cells_far_kernel takes it
+        const bool odd = __float_as_uint(mark2) >> 31;             // marked: far_part takes it
         const unsigned odds = __ballot_sync(kFullMask, odd);
         if (lane < 16) s.geo[warp][slot][lane] = make_float4(geo2.x, geo2.y, geo2.z, (odd || f + lane >= stop) ? 0.0f : coef2);
         const uint32_t from = stage3;
@@ -736,108 +834,21 @@ __device__ __forceinline__ void sums_block(const unsigned block, const bf16* __r
 
 template <int D, bool kGated>
 __global__ void __launch_bounds__(kSumThreads, D == 32 ? 3 : 2)
-cells_sums_kernel(const bf16* __restrict__ q, const bf16* __restrict__ dout, float* __restrict__ acc_dk, float* __restrict__ acc_dv,
-                  const __grid_constant__ Problem pr, const __grid_constant__ Slab sl, unsigned blocks) {
+cells_sums_kernel(const bf16* __restrict__ q, const bf16* __restrict__ dout, const float* __restrict__ offsets, float* __restrict__ acc_dk,
+                  float* __restrict__ acc_dv, const __grid_constant__ Problem pr, const __grid_constant__ Slab sl, unsigned blocks) {
     if constexpr (!kGated) {
-        sums_block<D>(blockIdx.x, q, dout, acc_dk, acc_dv, pr, sl);
+        if (blockIdx.x < blocks) sums_block<D>(blockIdx.x, q, dout, acc_dk, acc_dv, pr, sl);
+        else far_part<D, true>(blockIdx.x - blocks, gridDim.x - blocks, q, nullptr, nullptr, dout, offsets, acc_dk, acc_dv, pr, sl);
     } else {
         if (gated_off(pr)) return;
         for (unsigned block = blockIdx.x; block < blocks; block += gridDim.x) {
             sums_block<D>(block, q, dout, acc_dk, acc_dv, pr, sl);
             __syncthreads();
         }
+        far_part<D, true>(blockIdx.x, gridDim.x, q, nullptr, nullptr, dout, offsets, acc_dk, acc_dv, pr, sl);
     }
 }
 
-
-// ------------------------------------------------------------------------------------------------ beyond the bins
-// The samples in bin kBins of every tile, a warp per sample, row by row.  kScatter: their contributions to dK and dV, and those
-// of marked samples of the other bins; otherwise what cells_dots_kernel leaves for the others.
-template <int D, bool kScatter>
-__global__ void __launch_bounds__(256)
-cells_far_kernel(const bf16* __restrict__ q, const bf16* __restrict__ k, const bf16* __restrict__ v, const bf16* __restrict__ dout,
-                 const float* __restrict__ offsets, float* __restrict__ acc_dk, float* __restrict__ acc_dv, const Problem pr, const Slab sl,
-                 int tiles) {
-    if (gated_off(pr)) return;
-    constexpr int V = D / 32;                       // channels per lane
-    const int lane = threadIdx.x & 31, warps = gridDim.x * 8;
-    const long long tok = static_cast<long long>(pr.heads) * D;
-    const int per_head = sl.tiles_t * sl.tiles_y * sl.tiles_x;
-    [[maybe_unused]] const long long kv_extent = pr.N * pr.heads * D;
-    for (int base = (static_cast<int>(blockIdx.x) * 8 + static_cast<int>(threadIdx.x >> 5)) * 32; base < tiles; base += warps * 32) {
-        uint32_t mine = 0u;
-        if (base + lane < tiles) mine = __ldg(sl.seg + static_cast<long long>(base + lane) * (kBins + 1) + kBins);
-        const bool marked = kScatter && *sl.marked != 0;
-        if (marked) mine = ((mine & 0xffffu) + (mine >> 16)) << 16;        // all samples of the tile: those beyond the bins are its last
-        unsigned todo = __ballot_sync(kFullMask, (mine >> 16) != 0u);
-        while (todo) {
-            const int src = __ffs(static_cast<int>(todo)) - 1;
-            todo &= todo - 1u;
-            const uint32_t w = __shfl_sync(kFullMask, mine, src);
-            const long long tile = base + src;
-            const int m = sl.m0 + static_cast<int>(tile / per_head);
-            const uint32_t far_from = marked ? __ldg(sl.seg + tile * (kBins + 1) + kBins) & 0xffffu : 0u;
-            for (uint32_t i = 0; i < (w >> 16); ++i) {
-                const long long at = tile * (kRows * pr.P) + (w & 0xffffu) + i;
-                const int n = static_cast<int>(__ldg(sl.geo + at).x), p = static_cast<int>(__ldg(sl.meta + at) & 255u);
-                const int x = n % pr.W, y = (n / pr.W) % pr.H, t = n / (pr.W * pr.H);
-                const long long row = static_cast<long long>(n) * pr.heads + m;
-                const Sample smp = to_sample(pr, make_cell(pr, t, y, x, p, offsets + (row * pr.P + p) * 3));
-                const long long o0 = static_cast<long long>(m) * D + smp.base * tok + lane * V;
-                float qv[V], dv[V];
-#pragma unroll
-                for (int z = 0; z < V; ++z) {
-                    qv[z] = __bfloat162float(q[row * D + lane * V + z]);
-                    dv[z] = __bfloat162float(dout[row * D + lane * V + z]);
-                }
-                const float wt[2] = {1.0f - smp.ft, smp.ft}, wy[2] = {1.0f - smp.fy, smp.fy}, wx[2] = {1.0f - smp.fx, smp.fx};
-                const long long sy = static_cast<long long>(pr.W) * tok, st = static_cast<long long>(pr.H) * sy;
-                const long long sidx = sample_at(sl, pr, m, n, p);
-                if constexpr (kScatter) {
-                    const float2 cf = sl.coef[sidx];
-                    if (marked && i < far_from && !(__float_as_uint(cf.y) >> 31)) continue;
-                    for (int j = 0; j < 8; ++j) {
-                        const float wj = wt[j >> 2] * wy[(j >> 1) & 1] * wx[j & 1];
-                        const long long o = o0 + (j >> 2) * st + ((j >> 1) & 1) * sy + (j & 1) * tok;
-                        if (!((smp.mask >> j) & 1u) || wj == 0.0f || !DSA3D_IN_RANGE(pr, o, kv_extent, 7)) continue;
-#pragma unroll
-                        for (int z = 0; z < V; ++z) {
-                            atomicAdd(acc_dk + o + z, wj * cf.x * qv[z]);
-                            atomicAdd(acc_dv + o + z, wj * fabsf(cf.y) * dv[z]);
-                        }
-                    }
-                } else {
-                    float a[8], bb[8];
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const int ct = j >> 2, cy = (j >> 1) & 1, cx = j & 1;
-                        const bool needed = wt[ct] * wy[cy] * wx[cx] != 0.0f || wy[cy] * wx[cx] != 0.0f || wt[ct] * wx[cx] != 0.0f || wt[ct] * wy[cy] != 0.0f;
-                        const long long o = o0 + ct * st + cy * sy + cx * tok;
-                        a[j] = bb[j] = 0.0f;
-                        if (!((smp.mask >> j) & 1u) || !needed || !DSA3D_IN_RANGE(pr, o, kv_extent, 5)) continue;
-#pragma unroll
-                        for (int z = 0; z < V; ++z) {
-                            a[j] = fmaf(qv[z], __bfloat162float(k[o + z]), a[j]);
-                            bb[j] = fmaf(dv[z], __bfloat162float(v[o + z]), bb[j]);
-                        }
-                    }
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        a[j] = group_sum<32>(a[j], kFullMask);
-                        bb[j] = group_sum<32>(bb[j], kFullMask);
-                    }
-                    float r[8];
-                    trilerp_grad(a, smp.ft, smp.fy, smp.fx, r[0], r[1], r[2], r[3]);
-                    trilerp_grad(bb, smp.ft, smp.fy, smp.fx, r[4], r[5], r[6], r[7]);
-                    if (lane == 0) {
-#pragma unroll
-                        for (int z = 0; z < 8; ++z) sl.stats[sidx * 8 + z] = r[z];
-                    }
-                }
-            }
-        }
-    }
-}
 
 // ------------------------------------------------------------------------------------------------ host
 int floor_div4(int a) { return a >= 0 ? a / 4 : -((-a + 3) / 4); }
@@ -876,14 +887,14 @@ size_t lay_out(const Problem& pr, int m0, int heads, int f0, int f1, char* base,
 // the gated instances loop over their blocks.
 template <int D, bool kGated>
 cudaError_t launch_slab(const void* q_, const void* k_, const void* v_, const float* offsets, const float* lse, const void* dout_, void* dq_,
-                        float* acc_dk, float* acc_dv, float* doffsets, const Problem& pr, const Slab& s, cudaStream_t stream) {
+                        float* acc_dk, float* acc_dv, float* doffsets, const Problem& pr, const Slab& s, void* clear, size_t clear_bytes, cudaStream_t stream) {
     const bf16 *q = static_cast<const bf16*>(q_), *k = static_cast<const bf16*>(k_), *v = static_cast<const bf16*>(v_), *dout = static_cast<const bf16*>(dout_);
     const unsigned tiles = static_cast<unsigned>(s.heads * s.tiles_t * s.tiles_y * s.tiles_x), blocks = static_cast<unsigned>(s.heads * s.blocks_t * s.blocks_y * s.blocks_x);
     const unsigned inv_p = ((1u << 24) + static_cast<unsigned>(pr.P) - 1u) / static_cast<unsigned>(pr.P);
     auto grid = [](unsigned n) { return kGated && n > 148u * 8u ? 148u * 8u : n; };
     cudaError_t e = cudaSuccess;
     auto big = [&](auto kern, size_t smem) {           // allows the kernel its dynamic shared memory
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+        if (e == cudaSuccess && smem > 48 * 1024) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
         return kern;
     };
     const size_t bin_smem = static_cast<size_t>((kBins + 1) * kCopies + kRows * pr.P) * sizeof(uint32_t), dot_smem = sizeof(DotSmem<D>), sum_smem = sizeof(SumSmem<D>) + 256;
@@ -892,18 +903,18 @@ cudaError_t launch_slab(const void* q_, const void* k_, const void* v_, const fl
     auto dots = big(wide ? cells_dots_kernel<D, true, kGated> : cells_dots_kernel<D, false, kGated>, dot_smem);
     auto sums = big(cells_sums_kernel<D, kGated>, sum_smem);
     if (e != cudaSuccess) return e;
-    bin<<<grid(tiles), kBinThreads, bin_smem, stream>>>(offsets, pr, s, inv_p, tiles);
+    const long long clear_all = static_cast<long long>(clear_bytes / 16);
+    bin<<<grid(tiles), kBinThreads, bin_smem, stream>>>(offsets, pr, s, inv_p, tiles, static_cast<uint4*>(clear), (clear_all + tiles - 1) / tiles, clear_all);
     cells_sort_kernel<kGated><<<grid(blocks), kSortThreads, 0, stream>>>(pr, s, blocks);
-    dots<<<grid(blocks), kDotThreads, dot_smem, stream>>>(q, k, v, dout, pr, s, blocks);
-    const unsigned far_grid = tiles / 256 + 1 < 148 * 8 ? tiles / 256 + 1 : 148 * 8;
-    cells_far_kernel<D, false><<<far_grid, 256, 0, stream>>>(q, k, v, dout, offsets, acc_dk, acc_dv, pr, s, static_cast<int>(tiles));
+    static_assert(kDotThreads == 256 && kSumThreads == 256, "far_part");
+    const unsigned far_parts = tiles / 256 + 1 < 148 * 8 ? tiles / 256 + 1 : 148 * 8;
+    dots<<<grid(blocks + far_parts), kDotThreads, dot_smem, stream>>>(q, k, v, dout, offsets, pr, s, blocks);
     // As many queries per warp as have a lane for every sample.
     const int share = pr.P <= 8 ? 4 : pr.P <= 16 ? 2 : 1, per_block = kQueryWarps * share;
     const unsigned per_head = static_cast<unsigned>((static_cast<long long>(s.f1 - s.f0) * pr.H * pr.W + per_block - 1) / per_block), query_blocks = per_head * static_cast<unsigned>(s.heads);
     auto query = share == 4 ? cells_query_kernel<D, 4, kGated> : share == 2 ? cells_query_kernel<D, 2, kGated> : cells_query_kernel<D, 1, kGated>;
     query<<<grid(query_blocks), kQueryWarps * 32, 0, stream>>>(k, offsets, lse, static_cast<bf16*>(dq_), doffsets, pr, s, per_head, query_blocks);
-    sums<<<grid(blocks), kSumThreads, sum_smem, stream>>>(q, dout, acc_dk, acc_dv, pr, s, blocks);
-    cells_far_kernel<D, true><<<far_grid, 256, 0, stream>>>(q, k, v, dout, offsets, acc_dk, acc_dv, pr, s, static_cast<int>(tiles));
+    sums<<<grid(blocks + far_parts), kSumThreads, sum_smem, stream>>>(q, dout, offsets, acc_dk, acc_dv, pr, s, blocks);
     return cudaGetLastError();
 }
 
@@ -912,8 +923,8 @@ cudaError_t launch_slab(const void* q_, const void* k_, const void* v_, const fl
 // Splits the queries of `pr` (whole frames) into passes whose buffers fit `bytes`: by heads first (they share nothing),
 // then by frames.
 bool try_cells_backward(const void* q, const void* k, const void* v, const float* offsets, const float* lse, const void* dout, void* dq,
-                        float* acc_dk, float* acc_dv, float* doffsets, void* scratch, size_t bytes, const Problem& pr, cudaStream_t stream,
-                        cudaError_t* err) {
+                        float* acc_dk, float* acc_dv, float* doffsets, void* scratch, size_t bytes, void* clear, size_t clear_bytes, const Problem& pr,
+                        cudaStream_t stream, cudaError_t* err) {
     *err = cudaSuccess;
     const long long frame = static_cast<long long>(pr.H) * pr.W;
     const int f_begin = static_cast<int>(pr.q_begin / frame), f_end = f_begin + static_cast<int>(pr.q_count / frame);
@@ -931,7 +942,8 @@ bool try_cells_backward(const void* q, const void* k, const void* v, const float
             auto slab = pr.d == 128 ? (pr.gate ? launch_slab<128, true> : launch_slab<128, false>)
                         : pr.d == 64 ? (pr.gate ? launch_slab<64, true> : launch_slab<64, false>)
                                      : (pr.gate ? launch_slab<32, true> : launch_slab<32, false>);
-            *err = slab(q, k, v, offsets, lse, dout, dq, acc_dk, acc_dv, doffsets, pr, s, stream);
+            *err = slab(q, k, v, offsets, lse, dout, dq, acc_dk, acc_dv, doffsets, pr, s, clear, clear_bytes, stream);
+            clear_bytes = 0;                                        // the first pass clears for all
             if (*err != cudaSuccess) return true;
         }
     return true;

@@ -35,16 +35,17 @@ cudaError_t launch_scatter_tiles(const void* q, const void* dout, const float* o
 
 // The whole backward of the bf16 queries of `pr` (whole frames) on samples sorted by key cell (dsa3d_cells.cu): dq, doffsets, and
 // the contributions to the fp32 accumulators.  `scratch`: `bytes` of device memory, worked through in as many passes as
-// it takes; false: not even the smallest pass fits, nothing launched.
+// it takes; false: not even the smallest pass fits, nothing launched.  `clear_bytes` from `clear` on (the accumulators) are
+// zeroed first.
 bool try_cells_backward(const void* q, const void* k, const void* v, const float* offsets, const float* lse, const void* dout, void* dq,
-                        float* acc_dk, float* acc_dv, float* doffsets, void* scratch, size_t bytes, const Problem& pr, cudaStream_t stream,
-                        cudaError_t* err);
+                        float* acc_dk, float* acc_dv, float* doffsets, void* scratch, size_t bytes, void* clear, size_t clear_bytes,
+                        const Problem& pr, cudaStream_t stream, cudaError_t* err);
 
 // Dynamic shared memory of the tile kernel for this problem's tiling.
 size_t tile_smem_bytes(const Problem& pr);
 
-// fp32 accumulators -> bf16 outputs (round to nearest even).
-cudaError_t launch_convert_bf16(const float* acc, void* dst, long long count, cudaStream_t stream,
+// fp32 accumulators (those of dk, then those of dv, `count` each) -> bf16 outputs (round to nearest even).
+cudaError_t launch_convert_bf16(const float* acc, void* dk, void* dv, long long count, cudaStream_t stream,
                                 const int* gate = nullptr);
 // Zeroes `bytes` (a multiple of 16) at `dst` unless *gate is 0.
 cudaError_t launch_gated_clear(void* dst, size_t bytes, const int* gate, cudaStream_t stream);
