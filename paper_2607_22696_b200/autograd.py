@@ -155,13 +155,19 @@ class _OffsetsLinear(torch.autograd.Function):
 def dwconv3d(x, weight, bias, kernel):
     """Depthwise 3-D convolution of x [T, H, W, C] (first term of Eq. 1; first stage of the
     offset predictor); weight fp32 [kt*kh*kw, C], bias fp32 [C] or None."""
-    return _DwConv3d.apply(x, weight, bias, tuple(kernel))
+    kernel = tuple(int(s) for s in kernel)
+    if len(kernel) == 3:
+        y = _native().dwconv3d(x, weight, bias, *kernel)
+        if y is not None:
+            return y
+    return _DwConv3d.apply(x, weight, bias, kernel)
 
 
 def offsets_linear(u, w, bias):
     """offsets [tokens, O] (fp32) = u [tokens, C] . w [O, C]^T + bias [O] (fp32); the gradient of
     w is accumulated in fp32 and rounded once to w's dtype."""
-    return _OffsetsLinear.apply(u, w, bias)
+    out = _native().offsets_linear(u, w, bias)
+    return out if out is not None else _OffsetsLinear.apply(u, w, bias)
 
 
 def dsa3d(q, k, v, offsets, window, residual=None):

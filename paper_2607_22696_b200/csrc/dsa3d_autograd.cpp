@@ -44,13 +44,15 @@ bool taken_qkv(const Tensor& q, const Tensor& k, const Tensor& v) {
     return taken(k, q) && taken(v, q) && k.numel() == q.numel() && v.numel() == q.numel();
 }
 
+int code_of(const Tensor& t) { return t.scalar_type() == at::kBFloat16 ? DSA3D_BF16 : DSA3D_F32; }
+
 struct Shape {
     int T, H, W, heads, d, window[3], code;
     Shape(const Tensor& q, const int64_t* w)
         : T(static_cast<int>(q.size(0))), H(static_cast<int>(q.size(1))), W(static_cast<int>(q.size(2))),
           heads(static_cast<int>(q.size(3))), d(static_cast<int>(q.size(4))),
           window{static_cast<int>(w[0]), static_cast<int>(w[1]), static_cast<int>(w[2])},
-          code(q.scalar_type() == at::kBFloat16 ? DSA3D_BF16 : DSA3D_F32) {}
+          code(code_of(q)) {}
 };
 
 Tensor new_lse(const Tensor& q) {
@@ -135,6 +137,75 @@ struct Dsa3dFixedWindow : torch::autograd::Function<Dsa3dFixedWindow> {
     }
 };
 
+// x [T, H, W, C], weight fp32 [taps, C], bias fp32 [C] or none
+struct DwConv3d : torch::autograd::Function<DwConv3d> {
+    static Tensor forward(AutogradContext* ctx, const Tensor& x, const Tensor& weight, const std::optional<Tensor>& bias, int64_t kt,
+                          int64_t kh, int64_t kw) {
+        const c10::cuda::CUDAGuard guard(x.device());
+        const int kernel[3] = {static_cast<int>(kt), static_cast<int>(kh), static_cast<int>(kw)};
+        Tensor y = at::empty_like(x);
+        check(dsa3d_dwconv3d_forward(x.data_ptr(), weight.data_ptr<float>(), bias ? bias->data_ptr<float>() : nullptr,
+                                     static_cast<int>(x.size(0)), static_cast<int>(x.size(1)), static_cast<int>(x.size(2)),
+                                     static_cast<int>(x.size(3)), kernel, y.data_ptr(), code_of(x),
+                                     c10::cuda::getCurrentCUDAStream().stream()));
+        ctx->save_for_backward({x, weight});
+        const int64_t w[3] = {kt, kh, kw};
+        save_window(ctx, w);
+        ctx->saved_data["bias"] = bias.has_value();
+        return y;
+    }
+    static variable_list backward(AutogradContext* ctx, const variable_list& grads) {
+        const variable_list saved = ctx->get_saved_variables();
+        const Tensor &x = saved[0], &weight = saved[1];
+        const c10::cuda::CUDAGuard guard(x.device());
+        const Window w = saved_window(ctx);
+        const int kernel[3] = {static_cast<int>(w.w[0]), static_cast<int>(w.w[1]), static_cast<int>(w.w[2])};
+        const bool need_x = ctx->needs_input_grad(0), need_w = ctx->needs_input_grad(1);
+        const bool need_b = ctx->saved_data["bias"].toBool() && ctx->needs_input_grad(2);
+        const Tensor dy = grads[0].contiguous();
+        const Tensor dx = need_x ? at::empty_like(x) : Tensor(), dw = need_w || need_b ? at::empty_like(weight) : Tensor();
+        const Tensor db = need_b ? at::empty({x.size(3)}, x.options().dtype(at::kFloat)) : Tensor();
+        const Tensor ws = need_x ? new_workspace(x, dsa3d_dwconv3d_backward_workspace_bytes(static_cast<int>(x.size(3)), kernel)) : Tensor();
+        check(dsa3d_dwconv3d_backward(x.data_ptr(), weight.data_ptr<float>(), dy.data_ptr(), static_cast<int>(x.size(0)),
+                                      static_cast<int>(x.size(1)), static_cast<int>(x.size(2)), static_cast<int>(x.size(3)), kernel,
+                                      need_x ? dx.data_ptr() : nullptr, dw.defined() ? dw.data_ptr<float>() : nullptr,
+                                      need_b ? db.data_ptr<float>() : nullptr, need_x ? ws.data_ptr() : nullptr,
+                                      need_x ? static_cast<size_t>(ws.numel()) : 0, code_of(x),
+                                      c10::cuda::getCurrentCUDAStream().stream()));
+        return {dx, need_w ? dw : Tensor(), db, Tensor(), Tensor(), Tensor()};
+    }
+};
+
+// u [tokens, C], w [O, C] of one type, bias fp32 [O]
+struct OffsetsLinear : torch::autograd::Function<OffsetsLinear> {
+    static Tensor forward(AutogradContext* ctx, const Tensor& u, const Tensor& w, const Tensor& bias) {
+        const c10::cuda::CUDAGuard guard(u.device());
+        Tensor out = at::empty({u.size(0), w.size(0)}, u.options().dtype(at::kFloat));
+        check(dsa3d_offsets_linear_forward(u.data_ptr(), w.data_ptr(), bias.data_ptr<float>(), u.size(0), static_cast<int>(u.size(1)),
+                                           static_cast<int>(w.size(0)), out.data_ptr<float>(), code_of(u),
+                                           c10::cuda::getCurrentCUDAStream().stream()));
+        ctx->save_for_backward({u, w});
+        return out;
+    }
+    static variable_list backward(AutogradContext* ctx, const variable_list& grads) {
+        const variable_list saved = ctx->get_saved_variables();
+        const Tensor &u = saved[0], &w = saved[1];
+        const c10::cuda::CUDAGuard guard(u.device());
+        const int C = static_cast<int>(u.size(1)), O = static_cast<int>(w.size(0));
+        const bool need_u = ctx->needs_input_grad(0), need_w = ctx->needs_input_grad(1), need_b = ctx->needs_input_grad(2);
+        const Tensor g = grads[0].contiguous();
+        const auto f32 = u.options().dtype(at::kFloat);
+        const Tensor du = need_u ? at::empty_like(u) : Tensor(), dw = need_w ? at::empty({O, C}, f32) : Tensor();
+        const Tensor db = need_b ? at::empty({O}, f32) : Tensor();
+        const Tensor ws = new_workspace(u, dsa3d_offsets_linear_backward_workspace_bytes(u.size(0), C, O, code_of(u)));
+        check(dsa3d_offsets_linear_backward(u.data_ptr(), w.data_ptr(), g.data_ptr<float>(), u.size(0), C, O,
+                                            need_u ? du.data_ptr() : nullptr, need_w ? dw.data_ptr<float>() : nullptr,
+                                            need_b ? db.data_ptr<float>() : nullptr, ws.data_ptr(), static_cast<size_t>(ws.numel()),
+                                            code_of(u), c10::cuda::getCurrentCUDAStream().stream()));
+        return {du, need_w ? dw.to(w.scalar_type()) : Tensor(), db};
+    }
+};
+
 // Runs `call` without the interpreter lock; a Python exception that came up in it is raised where Python called.
 template <typename F> Tensor run(F call) {
     try {
@@ -165,9 +236,34 @@ std::optional<Tensor> dsa3d_fixed_window(const Tensor& q, const Tensor& k, const
     return run([&] { return Dsa3dFixedWindow::apply(q, k, v, kt, kh, kw); });
 }
 
+bool taken_f32(const Tensor& t, const Tensor& like, int64_t numel) {
+    return t.is_cuda() && t.device() == like.device() && t.scalar_type() == at::kFloat && t.is_contiguous() && t.numel() == numel;
+}
+
+bool taken_storage(const Tensor& t, int64_t dims) {
+    if (!taken(t, t) || t.dim() != dims || (t.scalar_type() != at::kFloat && t.scalar_type() != at::kBFloat16)) return false;
+    for (int64_t s : t.sizes()) if (s < 1 || s > INT_MAX) return false;
+    return true;
+}
+
+std::optional<Tensor> dwconv3d(const Tensor& x, const Tensor& weight, const std::optional<Tensor>& bias, int64_t kt, int64_t kh, int64_t kw) {
+    if (!taken_storage(x, 4) || !taken_window(kt, kh, kw) || weight.dim() != 2 || !taken_f32(weight, x, kt * kh * kw * x.size(3)) ||
+        (bias && !taken_f32(*bias, x, x.size(3))))
+        return std::nullopt;
+    return run([&] { return DwConv3d::apply(x, weight, bias, kt, kh, kw); });
+}
+
+std::optional<Tensor> offsets_linear(const Tensor& u, const Tensor& w, const Tensor& bias) {
+    if (!taken_storage(u, 2) || !taken_storage(w, 2) || !taken(w, u) || w.size(1) != u.size(1) || !taken_f32(bias, u, w.size(0)))
+        return std::nullopt;
+    return run([&] { return OffsetsLinear::apply(u, w, bias); });
+}
+
 }  // namespace
 
 PYBIND11_MODULE(_autograd_native, m) {
     m.def("dsa3d", &dsa3d);
     m.def("dsa3d_fixed_window", &dsa3d_fixed_window);
+    m.def("dwconv3d", &dwconv3d);
+    m.def("offsets_linear", &offsets_linear);
 }
