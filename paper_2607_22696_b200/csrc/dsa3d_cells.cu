@@ -884,14 +884,15 @@ size_t lay_out(const Problem& pr, int m0, int heads, int f0, int f1, char* base,
 }
 
 // Behind a gate that is mostly closed launching all CTAs would cost more than anything else (0.95 ms for 1.8 M of the query kernel):
-// the gated instances loop over their blocks.
+// the gated instances loop over their blocks, with about as many CTAs as an SM holds (four times as many cost an
+// empty chain 6 us more).
 template <int D, bool kGated>
 cudaError_t launch_slab(const void* q_, const void* k_, const void* v_, const float* offsets, const float* lse, const void* dout_, void* dq_,
                         float* acc_dk, float* acc_dv, float* doffsets, const Problem& pr, const Slab& s, void* clear, size_t clear_bytes, cudaStream_t stream) {
     const bf16 *q = static_cast<const bf16*>(q_), *k = static_cast<const bf16*>(k_), *v = static_cast<const bf16*>(v_), *dout = static_cast<const bf16*>(dout_);
     const unsigned tiles = static_cast<unsigned>(s.heads * s.tiles_t * s.tiles_y * s.tiles_x), blocks = static_cast<unsigned>(s.heads * s.blocks_t * s.blocks_y * s.blocks_x);
     const unsigned inv_p = ((1u << 24) + static_cast<unsigned>(pr.P) - 1u) / static_cast<unsigned>(pr.P);
-    auto grid = [](unsigned n) { return kGated && n > 148u * 8u ? 148u * 8u : n; };
+    auto grid = [](unsigned n, unsigned resident) { return kGated && n > 148u * resident ? 148u * resident : n; };
     cudaError_t e = cudaSuccess;
     auto big = [&](auto kern, size_t smem) {           // allows the kernel its dynamic shared memory
         if (e == cudaSuccess && smem > 48 * 1024) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
@@ -904,17 +905,17 @@ cudaError_t launch_slab(const void* q_, const void* k_, const void* v_, const fl
     auto sums = big(cells_sums_kernel<D, kGated>, sum_smem);
     if (e != cudaSuccess) return e;
     const long long clear_all = static_cast<long long>(clear_bytes / 16);
-    bin<<<grid(tiles), kBinThreads, bin_smem, stream>>>(offsets, pr, s, inv_p, tiles, static_cast<uint4*>(clear), (clear_all + tiles - 1) / tiles, clear_all);
-    cells_sort_kernel<kGated><<<grid(blocks), kSortThreads, 0, stream>>>(pr, s, blocks);
+    bin<<<grid(tiles, 2), kBinThreads, bin_smem, stream>>>(offsets, pr, s, inv_p, tiles, static_cast<uint4*>(clear), (clear_all + tiles - 1) / tiles, clear_all);
+    cells_sort_kernel<kGated><<<grid(blocks, 4), kSortThreads, 0, stream>>>(pr, s, blocks);
     static_assert(kDotThreads == 256 && kSumThreads == 256, "far_part");
     const unsigned far_parts = tiles / 256 + 1 < 148 * 8 ? tiles / 256 + 1 : 148 * 8;
-    dots<<<grid(blocks + far_parts), kDotThreads, dot_smem, stream>>>(q, k, v, dout, offsets, pr, s, blocks);
+    dots<<<grid(blocks + far_parts, 3), kDotThreads, dot_smem, stream>>>(q, k, v, dout, offsets, pr, s, blocks);
     // As many queries per warp as have a lane for every sample.
     const int share = pr.P <= 8 ? 4 : pr.P <= 16 ? 2 : 1, per_block = kQueryWarps * share;
     const unsigned per_head = static_cast<unsigned>((static_cast<long long>(s.f1 - s.f0) * pr.H * pr.W + per_block - 1) / per_block), query_blocks = per_head * static_cast<unsigned>(s.heads);
     auto query = share == 4 ? cells_query_kernel<D, 4, kGated> : share == 2 ? cells_query_kernel<D, 2, kGated> : cells_query_kernel<D, 1, kGated>;
-    query<<<grid(query_blocks), kQueryWarps * 32, 0, stream>>>(k, offsets, lse, static_cast<bf16*>(dq_), doffsets, pr, s, per_head, query_blocks);
-    sums<<<grid(blocks + far_parts), kSumThreads, sum_smem, stream>>>(q, dout, offsets, acc_dk, acc_dv, pr, s, blocks);
+    query<<<grid(query_blocks, 12), kQueryWarps * 32, 0, stream>>>(k, offsets, lse, static_cast<bf16*>(dq_), doffsets, pr, s, per_head, query_blocks);
+    sums<<<grid(blocks + far_parts, 2), kSumThreads, sum_smem, stream>>>(q, dout, offsets, acc_dk, acc_dv, pr, s, blocks);
     return cudaGetLastError();
 }
 

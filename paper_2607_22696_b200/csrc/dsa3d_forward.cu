@@ -457,7 +457,7 @@ static cudaError_t launch_gather_forward(const void* q, const void* k, const voi
     const long long per_head = (pr.q_count + kFwdWarps * share - 1) / (kFwdWarps * share);
     // behind a gate that is mostly closed, a CTA per two items would cost more to launch than to run (0.95 ms for 3.7 M items)
     const long long all = per_head * pr.heads;
-    const unsigned blocks = static_cast<unsigned>(gate && share == 1 && all > 148 * 64 ? 148 * 64 : all);
+    const unsigned blocks = static_cast<unsigned>(gate && share == 1 && all > 148 * 16 ? 148 * 16 : all);
     if (share > 1) {
         auto kern = share == 4 ? (addend ? gather_forward_small_kernel<D, 4, true> : gather_forward_small_kernel<D, 4, false>)
                                : (addend ? gather_forward_small_kernel<D, 2, true> : gather_forward_small_kernel<D, 2, false>);
