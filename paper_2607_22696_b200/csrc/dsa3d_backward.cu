@@ -597,7 +597,7 @@ cudaError_t launch_scatter_tiles(const void* q, const void* dout, const float* o
 
 __global__ void __launch_bounds__(256)
 convert_bf16_kernel(const float4* __restrict__ acc, uint2* __restrict__ dk, uint2* __restrict__ dv, long long count4, const int* __restrict__ gate) {
-    if (gate != nullptr && *gate == 0) return;      // the tile kernels of a bounded-offsets backward wrote dk and dv
+    if (gate != nullptr && gated_off_early(gate)) return;      // the tile kernels of a bounded-offsets backward wrote dk and dv
     const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
     uint2* dst = blockIdx.y ? dv : dk;
     if (blockIdx.y) acc += count4;
@@ -633,8 +633,11 @@ cudaError_t launch_convert_bf16(const float* acc, void* dk, void* dv, long long 
     long long blocks = (count4 + 255) / 256;
     if (blocks > 148LL * 8) blocks = 148LL * 8;
     if (blocks < 1) blocks = 1;
-    convert_bf16_kernel<<<dim3(static_cast<unsigned>(blocks), 2), 256, 0, stream>>>(
-        reinterpret_cast<const float4*>(acc), reinterpret_cast<uint2*>(dk), reinterpret_cast<uint2*>(dv), count4, gate);
+    const dim3 grid(static_cast<unsigned>(blocks), 2);
+    const float4* from = reinterpret_cast<const float4*>(acc);
+    uint2 *to_k = static_cast<uint2*>(dk), *to_v = static_cast<uint2*>(dv);
+    if (gate) return launch_gated(convert_bf16_kernel, grid, 256, 0, stream, from, to_k, to_v, count4, gate);
+    convert_bf16_kernel<<<grid, 256, 0, stream>>>(from, to_k, to_v, count4, gate);
     return cudaGetLastError();
 }
 

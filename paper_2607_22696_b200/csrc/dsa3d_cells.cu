@@ -131,7 +131,7 @@ cells_bin_kernel(const float* __restrict__ offsets, const __grid_constant__ Prob
     if constexpr (!kGated) {
         bin_block(blockIdx.x, offsets, pr, sl, inv_p, clear, clear_each, clear_all);
     } else {
-        if (gated_off(pr)) return;
+        if (gated_off_early(pr.gate)) return;
         for (unsigned block = blockIdx.x; block < blocks; block += gridDim.x) {
             bin_block(block, offsets, pr, sl, inv_p, clear, clear_each, clear_all);
             __syncthreads();
@@ -269,7 +269,7 @@ cells_sort_kernel(const __grid_constant__ Problem pr, const __grid_constant__ Sl
     if constexpr (!kGated) {
         sort_block(blockIdx.x, pr, sl);
     } else {
-        if (gated_off(pr)) return;
+        if (gated_off_early(pr.gate)) return;
         for (unsigned block = blockIdx.x; block < blocks; block += gridDim.x) {
             sort_block(block, pr, sl);
             __syncthreads();
@@ -516,7 +516,7 @@ cells_dots_kernel(const bf16* __restrict__ q, const bf16* __restrict__ k, const 
         if (blockIdx.x < blocks) dots_block<D, kWide>(blockIdx.x, q, k, v, dout, pr, sl);
         else far_part<D, false>(blockIdx.x - blocks, gridDim.x - blocks, q, k, v, dout, offsets, nullptr, nullptr, pr, sl);
     } else {
-        if (gated_off(pr)) return;
+        if (gated_off_early(pr.gate)) return;
         for (unsigned block = blockIdx.x; block < blocks; block += gridDim.x) {
             dots_block<D, kWide>(block, q, k, v, dout, pr, sl);
             __syncthreads();
@@ -640,7 +640,7 @@ cells_query_kernel(const bf16* __restrict__ k, const float* __restrict__ offsets
     if constexpr (!kGated) {
         query_block<D, G>(blockIdx.x, k, offsets, lse, dq, doffsets, pr, sl, blocks_per_head);
     } else {
-        if (gated_off(pr)) return;
+        if (gated_off_early(pr.gate)) return;
         for (unsigned block = blockIdx.x; block < blocks; block += gridDim.x) {
             query_block<D, G>(block, k, offsets, lse, dq, doffsets, pr, sl, blocks_per_head);
             __syncthreads();
@@ -840,7 +840,7 @@ cells_sums_kernel(const bf16* __restrict__ q, const bf16* __restrict__ dout, con
         if (blockIdx.x < blocks) sums_block<D>(blockIdx.x, q, dout, acc_dk, acc_dv, pr, sl);
         else far_part<D, true>(blockIdx.x - blocks, gridDim.x - blocks, q, nullptr, nullptr, dout, offsets, acc_dk, acc_dv, pr, sl);
     } else {
-        if (gated_off(pr)) return;
+        if (gated_off_early(pr.gate)) return;
         for (unsigned block = blockIdx.x; block < blocks; block += gridDim.x) {
             sums_block<D>(block, q, dout, acc_dk, acc_dv, pr, sl);
             __syncthreads();
@@ -904,19 +904,28 @@ cudaError_t launch_slab(const void* q_, const void* k_, const void* v_, const fl
     auto dots = big(wide ? cells_dots_kernel<D, true, kGated> : cells_dots_kernel<D, false, kGated>, dot_smem);
     auto sums = big(cells_sums_kernel<D, kGated>, sum_smem);
     if (e != cudaSuccess) return e;
+    auto launch = [&](auto kern, unsigned ctas, unsigned threads, size_t smem, const auto&... args) {
+        if (e != cudaSuccess) return;
+        if constexpr (kGated) {
+            e = launch_gated(kern, dim3(ctas), threads, smem, stream, args...);
+        } else {
+            kern<<<ctas, threads, smem, stream>>>(args...);
+            e = cudaGetLastError();
+        }
+    };
     const long long clear_all = static_cast<long long>(clear_bytes / 16);
-    bin<<<grid(tiles, 2), kBinThreads, bin_smem, stream>>>(offsets, pr, s, inv_p, tiles, static_cast<uint4*>(clear), (clear_all + tiles - 1) / tiles, clear_all);
-    cells_sort_kernel<kGated><<<grid(blocks, 4), kSortThreads, 0, stream>>>(pr, s, blocks);
+    launch(bin, grid(tiles, 2), kBinThreads, bin_smem, offsets, pr, s, inv_p, tiles, static_cast<uint4*>(clear), (clear_all + tiles - 1) / tiles, clear_all);
+    launch(cells_sort_kernel<kGated>, grid(blocks, 4), kSortThreads, 0, pr, s, blocks);
     static_assert(kDotThreads == 256 && kSumThreads == 256, "far_part");
     const unsigned far_parts = tiles / 256 + 1 < 148 * 8 ? tiles / 256 + 1 : 148 * 8;
-    dots<<<grid(blocks + far_parts, 3), kDotThreads, dot_smem, stream>>>(q, k, v, dout, offsets, pr, s, blocks);
+    launch(dots, grid(blocks + far_parts, 3), kDotThreads, dot_smem, q, k, v, dout, offsets, pr, s, blocks);
     // As many queries per warp as have a lane for every sample.
     const int share = pr.P <= 8 ? 4 : pr.P <= 16 ? 2 : 1, per_block = kQueryWarps * share;
     const unsigned per_head = static_cast<unsigned>((static_cast<long long>(s.f1 - s.f0) * pr.H * pr.W + per_block - 1) / per_block), query_blocks = per_head * static_cast<unsigned>(s.heads);
     auto query = share == 4 ? cells_query_kernel<D, 4, kGated> : share == 2 ? cells_query_kernel<D, 2, kGated> : cells_query_kernel<D, 1, kGated>;
-    query<<<grid(query_blocks, 12), kQueryWarps * 32, 0, stream>>>(k, offsets, lse, static_cast<bf16*>(dq_), doffsets, pr, s, per_head, query_blocks);
-    sums<<<grid(blocks + far_parts, 2), kSumThreads, sum_smem, stream>>>(q, dout, offsets, acc_dk, acc_dv, pr, s, blocks);
-    return cudaGetLastError();
+    launch(query, grid(query_blocks, 12), kQueryWarps * 32, 0, k, offsets, lse, static_cast<bf16*>(dq_), doffsets, pr, s, per_head, query_blocks);
+    launch(sums, grid(blocks + far_parts, 2), kSumThreads, sum_smem, q, dout, offsets, acc_dk, acc_dv, pr, s, blocks);
+    return e;
 }
 
 }  // namespace

@@ -38,6 +38,28 @@ struct Problem {
     const int* gate;
 };
 
+// The start of a kernel launched by launch_gated: true when it has nothing to do.  Its CTAs may be put in place while the
+// kernel before it still runs; they wait here until that has completed and its memory is visible.  Of a chain of kernels that
+// find their gate closed only 1 of 4 us each is left.  (When it is open the next kernel is not let in early: its waiting
+// CTAs cost the running one 9 %.)  The gate is final long before: ordinary launches lie between the check that writes it
+// and the chain.  Nothing else is read before the wait, and the loads behind it stand behind the branch on the gate.
+__device__ __forceinline__ bool gated_off_early(const int* gate) {
+    const bool off = *reinterpret_cast<const volatile int*>(gate) == 0;
+    if (off) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    return off;
+}
+template <typename... P, typename... A>
+cudaError_t launch_gated(void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t stream, const A&... args) {
+    cudaLaunchAttribute early;
+    early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    early.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t config = {};
+    config.gridDim = grid; config.blockDim = dim3(threads); config.dynamicSmemBytes = smem; config.stream = stream;
+    config.attrs = &early; config.numAttrs = 1;
+    return cudaLaunchKernelEx(&config, kern, static_cast<P>(args)...);
+}
+
 // True when a gated general kernel has nothing to do (see Problem::gate).
 __device__ __forceinline__ bool gated_off(const Problem& pr) { return pr.gate != nullptr && *pr.gate == 0; }
 
