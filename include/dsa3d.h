@@ -238,9 +238,9 @@ int dsa3d_backward_noalloc_last_cuda_error(void);
  * Timing hook (a measurement aid; the paper has no counterpart).  The six arguments are
  * cudaEvent_t handles created by the caller, or NULL.  While set (per calling thread),
  * dsa3d_forward records fwd_start / fwd_stop on its stream immediately around the forward
- * kernel, and dsa3d_backward records bwd_start / bwd_stop around its gather kernel and
- * scatter_start / scatter_stop around its tile scatter kernel (when that kernel runs), so a
- * caller can time those kernels alone inside a longer step.  Pass NULLs to switch it off.
+ * kernel, and dsa3d_backward records bwd_start / bwd_stop around its cell-sorted kernels or, where
+ * those do not run (fp32, DSA3D_TILE), around its gather kernel and scatter_start / scatter_stop around
+ * its tile scatter kernel (when that kernel runs), so a caller can time those kernels alone inside a longer step.  Pass NULLs to switch it off.
  */
 int dsa3d_set_profile_events(void* fwd_start, void* fwd_stop, void* bwd_start, void* bwd_stop,
                              void* scatter_start, void* scatter_stop);

@@ -269,13 +269,14 @@ gather_forward_small_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bflo
 #define DSA3D_FWD_MINBLOCKS 3
 #endif
 
-template <typename T, int D, int NV, bool kAdd>
-__global__ void __launch_bounds__(256, NV == 2 ? 2 : DSA3D_FWD_MINBLOCKS)
+// fp32 storage, and bf16 where launch_forward keeps it: a group of lanes per item.
+template <typename T, int D, bool kAdd>
+__global__ void __launch_bounds__(256, DSA3D_FWD_MINBLOCKS)
 forward_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
                const float* __restrict__ offsets, const T* addend, T* out, float* __restrict__ lse,
                const Problem pr, const int* __restrict__ gate) {
     if (gate && *gate == 0) return;                      // another kernel takes this call (see launch_forward)
-    using E = Elt<T, NV>;
+    using E = Elt<T, 1>;
     using Row = typename E::Row;
     constexpr int VEC = E::VEC;
     constexpr int LPR = D / VEC;
@@ -440,14 +441,6 @@ forward_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __rest
     }
 }
 
-// 16-byte vectors per lane.  One everywhere: two (8 lanes per 128-channel bf16 item) halves
-// the per-item bookkeeping but costs a block of occupancy, which the forward loses more by.
-#ifndef DSA3D_FWD_BF16_NV
-#define DSA3D_FWD_BF16_NV 1
-#endif
-template <typename T, int D> struct FwdLaneWidth { static constexpr int NV = 1; };
-template <> struct FwdLaneWidth<__nv_bfloat16, 128> { static constexpr int NV = DSA3D_FWD_BF16_NV; };
-
 template <int D>
 static cudaError_t launch_gather_forward(const void* q, const void* k, const void* v, const float* offsets, const void* addend, void* out,
                                          float* lse, const Problem& pr, cudaStream_t stream, const int* gate) {
@@ -484,17 +477,16 @@ template <typename T, int D>
 static cudaError_t launch_forward_t(const void* q, const void* k, const void* v, const float* offsets,
                                     const void* addend, void* out, float* lse, const Problem& pr,
                                     cudaStream_t stream, const int* gate) {
-    constexpr int NV = FwdLaneWidth<T, D>::NV;
-    constexpr int LPR = D / Elt<T, NV>::VEC;
+    constexpr int LPR = D / Elt<T, 1>::VEC;
     constexpr int threads = 256;
     const long long groups_per_block = threads / LPR;
     const long long blocks = (pr.items + groups_per_block - 1) / groups_per_block;
     if (addend)
-        forward_kernel<T, D, NV, true><<<static_cast<unsigned>(blocks), threads, 0, stream>>>(
+        forward_kernel<T, D, true><<<static_cast<unsigned>(blocks), threads, 0, stream>>>(
             static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v), offsets,
             static_cast<const T*>(addend), static_cast<T*>(out), lse, pr, gate);
     else
-        forward_kernel<T, D, NV, false><<<static_cast<unsigned>(blocks), threads, 0, stream>>>(
+        forward_kernel<T, D, false><<<static_cast<unsigned>(blocks), threads, 0, stream>>>(
             static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v), offsets, nullptr,
             static_cast<T*>(out), lse, pr, gate);
     return cudaGetLastError();
@@ -509,7 +501,7 @@ cudaError_t launch_forward(const void* q, const void* k, const void* v, const fl
 #define DSA3D_CASE(DD)                                                                                    \
     case DD:                                                                                              \
         return warp_per_item ? launch_gather_forward<DD>(q, k, v, offsets, addend, out, lse, pr, stream, gate)    \
-               : bf16 ? launch_forward_t<__nv_bfloat16, DD>(q, k, v, offsets, addend, out, lse, pr, stream, gate) \
+               : bf16 ? launch_forward_t<__nv_bfloat16, 32>(q, k, v, offsets, addend, out, lse, pr, stream, gate) \
                       : launch_forward_t<float, DD>(q, k, v, offsets, addend, out, lse, pr, stream, gate);
     switch (pr.d) {
         DSA3D_CASE(32)
