@@ -105,8 +105,10 @@ int dsa3d_forward(const void* q, const void* k, const void* v, const float* offs
  *                one-sided convention of the floor at integer positions (cell [i, i+1))
  * The sampling weights are recomputed, nothing of size N*P*d is stored.
  * `workspace` is device scratch of at least dsa3d_backward_workspace_bytes(...) bytes,
- * 16-byte aligned (bf16 storage: fp32 accumulators for dk and dv, two fp32 coefficients per
- * sample, and the bins of the tile pre-reduction; may be NULL when that size is 0).
+ * 16-byte aligned (bf16 storage: fp32 accumulators for dk and dv, then room in which the samples are
+ * sorted by key cell, as many heads at a time as fit; may be NULL when that size is 0).  fp32 storage runs with any
+ * workspace or none: what is given serves the sort, which makes large calls faster (1.4 times at 2.7 million samples
+ * of 64 channels).
  * Its contents on entry do not matter.  dk and dv are summed with floating-point atomics,
  * so their last bits can differ from run to run; dq, doffsets are deterministic.
  */
@@ -116,8 +118,8 @@ int dsa3d_backward(const void* q, const void* k, const void* v, const float* off
                    void* dq, void* dk, void* dv, float* doffsets,
                    void* workspace, size_t workspace_bytes, int dtype, void* stream);
 
-/* Scratch bytes dsa3d_backward needs for this problem (0 for DSA3D_F32; 0 also for
- * arguments the library would reject). */
+/* Scratch bytes dsa3d_backward needs for this problem (DSA3D_F32: what a large problem has use for, up to
+ * 1 GiB, and 0 for a small one; 0 also for arguments the library would reject). */
 size_t dsa3d_backward_workspace_bytes(int T, int H, int W, int heads, int d,
                                       const int window[3], int dtype);
 

@@ -97,9 +97,19 @@ struct BackwardWorkspace {
     long long entries_per_cta;
 };
 
+// fp32 storage: where the cell-sorted kernels are faster than the row kernels.  They cost seven launches more, and windows of
+// fewer samples fill the cells too thinly (64 channels, window (3,3,3): 166K samples 0.15 against 0.15 ms, 553K 0.31 against
+// 0.41, 2.7M 1.19 against 1.71; window (2,2,2) 400K 0.33 against 0.29).  On integer offsets the row kernels run and the
+// closed gates in front of them are all that is added: 0.02 to 0.03 ms, which is why the line lies above the first gains.
+constexpr int kF32CellsWindow = 16;
+constexpr long long kF32CellsSamples = 1000000;
+
 BackwardWorkspace backward_workspace(const dsa3d::Problem& pr, int dtype, bool tiled) {
     BackwardWorkspace w{};
-    if (dtype != DSA3D_BF16) return w;
+    if (dtype != DSA3D_BF16) {                       // nothing that has to be there: see backward_plan
+        w.total = pr.P >= kF32CellsWindow && pr.items * pr.P >= kF32CellsSamples ? dsa3d::cells_scratch_bytes(pr) : 0;
+        return w;
+    }
     w.acc_bytes = static_cast<size_t>(pr.items) * pr.d * sizeof(float) * 2;
     if (tiled && pr.tile_t >= 1) {
         // rounded up so that the 16-byte bin entries behind it stay 16-byte aligned
@@ -365,7 +375,7 @@ int backward_plan(int T, int H, int W, int heads, int d, const int* window, int 
     plan.bf16 = dtype == DSA3D_BF16;
     if (plan.bf16 && tiled) set_tiling(plan.pr);
     plan.ws = backward_workspace(plan.pr, dtype, tiled);
-    if (plan.ws.total > 0) {
+    if (plan.bf16 && plan.ws.total > 0) {
         if (!workspace || workspace_bytes < plan.ws.total) return DSA3D_ERR_WORKSPACE;
         if (!aligned16(workspace)) return DSA3D_ERR_MISALIGNED;
     }
@@ -380,6 +390,10 @@ int backward_plan(int T, int H, int W, int heads, int d, const int* window, int 
     if (plan.bf16 && !getenv("DSA3D_TILE")) {
         plan.cells = wsp + plan.ws.acc_bytes;
         plan.cells_bytes = workspace_bytes - plan.ws.acc_bytes;
+    }
+    if (!plan.bf16 && plan.ws.total > 0 && workspace && aligned16(workspace) && !getenv("DSA3D_TILE")) {
+        plan.cells = workspace;
+        plan.cells_bytes = workspace_bytes;
     }
     if (plan.coef) {
         int dev = 0, sms = 0;
@@ -428,12 +442,34 @@ dsa3d::Problem frames_of(const dsa3d::Problem& pr, int f0, int f1) {
 int backward_frames(const BackwardPlan& plan, const void* q, const void* k, const void* v, const float* offsets,
                     const float* lse, const void* dout, void* dq, float* doffsets, int f0, int f1,
                     bool clear, cudaStream_t stream, cudaEvent_t after_gather) {
-    const dsa3d::Problem pr = frames_of(plan.pr, f0, f1);
+    dsa3d::Problem pr = frames_of(plan.pr, f0, f1);
     cudaError_t e = record(2, stream);
     if (e != cudaSuccess) return cuda_failed(e);
-    if (plan.cells && dsa3d::try_cells_backward(q, k, v, offsets, lse, dout, dq, plan.acc_dk, plan.acc_dv, doffsets, plan.cells,
-                                                plan.cells_bytes, plan.workspace, clear ? plan.ws.acc_bytes : 0, pr, stream, &e)) {
+    const int* rows_gate = pr.gate;
+    if (!plan.bf16 && plan.cells) {                  // both routes are queued, each behind its gate
+        void* words = nullptr;
+        e = cudaGetSymbolAddress(&words, g_gate_words);
         if (e != cudaSuccess) return cuda_failed(e);
+        const unsigned next = g_next_gate.fetch_add(2u);
+        int *on_grid = static_cast<int*>(words) + next % kGateWords, *off_grid = static_cast<int*>(words) + (next + 1u) % kGateWords;
+        e = dsa3d::launch_cells_choose(offsets + pr.q_begin * pr.heads * pr.P * 3, pr.items * pr.P, on_grid, off_grid, stream);
+        if (e != cudaSuccess) return cuda_failed(e);
+        rows_gate = on_grid;
+        pr.gate = off_grid;
+    }
+    if (clear && !plan.bf16) {                       // two arrays of the caller's
+        const int rc = backward_clear(plan, stream);
+        if (rc != DSA3D_OK) return rc;
+        clear = false;
+    }
+    if (plan.cells && dsa3d::try_cells_backward(q, k, v, offsets, lse, dout, dq, plan.acc_dk, plan.acc_dv, doffsets, plan.cells,
+                                                plan.cells_bytes, plan.workspace, clear ? plan.ws.acc_bytes : 0, pr, plan.bf16, stream, &e)) {
+        if (e != cudaSuccess) return cuda_failed(e);
+        if (!plan.bf16) {
+            pr.gate = rows_gate;
+            e = dsa3d::launch_backward(q, k, v, offsets, lse, dout, dq, plan.acc_dk, plan.acc_dv, doffsets, plan.coef, pr, false, stream);
+            if (e != cudaSuccess) return cuda_failed(e);
+        }
         e = record(3, stream);
         if (e != cudaSuccess) return cuda_failed(e);
         if (after_gather) {
@@ -446,6 +482,7 @@ int backward_frames(const BackwardPlan& plan, const void* q, const void* k, cons
         const int rc = backward_clear(plan, stream);
         if (rc != DSA3D_OK) return rc;
     }
+    pr.gate = plan.pr.gate;
     e = dsa3d::launch_backward(q, k, v, offsets, lse, dout, dq, plan.acc_dk, plan.acc_dv, doffsets, plan.coef, pr,
                                plan.bf16, stream);
     if (e != cudaSuccess) return cuda_failed(e);

@@ -11,6 +11,8 @@
 //                        CTAs of the last two block kernels
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 #include "dsa3d_cells.cuh"
 #include "dsa3d_kernels.h"
 
@@ -299,24 +301,26 @@ __device__ __forceinline__ void load_box(unsigned char* dst, const bf16* __restr
 }
 
 // ------------------------------------------------------------------------------------------------ beyond the bins
-// The samples in bin kBins of every tile, a warp per sample, row by row: part `part` of `parts` (256 threads each).
+// The samples in bin kBins of every tile, a warp per sample, row by row: part `part` of `parts` (a CTA each).
 // kScatter: their contributions to dK and dV, and those of marked samples of the other bins; otherwise what the
 // products of cells_dots_kernel leave for the others.  There are none in nearly every call: the work rides in CTAs
 // behind those of the block kernels instead of two launches of its own.
-template <int D, bool kScatter>
-__device__ __noinline__ void far_part(const unsigned part, const unsigned parts, const bf16* __restrict__ q, const bf16* __restrict__ k, const bf16* __restrict__ v,
-                                      const bf16* __restrict__ dout, const float* __restrict__ offsets, float* __restrict__ acc_dk, float* __restrict__ acc_dv,
+template <typename T, int D, bool kScatter>
+__device__ __noinline__ void far_part(const unsigned part, const unsigned parts, const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
+                                      const T* __restrict__ dout, const float* __restrict__ offsets, float* __restrict__ acc_dk, float* __restrict__ acc_dv,
                                       const Problem& pr, const Slab& sl) {
     const int tiles = sl.heads * sl.tiles_t * sl.tiles_y * sl.tiles_x;
     constexpr int V = D / 32;                       // channels per lane
-    const int lane = threadIdx.x & 31, warps = static_cast<int>(parts) * 8;
+    const int lane = threadIdx.x & 31, warp = static_cast<int>(threadIdx.x >> 5), warps = static_cast<int>(blockDim.x >> 5);
     const long long tok = static_cast<long long>(pr.heads) * D;
     const int per_head = sl.tiles_t * sl.tiles_y * sl.tiles_x;
     [[maybe_unused]] const long long kv_extent = pr.N * pr.heads * D;
-    for (int base = (static_cast<int>(part) * 8 + static_cast<int>(threadIdx.x >> 5)) * 32; base < tiles; base += warps * 32) {
+    const bool marked = kScatter && *sl.marked != 0;
+    // a lane per tile finds those with something to do; the warps of the CTA then share a tile's samples
+    const int at_once = min(32, (tiles + static_cast<int>(parts) - 1) / static_cast<int>(parts));
+    for (int base = static_cast<int>(part) * at_once; base < tiles; base += static_cast<int>(parts) * at_once) {
         uint32_t mine = 0u;
-        if (base + lane < tiles) mine = __ldg(sl.seg + static_cast<long long>(base + lane) * (kBins + 1) + kBins);
-        const bool marked = kScatter && *sl.marked != 0;
+        if (lane < at_once && base + lane < tiles) mine = __ldg(sl.seg + static_cast<long long>(base + lane) * (kBins + 1) + kBins);
         if (marked) mine = ((mine & 0xffffu) + (mine >> 16)) << 16;        // all samples of the tile: those beyond the bins are its last
         unsigned todo = __ballot_sync(kFullMask, (mine >> 16) != 0u);
         while (todo) {
@@ -326,8 +330,21 @@ __device__ __noinline__ void far_part(const unsigned part, const unsigned parts,
             const long long tile = base + src;
             const int m = sl.m0 + static_cast<int>(tile / per_head);
             const uint32_t far_from = marked ? __ldg(sl.seg + tile * (kBins + 1) + kBins) & 0xffffu : 0u;
-            for (uint32_t i = 0; i < (w >> 16); ++i) {
-                const long long at = tile * (kRows * pr.P) + (w & 0xffffu) + i;
+            const long long list = tile * (kRows * pr.P) + (w & 0xffffu);
+            uint32_t next = static_cast<uint32_t>(warp) * 32u;
+            unsigned some = 0u;
+            while (true) {
+                while (some == 0u && next < (w >> 16)) {   // 32 samples at a time: which of them are beyond the bins or marked
+                    const uint32_t i = next + static_cast<uint32_t>(lane);
+                    bool take = i < (w >> 16);
+                    if (take && marked && i < far_from)
+                        take = __float_as_uint(sl.coef[sample_at(sl, pr, m, static_cast<int>(__ldg(sl.geo + list + i).x), static_cast<int>(__ldg(sl.meta + list + i) & 255u))].y) >> 31;
+                    some = __ballot_sync(kFullMask, take);
+                    next += static_cast<uint32_t>(warps) * 32u;
+                }
+                if (some == 0u) break;
+                const long long at = list + next - static_cast<uint32_t>(warps) * 32u + static_cast<uint32_t>(__ffs(static_cast<int>(some)) - 1);
+                some &= some - 1u;
                 const int n = static_cast<int>(__ldg(sl.geo + at).x), p = static_cast<int>(__ldg(sl.meta + at) & 255u);
                 const int x = n % pr.W, y = (n / pr.W) % pr.H, t = n / (pr.W * pr.H);
                 const long long row = static_cast<long long>(n) * pr.heads + m;
@@ -336,15 +353,14 @@ __device__ __noinline__ void far_part(const unsigned part, const unsigned parts,
                 float qv[V], dv[V];
 #pragma unroll
                 for (int z = 0; z < V; ++z) {
-                    qv[z] = __bfloat162float(q[row * D + lane * V + z]);
-                    dv[z] = __bfloat162float(dout[row * D + lane * V + z]);
+                    qv[z] = static_cast<float>(q[row * D + lane * V + z]);
+                    dv[z] = static_cast<float>(dout[row * D + lane * V + z]);
                 }
                 const float wt[2] = {1.0f - smp.ft, smp.ft}, wy[2] = {1.0f - smp.fy, smp.fy}, wx[2] = {1.0f - smp.fx, smp.fx};
                 const long long sy = static_cast<long long>(pr.W) * tok, st = static_cast<long long>(pr.H) * sy;
                 const long long sidx = sample_at(sl, pr, m, n, p);
                 if constexpr (kScatter) {
                     const float2 cf = sl.coef[sidx];
-                    if (marked && i < far_from && !(__float_as_uint(cf.y) >> 31)) continue;
                     for (int j = 0; j < 8; ++j) {
                         const float wj = wt[j >> 2] * wy[(j >> 1) & 1] * wx[j & 1];
                         const long long o = o0 + (j >> 2) * st + ((j >> 1) & 1) * sy + (j & 1) * tok;
@@ -366,8 +382,8 @@ __device__ __noinline__ void far_part(const unsigned part, const unsigned parts,
                         if (!((smp.mask >> j) & 1u) || !needed || !DSA3D_IN_RANGE(pr, o, kv_extent, 5)) continue;
 #pragma unroll
                         for (int z = 0; z < V; ++z) {
-                            a[j] = fmaf(qv[z], __bfloat162float(k[o + z]), a[j]);
-                            bb[j] = fmaf(dv[z], __bfloat162float(v[o + z]), bb[j]);
+                            a[j] = fmaf(qv[z], static_cast<float>(k[o + z]), a[j]);
+                            bb[j] = fmaf(dv[z], static_cast<float>(v[o + z]), bb[j]);
                         }
                     }
 #pragma unroll
@@ -514,14 +530,14 @@ cells_dots_kernel(const bf16* __restrict__ q, const bf16* __restrict__ k, const 
                   const float* __restrict__ offsets, const __grid_constant__ Problem pr, const __grid_constant__ Slab sl, unsigned blocks) {
     if constexpr (!kGated) {
         if (blockIdx.x < blocks) dots_block<D, kWide>(blockIdx.x, q, k, v, dout, pr, sl);
-        else far_part<D, false>(blockIdx.x - blocks, gridDim.x - blocks, q, k, v, dout, offsets, nullptr, nullptr, pr, sl);
+        else far_part<bf16, D, false>(blockIdx.x - blocks, gridDim.x - blocks, q, k, v, dout, offsets, nullptr, nullptr, pr, sl);
     } else {
         if (gated_off_early(pr.gate)) return;
         for (unsigned block = blockIdx.x; block < blocks; block += gridDim.x) {
             dots_block<D, kWide>(block, q, k, v, dout, pr, sl);
             __syncthreads();
         }
-        far_part<D, false>(blockIdx.x, gridDim.x, q, k, v, dout, offsets, nullptr, nullptr, pr, sl);
+        far_part<bf16, D, false>(blockIdx.x, gridDim.x, q, k, v, dout, offsets, nullptr, nullptr, pr, sl);
     }
 }
 
@@ -534,13 +550,13 @@ constexpr int kQueryWarps = 2;
 // in the forward (dsa3d_gather.cuh).  A sample with anything that is not finite (its rows of q, dO, K or V, or its
 // coefficients) is marked by the sign of cv: its contributions to dK and dV are formed one by one, so that they reach only
 // the corners with a weight.  Windows of at most 8 (16) samples: G = 4 (2) neighbouring queries share a warp.
-template <int D, int G>
-__device__ __forceinline__ void query_block(const unsigned block, const bf16* __restrict__ k, const float* __restrict__ offsets, const float* __restrict__ lse, bf16* __restrict__ dq,
+template <typename T, int D, int G>
+__device__ __forceinline__ void query_block(const unsigned block, const T* __restrict__ k, const float* __restrict__ offsets, const float* __restrict__ lse, T* __restrict__ dq,
                    float* __restrict__ doffsets, const Problem& pr, const Slab& sl, unsigned blocks_per_head) {
     __shared__ GatherList lists[kQueryWarps];
     constexpr int L = 32 / G;                       // lanes per query
-    constexpr int U = GatherStep<D>::U, PER = U > G ? U / G : 1, ITEMS = G > U ? G / U : 1;      // subgroups per query, queries per subgroup
-    constexpr int step = G == 1 ? GatherStep<D>::N : 4 * PER;
+    constexpr int CH = GatherStep<D, T>::CH, U = GatherStep<D, T>::U, PER = U > G ? U / G : 1, ITEMS = G > U ? G / U : 1;      // subgroups per query, queries per subgroup
+    constexpr int step = G == 1 ? GatherStep<D, T>::N : 4 * PER;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gl_lane = lane & (L - 1);
     GatherList& gl = lists[warp];
     const int frame = pr.H * pr.W, mh = static_cast<int>(block / blocks_per_head), per_head = frame * (sl.f1 - sl.f0);
@@ -554,8 +570,8 @@ __device__ __forceinline__ void query_block(const unsigned block, const bf16* __
     const float scale = rsqrtf(static_cast<float>(D)), lse2 = __ldg(lse + row) * kLog2e;
     const float* off_row = offsets + row * pr.P * 3;
     const float* st_row = sl.stats + item * pr.P * 8;
-    const uint32_t tok_bytes = static_cast<uint32_t>(pr.heads) * (D * 2);
-    const bf16* kh = k + static_cast<long long>(m) * D;
+    const uint32_t tok_bytes = static_cast<uint32_t>(pr.heads) * (D * static_cast<int>(sizeof(T)));
+    const T* kh = k + static_cast<long long>(m) * D;
     auto sample = [&](int p, Sample& s, float4& a, float4& b) {
         s.base = 0; s.mask = 0u; s.ft = s.fy = s.fx = 0.0f;
         a = b = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
@@ -577,9 +593,9 @@ __device__ __forceinline__ void query_block(const unsigned block, const bf16* __
         if (s2.mask) delta = fmaf(weight(a2.x), b2.x, delta);
     }
     delta = group_sum<L>(delta, kFullMask);
-    float acc[8];
+    float acc[CH];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) acc[e] = 0.0f;
+    for (int e = 0; e < CH; ++e) acc[e] = 0.0f;
     for (int pb = 0; pb < pr.P; pb += L) {
         const int p = pb + gl_lane;
         if (pb > 0) sample(p, s, a, b);
@@ -606,43 +622,43 @@ __device__ __forceinline__ void query_block(const unsigned block, const bf16* __
         gather_weights<G>(gl, part, ck, w, step);
         __syncwarp();
         if constexpr (G == 1) {
-            gather_sum<D>(gl, part.total, kh, tok_bytes, acc);
+            gather_sum<D, T>(gl, part.total, kh, tok_bytes, acc);
         } else {
-            constexpr int LPR = GatherStep<D>::LPR;
+            constexpr int LPR = GatherStep<D, T>::LPR;
 #pragma unroll
             for (int i = 0; i < ITEMS; ++i) {
                 const int u = lane / LPR, it = PER > 1 ? u / PER : u * ITEMS + i;
                 const int total = __shfl_sync(kFullMask, part.total, it * L);
 #pragma unroll
-                for (int e = 0; e < 8; ++e) acc[e] = 0.0f;
-                gather_sum_item<D, PER>(gl, it * (kGatherRows / G), total, PER > 1 ? u % PER : 0, kh, tok_bytes, acc);
+                for (int e = 0; e < CH; ++e) acc[e] = 0.0f;
+                gather_sum_item<D, PER, T>(gl, it * (kGatherRows / G), total, PER > 1 ? u % PER : 0, kh, tok_bytes, acc);
                 __syncwarp();
 #pragma unroll
                 for (int o = LPR; o < LPR * PER; o <<= 1)
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) acc[e] += __shfl_xor_sync(kFullMask, acc[e], o);
+                    for (int e = 0; e < CH; ++e) acc[e] += __shfl_xor_sync(kFullMask, acc[e], o);
                 if (warp_first + it < per_head && (PER == 1 || u % PER == 0))
-                    Elt<bf16, 1>::store(dq + (static_cast<long long>(frame * sl.f0 + warp_first + it) * pr.heads + m) * D + (lane % LPR) * 8, acc);
+                    Elt<T, 1>::store(dq + (static_cast<long long>(frame * sl.f0 + warp_first + it) * pr.heads + m) * D + (lane % LPR) * CH, acc);
             }
         }
         __syncwarp();
     }
     if constexpr (G == 1) {
         gather_finish<D>(acc);
-        if (lane < D / 8) Elt<bf16, 1>::store(dq + row * D + lane * 8, acc);
+        if (lane < D / CH) Elt<T, 1>::store(dq + row * D + lane * CH, acc);
     }
 }
 
-template <int D, int G, bool kGated>
+template <typename T, int D, int G, bool kGated>
 __global__ void __launch_bounds__(kQueryWarps * 32, 16)
-cells_query_kernel(const bf16* __restrict__ k, const float* __restrict__ offsets, const float* __restrict__ lse, bf16* __restrict__ dq,
+cells_query_kernel(const T* __restrict__ k, const float* __restrict__ offsets, const float* __restrict__ lse, T* __restrict__ dq,
                    float* __restrict__ doffsets, const __grid_constant__ Problem pr, const __grid_constant__ Slab sl, unsigned blocks_per_head, unsigned blocks) {
     if constexpr (!kGated) {
-        query_block<D, G>(blockIdx.x, k, offsets, lse, dq, doffsets, pr, sl, blocks_per_head);
+        query_block<T, D, G>(blockIdx.x, k, offsets, lse, dq, doffsets, pr, sl, blocks_per_head);
     } else {
         if (gated_off_early(pr.gate)) return;
         for (unsigned block = blockIdx.x; block < blocks; block += gridDim.x) {
-            query_block<D, G>(block, k, offsets, lse, dq, doffsets, pr, sl, blocks_per_head);
+            query_block<T, D, G>(block, k, offsets, lse, dq, doffsets, pr, sl, blocks_per_head);
             __syncthreads();
         }
     }
@@ -838,17 +854,182 @@ cells_sums_kernel(const bf16* __restrict__ q, const bf16* __restrict__ dout, con
                   float* __restrict__ acc_dv, const __grid_constant__ Problem pr, const __grid_constant__ Slab sl, unsigned blocks) {
     if constexpr (!kGated) {
         if (blockIdx.x < blocks) sums_block<D>(blockIdx.x, q, dout, acc_dk, acc_dv, pr, sl);
-        else far_part<D, true>(blockIdx.x - blocks, gridDim.x - blocks, q, nullptr, nullptr, dout, offsets, acc_dk, acc_dv, pr, sl);
+        else far_part<bf16, D, true>(blockIdx.x - blocks, gridDim.x - blocks, q, static_cast<const bf16*>(nullptr), static_cast<const bf16*>(nullptr), dout, offsets, acc_dk, acc_dv, pr, sl);
     } else {
         if (gated_off_early(pr.gate)) return;
         for (unsigned block = blockIdx.x; block < blocks; block += gridDim.x) {
             sums_block<D>(block, q, dout, acc_dk, acc_dv, pr, sl);
             __syncthreads();
         }
-        far_part<D, true>(blockIdx.x, gridDim.x, q, nullptr, nullptr, dout, offsets, acc_dk, acc_dv, pr, sl);
+        far_part<bf16, D, true>(blockIdx.x, gridDim.x, q, static_cast<const bf16*>(nullptr), static_cast<const bf16*>(nullptr), dout, offsets, acc_dk, acc_dv, pr, sl);
     }
 }
 
+
+// ------------------------------------------------------------------------------------------------ fp32 storage
+// The block kernels for fp32 storage, on fp32 FMAs.  A cell's samples follow one another through a group of D / 4 lanes (16
+// bytes of a row each; groups alternate between the two tensors) which holds the cell's eight corner rows - for the
+// sums, their accumulators - in registers: per sample one query row is read instead of eight key rows, and a cell's rows are
+// reduced into the accumulators once instead of once per sample (which bound the row kernels: 1.67 ms
+// for 99840 items of 64 channels, window (3,3,3), against 1.19 ms; the issue rate bounds these: 104 and 83 instructions of a
+// warp per sample).
+constexpr int kF32Ahead = 4;        // samples a group has in flight
+
+template <int D> struct F32Lanes {
+    static constexpr int LPR = D / 4, U = 32 / LPR, SP = U > 1 ? U / 2 : 1;       // groups of a warp; samples it takes at a time
+    int gl, tensor, sub, cell0, cell_step;
+    __device__ __forceinline__ F32Lanes() {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, slot = lane / LPR;
+        gl = lane % LPR;
+        tensor = U > 1 ? slot & 1 : warp & 1;
+        sub = slot >> 1;
+        cell0 = U > 1 ? warp : warp >> 1;
+        cell_step = static_cast<int>(blockDim.x) / (U > 1 ? 32 : 64);
+    }
+};
+
+template <int D, int kThreads>
+__global__ void __launch_bounds__(kThreads, 640 / kThreads)
+cells_dots_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v, const float* __restrict__ dout,
+                      const float* __restrict__ offsets, const __grid_constant__ Problem pr, const __grid_constant__ Slab sl, unsigned blocks) {
+    if (gated_off_early(pr.gate)) return;
+    if (blockIdx.x >= blocks) {
+        far_part<float, D, false>(blockIdx.x - blocks, gridDim.x - blocks, q, k, v, dout, offsets, nullptr, nullptr, pr, sl);
+        return;
+    }
+    using L = F32Lanes<D>;
+    constexpr int LPR = L::LPR, SP = L::SP;
+    const uint32_t* first = sl.first + static_cast<long long>(blockIdx.x) * (kCells + 1);
+    if (__ldg(first) == __ldg(first + kCells)) return;
+    const L ln;
+    const BlockPos b = block_pos(sl, blockIdx.x);
+    const long long tok = static_cast<long long>(pr.heads) * D, head = static_cast<long long>(b.m) * D + ln.gl * 4;
+    const float* keys = (ln.tensor ? v : k) + head;
+    const float* src = (ln.tensor ? dout : q) + head;
+    float* out = sl.stats + ln.tensor * 4 + ((ln.gl & (LPR / 2)) ? 2 : 0) + ((ln.gl & (LPR / 4)) ? 1 : 0);
+    const bool writes = (ln.gl & (LPR / 4 - 1)) == 0;
+    for (int cell = ln.cell0; cell < kCells; cell += ln.cell_step) {
+        const uint32_t f0 = __ldg(first + cell), f1 = __ldg(first + cell + 1);
+        if (f0 == f1) continue;
+        float4 rows[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const int t = b.t + cell_t(cell) + (c >> 2), y = b.y + cell_y(cell) + ((c >> 1) & 1), x = b.x + cell_x(cell) + (c & 1);
+            rows[c] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (static_cast<unsigned>(t) < static_cast<unsigned>(pr.T) && static_cast<unsigned>(y) < static_cast<unsigned>(pr.H) && static_cast<unsigned>(x) < static_cast<unsigned>(pr.W))
+                rows[c] = __ldg(reinterpret_cast<const float4*>(keys + ((static_cast<long long>(t) * pr.H + y) * pr.W + x) * tok));
+        }
+        for (uint32_t f = f0; f < f1; f += SP * kF32Ahead) {
+            float4 geo[kF32Ahead], r[kF32Ahead];
+            uint32_t at[kF32Ahead];
+#pragma unroll
+            for (int i = 0; i < kF32Ahead; ++i) {
+                const uint32_t s = min(f + static_cast<uint32_t>(i * SP + ln.sub), f1 - 1u);       // a missing sample repeats the last one
+                geo[i] = __ldg(sl.sorted + s);
+                at[i] = __ldg(sl.place + s);
+            }
+#pragma unroll
+            for (int i = 0; i < kF32Ahead; ++i) r[i] = __ldg(reinterpret_cast<const float4*>(src + __float_as_int(geo[i].w) * tok));
+#pragma unroll
+            for (int i = 0; i < kF32Ahead; ++i) {
+                if (f + static_cast<uint32_t>(i * SP) >= f1) break;
+                const float ft = geo[i].x, fy = geo[i].y, fx = geo[i].z;
+                float a[8];
+#pragma unroll
+                for (int c = 0; c < 8; ++c) a[c] = fmaf(r[i].w, rows[c].w, fmaf(r[i].z, rows[c].z, fmaf(r[i].y, rows[c].y, r[i].x * rows[c].x)));
+                // corners whose weight and weight derivatives are all zero do not enter (they may hold anything)
+                if (ft == 0.0f || fy == 0.0f || fx == 0.0f) {
+#pragma unroll
+                    for (int c = 0; c < 8; ++c)
+                        if (((c >> 2) && ft == 0.0f) + (((c >> 1) & 1) && fy == 0.0f) + ((c & 1) && fx == 0.0f) > 1) a[c] = 0.0f;
+                }
+                float n0, n1, n2, n3;
+                trilerp_grad(a, ft, fy, fx, n0, n1, n2, n3);
+                // four sums over the group, handing half of the numbers over at each of the first two steps
+                const bool up = ln.gl & (LPR / 2), up2 = ln.gl & (LPR / 4);
+                const float x0 = (up ? n2 : n0) + __shfl_xor_sync(kFullMask, up ? n0 : n2, LPR / 2);
+                const float x1 = (up ? n3 : n1) + __shfl_xor_sync(kFullMask, up ? n1 : n3, LPR / 2);
+                float x = (up2 ? x1 : x0) + __shfl_xor_sync(kFullMask, up2 ? x0 : x1, LPR / 4);
+#pragma unroll
+                for (int o = LPR / 8; o > 0; o >>= 1) x += __shfl_xor_sync(kFullMask, x, o);
+                if (writes && f + static_cast<uint32_t>(i * SP + ln.sub) < f1) out[static_cast<size_t>(at[i]) * 8] = x;
+            }
+        }
+    }
+}
+
+template <int D, int kThreads>
+__global__ void __launch_bounds__(kThreads, 640 / kThreads)
+cells_sums_f32_kernel(const float* __restrict__ q, const float* __restrict__ dout, const float* __restrict__ offsets, float* __restrict__ acc_dk,
+                      float* __restrict__ acc_dv, const __grid_constant__ Problem pr, const __grid_constant__ Slab sl, unsigned blocks) {
+    if (gated_off_early(pr.gate)) return;
+    if (blockIdx.x >= blocks) {
+        far_part<float, D, true>(blockIdx.x - blocks, gridDim.x - blocks, q, static_cast<const float*>(nullptr), static_cast<const float*>(nullptr), dout, offsets, acc_dk, acc_dv, pr, sl);
+        return;
+    }
+    using L = F32Lanes<D>;
+    constexpr int LPR = L::LPR, SP = L::SP;
+    const uint32_t* first = sl.first + static_cast<long long>(blockIdx.x) * (kCells + 1);
+    if (__ldg(first) == __ldg(first + kCells)) return;
+    const L ln;
+    const BlockPos b = block_pos(sl, blockIdx.x);
+    [[maybe_unused]] const long long kv_extent = pr.N * pr.heads * D;
+    const long long tok = static_cast<long long>(pr.heads) * D, head = static_cast<long long>(b.m) * D + ln.gl * 4;
+    const float* src = (ln.tensor ? dout : q) + head;
+    float* const base = ln.tensor ? acc_dv : acc_dk;
+    for (int cell = ln.cell0; cell < kCells; cell += ln.cell_step) {
+        const uint32_t f0 = __ldg(first + cell), f1 = __ldg(first + cell + 1);
+        if (f0 == f1) continue;
+        float acc[8][4];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) acc[c][0] = acc[c][1] = acc[c][2] = acc[c][3] = 0.0f;
+        unsigned used = 0u;                            // corners that a sample has a weight for
+        for (uint32_t f = f0; f < f1; f += SP * kF32Ahead) {
+            float4 geo[kF32Ahead], r[kF32Ahead];
+            float2 cf[kF32Ahead];
+#pragma unroll
+            for (int i = 0; i < kF32Ahead; ++i) {
+                const uint32_t s = min(f + static_cast<uint32_t>(i * SP + ln.sub), f1 - 1u);
+                geo[i] = __ldg(sl.sorted + s);
+                cf[i] = __ldg(sl.coef + __ldg(sl.place + s));
+                r[i] = __ldg(reinterpret_cast<const float4*>(src + __float_as_int(geo[i].w) * tok));
+            }
+#pragma unroll
+            for (int i = 0; i < kF32Ahead; ++i) {
+                // beyond the cell, or marked (far_part takes it)
+                if (f + static_cast<uint32_t>(i * SP + ln.sub) >= f1 || (__float_as_uint(cf[i].y) >> 31)) continue;
+                const float ft = geo[i].x, fy = geo[i].y, fx = geo[i].z, co = ln.tensor ? cf[i].y : cf[i].x;
+                used |= weighted_corners(0xffu, ft, fy, fx);
+                const float wt[2] = {1.0f - ft, ft}, wy[2] = {1.0f - fy, fy}, wx[2] = {(1.0f - fx) * co, fx * co};
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    const float w = wt[c >> 2] * wy[(c >> 1) & 1] * wx[c & 1];
+                    fma2(acc[c][0], acc[c][1], w, w, r[i].x, r[i].y);
+                    fma2(acc[c][2], acc[c][3], w, w, r[i].z, r[i].w);
+                }
+            }
+        }
+#pragma unroll
+        for (int o = 2 * LPR; o < 32; o <<= 1) {       // groups that shared the cell's samples
+            used |= __shfl_xor_sync(kFullMask, used, o);
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) acc[c][e] += __shfl_xor_sync(kFullMask, acc[c][e], o);
+        }
+        if (ln.sub != 0) continue;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const int t = b.t + cell_t(cell) + (c >> 2), y = b.y + cell_y(cell) + ((c >> 1) & 1), x = b.x + cell_x(cell) + (c & 1);
+            if (!((used >> c) & 1u) || static_cast<unsigned>(t) >= static_cast<unsigned>(pr.T) || static_cast<unsigned>(y) >= static_cast<unsigned>(pr.H) ||
+                static_cast<unsigned>(x) >= static_cast<unsigned>(pr.W))
+                continue;
+            float* to = base + ((static_cast<long long>(t) * pr.H + y) * pr.W + x) * tok + head;
+            if (DSA3D_IN_RANGE(pr, to - base, kv_extent, 10))
+                red_add_v4(to, acc[c][0], acc[c][1], acc[c][2], acc[c][3]);
+        }
+    }
+}
 
 // ------------------------------------------------------------------------------------------------ host
 int floor_div4(int a) { return a >= 0 ? a / 4 : -((-a + 3) / 4); }
@@ -886,10 +1067,11 @@ size_t lay_out(const Problem& pr, int m0, int heads, int f0, int f1, char* base,
 // Behind a gate that is mostly closed launching all CTAs would cost more than anything else (0.95 ms for 1.8 M of the query kernel):
 // the gated instances loop over their blocks, with about as many CTAs as an SM holds (four times as many cost an
 // empty chain 6 us more).
-template <int D, bool kGated>
+template <typename T, int D, bool kGated>
 cudaError_t launch_slab(const void* q_, const void* k_, const void* v_, const float* offsets, const float* lse, const void* dout_, void* dq_,
                         float* acc_dk, float* acc_dv, float* doffsets, const Problem& pr, const Slab& s, void* clear, size_t clear_bytes, cudaStream_t stream) {
-    const bf16 *q = static_cast<const bf16*>(q_), *k = static_cast<const bf16*>(k_), *v = static_cast<const bf16*>(v_), *dout = static_cast<const bf16*>(dout_);
+    constexpr bool kF32 = std::is_same<T, float>::value;
+    const T *q = static_cast<const T*>(q_), *k = static_cast<const T*>(k_), *v = static_cast<const T*>(v_), *dout = static_cast<const T*>(dout_);
     const unsigned tiles = static_cast<unsigned>(s.heads * s.tiles_t * s.tiles_y * s.tiles_x), blocks = static_cast<unsigned>(s.heads * s.blocks_t * s.blocks_y * s.blocks_x);
     const unsigned inv_p = ((1u << 24) + static_cast<unsigned>(pr.P) - 1u) / static_cast<unsigned>(pr.P);
     auto grid = [](unsigned n, unsigned resident) { return kGated && n > 148u * resident ? 148u * resident : n; };
@@ -898,15 +1080,19 @@ cudaError_t launch_slab(const void* q_, const void* k_, const void* v_, const fl
         if (e == cudaSuccess && smem > 48 * 1024) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
         return kern;
     };
-    const size_t bin_smem = static_cast<size_t>((kBins + 1) * kCopies + kRows * pr.P) * sizeof(uint32_t), dot_smem = sizeof(DotSmem<D>), sum_smem = sizeof(SumSmem<D>) + 256;
+    const size_t bin_smem = static_cast<size_t>((kBins + 1) * kCopies + kRows * pr.P) * sizeof(uint32_t), dot_smem = kF32 ? 0 : sizeof(DotSmem<D>), sum_smem = kF32 ? 0 : sizeof(SumSmem<D>) + 256;
     const bool wide = ((reinterpret_cast<uintptr_t>(q) | reinterpret_cast<uintptr_t>(dout)) & 31u) == 0;
+    // fp32: a warp takes cell after cell; CTAs of four warps while they fill the chip three times (five to an SM: the smallest
+    // loss at the end of a block), beyond that many warps to a block so that each has few cells
+    [[maybe_unused]] const unsigned f32_threads = blocks >= 3u * 5u * 148u ? 128u : 512u;
     auto bin = big(cells_bin_kernel<kGated>, bin_smem);
-    auto dots = big(wide ? cells_dots_kernel<D, true, kGated> : cells_dots_kernel<D, false, kGated>, dot_smem);
-    auto sums = big(cells_sums_kernel<D, kGated>, sum_smem);
+    auto dots = [&] { if constexpr (kF32) return f32_threads == 128u ? cells_dots_f32_kernel<D, 128> : cells_dots_f32_kernel<D, 512>; else return big(wide ? cells_dots_kernel<D, true, kGated> : cells_dots_kernel<D, false, kGated>, dot_smem); }();
+    auto sums = [&] { if constexpr (kF32) return f32_threads == 128u ? cells_sums_f32_kernel<D, 128> : cells_sums_f32_kernel<D, 512>; else return big(cells_sums_kernel<D, kGated>, sum_smem); }();
     if (e != cudaSuccess) return e;
+    bool ordinary = kF32;                              // the kernel that writes the gate may be the one before
     auto launch = [&](auto kern, unsigned ctas, unsigned threads, size_t smem, const auto&... args) {
         if (e != cudaSuccess) return;
-        if constexpr (kGated) {
+        if (kGated && !ordinary) {
             e = launch_gated(kern, dim3(ctas), threads, smem, stream, args...);
         } else {
             kern<<<ctas, threads, smem, stream>>>(args...);
@@ -915,26 +1101,61 @@ cudaError_t launch_slab(const void* q_, const void* k_, const void* v_, const fl
     };
     const long long clear_all = static_cast<long long>(clear_bytes / 16);
     launch(bin, grid(tiles, 2), kBinThreads, bin_smem, offsets, pr, s, inv_p, tiles, static_cast<uint4*>(clear), (clear_all + tiles - 1) / tiles, clear_all);
+    ordinary = false;
     launch(cells_sort_kernel<kGated>, grid(blocks, 4), kSortThreads, 0, pr, s, blocks);
-    static_assert(kDotThreads == 256 && kSumThreads == 256, "far_part");
-    const unsigned far_parts = tiles / 256 + 1 < 148 * 8 ? tiles / 256 + 1 : 148 * 8;
-    launch(dots, grid(blocks + far_parts, 3), kDotThreads, dot_smem, q, k, v, dout, offsets, pr, s, blocks);
+    const unsigned far_parts = tiles < 148u * 4u ? tiles : 148u * 4u;
+    launch(dots, grid(blocks + far_parts, kF32 ? 1u << 20 : 3u), kF32 ? f32_threads : kDotThreads, dot_smem, q, k, v, dout, offsets, pr, s, blocks);
     // As many queries per warp as have a lane for every sample.
     const int share = pr.P <= 8 ? 4 : pr.P <= 16 ? 2 : 1, per_block = kQueryWarps * share;
     const unsigned per_head = static_cast<unsigned>((static_cast<long long>(s.f1 - s.f0) * pr.H * pr.W + per_block - 1) / per_block), query_blocks = per_head * static_cast<unsigned>(s.heads);
-    auto query = share == 4 ? cells_query_kernel<D, 4, kGated> : share == 2 ? cells_query_kernel<D, 2, kGated> : cells_query_kernel<D, 1, kGated>;
-    launch(query, grid(query_blocks, 12), kQueryWarps * 32, 0, k, offsets, lse, static_cast<bf16*>(dq_), doffsets, pr, s, per_head, query_blocks);
-    launch(sums, grid(blocks + far_parts, 2), kSumThreads, sum_smem, q, dout, offsets, acc_dk, acc_dv, pr, s, blocks);
+    auto query = share == 4 ? cells_query_kernel<T, D, 4, kGated> : share == 2 ? cells_query_kernel<T, D, 2, kGated> : cells_query_kernel<T, D, 1, kGated>;
+    launch(query, grid(query_blocks, 12), kQueryWarps * 32, 0, k, offsets, lse, static_cast<T*>(dq_), doffsets, pr, s, per_head, query_blocks);
+    launch(sums, grid(blocks + far_parts, kF32 ? 1u << 20 : 2u), kF32 ? f32_threads : kSumThreads, sum_smem, q, dout, offsets, acc_dk, acc_dv, pr, s, blocks);
     return e;
 }
 
+// fp32 storage: *on_grid = 1 if most of up to 4096 samples spread over the offsets lie on grid positions, *off_grid = 1 if not.
+__global__ void __launch_bounds__(1024)
+cells_choose_kernel(const float* __restrict__ offsets, long long samples, int* __restrict__ on_grid, int* __restrict__ off_grid) {
+    int off = 0, seen = 0;
+    for (int i = 0; i < 4; ++i) {
+        const long long s = (samples * (4 * static_cast<int>(threadIdx.x) + i)) >> 12;
+        if (i > 0 && s == (samples * (4 * static_cast<int>(threadIdx.x) + i - 1)) >> 12) continue;
+        const float a = offsets[3 * s], b = offsets[3 * s + 1], c = offsets[3 * s + 2];
+        ++seen;
+        off += floorf(a) != a || floorf(b) != b || floorf(c) != c;
+    }
+    const int votes = __syncthreads_count(2 * off > seen);
+    if (threadIdx.x == 0) {
+        *on_grid = 2 * votes <= 1024;
+        *off_grid = 2 * votes > 1024;
+    }
+}
 }  // namespace
+
+cudaError_t launch_cells_choose(const float* offsets, long long samples, int* on_grid, int* off_grid, cudaStream_t stream) {
+    cells_choose_kernel<<<1, 1024, 0, stream>>>(offsets, samples, on_grid, off_grid);
+    return cudaGetLastError();
+}
+
+// Scratch the fp32 route asks for: the whole problem in one pass up to 1 GiB, passes of at most that beyond.
+size_t cells_scratch_bytes(const Problem& pr) {
+    int heads = pr.heads, frames = pr.T;
+    Slab s;
+    size_t bytes;
+    while ((bytes = lay_out(pr, 0, heads, 0, frames, nullptr, s)) > (static_cast<size_t>(1) << 30)) {
+        if (heads > 1) heads = (heads + 1) / 2;
+        else if (frames > 4) frames = ((frames + 1) / 2 + 3) / 4 * 4;
+        else return 0;
+    }
+    return bytes;
+}
 
 // Splits the queries of `pr` (whole frames) into passes whose buffers fit `bytes`: by heads first (they share nothing),
 // then by frames.
 bool try_cells_backward(const void* q, const void* k, const void* v, const float* offsets, const float* lse, const void* dout, void* dq,
                         float* acc_dk, float* acc_dv, float* doffsets, void* scratch, size_t bytes, void* clear, size_t clear_bytes, const Problem& pr,
-                        cudaStream_t stream, cudaError_t* err) {
+                        bool bf16_storage, cudaStream_t stream, cudaError_t* err) {
     *err = cudaSuccess;
     const long long frame = static_cast<long long>(pr.H) * pr.W;
     const int f_begin = static_cast<int>(pr.q_begin / frame), f_end = f_begin + static_cast<int>(pr.q_count / frame);
@@ -949,9 +1170,10 @@ bool try_cells_backward(const void* q, const void* k, const void* v, const float
         for (int m = 0; m < pr.heads; m += heads) {
             const int f1 = f + frames < f_end ? f + frames : f_end, mh = m + heads < pr.heads ? heads : pr.heads - m;
             lay_out(pr, m, mh, f, f1, static_cast<char*>(scratch), s);
-            auto slab = pr.d == 128 ? (pr.gate ? launch_slab<128, true> : launch_slab<128, false>)
-                        : pr.d == 64 ? (pr.gate ? launch_slab<64, true> : launch_slab<64, false>)
-                                     : (pr.gate ? launch_slab<32, true> : launch_slab<32, false>);
+            auto slab = !bf16_storage ? (pr.d == 128 ? launch_slab<float, 128, true> : pr.d == 64 ? launch_slab<float, 64, true> : launch_slab<float, 32, true>)
+                        : pr.d == 128 ? (pr.gate ? launch_slab<bf16, 128, true> : launch_slab<bf16, 128, false>)
+                        : pr.d == 64  ? (pr.gate ? launch_slab<bf16, 64, true> : launch_slab<bf16, 64, false>)
+                                      : (pr.gate ? launch_slab<bf16, 32, true> : launch_slab<bf16, 32, false>);
             *err = slab(q, k, v, offsets, lse, dout, dq, acc_dk, acc_dv, doffsets, pr, s, clear, clear_bytes, stream);
             clear_bytes = 0;                                        // the first pass clears for all
             if (*err != cudaSuccess) return true;

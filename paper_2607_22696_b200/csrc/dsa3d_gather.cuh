@@ -208,25 +208,27 @@ __device__ __forceinline__ void gather_dots_pair(GatherList& gl, int ra, int ta,
     }
 }
 
-// acc += sum of value[i] * row i: D / 8 lanes per row, 8 channels per lane; the subgroups of a warp take four rows each in turn and
-// their sums are added up by gather_finish.  The list is padded to a multiple of kGatherStep.
-template <int D> struct GatherStep { static constexpr int LPR = D / 8, U = 32 / LPR, N = D == 128 ? 16 : 4 * U; };
-template <int D>
-__device__ __forceinline__ void gather_sum(const GatherList& gl, int total, const __nv_bfloat16* __restrict__ rows, uint32_t tok_bytes, float (&acc)[8]) {
-    using E = Elt<__nv_bfloat16, 1>;
-    constexpr int LPR = GatherStep<D>::LPR, U = GatherStep<D>::U, B = GatherStep<D>::N / (4 * U);    // B batches of four rows in flight
+// acc += sum of value[i] * row i: 16 bytes of a row per lane (LPR lanes per row, CH channels each); the subgroups of a warp take four
+// rows each in turn and their sums are added up by gather_finish.  The list is padded to a multiple of GatherStep::N.
+template <int D, typename T = __nv_bfloat16> struct GatherStep {
+    static constexpr int CH = 16 / static_cast<int>(sizeof(T)), LPR = D / CH, U = 32 / LPR, N = LPR >= 16 ? 8 * U : 4 * U;
+};
+template <int D, typename T = __nv_bfloat16>
+__device__ __forceinline__ void gather_sum(const GatherList& gl, int total, const T* __restrict__ rows, uint32_t tok_bytes, float (&acc)[16 / sizeof(T)]) {
+    using E = Elt<T, 1>;
+    constexpr int LPR = GatherStep<D, T>::LPR, U = GatherStep<D, T>::U, B = GatherStep<D, T>::N / (4 * U);    // B batches of four rows in flight
     const int lane = threadIdx.x & 31;
     const char* src = reinterpret_cast<const char*>(rows) + (lane % LPR) * 16;
     const int u4 = (lane / LPR) * 4;
 _Pragma("unroll 1")
-    for (int s = 0; s < total; s += GatherStep<D>::N) {
-        E::Row r[4 * B];
+    for (int s = 0; s < total; s += GatherStep<D, T>::N) {
+        typename E::Row r[4 * B];
 #pragma unroll
         for (int b = 0; b < B; ++b) {
             const uint4 t = *reinterpret_cast<const uint4*>(gl.token + s + b * 4 * U + u4);
             const uint32_t tk[4] = {t.x, t.y, t.z, t.w};
 #pragma unroll
-            for (int i = 0; i < 4; ++i) r[4 * b + i] = E::load(reinterpret_cast<const __nv_bfloat16*>(src + static_cast<uint64_t>(tk[i]) * tok_bytes));
+            for (int i = 0; i < 4; ++i) r[4 * b + i] = E::load(reinterpret_cast<const T*>(src + static_cast<uint64_t>(tk[i]) * tok_bytes));
         }
 #pragma unroll
         for (int b = 0; b < B; ++b) {
@@ -241,17 +243,17 @@ _Pragma("unroll 1")
 
 // The same for the item whose entries start at `region` by PER neighbouring subgroups of the warp (`sub`: which of them this is); the
 // list is padded to a multiple of 4 * PER.
-template <int D, int PER>
-__device__ __forceinline__ void gather_sum_item(const GatherList& gl, int region, int total, int sub, const __nv_bfloat16* __restrict__ rows, uint32_t tok_bytes,
-                                                float (&acc)[8]) {
-    using E = Elt<__nv_bfloat16, 1>;
-    const char* src = reinterpret_cast<const char*>(rows) + ((threadIdx.x & 31) % GatherStep<D>::LPR) * 16;
+template <int D, int PER, typename T = __nv_bfloat16>
+__device__ __forceinline__ void gather_sum_item(const GatherList& gl, int region, int total, int sub, const T* __restrict__ rows, uint32_t tok_bytes,
+                                                float (&acc)[16 / sizeof(T)]) {
+    using E = Elt<T, 1>;
+    const char* src = reinterpret_cast<const char*>(rows) + ((threadIdx.x & 31) % GatherStep<D, T>::LPR) * 16;
     for (int s = region + sub * 4; s < region + total; s += 4 * PER) {
         const uint4 t = *reinterpret_cast<const uint4*>(gl.token + s);
         const uint32_t tk[4] = {t.x, t.y, t.z, t.w};
-        E::Row r[4];
+        typename E::Row r[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) r[i] = E::load(reinterpret_cast<const __nv_bfloat16*>(src + static_cast<uint64_t>(tk[i]) * tok_bytes));
+        for (int i = 0; i < 4; ++i) r[i] = E::load(reinterpret_cast<const T*>(src + static_cast<uint64_t>(tk[i]) * tok_bytes));
         const float4 w = *reinterpret_cast<const float4*>(gl.value + s);
         E::axpy_paired(w.x, r[0], acc);
         E::axpy_paired(w.y, r[1], acc);
@@ -260,12 +262,12 @@ __device__ __forceinline__ void gather_sum_item(const GatherList& gl, int region
     }
 }
 
-// Adds the subgroups' sums up: every lane then holds the whole sums of its eight channels.
-template <int D> __device__ __forceinline__ void gather_finish(float (&acc)[8]) {
+// Adds the subgroups' sums up: every lane then holds the whole sums of its channels.
+template <int D, int CH> __device__ __forceinline__ void gather_finish(float (&acc)[CH]) {
 #pragma unroll
-    for (int o = GatherStep<D>::LPR; o < 32; o <<= 1)
+    for (int o = D / CH; o < 32; o <<= 1)
 #pragma unroll
-        for (int e = 0; e < 8; ++e) acc[e] += __shfl_xor_sync(kFullMask, acc[e], o);
+        for (int e = 0; e < CH; ++e) acc[e] += __shfl_xor_sync(kFullMask, acc[e], o);
 }
 
 }  // namespace dsa3d

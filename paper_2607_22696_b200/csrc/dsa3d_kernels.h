@@ -33,13 +33,17 @@ cudaError_t launch_scatter_tiles(const void* q, const void* dout, const float* o
                                  float* acc_dk, float* acc_dv, void* scratch, int ctas,
                                  long long entries_per_cta, const Problem& pr, cudaStream_t stream);
 
-// The whole backward of the bf16 queries of `pr` (whole frames) on samples sorted by key cell (dsa3d_cells.cu): dq, doffsets, and
+// The whole backward of the queries of `pr` (whole frames) on samples sorted by key cell (dsa3d_cells.cu): dq, doffsets, and
 // the contributions to the fp32 accumulators.  `scratch`: `bytes` of device memory, worked through in as many passes as
 // it takes; false: not even the smallest pass fits, nothing launched.  `clear_bytes` from `clear` on (the accumulators) are
 // zeroed first.
 bool try_cells_backward(const void* q, const void* k, const void* v, const float* offsets, const float* lse, const void* dout, void* dq,
                         float* acc_dk, float* acc_dv, float* doffsets, void* scratch, size_t bytes, void* clear, size_t clear_bytes,
-                        const Problem& pr, cudaStream_t stream, cudaError_t* err);
+                        const Problem& pr, bool bf16_storage, cudaStream_t stream, cudaError_t* err);
+size_t cells_scratch_bytes(const Problem& pr);
+// fp32 storage: leaves 1 in one of two gate words and 0 in the other: whether the samples lie on grid positions (then the
+// row kernels are faster: they read and write only the one corner that has a weight) or not.
+cudaError_t launch_cells_choose(const float* offsets, long long samples, int* on_grid, int* off_grid, cudaStream_t stream);
 
 // Dynamic shared memory of the tile kernel for this problem's tiling.
 size_t tile_smem_bytes(const Problem& pr);
