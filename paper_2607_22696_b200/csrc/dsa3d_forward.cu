@@ -110,7 +110,7 @@ _Pragma("unroll 1")
             s.base = 0; s.mask = 0u; s.ft = s.fy = s.fx = 0.0f;
             if (have) s = to_sample(pr, make_cell(pr, t, y, x, pb + lane, offsets ? offsets + (row * pr.P + pb + lane) * 3 : kZeroOffset));
             const unsigned mask = checked_corners(pr, weighted_corners(s.mask, s.ft, s.fy, s.fx), s.base, 2);
-            const GatherPart part = gather_list(gl, mask, s.base, pr, step);
+            const GatherPart part = gather_list<1, (D < 128)>(gl, mask, s.base, pr, step);
             __syncwarp();
             gather_dots<D>(gl, part.total, qr, kh, tok_bytes);
             __syncwarp();
