@@ -25,12 +25,18 @@ using bf16 = __nv_bfloat16;
 // ------------------------------------------------------------------------------------------------ binning
 constexpr int kBinThreads = 512, kBinWarps = kBinThreads / 32, kCopies = 8;
 
+// kKeep: the fractions wait in shared memory for the samples' places (windows up to kBinKeep samples: three CTAs per SM still);
+// else the cells are worked out twice.  (Three CTAs against two: 403 -> 381 us for
+// 566 K items, window (3,3,3); kept: 359.)
+constexpr int kBinKeep = 36;
+template <bool kKeep>
 __device__ __forceinline__ void bin_block(const unsigned block, const float* __restrict__ offsets, const Problem& pr, const Slab& sl, unsigned inv_p,
                                           uint4* __restrict__ clear, long long clear_each, long long clear_all) {
     extern __shared__ __align__(16) unsigned char raw[];
     uint32_t* counters = reinterpret_cast<uint32_t*>(raw);                 // [kBins + 1][kCopies]: lanes of a warp mostly hit the same bin
     uint32_t* words = counters + (kBins + 1) * kCopies;                     // [kRows * P]: bin (9 bits), cell (6), rank in its counter (16)
     __shared__ uint32_t scan[kBinWarps];
+    float* kept = kKeep ? reinterpret_cast<float*>(words + kRows * pr.P) : nullptr;     // [3][kRows * P]: the samples' fractions
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const long long tile = block;
     int r = static_cast<int>(tile % (sl.tiles_t * sl.tiles_y * sl.tiles_x));
@@ -62,6 +68,7 @@ __device__ __forceinline__ void bin_block(const unsigned block, const float* __r
             int n;
             const Cell c = cell_of(s, n);
             if (c.mask == 0u) continue;
+            if constexpr (kKeep) { kept[s] = c.ft; kept[samples + s] = c.fy; kept[2 * samples + s] = c.fx; }
             const int rt = c.it - t0 + kReach, ry = c.iy - y0 + kReach, rx = c.ix - x0 + kReach;
             uint32_t bin = kBins, cell = 0u;
             if (static_cast<unsigned>(rt) < 4u * kBinsT && static_cast<unsigned>(ry) < 4u * kBinsY && static_cast<unsigned>(rx) < 3u * kBinsX) {
@@ -119,23 +126,31 @@ __device__ __forceinline__ void bin_block(const unsigned block, const float* __r
         const uint32_t w = words[s];
         if (w == 0xffffffffu) continue;
         int n;
-        const Cell cl = cell_of(s, n);                 // once more from the offsets, in L1 or L2 by now
+        float ft, fy, fx;
+        if constexpr (kKeep) {
+            const int row = row_of(s), ty = row / kTileX;
+            n = ((t0 + (ty >> 2)) * pr.H + y0 + (ty & 3)) * pr.W + x0 + row - ty * kTileX;
+            ft = kept[s]; fy = kept[samples + s]; fx = kept[2 * samples + s];
+        } else {
+            const Cell cl = cell_of(s, n);             // once more from the offsets, in L1 or L2 by now
+            ft = cl.ft; fy = cl.fy; fx = cl.fx;
+        }
         const uint32_t at = counters[(w & 511u) * kCopies + (lane & (kCopies - 1))] + (w >> 15);
-        geo[at] = make_uint4(static_cast<uint32_t>(n), __float_as_uint(cl.ft), __float_as_uint(cl.fy), __float_as_uint(cl.fx));
+        geo[at] = make_uint4(static_cast<uint32_t>(n), __float_as_uint(ft), __float_as_uint(fy), __float_as_uint(fx));
         meta[at] = static_cast<uint16_t>(static_cast<uint32_t>(s - row_of(s) * pr.P) | (((w >> 9) & 63u) << 8));
     }
 }
 
-template <bool kGated>
-__global__ void __launch_bounds__(kBinThreads, 2)
+template <bool kGated, bool kKeep>
+__global__ void __launch_bounds__(kBinThreads, 3)
 cells_bin_kernel(const float* __restrict__ offsets, const __grid_constant__ Problem pr, const __grid_constant__ Slab sl, unsigned inv_p, unsigned blocks,
                  uint4* __restrict__ clear, long long clear_each, long long clear_all) {
     if constexpr (!kGated) {
-        bin_block(blockIdx.x, offsets, pr, sl, inv_p, clear, clear_each, clear_all);
+        bin_block<kKeep>(blockIdx.x, offsets, pr, sl, inv_p, clear, clear_each, clear_all);
     } else {
         if (gated_off_early(pr.gate)) return;
         for (unsigned block = blockIdx.x; block < blocks; block += gridDim.x) {
-            bin_block(block, offsets, pr, sl, inv_p, clear, clear_each, clear_all);
+            bin_block<kKeep>(block, offsets, pr, sl, inv_p, clear, clear_each, clear_all);
             __syncthreads();
         }
     }
@@ -1080,12 +1095,13 @@ cudaError_t launch_slab(const void* q_, const void* k_, const void* v_, const fl
         if (e == cudaSuccess && smem > 48 * 1024) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
         return kern;
     };
-    const size_t bin_smem = static_cast<size_t>((kBins + 1) * kCopies + kRows * pr.P) * sizeof(uint32_t), dot_smem = kF32 ? 0 : sizeof(DotSmem<D>), sum_smem = kF32 ? 0 : sizeof(SumSmem<D>) + 256;
+    const bool keep = pr.P <= kBinKeep;
+    const size_t bin_smem = static_cast<size_t>((kBins + 1) * kCopies + kRows * pr.P * (keep ? 4 : 1)) * sizeof(uint32_t), dot_smem = kF32 ? 0 : sizeof(DotSmem<D>), sum_smem = kF32 ? 0 : sizeof(SumSmem<D>) + 256;
     const bool wide = ((reinterpret_cast<uintptr_t>(q) | reinterpret_cast<uintptr_t>(dout)) & 31u) == 0;
     // fp32: a warp takes cell after cell; CTAs of four warps while they fill the chip three times (five to an SM: the smallest
     // loss at the end of a block), beyond that many warps to a block so that each has few cells
     [[maybe_unused]] const unsigned f32_threads = blocks >= 3u * 5u * 148u ? 128u : 512u;
-    auto bin = big(cells_bin_kernel<kGated>, bin_smem);
+    auto bin = big(keep ? cells_bin_kernel<kGated, true> : cells_bin_kernel<kGated, false>, bin_smem);
     auto dots = [&] { if constexpr (kF32) return f32_threads == 128u ? cells_dots_f32_kernel<D, 128> : cells_dots_f32_kernel<D, 512>; else return big(wide ? cells_dots_kernel<D, true, kGated> : cells_dots_kernel<D, false, kGated>, dot_smem); }();
     auto sums = [&] { if constexpr (kF32) return f32_threads == 128u ? cells_sums_f32_kernel<D, 128> : cells_sums_f32_kernel<D, 512>; else return big(cells_sums_kernel<D, kGated>, sum_smem); }();
     if (e != cudaSuccess) return e;
