@@ -74,6 +74,15 @@ __device__ __noinline__ void forward_item_plain(const __nv_bfloat16* q, const __
     if (lane == 0) lse[row] = (m_run + log2f(l_run)) * kLn2;
 }
 
+// CTAs are handed to the SMs in turn: a wave's CTA numbers are permuted so that kRun consecutive blocks of items, whose samples
+// share K and V rows, run on one SM (64 channels: 13.18 -> 12.95 ms for 4.2 M items; 128 channels 32.19 -> 32.06 for 5.5 M;
+// runs of 8 and 16 gain less).
+__device__ __forceinline__ unsigned sm_neighbours(unsigned block, unsigned blocks) {
+    constexpr unsigned kSms = 148u, kRun = 4, kWave = kSms * kRun;
+    const unsigned wave = block / kWave, r = block - wave * kWave;
+    return (wave + 1u) * kWave <= blocks ? wave * kWave + (r % kSms) * kRun + r / kSms : block;
+}
+
 template <int D, bool kAdd, bool kGated>
 __global__ void __launch_bounds__(kFwdWarps * 32, 16)
 gather_forward_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v,
@@ -85,7 +94,7 @@ gather_forward_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* 
     GatherList& gl = lists[warp];
     // One block of items per CTA; behind a gate (a small launch, see launch_gather_forward) a loop over them.  The loop costs the
     // kernel 2 - 15 %, so only the gated instance has it.
-    unsigned block = blockIdx.x;
+    unsigned block = kGated ? blockIdx.x : sm_neighbours(blockIdx.x, gridDim.x);
 _Pragma("unroll 1")
     do {
         const int m = static_cast<int>(block / blocks_per_head);
