@@ -71,7 +71,7 @@ def _compile(lib: str, force: bool, verbose: bool, debug: bool) -> str:
     flags = list(NVCC_FLAGS) + os.environ.get("DSA3D_NVCC_EXTRA", "").split() + (["-DDSA3D_DEBUG"] if debug else [])
     if verbose:
         flags += ["-Xptxas", "-v"]
-    cmd = [_nvcc(), "-shared", "-o", lib] + flags + [os.path.join(CSRC, s) for s in SOURCES]
+    cmd = [_nvcc(), "-t", "0", "-shared", "-o", lib] + flags + [os.path.join(CSRC, s) for s in SOURCES]
     res = subprocess.run(cmd, capture_output=True, text=True)
     if verbose:
         sys.stderr.write(res.stderr)
