@@ -82,6 +82,8 @@ def _declare(lib) -> None:
     lib.dsa3d_backward_noalloc_max_elements.argtypes = []
     lib.dsa3d_backward_noalloc_last_cuda_error.restype = i
     lib.dsa3d_backward_noalloc_last_cuda_error.argtypes = []
+    lib.dsa3d_test_backward_passes.restype = i
+    lib.dsa3d_test_backward_passes.argtypes = [i, i, i, i, i, win, i, sz, ctypes.POINTER(i), ctypes.POINTER(sz)]
     dptr = ctypes.POINTER(ctypes.c_double)
     lib.dsa3d_probe_gather.restype = i
     lib.dsa3d_probe_gather.argtypes = [p, sz, i, dptr, p]
@@ -341,6 +343,14 @@ def dsa3d_check_device_timeout() -> None:
 def dsa3d_clear_device_timeout() -> None:
     """Resets the (sticky) timeout flag."""
     _check(load().dsa3d_clear_device_timeout())
+
+
+def dsa3d_test_backward_passes(T, H, W, heads, d, window, dtype, scratch_bytes):
+    """(passes of the cell-sorted backward in so much scratch, most bytes one of them uses)."""
+    passes, largest = ctypes.c_int(0), ctypes.c_size_t(0)
+    _check(load().dsa3d_test_backward_passes(T, H, W, heads, d, _window(window), _DTYPES[dtype], scratch_bytes,
+                                             ctypes.byref(passes), ctypes.byref(largest)))
+    return passes.value, largest.value
 
 
 def dsa3d_test_wait_timeout(polls: int, stream=None) -> None:

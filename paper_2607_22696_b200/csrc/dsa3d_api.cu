@@ -950,6 +950,15 @@ int dsa3d_backward_batch(const void* q, const void* k, const void* v, const floa
     return DSA3D_OK;
 }
 
+int dsa3d_test_backward_passes(int T, int H, int W, int heads, int d, const int window[3], int dtype, size_t scratch_bytes,
+                               int* passes, size_t* largest) {
+    if (!passes || !largest) return DSA3D_ERR_NULL_POINTER;
+    dsa3d::Problem pr;
+    const int rc = make_problem(T, H, W, heads, d, window, dtype, pr);
+    if (rc == DSA3D_OK) *passes = dsa3d::cells_passes(pr, scratch_bytes, largest);
+    return rc;
+}
+
 int dsa3d_debug_build(void) {
 #ifdef DSA3D_DEBUG
     return 1;

@@ -1051,10 +1051,13 @@ int floor_div4(int a) { return a >= 0 ? a / 4 : -((-a + 3) / 4); }
 
 size_t round256(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
 
-// Lays a slab's buffers out at `base` (may be NULL); returns their bytes.
+// Lays a slab's buffers out at `base` (may be NULL); returns their bytes.  They depend on how many heads and frames the slab has and
+// not on where its frames lie, and fewer need no more: a slab at the video's start has only one layer of blocks below
+// its tiles, one in the middle three, so room is taken for the most that any can have - three below and three above, and
+// no more than blocks of four cut the cells -1 .. T - 1 into wherever they begin.
 size_t lay_out(const Problem& pr, int m0, int heads, int f0, int f1, char* base, Slab& s) {
     s.m0 = m0; s.heads = heads; s.f0 = f0; s.f1 = f1;
-    s.tiles_t = (f1 - f0 + 3) / 4; s.tiles_y = (pr.H + 3) / 4; s.tiles_x = (pr.W + kTileX - 1) / kTileX;
+    s.tiles_t = (f1 - f0 - 1) / 4 + 1; s.tiles_y = (pr.H + 3) / 4; s.tiles_x = (pr.W + kTileX - 1) / kTileX;
     const int lo = floor_div4(-1 - f0), hi = floor_div4(pr.T - 1 - f0);
     s.bt0 = lo < -3 ? -3 : lo;
     const int top = s.tiles_t - 1 + 3 < hi ? s.tiles_t - 1 + 3 : hi;
@@ -1068,7 +1071,9 @@ size_t lay_out(const Problem& pr, int m0, int heads, int f0, int f1, char* base,
     s.geo = reinterpret_cast<uint4*>(base + at); at += round256(samples * sizeof(uint4));
     s.meta = reinterpret_cast<uint16_t*>(base + at); at += round256(samples * sizeof(uint16_t));
     s.seg = reinterpret_cast<uint32_t*>(base + at); at += round256(tiles * (kBins + 1) * sizeof(uint32_t));
-    const size_t blocks = static_cast<size_t>(heads) * s.blocks_t * s.blocks_y * s.blocks_x;
+    const int layers = s.tiles_t + 6 < (pr.T - 1) / 4 + 2 ? s.tiles_t + 6 : (pr.T - 1) / 4 + 2;
+    if (s.blocks_t > layers) return ~static_cast<size_t>(0);
+    const size_t blocks = static_cast<size_t>(heads) * layers * s.blocks_y * s.blocks_x;
     s.sorted = reinterpret_cast<float4*>(base + at); at += round256(live * sizeof(float4));
     s.place = reinterpret_cast<uint32_t*>(base + at); at += round256(live * sizeof(uint32_t));
     s.first = reinterpret_cast<uint32_t*>(base + at); at += round256(blocks * (kCells + 1) * sizeof(uint32_t));
@@ -1154,38 +1159,56 @@ cudaError_t launch_cells_choose(const float* offsets, long long samples, int* on
     return cudaGetLastError();
 }
 
-// Scratch the fp32 route asks for: the whole problem in one pass up to 1 GiB, passes of at most that beyond.
-size_t cells_scratch_bytes(const Problem& pr) {
-    int heads = pr.heads, frames = pr.T;
+// The heads and frames of a pass over `pr`'s heads and `frames` of its frames whose buffers fit `bytes`: divided by heads first
+// (they share nothing), then by frames.  Returns the bytes of the largest pass, 0 if the smallest does not fit.
+static size_t divide(const Problem& pr, size_t bytes, int& heads, int& frames) {
+    heads = pr.heads;
     Slab s;
-    size_t bytes;
-    while ((bytes = lay_out(pr, 0, heads, 0, frames, nullptr, s)) > (static_cast<size_t>(1) << 30)) {
+    size_t need;
+    while ((need = lay_out(pr, 0, heads, 0, frames, nullptr, s)) > bytes) {
         if (heads > 1) heads = (heads + 1) / 2;
         else if (frames > 4) frames = ((frames + 1) / 2 + 3) / 4 * 4;
         else return 0;
     }
-    return bytes;
+    return need;
 }
 
-// Splits the queries of `pr` (whole frames) into passes whose buffers fit `bytes`: by heads first (they share nothing),
-// then by frames.
+// Scratch the fp32 route asks for: the whole problem in one pass up to 1 GiB, passes of at most that beyond.
+size_t cells_scratch_bytes(const Problem& pr) {
+    int heads, frames = pr.T;
+    return divide(pr, static_cast<size_t>(1) << 30, heads, frames);
+}
+
+int cells_passes(const Problem& pr, size_t bytes, size_t* largest) {
+    *largest = 0;
+    int heads, frames = pr.T;
+    if (divide(pr, bytes, heads, frames) == 0) return 0;
+    Slab s;
+    int passes = 0;
+    for (int f = 0; f < pr.T; f += frames)
+        for (int m = 0; m < pr.heads; m += heads, ++passes) {
+            const int f1 = f + frames < pr.T ? f + frames : pr.T, mh = m + heads < pr.heads ? heads : pr.heads - m;
+            const size_t used = lay_out(pr, m, mh, f, f1, nullptr, s);
+            const uint32_t* first_end = s.first + static_cast<size_t>(mh) * s.blocks_t * s.blocks_y * s.blocks_x * (kCells + 1);
+            if (first_end > reinterpret_cast<const uint32_t*>(s.stats)) { *largest = ~static_cast<size_t>(0); return passes + 1; }
+            if (used > *largest) *largest = used;
+        }
+    return passes;
+}
+
 bool try_cells_backward(const void* q, const void* k, const void* v, const float* offsets, const float* lse, const void* dout, void* dq,
                         float* acc_dk, float* acc_dv, float* doffsets, void* scratch, size_t bytes, void* clear, size_t clear_bytes, const Problem& pr,
                         bool bf16_storage, cudaStream_t stream, cudaError_t* err) {
     *err = cudaSuccess;
     const long long frame = static_cast<long long>(pr.H) * pr.W;
     const int f_begin = static_cast<int>(pr.q_begin / frame), f_end = f_begin + static_cast<int>(pr.q_count / frame);
-    int heads = pr.heads, frames = f_end - f_begin;
+    int heads, frames = f_end - f_begin;
+    if (divide(pr, bytes, heads, frames) == 0) return false;
     Slab s;
-    while (lay_out(pr, 0, heads, f_begin, f_begin + frames, nullptr, s) > bytes) {
-        if (heads > 1) heads = (heads + 1) / 2;
-        else if (frames > 4) frames = ((frames + 1) / 2 + 3) / 4 * 4;
-        else return false;
-    }
     for (int f = f_begin; f < f_end; f += frames)
         for (int m = 0; m < pr.heads; m += heads) {
             const int f1 = f + frames < f_end ? f + frames : f_end, mh = m + heads < pr.heads ? heads : pr.heads - m;
-            lay_out(pr, m, mh, f, f1, static_cast<char*>(scratch), s);
+            if (lay_out(pr, m, mh, f, f1, static_cast<char*>(scratch), s) > bytes) { *err = cudaErrorInvalidValue; return true; }
             auto slab = !bf16_storage ? (pr.d == 128 ? launch_slab<float, 128, true> : pr.d == 64 ? launch_slab<float, 64, true> : launch_slab<float, 32, true>)
                         : pr.d == 128 ? (pr.gate ? launch_slab<bf16, 128, true> : launch_slab<bf16, 128, false>)
                         : pr.d == 64  ? (pr.gate ? launch_slab<bf16, 64, true> : launch_slab<bf16, 64, false>)

@@ -41,6 +41,9 @@ bool try_cells_backward(const void* q, const void* k, const void* v, const float
                         float* acc_dk, float* acc_dv, float* doffsets, void* scratch, size_t bytes, void* clear, size_t clear_bytes,
                         const Problem& pr, bool bf16_storage, cudaStream_t stream, cudaError_t* err);
 size_t cells_scratch_bytes(const Problem& pr);
+// Passes that try_cells_backward makes over all of `pr` with `bytes` of scratch (0: they do not suffice), and the most bytes
+// that one of them lays out.  Host only.
+int cells_passes(const Problem& pr, size_t bytes, size_t* largest);
 // fp32 storage: leaves 1 in one of two gate words and 0 in the other: whether the samples lie on grid positions (then the
 // row kernels are faster: they read and write only the one corner that has a weight) or not.
 cudaError_t launch_cells_choose(const float* offsets, long long samples, int* on_grid, int* off_grid, cudaStream_t stream);

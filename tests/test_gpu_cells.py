@@ -91,6 +91,38 @@ def test_fp32_storage_from_a_million_samples_on(d, window, shape, sigma, kind, m
             assert float((other - c).abs().max()) <= pu.F32_BWD_ATOL * scale, name
 
 
+@pytest.mark.parametrize("dtype,dims,window,scratch", [
+    (F32, (26, 40, 48, 1, 64), (3, 3, 3), 36 << 20),     # four passes, the last of two frames
+    (F32, (30, 24, 90, 1, 32), (4, 2, 2), 12 << 20),     # eight of four frames
+    (BF16, (64, 68, 120, 1, 32), (1, 1, 2), None),       # the workspace the library asks for
+])
+def test_passes_over_frames_stay_inside_the_workspace(dtype, dims, window, scratch):
+    """Passes in the middle of the video use the most scratch.  Bytes behind the workspace keep their pattern, and the gradients
+    are those of the row kernels (tolerances as in the tests around this one)."""
+    T, H, W, heads, d = dims
+    acc = 8 * T * H * W * heads * d if dtype == BF16 else 0
+    nbytes = scratch or binding.dsa3d_backward_workspace_bytes(*dims, window, dtype)
+    passes, largest = binding.dsa3d_test_backward_passes(*dims, window, dtype, nbytes - acc)
+    assert passes >= 3 and largest <= nbytes - acc
+    q, k, v, off, dout = (z.cuda() for z in small_problem(*dims, window, dtype, 1.5, 740 + T))
+    _, lse = pu.gpu_forward(q, k, v, off, dims, window)
+    guard = 4 << 20
+
+    def backward():
+        buf = torch.full((nbytes + guard,), 0xA5, dtype=torch.uint8, device="cuda")
+        g = [torch.full_like(z, float("nan")) for z in (q, q, q, off)]
+        binding.dsa3d_backward(q, k, v, off, lse, dout, *dims, window, *g, buf[:nbytes])
+        assert bool((buf[nbytes:] == 0xA5).all())
+        return g
+
+    got = backward()
+    with pytest.MonkeyPatch.context() as mp:
+        mp.setenv("DSA3D_TILE", "0")
+        want = backward()
+    for name, a, b in zip(("dq", "dk", "dv", "doffsets"), got, want):
+        pu.assert_close(name, a, b.cpu(), dtype, backward=True)
+
+
 @pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("window,shape", [((2, 2, 2), (3, 5, 7, 2)), ((3, 3, 3), (1, 4, 8, 3)), ((3, 5, 5), (3, 7, 11, 1)),
                                           ((3, 7, 7), (4, 9, 17, 2))])
