@@ -234,8 +234,8 @@ size_t dsa3d_backward_noalloc_max_elements(void);
 
 /*
  * Test aid: how the cell-sorted kernels of dsa3d_backward divide a problem when they are given `scratch_bytes` of
- * device memory (bf16: what the workspace holds behind the fp32 accumulators, 8 * T*H*W*heads*d bytes).  *passes: their
- * passes over heads and frames, 0 if the smallest does not fit; *largest: the most bytes any of them uses.
+ * device memory (what the workspace holds behind the fp32 accumulators, 8 * T*H*W*heads*d bytes, or, for fp32, behind its
+ * first 256 bytes).  *passes: their passes over heads and frames, 0 if the smallest does not fit; *largest: the most bytes any of them uses.
  * Host arithmetic only.
  */
 int dsa3d_test_backward_passes(int T, int H, int W, int heads, int d, const int window[3], int dtype,

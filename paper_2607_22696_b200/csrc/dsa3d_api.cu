@@ -103,11 +103,15 @@ struct BackwardWorkspace {
 // closed gates in front of them are all that is added: 0.02 to 0.03 ms, which is why the line lies above the first gains.
 constexpr int kF32CellsWindow = 16;
 constexpr long long kF32CellsSamples = 1000000;
+// The two gate words of that route stand at the front of its workspace: calls that do not share a workspace share nothing,
+// and a captured call can be replayed beside any others.
+constexpr size_t kF32GateBytes = 256;
 
 BackwardWorkspace backward_workspace(const dsa3d::Problem& pr, int dtype, bool tiled) {
     BackwardWorkspace w{};
     if (dtype != DSA3D_BF16) {                       // nothing that has to be there: see backward_plan
-        w.total = pr.P >= kF32CellsWindow && pr.items * pr.P >= kF32CellsSamples ? dsa3d::cells_scratch_bytes(pr) : 0;
+        const size_t cells = pr.P >= kF32CellsWindow && pr.items * pr.P >= kF32CellsSamples ? dsa3d::cells_scratch_bytes(pr) : 0;
+        w.total = cells ? kF32GateBytes + cells : 0;
         return w;
     }
     w.acc_bytes = static_cast<size_t>(pr.items) * pr.d * sizeof(float) * 2;
@@ -391,9 +395,9 @@ int backward_plan(int T, int H, int W, int heads, int d, const int* window, int 
         plan.cells = wsp + plan.ws.acc_bytes;
         plan.cells_bytes = workspace_bytes - plan.ws.acc_bytes;
     }
-    if (!plan.bf16 && plan.ws.total > 0 && workspace && aligned16(workspace) && !getenv("DSA3D_TILE")) {
-        plan.cells = workspace;
-        plan.cells_bytes = workspace_bytes;
+    if (!plan.bf16 && plan.ws.total > 0 && workspace && aligned16(workspace) && workspace_bytes > kF32GateBytes && !getenv("DSA3D_TILE")) {
+        plan.cells = wsp + kF32GateBytes;
+        plan.cells_bytes = workspace_bytes - kF32GateBytes;
     }
     if (plan.coef) {
         int dev = 0, sms = 0;
@@ -446,12 +450,9 @@ int backward_frames(const BackwardPlan& plan, const void* q, const void* k, cons
     cudaError_t e = record(2, stream);
     if (e != cudaSuccess) return cuda_failed(e);
     const int* rows_gate = pr.gate;
-    if (!plan.bf16 && plan.cells) {                  // both routes are queued, each behind its gate
-        void* words = nullptr;
-        e = cudaGetSymbolAddress(&words, g_gate_words);
-        if (e != cudaSuccess) return cuda_failed(e);
-        const unsigned next = g_next_gate.fetch_add(2u);
-        int *on_grid = static_cast<int*>(words) + next % kGateWords, *off_grid = static_cast<int*>(words) + (next + 1u) % kGateWords;
+    const bool cells = plan.cells && dsa3d::cells_fit(pr, plan.cells_bytes);
+    if (!plan.bf16 && cells) {                       // both routes are queued, each behind its gate
+        int *on_grid = static_cast<int*>(plan.workspace), *off_grid = on_grid + 1;
         e = dsa3d::launch_cells_choose(offsets + pr.q_begin * pr.heads * pr.P * 3, pr.items * pr.P, on_grid, off_grid, stream);
         if (e != cudaSuccess) return cuda_failed(e);
         rows_gate = on_grid;
@@ -462,8 +463,9 @@ int backward_frames(const BackwardPlan& plan, const void* q, const void* k, cons
         if (rc != DSA3D_OK) return rc;
         clear = false;
     }
-    if (plan.cells && dsa3d::try_cells_backward(q, k, v, offsets, lse, dout, dq, plan.acc_dk, plan.acc_dv, doffsets, plan.cells,
-                                                plan.cells_bytes, plan.workspace, clear ? plan.ws.acc_bytes : 0, pr, plan.bf16, stream, &e)) {
+    if (cells) {
+        e = dsa3d::launch_cells_backward(q, k, v, offsets, lse, dout, dq, plan.acc_dk, plan.acc_dv, doffsets, plan.cells,
+                                         plan.cells_bytes, plan.workspace, clear ? plan.ws.acc_bytes : 0, pr, plan.bf16, stream);
         if (e != cudaSuccess) return cuda_failed(e);
         if (!plan.bf16) {
             pr.gate = rows_gate;
@@ -482,7 +484,6 @@ int backward_frames(const BackwardPlan& plan, const void* q, const void* k, cons
         const int rc = backward_clear(plan, stream);
         if (rc != DSA3D_OK) return rc;
     }
-    pr.gate = plan.pr.gate;
     e = dsa3d::launch_backward(q, k, v, offsets, lse, dout, dq, plan.acc_dk, plan.acc_dv, doffsets, plan.coef, pr,
                                plan.bf16, stream);
     if (e != cudaSuccess) return cuda_failed(e);

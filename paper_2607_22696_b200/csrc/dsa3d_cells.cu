@@ -1196,28 +1196,33 @@ int cells_passes(const Problem& pr, size_t bytes, size_t* largest) {
     return passes;
 }
 
-bool try_cells_backward(const void* q, const void* k, const void* v, const float* offsets, const float* lse, const void* dout, void* dq,
-                        float* acc_dk, float* acc_dv, float* doffsets, void* scratch, size_t bytes, void* clear, size_t clear_bytes, const Problem& pr,
-                        bool bf16_storage, cudaStream_t stream, cudaError_t* err) {
-    *err = cudaSuccess;
-    const long long frame = static_cast<long long>(pr.H) * pr.W;
-    const int f_begin = static_cast<int>(pr.q_begin / frame), f_end = f_begin + static_cast<int>(pr.q_count / frame);
+static int frames_in(const Problem& pr) { return static_cast<int>(pr.q_count / (static_cast<long long>(pr.H) * pr.W)); }
+
+bool cells_fit(const Problem& pr, size_t bytes) {
+    int heads, frames = frames_in(pr);
+    return divide(pr, bytes, heads, frames) != 0;
+}
+
+cudaError_t launch_cells_backward(const void* q, const void* k, const void* v, const float* offsets, const float* lse, const void* dout, void* dq,
+                                  float* acc_dk, float* acc_dv, float* doffsets, void* scratch, size_t bytes, void* clear, size_t clear_bytes,
+                                  const Problem& pr, bool bf16_storage, cudaStream_t stream) {
+    const int f_begin = static_cast<int>(pr.q_begin / (static_cast<long long>(pr.H) * pr.W)), f_end = f_begin + frames_in(pr);
     int heads, frames = f_end - f_begin;
-    if (divide(pr, bytes, heads, frames) == 0) return false;
+    if (divide(pr, bytes, heads, frames) == 0) return cudaErrorInvalidValue;
     Slab s;
     for (int f = f_begin; f < f_end; f += frames)
         for (int m = 0; m < pr.heads; m += heads) {
             const int f1 = f + frames < f_end ? f + frames : f_end, mh = m + heads < pr.heads ? heads : pr.heads - m;
-            if (lay_out(pr, m, mh, f, f1, static_cast<char*>(scratch), s) > bytes) { *err = cudaErrorInvalidValue; return true; }
+            if (lay_out(pr, m, mh, f, f1, static_cast<char*>(scratch), s) > bytes) return cudaErrorInvalidValue;
             auto slab = !bf16_storage ? (pr.d == 128 ? launch_slab<float, 128, true> : pr.d == 64 ? launch_slab<float, 64, true> : launch_slab<float, 32, true>)
                         : pr.d == 128 ? (pr.gate ? launch_slab<bf16, 128, true> : launch_slab<bf16, 128, false>)
                         : pr.d == 64  ? (pr.gate ? launch_slab<bf16, 64, true> : launch_slab<bf16, 64, false>)
                                       : (pr.gate ? launch_slab<bf16, 32, true> : launch_slab<bf16, 32, false>);
-            *err = slab(q, k, v, offsets, lse, dout, dq, acc_dk, acc_dv, doffsets, pr, s, clear, clear_bytes, stream);
+            const cudaError_t e = slab(q, k, v, offsets, lse, dout, dq, acc_dk, acc_dv, doffsets, pr, s, clear, clear_bytes, stream);
             clear_bytes = 0;                                        // the first pass clears for all
-            if (*err != cudaSuccess) return true;
+            if (e != cudaSuccess) return e;
         }
-    return true;
+    return cudaSuccess;
 }
 
 }  // namespace dsa3d

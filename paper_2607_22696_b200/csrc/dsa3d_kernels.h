@@ -35,13 +35,13 @@ cudaError_t launch_scatter_tiles(const void* q, const void* dout, const float* o
 
 // The whole backward of the queries of `pr` (whole frames) on samples sorted by key cell (dsa3d_cells.cu): dq, doffsets, and
 // the contributions to the fp32 accumulators.  `scratch`: `bytes` of device memory, worked through in as many passes as
-// it takes; false: not even the smallest pass fits, nothing launched.  `clear_bytes` from `clear` on (the accumulators) are
-// zeroed first.
-bool try_cells_backward(const void* q, const void* k, const void* v, const float* offsets, const float* lse, const void* dout, void* dq,
-                        float* acc_dk, float* acc_dv, float* doffsets, void* scratch, size_t bytes, void* clear, size_t clear_bytes,
-                        const Problem& pr, bool bf16_storage, cudaStream_t stream, cudaError_t* err);
+// it takes (cells_fit: it does for the smallest pass).  `clear_bytes` from `clear` on (the accumulators) are zeroed first.
+cudaError_t launch_cells_backward(const void* q, const void* k, const void* v, const float* offsets, const float* lse, const void* dout, void* dq,
+                                  float* acc_dk, float* acc_dv, float* doffsets, void* scratch, size_t bytes, void* clear, size_t clear_bytes,
+                                  const Problem& pr, bool bf16_storage, cudaStream_t stream);
+bool cells_fit(const Problem& pr, size_t bytes);
 size_t cells_scratch_bytes(const Problem& pr);
-// Passes that try_cells_backward makes over all of `pr` with `bytes` of scratch (0: they do not suffice), and the most bytes
+// Passes that launch_cells_backward makes over all of `pr` with `bytes` of scratch (0: they do not suffice), and the most bytes
 // that one of them lays out.  Host only.
 int cells_passes(const Problem& pr, size_t bytes, size_t* largest);
 // fp32 storage: leaves 1 in one of two gate words and 0 in the other: whether the samples lie on grid positions (then the

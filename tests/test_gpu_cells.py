@@ -100,10 +100,10 @@ def test_passes_over_frames_stay_inside_the_workspace(dtype, dims, window, scrat
     """Passes in the middle of the video use the most scratch.  Bytes behind the workspace keep their pattern, and the gradients
     are those of the row kernels (tolerances as in the tests around this one)."""
     T, H, W, heads, d = dims
-    acc = 8 * T * H * W * heads * d if dtype == BF16 else 0
+    front = 8 * T * H * W * heads * d if dtype == BF16 else 256          # accumulators, or gate words
     nbytes = scratch or binding.dsa3d_backward_workspace_bytes(*dims, window, dtype)
-    passes, largest = binding.dsa3d_test_backward_passes(*dims, window, dtype, nbytes - acc)
-    assert passes >= 3 and largest <= nbytes - acc
+    passes, largest = binding.dsa3d_test_backward_passes(*dims, window, dtype, nbytes - front)
+    assert passes >= 3 and largest <= nbytes - front
     q, k, v, off, dout = (z.cuda() for z in small_problem(*dims, window, dtype, 1.5, 740 + T))
     _, lse = pu.gpu_forward(q, k, v, off, dims, window)
     guard = 4 << 20
@@ -121,6 +121,48 @@ def test_passes_over_frames_stay_inside_the_workspace(dtype, dims, window, scrat
         want = backward()
     for name, a, b in zip(("dq", "dk", "dv", "doffsets"), got, want):
         pu.assert_close(name, a, b.cpu(), dtype, backward=True)
+
+
+def test_a_captured_fp32_call_shares_nothing_with_calls_on_other_streams():
+    """The fp32 route is chosen on the device by the offsets.  A graph of a call with real-valued offsets, replayed on one stream
+    while more than 512 calls with integer ones run on another, gives what the call gives alone."""
+    window, dims = (3, 3, 3), (6, 32, 40, 5, 32)
+    q, k, v, off, dout = (z.cuda() for z in small_problem(*dims, window, F32, 1.5, 761))
+    grid = inputs.uniform_int(tuple(off.shape), 762, 3, -2, 2, F32).cuda()
+    nbytes = binding.dsa3d_backward_workspace_bytes(*dims, window, F32)
+    assert nbytes > 0
+    lse = {id(o): pu.gpu_forward(q, k, v, o, dims, window)[1] for o in (off, grid)}
+
+    class Call:
+        def __init__(self, offsets):
+            self.offsets, self.g = offsets, [torch.full_like(z, float("nan")) for z in (q, q, q, off)]
+            self.ws = torch.full((nbytes,), 0xFF, dtype=torch.uint8, device="cuda")
+
+        def __call__(self):
+            binding.dsa3d_backward(q, k, v, self.offsets, lse[id(self.offsets)], dout, *dims, window, *self.g, self.ws)
+
+        def check(self, want):
+            for name, a, b in zip(("dq", "dk", "dv", "doffsets"), self.g, want):
+                assert float((a - b).abs().max()) <= pu.F32_BWD_ATOL * max(1.0, float(b.abs().max())), name
+
+    alone = {}
+    for o in (off, grid):
+        c = Call(o)
+        c()
+        alone[id(o)] = c.g
+    captured, eager = Call(off), Call(grid)
+    torch.cuda.synchronize()
+    graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(graph):
+        captured()
+    with torch.cuda.stream(side):
+        for _ in range(600):
+            eager()
+    for _ in range(300):
+        graph.replay()
+        captured.check(alone[id(off)])
+    torch.cuda.synchronize()
+    eager.check(alone[id(grid)])
 
 
 @pytest.mark.parametrize("d", [64, 128])
