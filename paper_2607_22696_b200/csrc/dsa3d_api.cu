@@ -107,10 +107,17 @@ constexpr long long kF32CellsSamples = 1000000;
 // and a captured call can be replayed beside any others.
 constexpr size_t kF32GateBytes = 256;
 
+// Whether the queries of `pr` (the whole video or some frames of it) are enough for that route.  Its tiles are four frames
+// deep: fewer out of a longer video leave most of them empty.
+bool f32_cells(const dsa3d::Problem& pr) {
+    return pr.P >= kF32CellsWindow && pr.items * pr.P >= kF32CellsSamples &&
+           (pr.q_count == pr.N || pr.q_count >= 4ll * pr.H * pr.W);
+}
+
 BackwardWorkspace backward_workspace(const dsa3d::Problem& pr, int dtype, bool tiled) {
     BackwardWorkspace w{};
     if (dtype != DSA3D_BF16) {                       // nothing that has to be there: see backward_plan
-        const size_t cells = pr.P >= kF32CellsWindow && pr.items * pr.P >= kF32CellsSamples ? dsa3d::cells_scratch_bytes(pr) : 0;
+        const size_t cells = f32_cells(pr) ? dsa3d::cells_scratch_bytes(pr) : 0;
         w.total = cells ? kF32GateBytes + cells : 0;
         return w;
     }
@@ -395,7 +402,7 @@ int backward_plan(int T, int H, int W, int heads, int d, const int* window, int 
         plan.cells = wsp + plan.ws.acc_bytes;
         plan.cells_bytes = workspace_bytes - plan.ws.acc_bytes;
     }
-    if (!plan.bf16 && plan.ws.total > 0 && workspace && aligned16(workspace) && workspace_bytes > kF32GateBytes && !getenv("DSA3D_TILE")) {
+    if (!plan.bf16 && workspace && aligned16(workspace) && workspace_bytes > kF32GateBytes && !getenv("DSA3D_TILE")) {
         plan.cells = wsp + kF32GateBytes;
         plan.cells_bytes = workspace_bytes - kF32GateBytes;
     }
@@ -450,7 +457,7 @@ int backward_frames(const BackwardPlan& plan, const void* q, const void* k, cons
     cudaError_t e = record(2, stream);
     if (e != cudaSuccess) return cuda_failed(e);
     const int* rows_gate = pr.gate;
-    const bool cells = plan.cells && dsa3d::cells_fit(pr, plan.cells_bytes);
+    const bool cells = plan.cells && (plan.bf16 || f32_cells(pr)) && dsa3d::cells_fit(pr, plan.cells_bytes);
     if (!plan.bf16 && cells) {                       // both routes are queued, each behind its gate
         int *on_grid = static_cast<int*>(plan.workspace), *off_grid = on_grid + 1;
         e = dsa3d::launch_cells_choose(offsets + pr.q_begin * pr.heads * pr.P * 3, pr.items * pr.P, on_grid, off_grid, stream);
@@ -550,6 +557,14 @@ namespace {
 
 size_t round256(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
 
+constexpr int kMaxSlabs = 8;
+
+// Frames of a slab of dsa3d_step_host: at most kMaxSlabs of them, starting on tile boundaries where there are tiles.
+int step_slab_frames(const dsa3d::Problem& pr) {
+    const int unit = pr.tile_t >= 1 ? pr.tile_t : 1, frames = (pr.T - 1) / kMaxSlabs + 1;
+    return (frames + unit - 1) / unit * unit;
+}
+
 // Layout of the device arena of dsa3d_step_host: offsets of each buffer, total in `total`.
 struct Arena {
     size_t q, k, v, k2, v2, dout, out, dq, dk, dv, offsets, doffsets, lse, workspace, total;
@@ -563,9 +578,10 @@ Arena arena_layout(const dsa3d::Problem& pr, int dtype) {
     a.off_bytes = static_cast<size_t>(pr.items) * pr.P * 3 * sizeof(float);
     a.lse_bytes = static_cast<size_t>(pr.items) * sizeof(float);
     {
-        dsa3d::Problem tiled = pr;
-        if (dtype == DSA3D_BF16) set_tiling(tiled);
-        a.ws_bytes = backward_workspace(tiled, dtype, true).total;
+        dsa3d::Problem all = pr;
+        if (dtype == DSA3D_BF16) set_tiling(all);
+        const int slab = step_slab_frames(all);
+        a.ws_bytes = backward_workspace(dtype == DSA3D_BF16 || slab >= pr.T ? all : frames_of(all, 0, slab), dtype, true).total;
     }
     size_t at = 0;
     // K and V twice: the pipelined step uploads the next call's K/V while this call's kernels read theirs
@@ -581,7 +597,6 @@ Arena arena_layout(const dsa3d::Problem& pr, int dtype) {
 
 // Two side streams and the events of the copy/compute pipeline of dsa3d_step_host, per
 // (thread, device); created on first use and kept for the life of the thread.
-constexpr int kMaxSlabs = 8;
 struct HostStep {
     int device = -1;
     cudaStream_t in = nullptr, out = nullptr;
@@ -649,8 +664,11 @@ int step_host_body(const void* q_h, const void* k_h, const void* v_h, const floa
     const int rc = make_problem(T, H, W, heads, d, window, dtype, pr);
     if (rc != DSA3D_OK) return rc;
     if ((reinterpret_cast<uintptr_t>(arena) & 255u) != 0) return DSA3D_ERR_MISALIGNED;
-    const Arena a = arena_layout(pr, dtype);
-    if (arena_bytes < a.total) return DSA3D_ERR_WORKSPACE;
+    Arena a = arena_layout(pr, dtype);
+    if (dtype != DSA3D_BF16 && arena_bytes >= a.workspace && arena_bytes - a.workspace < a.ws_bytes)
+        a.ws_bytes = arena_bytes - a.workspace;          // fp32 does without, and the workspace comes last
+    else if (arena_bytes < a.total)
+        return DSA3D_ERR_WORKSPACE;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     char* base = static_cast<char*>(arena);
     HostStep* hs = host_step_resources();
@@ -672,9 +690,7 @@ int step_host_body(const void* q_h, const void* k_h, const void* v_h, const floa
     int st = backward_plan(T, H, W, heads, d, window, dtype, true, base + a.dk, base + a.dv,
                            a.ws_bytes ? base + a.workspace : nullptr, a.ws_bytes, plan);
     if (st != DSA3D_OK) return st;
-    const int unit = plan.pr.tile_t >= 1 ? plan.pr.tile_t : 1;          // slabs start on tile boundaries
-    int slab_frames = (T + kMaxSlabs - 1) / kMaxSlabs;
-    slab_frames = (slab_frames + unit - 1) / unit * unit;
+    const int slab_frames = step_slab_frames(plan.pr);
     const int slabs = (T + slab_frames - 1) / slab_frames;
     const size_t elt = bf16 ? 2 : 4;
     const size_t frame_rows = static_cast<size_t>(H) * W * heads;

@@ -1173,9 +1173,11 @@ static size_t divide(const Problem& pr, size_t bytes, int& heads, int& frames) {
     return need;
 }
 
-// Scratch the fp32 route asks for: the whole problem in one pass up to 1 GiB, passes of at most that beyond.
+static int frames_in(const Problem& pr) { return static_cast<int>(pr.q_count / (static_cast<long long>(pr.H) * pr.W)); }
+
+// Scratch the fp32 route asks for: all queries of `pr` in one pass up to 1 GiB, passes of at most that beyond.
 size_t cells_scratch_bytes(const Problem& pr) {
-    int heads, frames = pr.T;
+    int heads, frames = frames_in(pr);
     return divide(pr, static_cast<size_t>(1) << 30, heads, frames);
 }
 
@@ -1195,8 +1197,6 @@ int cells_passes(const Problem& pr, size_t bytes, size_t* largest) {
         }
     return passes;
 }
-
-static int frames_in(const Problem& pr) { return static_cast<int>(pr.q_count / (static_cast<long long>(pr.H) * pr.W)); }
 
 bool cells_fit(const Problem& pr, size_t bytes) {
     int heads, frames = frames_in(pr);

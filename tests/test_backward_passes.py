@@ -50,3 +50,17 @@ def test_every_pass_fits_whatever_scratch_it_is_given():
         assert largest <= scratch
         divided += passes > dims[3]
     assert divided > 300
+
+
+def test_fp32_host_step_asks_for_what_its_slabs_can_use():
+    """The host step runs by slabs of an eighth of the video.  Slabs too small to be sorted ask for no room to sort in."""
+    def extra(dims, window=(3, 3, 3)):
+        T, H, W, heads, d = dims
+        items, up = T * H * W * heads, lambda x: (x + 255) // 256 * 256
+        buffers = 10 * up(items * d * 4) + 2 * up(items * 27 * 12) + up(items * 4)
+        return binding.dsa3d_step_host_arena_bytes(*dims, window, F32) - buffers
+
+    assert extra((8, 30, 52, 8, 64)) == 0                    # slabs of one frame
+    assert extra((64, 12, 10, 8, 64)) == 0                   # of eight, 207,360 samples
+    whole = binding.dsa3d_backward_workspace_bytes(64, 30, 52, 8, 64, (3, 3, 3), F32)
+    assert 0 < extra((64, 30, 52, 8, 64)) < whole            # of eight, 2.7 million

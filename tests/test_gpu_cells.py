@@ -165,6 +165,31 @@ def test_a_captured_fp32_call_shares_nothing_with_calls_on_other_streams():
     eager.check(alone[id(grid)])
 
 
+@pytest.mark.parametrize("frames", [6, 34])             # slabs of one frame, and of five with enough samples to be sorted
+@pytest.mark.parametrize("old_arena", [False, True])
+def test_fp32_host_step_with_and_without_room_for_the_sort(frames, old_arena):
+    """The sort's workspace comes last in the arena and fp32 does without it: an arena that ends before it is taken too."""
+    window, dims = (3, 3, 3), (frames, 30, 52, 5, 32)
+    host = small_problem(*dims, window, F32, 1.5, 763)
+    q, k, v, off, dout = host
+    nbytes = binding.dsa3d_step_host_arena_bytes(*dims, window, F32)
+    buffers = sum((z.numel() * 4 + 255) // 256 * 256 * n for z, n in ((q, 10), (off, 2), (q[..., 0], 1)))
+    assert (nbytes > buffers) == (frames == 34) and nbytes >= buffers
+    if old_arena:
+        nbytes = buffers
+    hin = [z.clone().pin_memory() for z in host]
+    hout = [torch.full(z.shape, float("nan")).pin_memory() for z in (q, q[..., 0], q, k, v, off)]     # out, lse, dq, dk, dv, doffsets
+    buf = torch.full((nbytes + 4096,), 0xA5, dtype=torch.uint8, device="cuda")
+    binding.dsa3d_step_host(*hin, *dims, window, *hout, buf[:nbytes])
+    torch.cuda.synchronize()
+    assert bool((buf[nbytes:] == 0xA5).all())
+    dev = [z.cuda() for z in host]
+    out, lse = pu.gpu_forward(*dev[:4], dims, window)
+    want = (out, lse) + tuple(pu.gpu_backward(*dev[:4], lse, dev[4], dims, window))
+    for name, a, b in zip(("out", "lse", "dq", "dk", "dv", "doffsets"), hout, want):
+        assert float((a - b.cpu()).abs().max()) <= pu.F32_BWD_ATOL * max(1.0, float(b.abs().max())), name
+
+
 @pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("window,shape", [((2, 2, 2), (3, 5, 7, 2)), ((3, 3, 3), (1, 4, 8, 3)), ((3, 5, 5), (3, 7, 11, 1)),
                                           ((3, 7, 7), (4, 9, 17, 2))])
