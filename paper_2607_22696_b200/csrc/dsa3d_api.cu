@@ -471,8 +471,10 @@ int backward_frames(const BackwardPlan& plan, const void* q, const void* k, cons
         clear = false;
     }
     if (cells) {
+        // fp32: dq and doffsets may still come from the row kernels behind
         e = dsa3d::launch_cells_backward(q, k, v, offsets, lse, dout, dq, plan.acc_dk, plan.acc_dv, doffsets, plan.cells,
-                                         plan.cells_bytes, plan.workspace, clear ? plan.ws.acc_bytes : 0, pr, plan.bf16, stream);
+                                         plan.cells_bytes, plan.workspace, clear ? plan.ws.acc_bytes : 0, pr, plan.bf16, stream,
+                                         plan.bf16 ? after_gather : nullptr);
         if (e != cudaSuccess) return cuda_failed(e);
         if (!plan.bf16) {
             pr.gate = rows_gate;
@@ -481,7 +483,7 @@ int backward_frames(const BackwardPlan& plan, const void* q, const void* k, cons
         }
         e = record(3, stream);
         if (e != cudaSuccess) return cuda_failed(e);
-        if (after_gather) {
+        if (after_gather && !plan.bf16) {
             e = cudaEventRecord(after_gather, stream);
             if (e != cudaSuccess) return cuda_failed(e);
         }

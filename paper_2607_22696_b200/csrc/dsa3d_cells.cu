@@ -1089,7 +1089,8 @@ size_t lay_out(const Problem& pr, int m0, int heads, int f0, int f1, char* base,
 // empty chain 6 us more).
 template <typename T, int D, bool kGated>
 cudaError_t launch_slab(const void* q_, const void* k_, const void* v_, const float* offsets, const float* lse, const void* dout_, void* dq_,
-                        float* acc_dk, float* acc_dv, float* doffsets, const Problem& pr, const Slab& s, void* clear, size_t clear_bytes, cudaStream_t stream) {
+                        float* acc_dk, float* acc_dv, float* doffsets, const Problem& pr, const Slab& s, void* clear, size_t clear_bytes, cudaStream_t stream,
+                        cudaEvent_t queries_done) {
     constexpr bool kF32 = std::is_same<T, float>::value;
     const T *q = static_cast<const T*>(q_), *k = static_cast<const T*>(k_), *v = static_cast<const T*>(v_), *dout = static_cast<const T*>(dout_);
     const unsigned tiles = static_cast<unsigned>(s.heads * s.tiles_t * s.tiles_y * s.tiles_x), blocks = static_cast<unsigned>(s.heads * s.blocks_t * s.blocks_y * s.blocks_x);
@@ -1131,6 +1132,7 @@ cudaError_t launch_slab(const void* q_, const void* k_, const void* v_, const fl
     const unsigned per_head = static_cast<unsigned>((static_cast<long long>(s.f1 - s.f0) * pr.H * pr.W + per_block - 1) / per_block), query_blocks = per_head * static_cast<unsigned>(s.heads);
     auto query = share == 4 ? cells_query_kernel<T, D, 4, kGated> : share == 2 ? cells_query_kernel<T, D, 2, kGated> : cells_query_kernel<T, D, 1, kGated>;
     launch(query, grid(query_blocks, 12), kQueryWarps * 32, 0, k, offsets, lse, static_cast<T*>(dq_), doffsets, pr, s, per_head, query_blocks);
+    if (e == cudaSuccess && queries_done) e = cudaEventRecord(queries_done, stream);
     launch(sums, grid(blocks + far_parts, kF32 ? 1u << 20 : 2u), kF32 ? f32_threads : kSumThreads, sum_smem, q, dout, offsets, acc_dk, acc_dv, pr, s, blocks);
     return e;
 }
@@ -1205,7 +1207,7 @@ bool cells_fit(const Problem& pr, size_t bytes) {
 
 cudaError_t launch_cells_backward(const void* q, const void* k, const void* v, const float* offsets, const float* lse, const void* dout, void* dq,
                                   float* acc_dk, float* acc_dv, float* doffsets, void* scratch, size_t bytes, void* clear, size_t clear_bytes,
-                                  const Problem& pr, bool bf16_storage, cudaStream_t stream) {
+                                  const Problem& pr, bool bf16_storage, cudaStream_t stream, cudaEvent_t queries_done) {
     const int f_begin = static_cast<int>(pr.q_begin / (static_cast<long long>(pr.H) * pr.W)), f_end = f_begin + frames_in(pr);
     int heads, frames = f_end - f_begin;
     if (divide(pr, bytes, heads, frames) == 0) return cudaErrorInvalidValue;
@@ -1218,7 +1220,8 @@ cudaError_t launch_cells_backward(const void* q, const void* k, const void* v, c
                         : pr.d == 128 ? (pr.gate ? launch_slab<bf16, 128, true> : launch_slab<bf16, 128, false>)
                         : pr.d == 64  ? (pr.gate ? launch_slab<bf16, 64, true> : launch_slab<bf16, 64, false>)
                                       : (pr.gate ? launch_slab<bf16, 32, true> : launch_slab<bf16, 32, false>);
-            const cudaError_t e = slab(q, k, v, offsets, lse, dout, dq, acc_dk, acc_dv, doffsets, pr, s, clear, clear_bytes, stream);
+            const bool last = f1 == f_end && m + mh == pr.heads;
+            const cudaError_t e = slab(q, k, v, offsets, lse, dout, dq, acc_dk, acc_dv, doffsets, pr, s, clear, clear_bytes, stream, last ? queries_done : nullptr);
             clear_bytes = 0;                                        // the first pass clears for all
             if (e != cudaSuccess) return e;
         }

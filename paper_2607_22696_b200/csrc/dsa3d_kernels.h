@@ -36,9 +36,10 @@ cudaError_t launch_scatter_tiles(const void* q, const void* dout, const float* o
 // The whole backward of the queries of `pr` (whole frames) on samples sorted by key cell (dsa3d_cells.cu): dq, doffsets, and
 // the contributions to the fp32 accumulators.  `scratch`: `bytes` of device memory, worked through in as many passes as
 // it takes (cells_fit: it does for the smallest pass).  `clear_bytes` from `clear` on (the accumulators) are zeroed first.
+// `queries_done` (may be NULL) is recorded as soon as dq and doffsets are final, before the last sums of dk and dv.
 cudaError_t launch_cells_backward(const void* q, const void* k, const void* v, const float* offsets, const float* lse, const void* dout, void* dq,
                                   float* acc_dk, float* acc_dv, float* doffsets, void* scratch, size_t bytes, void* clear, size_t clear_bytes,
-                                  const Problem& pr, bool bf16_storage, cudaStream_t stream);
+                                  const Problem& pr, bool bf16_storage, cudaStream_t stream, cudaEvent_t queries_done);
 bool cells_fit(const Problem& pr, size_t bytes);
 size_t cells_scratch_bytes(const Problem& pr);
 // Passes that launch_cells_backward makes over all of `pr` with `bytes` of scratch (0: they do not suffice), and the most bytes
