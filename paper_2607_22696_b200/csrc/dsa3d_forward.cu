@@ -13,7 +13,7 @@
 // (gather_forward_small_kernel: the same for two or four items per warp where the window is small: 32 x 45 x 80, 16 heads of 128, window
 // (2,2,2): 3.83 -> 3.24 ms, integer offsets 1.25 -> 0.94 ms.)
 //
-// forward_kernel (fp32; bf16 with 32 channels and few samples): one group of LPR = d / VEC lanes owns one item; each lane holds VEC consecutive channels
+// forward_kernel (fp32; bf16 with 32 channels and few samples or 128 channels in long calls, see launch_forward): one group of LPR = d / VEC lanes owns one item; each lane holds VEC consecutive channels
 // (16 bytes) of every row it touches.  Per sample: the 8 corner rows of K and of V are loaded with 16-byte loads, the
 // logit is the weighted sum of the corner dot products, and the output is accumulated in fp32 registers.  A sample whose 8
 // corners are all inside the grid with non-zero weights (the usual case for real-valued offsets) takes a branch-free path
@@ -501,23 +501,33 @@ static cudaError_t launch_forward_t(const void* q, const void* k, const void* v,
     return cudaGetLastError();
 }
 
+// Calls from this many samples on last long enough for the card's power limit to set the clock.
+constexpr long long kPowerLimitedSamples = 300000000;
+
 cudaError_t launch_forward(const void* q, const void* k, const void* v, const float* offsets, const void* addend,
                            void* out, float* lse, const Problem& pr, bool bf16, cudaStream_t stream, const int* gate) {
-    // At 32 channels and up to 32 samples the row traffic is too small to pay for the list: 0.94 - 0.97x of the other kernel.
-    // Elsewhere (32 x 45 x 80, 16 heads of 128): window (2,2,2) 1.18x (integer offsets 1.34x), (3,3,3) 1.02 - 1.20x, 64 channels 1.08 -
-    // 1.14x; (3,7,7) 1.9x; grids of a few hundred tokens 1.7x.
-    const bool warp_per_item = bf16 && !(pr.d == 32 && pr.P <= 32);
-#define DSA3D_CASE(DD)                                                                                    \
-    case DD:                                                                                              \
-        return warp_per_item ? launch_gather_forward<DD>(q, k, v, offsets, addend, out, lse, pr, stream, gate)    \
-               : bf16 ? launch_forward_t<__nv_bfloat16, 32>(q, k, v, offsets, addend, out, lse, pr, stream, gate) \
-                      : launch_forward_t<float, DD>(q, k, v, offsets, addend, out, lse, pr, stream, gate);
-    switch (pr.d) {
-        DSA3D_CASE(32)
-        DSA3D_CASE(64)
-        DSA3D_CASE(128)
+    // Which bf16 calls a warp per item serves, and which the rows of forward_kernel (time by rows over time by a warp per item):
+    // 32 channels, up to 32 samples: the row traffic is too small to pay for the list (0.94 - 0.97); more samples 1.9 - 2.9.
+    // 64 channels, window (3,3,3): 1.14 - 1.36 on 8 x 45 x 80, 16 heads, 1.03 - 1.14 on 16 x 68 x 120, 32 heads, 0.97 - 1.03 on
+    // 64 x 68 x 120, the larger the offsets the more; integer offsets 1.03 - 0.85.
+    // 128 channels: window (2,2,2) 1.4, (3,3,3) 1.03 - 1.17 on 32 x 45 x 80, 16 heads, at the full clock.  But it draws more power, and
+    // in training steps back to back the clock follows: steps by rows over steps by a warp per item, offsets N(0, 2), 16 heads,
+    // 1.02 for 32 x 45 x 80, 0.996 for 64 x 45 x 80 x 24, 0.98 for 128 x 68 x 120 and for 256 x 68 x 120 (574 -> 561 ms, the forward
+    // itself 220 -> 209), so windows of 17 to 32 samples go by rows from kPowerLimitedSamples on.  More samples 1.0 - 1.9 (147: 9.8
+    // against 18.5 ms).
+    switch (bf16 ? pr.d : -pr.d) {
+        case 32:
+            return pr.P <= 32 ? launch_forward_t<__nv_bfloat16, 32>(q, k, v, offsets, addend, out, lse, pr, stream, gate)
+                              : launch_gather_forward<32>(q, k, v, offsets, addend, out, lse, pr, stream, gate);
+        case 64: return launch_gather_forward<64>(q, k, v, offsets, addend, out, lse, pr, stream, gate);
+        case 128:
+            return pr.P > 16 && pr.P <= 32 && pr.items * pr.P >= kPowerLimitedSamples && !gate
+                       ? launch_forward_t<__nv_bfloat16, 128>(q, k, v, offsets, addend, out, lse, pr, stream, gate)
+                       : launch_gather_forward<128>(q, k, v, offsets, addend, out, lse, pr, stream, gate);
+        case -32: return launch_forward_t<float, 32>(q, k, v, offsets, addend, out, lse, pr, stream, gate);
+        case -64: return launch_forward_t<float, 64>(q, k, v, offsets, addend, out, lse, pr, stream, gate);
+        case -128: return launch_forward_t<float, 128>(q, k, v, offsets, addend, out, lse, pr, stream, gate);
     }
-#undef DSA3D_CASE
     return cudaErrorInvalidValue;
 }
 
