@@ -44,8 +44,8 @@ int make_problem(int T, int H, int W, int heads, int d, const int* window, int d
     if (d != 32 && d != 64 && d != 128) return DSA3D_ERR_UNSUPPORTED;
     const long long P = static_cast<long long>(window[0]) * window[1] * window[2];
     if (P > 256) return DSA3D_ERR_UNSUPPORTED;
-    // one CUDA block covers at least 8 items, and the grid has at most 2^31 - 1 blocks
-    if (N * heads / 8 >= (1LL << 31) - 1) return DSA3D_ERR_BAD_SHAPE;
+    // a CUDA block of the kernels with a warp per item covers two items, and a grid has at most 2^31 - 1 blocks
+    if ((N + 1) / 2 * heads > (1LL << 31) - 1) return DSA3D_ERR_BAD_SHAPE;
     pr.T = T; pr.H = H; pr.W = W; pr.heads = heads; pr.d = d;
     pr.kt = window[0]; pr.kh = window[1]; pr.kw = window[2];
     pr.inv_kw = ((1u << 20) + static_cast<unsigned>(pr.kw) - 1u) / static_cast<unsigned>(pr.kw);

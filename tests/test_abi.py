@@ -60,6 +60,18 @@ def test_workspace_size(lib):
     assert lib.dsa3d_backward_workspace_bytes(4, 8, 8, 2, 48, win, 1) == 0      # rejected shape
 
 
+def test_problems_beyond_the_largest_grid_of_blocks_are_refused(lib):
+    """A warp per item, two warps per block: more than 2^32 - 2 items do not fit one launch."""
+    win = (ctypes.c_int * 3)(3, 3, 3)
+    a = 4096                                     # fake, aligned, never dereferenced
+
+    def forward(T, heads):
+        return lib.dsa3d_forward(a + 4, a, a, a, T, 1, 1, heads, 32, win, a, a, 1, None)      # misaligned: checked after the shape
+
+    assert forward(1 << 30, 4) == 2 and forward(1 << 22, 1024) == 2 and forward((1 << 20) - 1, 4096) == 2
+    assert forward((1 << 30) - 2, 4) == 4 and forward((1 << 22) - 2, 1024) == 4
+
+
 def test_forward_rejects_bad_arguments_without_launching(lib):
     win = (ctypes.c_int * 3)(3, 3, 3)
     a = 4096                                     # fake, aligned, never dereferenced
