@@ -69,7 +69,12 @@ class _Dsa3d(torch.autograd.Function):
         dq, dk, dv = torch.empty_like(q), torch.empty_like(q), torch.empty_like(q)
         doff = torch.empty_like(offsets)
         nbytes = binding.dsa3d_backward_workspace_bytes(T, H, W, heads, d, ctx.window, q.dtype)
-        ws = torch.empty(max(nbytes, 16), dtype=torch.uint8, device=q.device)
+        try:
+            ws = torch.empty(max(nbytes, 16), dtype=torch.uint8, device=q.device)
+        except torch.OutOfMemoryError:
+            if q.dtype != torch.float32:
+                raise
+            ws = None                                    # fp32 runs without the sort's room
         binding.dsa3d_backward(q, k, v, offsets, lse, dout, T, H, W, heads, d, ctx.window, dq, dk, dv, doff, ws)
         return dq, dk, dv, doff, (dout if ctx.has_residual else None), None
 

@@ -63,6 +63,17 @@ Tensor new_workspace(const Tensor& q, size_t bytes) {
     return at::empty({static_cast<int64_t>(bytes < 16 ? 16 : bytes)}, q.options().dtype(at::kByte));
 }
 
+// fp32 runs with any workspace or none: on a card too full for the sort's room it goes without, as it did before there was one.
+Tensor new_backward_workspace(const Tensor& q, const Shape& s) {
+    const size_t bytes = dsa3d_backward_workspace_bytes(s.T, s.H, s.W, s.heads, s.d, s.window, s.code);
+    if (s.code != DSA3D_F32) return new_workspace(q, bytes);
+    try {
+        return new_workspace(q, bytes);
+    } catch (const c10::OutOfMemoryError&) {
+        return Tensor();
+    }
+}
+
 struct Window { int64_t w[3]; };
 
 void save_window(AutogradContext* ctx, const int64_t* w) {
@@ -99,11 +110,11 @@ struct Dsa3d : torch::autograd::Function<Dsa3d> {
         const Shape s(q, w.w);
         const Tensor dout = grads[0].contiguous();
         Tensor dq = at::empty_like(q), dk = at::empty_like(q), dv = at::empty_like(q), doffsets = at::empty_like(offsets);
-        const Tensor ws = new_workspace(q, dsa3d_backward_workspace_bytes(s.T, s.H, s.W, s.heads, s.d, s.window, s.code));
+        const Tensor ws = new_backward_workspace(q, s);
         check(dsa3d_backward(q.data_ptr(), k.data_ptr(), v.data_ptr(), offsets.data_ptr<float>(), lse.data_ptr<float>(),
                              dout.data_ptr(), s.T, s.H, s.W, s.heads, s.d, s.window, dq.data_ptr(), dk.data_ptr(), dv.data_ptr(),
-                             doffsets.data_ptr<float>(), ws.data_ptr(), static_cast<size_t>(ws.numel()), s.code,
-                             c10::cuda::getCurrentCUDAStream().stream()));
+                             doffsets.data_ptr<float>(), ws.defined() ? ws.data_ptr() : nullptr,
+                             ws.defined() ? static_cast<size_t>(ws.numel()) : 0, s.code, c10::cuda::getCurrentCUDAStream().stream()));
         return {dq, dk, dv, doffsets, ctx->saved_data["residual"].toBool() ? dout : Tensor(), Tensor(), Tensor(), Tensor()};
     }
 };

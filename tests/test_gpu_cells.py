@@ -230,3 +230,30 @@ def test_autograd_takes_what_has_to_be_converted_and_raises_what_the_library_ref
     buf = torch.zeros(dout.numel() + 1, dtype=BF16, device="cuda")
     with pytest.raises(binding.Dsa3dError):              # a gradient off its 16-byte alignment, refused in the backward
         torch.autograd.grad(out, leaves, buf[1:].view(dout.shape))
+
+
+@pytest.mark.parametrize("contiguous", [True, False])    # the compiled function, and the one that converts
+def test_fp32_backward_on_a_card_too_full_for_the_sort(contiguous):
+    """The room to sort in is several times the tensors; where it does not fit, the row kernels run."""
+    window, dims = (3, 3, 3), (8, 30, 52, 8, 32)
+    q, k, v, off, dout = (z.cuda() for z in small_problem(*dims, window, F32, 1.5, 780))
+    if not contiguous:
+        q = q.transpose(1, 2).contiguous().transpose(1, 2)
+    leaves = [z.requires_grad_() for z in (q, k, v, off)]
+    want = torch.autograd.grad(ops.dsa3d(*leaves, window), leaves, dout)
+    nbytes = binding.dsa3d_backward_workspace_bytes(*dims, window, F32)
+    out = ops.dsa3d(*leaves, window)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    total = torch.cuda.get_device_properties(0).total_memory
+    room = torch.cuda.memory_reserved() + 3 * q.numel() * 4 + off.numel() * 4 + (64 << 20)
+    assert nbytes > 128 << 20
+    torch.cuda.set_per_process_memory_fraction(room / total)
+    try:
+        with pytest.raises(torch.OutOfMemoryError):
+            torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+        got = torch.autograd.grad(out, leaves, dout)
+    finally:
+        torch.cuda.set_per_process_memory_fraction(1.0)
+    for name, a, b in zip(("dq", "dk", "dv", "doffsets"), got, want):
+        assert float((a - b).abs().max()) <= pu.F32_BWD_ATOL * max(1.0, float(b.abs().max())), name
