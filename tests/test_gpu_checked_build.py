@@ -5,7 +5,8 @@ to be added to and every bin and scratch slot of the dK/dV pre-reduction is test
 extent of its tensor first; a violation would be recorded in a device word (and the access
 skipped: nothing traps).  The small parity cases run once through it: the results must match the
 oracle as in the normal build and the record must stay empty - on problems whose offsets reach far
-outside the grid, are NaN or infinite, on grids with extents of one, and through both dK/dV paths."""
+outside the grid, are NaN or infinite, on grids with extents of one, and through every route of the backward: samples
+sorted by key cell, the tile pre-reduction, and the gather kernel's own scatter."""
 import ctypes
 
 import pytest
@@ -50,21 +51,22 @@ def _violation(lib):
 CASES = [
     # (T, H, W, heads, d), window, dtype, sigma, what the offsets are made of
     ((4, 8, 8, 2, 32), (3, 3, 3), torch.float32, 0.5, "normal"),
-    ((5, 7, 9, 3, 128), (3, 3, 3), torch.bfloat16, 2.5, "normal"),       # the tile pre-reduction of dK/dV
+    ((5, 7, 9, 3, 128), (3, 3, 3), torch.bfloat16, 2.5, "normal"),
     ((4, 9, 10, 2, 64), (3, 5, 5), torch.bfloat16, 1.5, "normal"),
     ((1, 1, 40, 2, 128), (3, 3, 3), torch.bfloat16, 0.7, "normal"),      # extents of one
     ((4, 5, 6, 2, 32), (3, 3, 3), torch.float32, 1.0, "wild"),           # NaN, +-inf, 3e38, far outside
     ((5, 6, 7, 2, 64), (3, 3, 3), torch.bfloat16, 0.0, "integer"),       # positions exactly at -1 and at size
+    ((7, 32, 42, 4, 32), (3, 3, 3), torch.float32, 1.5, "normal"),       # enough samples for fp32 to be sorted
+    ((7, 32, 42, 4, 32), (3, 3, 3), torch.float32, 0.0, "integer"),      # as many, left to the gather kernel by their offsets
 ]
+# DSA3D_TILE: unset, tiles, no tiles (fp32 has no tiles)
+RUNS = [(c, t) for c in CASES for t in ([None, "4,8,8,6", "0"] if c[2] == torch.bfloat16 else [None, "0"])]
 
 
-@pytest.mark.parametrize("key_blocks", [False, True])
-@pytest.mark.parametrize("dims,window,dtype,sigma,kind", CASES)
-def test_parity_cases_leave_no_violation_in_the_checked_build(dims, window, dtype, sigma, kind, key_blocks, monkeypatch):
-    if key_blocks:
-        if dtype != torch.bfloat16 or dims[4] < 64:
-            pytest.skip("the key-block kernel takes bf16 rows of 64 or 128 channels")
-        monkeypatch.setenv("DSA3D_KEY_BLOCKS", "1")       # dK/dV on the tensor cores instead of the tile kernel
+@pytest.mark.parametrize("case,tile", RUNS)
+def test_parity_cases_leave_no_violation_in_the_checked_build(case, tile, monkeypatch):
+    dims, window, dtype, sigma, kind = case
+    monkeypatch.delenv("DSA3D_TILE", raising=False) if tile is None else monkeypatch.setenv("DSA3D_TILE", tile)
     lib = binding.load_checked_build()
     assert lib.dsa3d_debug_build() == 1 and binding.load().dsa3d_debug_build() == 0
     assert lib.dsa3d_debug_clear() == 0
