@@ -49,11 +49,13 @@
  *
  * Experiment switches.  A few environment variables, read on each call, select an alternative
  * kernel for the same result (they exist to measure one variant against another; none changes
- * what is computed beyond fp32 summation order):
+ * what is computed beyond fp32 summation order, and the 2^-17 noted at DSA3D_TILE):
  *   DSA3D_TILE="tt,ty,tx,halo"     dsa3d_backward (bf16) by the gather kernel and a tile kernel that pre-reduces dK/dV per
  *                                  tile of queries ("0" = no tiling, every contribution is an atomic add)
- *                                  instead of on samples sorted by key cell; also changes
- *                                  dsa3d_backward_workspace_bytes
+ *                                  instead of on samples sorted by key cell, whose dk and dv sums
+ *                                  take each coefficient as two bf16 numbers, 2^-17 of it off at most (here fp32; the
+ *                                  results are rounded to bf16, 2^-9); fp32: by the gather kernel alone;
+ *                                  also changes dsa3d_backward_workspace_bytes
  *   DSA3D_NO_TENSOR_FIXED_WINDOW   dsa3d_forward_fixed_window and dsa3d_forward_bounded_offsets use the general
  *                                  kernel, dsa3d_backward_bounded_offsets the kernels of dsa3d_backward;
  *                                  dsa3d_backward_fixed_window uses its per-row CUDA-core kernels only
@@ -108,7 +110,7 @@ int dsa3d_forward(const void* q, const void* k, const void* v, const float* offs
  * 16-byte aligned (bf16 storage: fp32 accumulators for dk and dv, then room in which the samples are
  * sorted by key cell, as many heads at a time as fit; may be NULL when that size is 0).  fp32 storage runs with any
  * workspace or none: what is given serves the sort, which makes large calls faster (1.4 times at 2.7 million samples
- * of 64 channels).
+ * of 64 channels).  Calls that may overlap need workspaces of their own.
  * Its contents on entry do not matter.  dk and dv are summed with floating-point atomics,
  * so their last bits can differ from run to run; dq, doffsets are deterministic.
  */
@@ -220,8 +222,9 @@ size_t dsa3d_forward_host_arena_bytes(int T, int H, int W, int heads, int d, con
  *     process that resets a device must not call this function on it again;
  *   - all calls share the one array, which keeps the previous call's contents; every call
  *     clears it on `stream` before use.  Two calls whose GPU work can overlap (different
- *     streams, or different threads on one device) race on it and give wrong dk/dv:
- *     serialise them.
+ *     streams, or different threads on one device) race on it: serialise them.  The array holds the
+ *     sums and, where it has room, the lists of samples that the kernels index with, so the race is
+ *     undefined behaviour and not only a wrong dk or dv.
  */
 #define DSA3D_NOALLOC_MAX_ELEMENTS (8u * 1024u * 1024u)
 int dsa3d_backward_noalloc(const void* q, const void* k, const void* v, const float* offsets,
@@ -250,8 +253,10 @@ int dsa3d_backward_noalloc_last_cuda_error(void);
  * cudaEvent_t handles created by the caller, or NULL.  While set (per calling thread),
  * dsa3d_forward records fwd_start / fwd_stop on its stream immediately around the forward
  * kernel, and dsa3d_backward records bwd_start / bwd_stop around its cell-sorted kernels or, where
- * those do not run (fp32, DSA3D_TILE), around its gather kernel and scatter_start / scatter_stop around
- * its tile scatter kernel (when that kernel runs), so a caller can time those kernels alone inside a longer step.  Pass NULLs to switch it off.
+ * those do not run (small fp32 calls, DSA3D_TILE), around its gather kernel and scatter_start / scatter_stop around
+ * its tile scatter kernel (when that kernel runs), so a caller can time those kernels alone inside a longer step.
+ * Large fp32 calls queue both and the offsets decide which works: bwd_start / bwd_stop enclose the two.  Pass NULLs to
+ * switch it off.
  */
 int dsa3d_set_profile_events(void* fwd_start, void* fwd_stop, void* bwd_start, void* bwd_stop,
                              void* scatter_start, void* scatter_stop);

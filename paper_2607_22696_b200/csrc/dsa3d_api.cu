@@ -97,10 +97,11 @@ struct BackwardWorkspace {
     long long entries_per_cta;
 };
 
-// fp32 storage: where the cell-sorted kernels are faster than the row kernels.  They cost seven launches more, and windows of
+// fp32 storage: where the cell-sorted kernels are faster than the row kernels.  They cost six launches more, and windows of
 // fewer samples fill the cells too thinly (64 channels, window (3,3,3): 166K samples 0.15 against 0.15 ms, 553K 0.31 against
 // 0.41, 2.7M 1.19 against 1.71; window (2,2,2) 400K 0.33 against 0.29).  On integer offsets the row kernels run and the
-// closed gates in front of them are all that is added: 0.02 to 0.03 ms, which is why the line lies above the first gains.
+// closed gates in front of them are all that is added: 0.03 ms at 1.2M samples, 0.07 at 6.2M (0.90 - 0.98 of the row kernels alone; real-
+// valued offsets gain 1.2 - 1.6), which is why the line lies above the first gains.
 constexpr int kF32CellsWindow = 16;
 constexpr long long kF32CellsSamples = 1000000;
 // The two gate words of that route stand at the front of its workspace: calls that do not share a workspace share nothing,

@@ -6,6 +6,7 @@ through the autograd wrappers; there is no PyTorch fallback.
 Q, K and V are inputs (their projections from X are dense layers outside this operator).  The
 offset predictor's linear layer starts at zero, so a fresh module attends over the fixed
 window (the zero-offset variant of the paper's ablation) and learns its deformation from there.
+With fp32 tensors the backward allocates up to 1 GiB of scratch while it runs (see dsa3d_backward_workspace_bytes).
 """
 from __future__ import annotations
 
