@@ -146,3 +146,27 @@ def test_cpu_baseline_sample_is_an_exact_crop_of_the_workload():
     for name, got, ref in (("out", out_c, out_f.view(-1, heads, d)[tok]), ("lse", lse_c, lse_f.view(-1, heads)[tok]),
                            ("dq", dq_c, dq_f.view(-1, heads, d)[tok]), ("doffsets", doff_c, doff_f.view(-1, heads, P, 3)[tok])):
         assert float((got - ref).abs().max()) <= 1e-5 * max(float(ref.abs().max()), 1.0), name
+
+
+def test_routes_and_launch_counts_follow_the_library(monkeypatch):
+    """What bench.py says runs: fp32 problems large enough for the sort queue both chains and their offsets decide; the passes are
+    the library's own count."""
+    import dataclasses
+    import bench
+    from paper_2607_22696_b200 import binding, build, inputs
+    build.build()
+    monkeypatch.delenv("DSA3D_TILE", raising=False)
+    small = inputs.WORKLOADS["tiny_f32"]
+    assert bench.backward_route(small, False, False) == "rows" and bench.launches_per_step(small, False, False) == 2
+    large = dataclasses.replace(small, T=8, H=30, W=52, heads=8, d=64)
+    dims = (large.T, large.H, large.W, large.heads, large.d)
+    assert bench.backward_route(large, False, False) == "cells"
+    assert bench.backward_route(dataclasses.replace(large, offsets="int"), False, False) == "rows"
+    passes = binding.dsa3d_test_backward_passes(*dims, large.window, large.dtype, bench.workspace_bytes(large) - 256)[0]
+    assert passes == 1 and bench.launches_per_step(large, False, False) == 1 + 1 + 5 + 1
+    big = inputs.WORKLOADS["1080p_256f_bf16"]
+    assert bench.forward_route(big) == "forward_kernel" and bench.forward_route(dataclasses.replace(big, T=16)) == "gather_forward_kernel"
+    assert bench.cells_passes(big) == 16 and bench.launches_per_step(big, False, False) == 1 + 5 * 16 + 1
+    monkeypatch.setenv("DSA3D_TILE", "0")
+    assert bench.backward_route(large, False, False) == bench.backward_route(big, False, False) == "rows"
+    assert bench.launches_per_step(large, False, False) == 2
