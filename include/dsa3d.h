@@ -49,13 +49,11 @@
  *
  * Experiment switches.  A few environment variables, read on each call, select an alternative
  * kernel for the same result (they exist to measure one variant against another; none changes
- * what is computed beyond fp32 summation order, and the 2^-17 noted at DSA3D_TILE):
+ * what is computed beyond fp32 summation order):
  *   DSA3D_TILE="tt,ty,tx,halo"     dsa3d_backward (bf16) by the gather kernel and a tile kernel that pre-reduces dK/dV per
  *                                  tile of queries ("0" = no tiling, every contribution is an atomic add)
- *                                  instead of on samples sorted by key cell, whose dk and dv sums
- *                                  take each coefficient as two bf16 numbers, 2^-17 of it off at most (here fp32; the
- *                                  results are rounded to bf16, 2^-9); fp32: by the gather kernel alone;
- *                                  also changes dsa3d_backward_workspace_bytes
+ *                                  instead of on samples sorted by key cell; fp32: by the gather
+ *                                  kernel alone; also changes dsa3d_backward_workspace_bytes
  *   DSA3D_NO_TENSOR_FIXED_WINDOW   dsa3d_forward_fixed_window and dsa3d_forward_bounded_offsets use the general
  *                                  kernel, dsa3d_backward_bounded_offsets the kernels of dsa3d_backward;
  *                                  dsa3d_backward_fixed_window uses its per-row CUDA-core kernels only

@@ -3,7 +3,7 @@
 // A sample reads (and its gradient writes) the eight corner rows of the grid cell it falls into.  All samples of a cell,
 // whichever query they belong to, share those eight rows.  So the samples are first sorted by key cell: then the dot
 // products of 16 samples with their eight corners are one m16n8k16 product chain (16 query rows x 8 key rows), the
-// dK / dV contributions of 16 samples another (8 corners, head and remainder of the weights, x 16 query rows), and the
+// dK / dV contributions of 16 samples another (corners, the weights in three bf16 parts, x 16 query rows), and the
 // row traffic per sample falls from eight key rows to one query row.  Nothing depends on how far the offsets reach.
 // (The groups are 16 samples of one cell, so the warp-level product is the one that fits: a tcgen05 tile would hold
 // 128 rows of which a cell fills 27.)

@@ -64,8 +64,7 @@ def test_zero_integer_and_dead_offsets(route):
 
 @pytest.mark.parametrize("dims", [(10, 14, 18, 3, 128), (7, 9, 22, 2, 64), (5, 12, 13, 3, 32)])
 def test_routes_agree(dims, monkeypatch):
-    """The routes sum the same fp32 terms in other orders (the sorted one with weights that keep 16 bits); rounded to bf16 two
-    results are at most one step apart, 2^-7 of a value or, near zero, of the tensor's size.  doffsets stays fp32: 54 dot
+    """The routes sum the same fp32 terms in other orders; rounded to bf16 two results are at most one step apart, 2^-7 of a value or, near zero, of the tensor's size.  doffsets stays fp32: 54 dot
     products of 128 terms at 2^-24 each, far below 1e-4."""
     window = (3, 3, 3)
     q, k, v, off, dout = small_problem(*dims, window, BF16, 2.0, 930)
@@ -83,6 +82,34 @@ def test_routes_agree(dims, monkeypatch):
         a, b = got["cells"][3], got[other][3]
         assert float((a - b).abs().max()) <= 1e-4 * max(1.0, float(b.abs().max()))
     assert torch.equal(got["tiles"][0], got["rows"][0]) and torch.equal(got["tiles"][3], got["rows"][3])      # the same gather kernel
+
+
+@pytest.mark.parametrize("d", [32, 64, 128])
+def test_weights_of_dv_keep_their_32_bits(d, route):
+    """Pairs of queries sample almost the same position with opposite dO: a key's dV is the difference of two weights in
+    (0, 1) that agree in 15 to 18 bits.  Grid positions below 8 leave fractions of 2^-21, so the weights are exact in fp32
+    (lse 0, one sample: alpha is 1) and only their products and the sum round: 2^-23 of |dO| <= 2 each, twice, beside
+    the rounding of the result, 2^-9 of it."""
+    T, H, W, heads = 3, 6, 8, 2
+    g = torch.Generator().manual_seed(951)
+    q = torch.zeros(T, H, W, heads, d, dtype=BF16)
+    k, v = (torch.randn(q.shape, generator=g).to(BF16) for _ in range(2))
+    dout = torch.randn(T, H, W // 2, 1, heads, d, generator=g).clamp_(-2, 2).to(BF16)
+    dout = torch.cat([dout, -dout], dim=3).view(q.shape).contiguous()
+    f = torch.randint(100000, 2000000, (T, H, W // 2, heads), generator=g)
+    near = f + torch.randint(8, 64, f.shape, generator=g)
+    frac = torch.stack([f, near], dim=3).view(T, H, W, heads).double() * 2.0 ** -21
+    x = torch.arange(W).view(1, 1, W, 1)
+    off = torch.zeros(T, H, W, heads, 1, 3)
+    off[..., 0, 2] = ((x // 2 * 2).double() + frac - x).float()
+    assert torch.equal(x.float() + off[..., 0, 2], ((x // 2 * 2).double() + frac).float())
+    dims = (T, H, W, heads, d)
+    dev = [z.cuda() for z in (q, k, v, off, dout)]
+    out, lse = pu.gpu_forward(*dev[:4], dims, (1, 1, 1))
+    dv = pu.gpu_backward(*dev[:4], lse, dev[4], dims, (1, 1, 1))[2].cpu().double()
+    ref = oracle.backward(q, k, v, off, dout, T, H, W, heads, d, (1, 1, 1))[2].view(q.shape)
+    assert float(ref.abs().max()) > 2.0 ** -17
+    assert bool(((dv - ref).abs() <= ref.abs() * 2.0 ** -8 + 2.0 ** -21).all())
 
 
 @pytest.mark.parametrize("shape", [(19, 9, 10, 2, 128), (6, 10, 12, 3, 64)])
