@@ -388,8 +388,8 @@ int dsa3d_forward_residual(const void* q, const void* k, const void* v, const fl
  * d = 64 or 128 it runs as dense tile attention on the tensor cores: windows (3,3,3) and (2,2,2)
  * with the scores of a 4x4x8 query tile against its whole halo region in one tcgen05 tile, window
  * mask, softmax and the weighted sum from shared memory; windows (3,5,5) and (3,7,7) (the paper's
- * own) one region plane at a time with the weighted sum on the tensor cores too, each fp32 weight
- * entering as a bf16 head plus a bf16 remainder.  Every other supported shape runs the general
+ * own) one region plane at a time, x-row by x-row, with the weighted sum on the tensor cores too, each
+ * fp32 weight entering as a bf16 head plus a bf16 remainder.  Every other supported shape runs the general
  * kernel with zero offsets.  The environment variable DSA3D_NO_TENSOR_FIXED_WINDOW forces the
  * general kernel.  The backward of this variant is dsa3d_backward with a zero offsets
  * tensor.  Bounded waits as in dsa3d_offsets_linear_forward (dsa3d_device_timeout_flag).
@@ -404,9 +404,9 @@ int dsa3d_forward_fixed_window(const void* q, const void* k, const void* v, int 
  * summation order).  A first kernel checks the offsets tensor; if every component is finite and below 1
  * in size, every corner of every sample lies in the box "window grown by one position on each side" and
  * the operator runs as dense tile attention on the tensor cores for bf16, d = 64 or 128 and window (3,3,3):
- * scores of a 4x4x8 query tile against its region by tcgen05, plane by plane; each logit the trilinear
- * combination of eight entries of the score tile; the softmax weights times the corner weights summed
- * per box position; the weighted sum as a second tcgen05 product (weights as bf16 head + remainder).
+ * scores of a 4x4x8 query tile against its region, plane by plane; each logit the trilinear combination
+ * of eight scores of the query's box; the softmax weights times the corner weights summed per box
+ * position; the weighted sum as a second product (weights as bf16 head + remainder).
  * Otherwise - some offset too large, or another shape - the general kernel runs, so the call is correct
  * for any offsets; the decision is taken on the device, the call stays asynchronous.  Calls that are in
  * flight at the same time each use their own gate word (out of 1024).  The environment variable
