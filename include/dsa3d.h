@@ -151,7 +151,10 @@ int dsa3d_backward_batch(const void* q, const void* k, const void* v, const floa
  * and the backward workspace; the library allocates no memory.  The step is pipelined over
  * slabs of whole frames: K and V go up first, then each slab's q, offsets and dout while
  * earlier slabs compute, and each slab's out, lse, dq and doffsets come back while later
- * slabs compute; dk and dv follow the last slab.  This uses two side streams the library
+ * slabs compute; dk and dv follow the last slab.  Tensors of 8 MB and more in page-locked
+ * memory, with heads for at least four groups of 512 bytes per token, go by groups of heads
+ * instead, by strided copies: heads share nothing, so K, V, dk and dv of a group too move
+ * while other groups compute.  This uses two side streams the library
  * creates on the calling thread's first call (with a few dozen events; they are kept for
  * the life of the thread); everything is ordered after the work
  * already in `stream`, and the step is complete when `stream` is.  The host buffers must
@@ -175,8 +178,8 @@ int dsa3d_step_host(const void* q_h, const void* k_h, const void* v_h, const flo
  * pipelined call has been flushed.  Results of call i are final on the host no later than that.
  * The arena must not be in use by other work queued in `stream` (the uploads do not wait for it).
  * A call whose arena, shape or dtype differs from the previous one first waits for all of the
- * previous call.  dsa3d_step_host is this call followed by the flush, with the uploads ordered
- * after `stream`.  dsa3d_step_host_flush makes `stream` wait for every transfer the calling
+ * previous call.  dsa3d_step_host by slabs of frames is this call followed by the flush, with the
+ * uploads ordered after `stream`.  dsa3d_step_host_flush makes `stream` wait for every transfer the calling
  * thread's earlier steps queued.
  */
 int dsa3d_step_host_pipelined(const void* q_h, const void* k_h, const void* v_h, const float* offsets_h,

@@ -653,6 +653,107 @@ size_t dsa3d_step_host_arena_bytes(int T, int H, int W, int heads, int d, const 
 
 namespace {
 
+// dsa3d_step_host takes the video by groups of heads where there are enough of them: heads share nothing, so that only the first group's
+// upload and the last one's results are not hidden behind other copies and kernels, K, V, dK and dV included.  Strided copies into buffers
+// that hold the groups one after the other: rows of 1 KB where that leaves four groups, or of 512 bytes (copies both ways at once 46 GB/s
+// each for 512 bytes, 37 for 256).  Steps by frames and by groups of 512 bytes and of 1 KB: 8 x 45 x 80, 16 heads of 128, 20.8, 17.1 and
+// 16.3 ms; 12 heads of 128 on 12 x 45 x 80 22.9 and 18.3; 32 heads of 64 36.7, 31.1 and 30.6; 4 x 30 x 52, 16 heads of 64 (13 MB a
+// tensor) 3.35 and 2.49; fp32, 8 heads of 64, 10.9 and 9.3.  Heads per group; 0: too few heads, or too little to copy.
+constexpr size_t kGroupLeastBytes = size_t(8) << 20;
+int step_group_heads(const dsa3d::Problem& pr, size_t row_bytes) {
+    if (row_bytes < kGroupLeastBytes) return 0;
+    const size_t head_bytes = row_bytes / (static_cast<size_t>(pr.N) * pr.heads);
+    for (size_t bytes : {size_t(1024), size_t(512)}) {
+        int group = static_cast<int>((bytes + head_bytes - 1) / head_bytes);
+        if (group < (pr.heads + kMaxSlabs - 1) / kMaxSlabs) group = (pr.heads + kMaxSlabs - 1) / kMaxSlabs;
+        if (pr.heads > 3 * group) return group;
+    }
+    return 0;
+}
+
+int step_host_heads(const dsa3d::Problem& pr, int group, const void* q_h, const void* k_h, const void* v_h, const float* offsets_h, const void* dout_h,
+                    const int window[3], void* out_h, float* lse_h, void* dq_h, void* dk_h, void* dv_h, float* doffsets_h, char* base, const Arena& a,
+                    int dtype, HostStep* hs, cudaStream_t stream) {
+    cudaError_t e;
+#define DSA3D_TRY(call)                         \
+    do {                                        \
+        e = (call);                             \
+        if (e != cudaSuccess) return cuda_failed(e); \
+    } while (0)
+    const bool bf16 = dtype == DSA3D_BF16;
+    const size_t elt = bf16 ? 2 : 4, N = static_cast<size_t>(pr.N);
+    // whatever pipelined steps may still have in flight comes first, and a later one shares no ordering per slab with this call
+    DSA3D_TRY(cudaStreamWaitEvent(stream, hs->out_done, 0));
+    DSA3D_TRY(cudaStreamWaitEvent(stream, hs->main_done, 0));
+    hs->last_arena = nullptr;
+    DSA3D_TRY(cudaEventRecord(hs->start, stream));
+    DSA3D_TRY(cudaStreamWaitEvent(hs->in, hs->start, 0));
+    DSA3D_TRY(cudaStreamWaitEvent(hs->out, hs->start, 0));
+    struct Group { int m0, heads; char *q, *k, *v, *dout, *out, *dq, *dk, *dv; float *offsets, *doffsets, *lse; };
+    Group groups[kMaxSlabs];
+    int count = 0;
+    size_t at = 0;                                       // the second pair of K and V buffers leaves room for the rounding
+    auto take = [&](size_t bytes) { char* p = base + at; at += round256(bytes); return p; };
+    for (int m0 = 0; m0 < pr.heads; m0 += group) {
+        Group& g = groups[count++];
+        g.m0 = m0;
+        g.heads = pr.heads - m0 < group ? pr.heads - m0 : group;
+        const size_t items = N * g.heads, rows = items * pr.d * elt, offs = items * pr.P * 3 * sizeof(float);
+        for (char** p : {&g.q, &g.k, &g.v, &g.dout, &g.out, &g.dq, &g.dk, &g.dv}) *p = take(rows);
+        g.offsets = reinterpret_cast<float*>(take(offs));
+        g.doffsets = reinterpret_cast<float*>(take(offs));
+        g.lse = reinterpret_cast<float*>(take(items * sizeof(float)));
+    }
+    if (at > a.workspace) return DSA3D_ERR_WORKSPACE;
+    // a group's part of a host tensor of `head_bytes` per (token, head)
+    auto up = [&](void* dst, const void* src, size_t head_bytes, const Group& g) {
+        return cudaMemcpy2DAsync(dst, g.heads * head_bytes, static_cast<const char*>(src) + g.m0 * head_bytes, pr.heads * head_bytes, g.heads * head_bytes, N, cudaMemcpyHostToDevice, hs->in);
+    };
+    auto down = [&](void* dst, const void* src, size_t head_bytes, const Group& g) {
+        return cudaMemcpy2DAsync(static_cast<char*>(dst) + g.m0 * head_bytes, pr.heads * head_bytes, src, g.heads * head_bytes, g.heads * head_bytes, N, cudaMemcpyDeviceToHost, hs->out);
+    };
+    const size_t row = pr.d * elt, off = pr.P * 3 * sizeof(float);
+    for (int i = 0; i < count; ++i) {
+        const Group& g = groups[i];
+        DSA3D_TRY(up(g.k, k_h, row, g));
+        DSA3D_TRY(up(g.v, v_h, row, g));
+        DSA3D_TRY(up(g.q, q_h, row, g));
+        DSA3D_TRY(up(g.offsets, offsets_h, off, g));
+        DSA3D_TRY(cudaEventRecord(hs->q_ready[i], hs->in));
+        DSA3D_TRY(up(g.dout, dout_h, row, g));
+        DSA3D_TRY(cudaEventRecord(hs->dout_ready[i], hs->in));
+    }
+    for (int i = 0; i < count; ++i) {
+        const Group& g = groups[i];
+        BackwardPlan plan;
+        int st = backward_plan(pr.T, pr.H, pr.W, g.heads, pr.d, window, dtype, true, g.dk, g.dv, a.ws_bytes ? base + a.workspace : nullptr, a.ws_bytes, plan);
+        if (st != DSA3D_OK) return st;
+        DSA3D_TRY(cudaStreamWaitEvent(stream, hs->q_ready[i], 0));
+        st = forward_frames(plan.pr, g.q, g.k, g.v, g.offsets, g.out, g.lse, bf16, 0, pr.T, stream);
+        if (st != DSA3D_OK) return st;
+        DSA3D_TRY(cudaEventRecord(hs->fwd_done[i], stream));
+        DSA3D_TRY(cudaStreamWaitEvent(hs->out, hs->fwd_done[i], 0));
+        DSA3D_TRY(down(out_h, g.out, row, g));
+        DSA3D_TRY(down(lse_h, g.lse, sizeof(float), g));
+        DSA3D_TRY(cudaStreamWaitEvent(stream, hs->dout_ready[i], 0));
+        st = backward_frames(plan, g.q, g.k, g.v, g.offsets, g.lse, g.dout, g.dq, g.doffsets, 0, pr.T, true, stream, hs->gather_done[i]);
+        if (st != DSA3D_OK) return st;
+        st = backward_finish(plan, g.dk, g.dv, stream);
+        if (st != DSA3D_OK) return st;
+        DSA3D_TRY(cudaEventRecord(hs->slab_in_free[i], stream));
+        DSA3D_TRY(cudaStreamWaitEvent(hs->out, hs->gather_done[i], 0));
+        DSA3D_TRY(down(dq_h, g.dq, row, g));
+        DSA3D_TRY(down(doffsets_h, g.doffsets, off, g));
+        DSA3D_TRY(cudaStreamWaitEvent(hs->out, hs->slab_in_free[i], 0));
+        DSA3D_TRY(down(dk_h, g.dk, row, g));
+        DSA3D_TRY(down(dv_h, g.dv, row, g));
+    }
+    DSA3D_TRY(cudaEventRecord(hs->main_done, stream));
+    DSA3D_TRY(cudaEventRecord(hs->out_done, hs->out));
+#undef DSA3D_TRY
+    return DSA3D_OK;
+}
+
 // One step enqueued on `stream_` and the two side streams.  ordered_start: uploads wait for the
 // work already on the stream (the plain entry point); otherwise only for the buffers they
 // overwrite, so that they overlap the previous call's kernels (the pipelined entry point).
@@ -676,6 +777,21 @@ int step_host_body(const void* q_h, const void* k_h, const void* v_h, const floa
     char* base = static_cast<char*>(arena);
     HostStep* hs = host_step_resources();
     if (!hs) return cuda_failed(cudaGetLastError());     // side streams / events could not be created
+    // (strided copies from and to memory that is not page-locked are staged row by row)
+    auto locked = [](const void* p) {
+        cudaPointerAttributes at;
+        if (cudaPointerGetAttributes(&at, p) == cudaSuccess) return at.type == cudaMemoryTypeHost;
+        cudaGetLastError();
+        return false;
+    };
+    const int group = ordered_start ? step_group_heads(pr, a.row_bytes) : 0;
+    if (group) {
+        const void* host[] = {q_h, k_h, v_h, offsets_h, dout_h, out_h, lse_h, dq_h, dk_h, dv_h, doffsets_h};
+        bool all = true;
+        for (const void* p : host) all = all && locked(p);
+        if (all)
+            return step_host_heads(pr, group, q_h, k_h, v_h, offsets_h, dout_h, window, out_h, lse_h, dq_h, dk_h, dv_h, doffsets_h, base, a, dtype, hs, stream);
+    }
     cudaError_t e;
 #define DSA3D_TRY(call)                         \
     do {                                        \
