@@ -1305,11 +1305,10 @@ cudaError_t launch_wgrad(const void* x, const void* dy, float* dweight, float* d
 // src [rows, cols] (row pitch lds) -> dstT [cols, rows] bf16 (row pitch ldt, a multiple of 8); when
 // `dst` is given also the untransposed bf16 copy (row pitch ldd, a multiple of 8: whole words are
 // written, the padding columns included), and when `colsum` is given the fp32 column sums of src
-// (one atomic per column and block).  A block owns a 64-column strip of up to kTrRowsPerBlock
+// (one atomic per column and block).  A block owns a 64-column strip of up to rows_per_block
 // rows and walks it in 64 x 64 tiles through shared memory; a thread moves pairs: two
 // neighbouring columns on the way in, two neighbouring rows on the way out, so every warp
 // access is 128 contiguous bytes (256 for fp32 sources).
-constexpr int kTrRowsPerBlock = 1024;
 template <typename S> struct SrcPair;
 template <> struct SrcPair<float> {
     static __device__ __forceinline__ float2 load(const float* p, bool vec, bool second) {
@@ -1331,13 +1330,13 @@ template <typename S>
 __global__ void __launch_bounds__(256)
 transpose_to_bf16_kernel(const S* __restrict__ src, long long lds, long long rows, int cols,
                          __nv_bfloat16* __restrict__ dstT, long long ldt, __nv_bfloat16* __restrict__ dst, long long ldd,
-                         float* __restrict__ colsum) {
+                         float* __restrict__ colsum, int rows_per_block) {
     __shared__ uint32_t tile[64][33];                                // [row][column pair]
     __shared__ float sums[8][64];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;          // 32 pairs x 8 phases
     const int c0 = blockIdx.x * 64;
-    const long long rb = static_cast<long long>(blockIdx.y) * kTrRowsPerBlock;
-    const long long re = rb + kTrRowsPerBlock < rows ? rb + kTrRowsPerBlock : rows;
+    const long long rb = static_cast<long long>(blockIdx.y) * rows_per_block;
+    const long long re = rb + rows_per_block < rows ? rb + rows_per_block : rows;
     const int c = c0 + 2 * tx;
     const bool in0 = c < cols, in1 = c + 1 < cols;
     // a pair is one aligned vector when the row pitch keeps pairs aligned and both columns exist
@@ -1387,14 +1386,14 @@ transpose_to_bf16_kernel(const S* __restrict__ src, long long lds, long long row
 }
 
 // fp32 [rows, cols] -> bf16 copy (row pitch ldd) plus fp32 column sums, for cols a multiple of 4:
-// a thread owns four neighbouring columns and walks down kCvtRows rows, so a block reads whole
-// rows front to back (one contiguous stream per block) and issues one atomic per column.
-constexpr int kCvtRows = 512;
+// a thread owns four neighbouring columns and walks down rows_per_block rows, so a block reads whole
+// rows front to back (one contiguous stream per block) and issues one atomic per column.  Bound by memory, given
+// enough blocks (rows_per_block).
 __global__ void __launch_bounds__(1024)
 convert_rows_bf16_kernel(const float* __restrict__ src, long long rows, int cols, __nv_bfloat16* __restrict__ dst,
-                         long long ldd, float* __restrict__ colsum) {
-    const long long rb = static_cast<long long>(blockIdx.x) * kCvtRows;
-    const long long re = rb + kCvtRows < rows ? rb + kCvtRows : rows;
+                         long long ldd, float* __restrict__ colsum, int rows_per_block) {
+    const long long rb = static_cast<long long>(blockIdx.x) * rows_per_block;
+    const long long re = rb + rows_per_block < rows ? rb + rows_per_block : rows;
     for (int c = threadIdx.x * 4; c < cols; c += blockDim.x * 4) {
         float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
         const float* sp = src + rb * cols + c;
@@ -1414,6 +1413,14 @@ convert_rows_bf16_kernel(const float* __restrict__ src, long long rows, int cols
             atomicAdd(colsum + c + 3, sum.w);
         }
     }
+}
+
+// Rows of a block of the two kernels above: 512, and fewer (a multiple of 64) where those would be less than three blocks per SM.  Blocks of 512
+// rows leave a call of 24,960 tokens, 1296 outputs, a third of the SMs: conversion 210 -> 56 us with 64.  On 262,144 tokens 320 rows
+// were no faster than 512 (whole linear-layer backward 2.78 and 2.69 ms).
+int rows_per_block(long long rows) {
+    const long long each = rows / (148 * 3) / 64 * 64;
+    return static_cast<int>(each < 64 ? 64 : each > 512 ? 512 : each);
 }
 
 // fp32 storage: plain loops, one thread per output element.
@@ -1681,25 +1688,25 @@ int dsa3d_offsets_linear_backward(const void* u, const void* w, const float* dof
     if (dw && (e = cudaMemsetAsync(dw, 0, static_cast<size_t>(O) * C * sizeof(float), st)) != cudaSuccess) return cuda_failed(e);
     if (dbias && (e = cudaMemsetAsync(dbias, 0, static_cast<size_t>(O) * sizeof(float), st)) != cudaSuccess) return cuda_failed(e);
     if (du) {                                                        // w [O, C] -> w^T [C, O]
-        const dim3 grid((C + 63) / 64, static_cast<unsigned>((O + kTrRowsPerBlock - 1) / kTrRowsPerBlock));
+        const dim3 grid((C + 63) / 64, static_cast<unsigned>((O + 63) / 64));
         transpose_to_bf16_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(w), C, O, C, wt,
-                                                                      plan.ld_o, nullptr, 0, nullptr);
+                                                                      plan.ld_o, nullptr, 0, nullptr, 64);
         if ((e = cudaGetLastError()) != cudaSuccess) return cuda_failed(e);
     }
     bool unsupported = false;
     for (long long s0 = 0; s0 < tokens; s0 += plan.slab) {
         const long long ns = tokens - s0 < plan.slab ? tokens - s0 : plan.slab;
-        const unsigned row_blocks = static_cast<unsigned>((ns + kTrRowsPerBlock - 1) / kTrRowsPerBlock);
+        const int rows = rows_per_block(ns);
+        const unsigned row_blocks = static_cast<unsigned>((ns + rows - 1) / rows);
         if (O % 4 == 0) {   // doffsets slab -> bf16 copy and column sums
             int threads = ((O / 4 + 31) / 32) * 32;
             if (threads > 1024) threads = 1024;
-            convert_rows_bf16_kernel<<<static_cast<unsigned>((ns + kCvtRows - 1) / kCvtRows), threads, 0, st>>>(
-                doffsets + s0 * O, ns, O, g, plan.ld_o, dbias);
+            convert_rows_bf16_kernel<<<row_blocks, threads, 0, st>>>(doffsets + s0 * O, ns, O, g, plan.ld_o, dbias, rows);
             if ((e = cudaGetLastError()) != cudaSuccess) return cuda_failed(e);
         } else {            // rows that do not start on a 16-byte boundary: the pairwise kernel
             const dim3 grid((O + 63) / 64, row_blocks);
             transpose_to_bf16_kernel<float><<<grid, 256, 0, st>>>(doffsets + s0 * O, O, ns, O, nullptr, 0, g, plan.ld_o,
-                                                                  dbias);
+                                                                  dbias, rows);
             if ((e = cudaGetLastError()) != cudaSuccess) return cuda_failed(e);
         }
         if (du) {                                                    // du[slab] = g . (w^T)^T
