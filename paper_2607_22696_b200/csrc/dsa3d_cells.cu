@@ -565,7 +565,12 @@ constexpr int kQueryWarps = 2;
 // in the forward (dsa3d_gather.cuh).  A sample with anything that is not finite (its rows of q, dO, K or V, or its
 // coefficients) is marked by the sign of cv: its contributions to dK and dV are formed one by one, so that they reach only
 // the corners with a weight.  Windows of at most 8 (16) samples: G = 4 (2) neighbouring queries share a warp.
-template <typename T, int D, int G>
+// Bound by the latency of the row loads at 32 warps an SM (60 % of the data pipe and of the issue slots), so what an item does before its
+// first row counts: the statistics are asked for beside the offsets (backward 0.5 - 2.4 % faster), and windows of at most 32 samples have
+// an instance of one round (kOne), which keeps nothing for a next one.  Backward, window (3,3,3), 16 x 68 x 120, 16 heads: 128 channels
+// 21.9 -> 20.0 ms, 64 channels 15.1 -> 13.4; (2,2,2), integer offsets, 16 x 45 x 80: 4.00 -> 3.92 ms; (3,7,7) 16.8 -> 16.3 ms (8 x 68 x 120,
+// 6 heads).  (Rows of the next batch ahead of the sums, or the first rows ahead of the statistics: with one round 2 % slower, for registers.)
+template <typename T, int D, int G, bool kOne>
 __device__ __forceinline__ void query_block(const unsigned block, const T* __restrict__ k, const float* __restrict__ offsets, const float* __restrict__ lse, T* __restrict__ dq,
                    float* __restrict__ doffsets, const Problem& pr, const Slab& sl, unsigned blocks_per_head) {
     __shared__ GatherList lists[kQueryWarps];
@@ -591,17 +596,17 @@ __device__ __forceinline__ void query_block(const unsigned block, const T* __res
         s.base = 0; s.mask = 0u; s.ft = s.fy = s.fx = 0.0f;
         a = b = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         if (p >= pr.P) return;
-        s = to_sample(pr, make_cell(pr, t, y, x, p, off_row + p * 3));
-        if (s.mask == 0u) return;                   // a dead sample has g = 0
+        // asked for beside the offsets, not behind them; what stands there for a dead sample is not used (it has g = 0)
         a = __ldg(reinterpret_cast<const float4*>(st_row + p * 8));
         b = __ldg(reinterpret_cast<const float4*>(st_row + p * 8) + 1);
+        s = to_sample(pr, make_cell(pr, t, y, x, p, off_row + p * 3));
     };
     auto weight = [&](float sv) { return exp2f(fmaf(sv, scale * kLog2e, -lse2)); };
     Sample s;
     float4 a, b;
     sample(gl_lane, s, a, b);
     float delta = s.mask ? weight(a.x) * b.x : 0.0f;
-    for (int p = gl_lane + L; p < pr.P; p += L) {   // (one sample per lane when G > 1)
+    for (int p = gl_lane + L; !kOne && p < pr.P; p += L) {
         Sample s2;
         float4 a2, b2;
         sample(p, s2, a2, b2);
@@ -611,9 +616,9 @@ __device__ __forceinline__ void query_block(const unsigned block, const T* __res
     float acc[CH];
 #pragma unroll
     for (int e = 0; e < CH; ++e) acc[e] = 0.0f;
-    for (int pb = 0; pb < pr.P; pb += L) {
+    for (int pb = 0; kOne ? pb == 0 : pb < pr.P; pb += L) {
         const int p = pb + gl_lane;
-        if (pb > 0) sample(p, s, a, b);
+        if (!kOne && pb > 0) sample(p, s, a, b);
         float ck = 0.0f, d0 = 0.0f, d1 = 0.0f, d2 = 0.0f;
         if (s.mask != 0u) {
             const float alpha = weight(a.x);
@@ -664,16 +669,16 @@ __device__ __forceinline__ void query_block(const unsigned block, const T* __res
     }
 }
 
-template <typename T, int D, int G, bool kGated>
+template <typename T, int D, int G, bool kOne, bool kGated>
 __global__ void __launch_bounds__(kQueryWarps * 32, 16)
 cells_query_kernel(const T* __restrict__ k, const float* __restrict__ offsets, const float* __restrict__ lse, T* __restrict__ dq,
                    float* __restrict__ doffsets, const __grid_constant__ Problem pr, const __grid_constant__ Slab sl, unsigned blocks_per_head, unsigned blocks) {
     if constexpr (!kGated) {
-        query_block<T, D, G>(blockIdx.x, k, offsets, lse, dq, doffsets, pr, sl, blocks_per_head);
+        query_block<T, D, G, kOne>(blockIdx.x, k, offsets, lse, dq, doffsets, pr, sl, blocks_per_head);
     } else {
         if (gated_off_early(pr.gate)) return;
         for (unsigned block = blockIdx.x; block < blocks; block += gridDim.x) {
-            query_block<T, D, G>(block, k, offsets, lse, dq, doffsets, pr, sl, blocks_per_head);
+            query_block<T, D, G, kOne>(block, k, offsets, lse, dq, doffsets, pr, sl, blocks_per_head);
             __syncthreads();
         }
     }
@@ -1140,7 +1145,7 @@ cudaError_t launch_slab(const void* q_, const void* k_, const void* v_, const fl
     // As many queries per warp as have a lane for every sample.
     const int share = pr.P <= 8 ? 4 : pr.P <= 16 ? 2 : 1, per_block = kQueryWarps * share;
     const unsigned per_head = static_cast<unsigned>((static_cast<long long>(s.f1 - s.f0) * pr.H * pr.W + per_block - 1) / per_block), query_blocks = per_head * static_cast<unsigned>(s.heads);
-    auto query = share == 4 ? cells_query_kernel<T, D, 4, kGated> : share == 2 ? cells_query_kernel<T, D, 2, kGated> : cells_query_kernel<T, D, 1, kGated>;
+    auto query = share == 4 ? cells_query_kernel<T, D, 4, true, kGated> : share == 2 ? cells_query_kernel<T, D, 2, true, kGated> : pr.P <= 32 ? cells_query_kernel<T, D, 1, true, kGated> : cells_query_kernel<T, D, 1, false, kGated>;
     launch(query, grid(query_blocks, 12), kQueryWarps * 32, 0, k, offsets, lse, static_cast<T*>(dq_), doffsets, pr, s, per_head, query_blocks);
     if (e == cudaSuccess && queries_done) e = cudaEventRecord(queries_done, stream);
     launch(sums, grid(blocks + far_parts, kF32 ? 1u << 20 : 2u), kF32 ? f32_threads : kSumThreads, sum_smem, q, dout, offsets, acc_dk, acc_dv, pr, s, blocks);
