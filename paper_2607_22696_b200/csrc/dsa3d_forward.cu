@@ -85,8 +85,12 @@ __device__ __forceinline__ unsigned sm_neighbours(unsigned block, unsigned block
     return (wave + 1u) * kWave <= blocks ? wave * kWave + (r % kSms) * kRun + r / kSms : block;
 }
 
-template <int D, bool kAdd, bool kGated>
-__global__ void __launch_bounds__(kFwdWarps * 32, 16)
+// Bound by the L1 data pipe (87 % at 128 channels, 80 % at 64).  Windows of 17 to 32 samples have an instance of one round (kOne), which
+// keeps nothing for a next one: window (3,3,3), 16 x 68 x 120, 16 heads of 128, N(0, 1.5) 11.72 -> 10.92 ms, 16 x 45 x 80 integer offsets
+// 1.54 -> 1.26 ms, N(0, 0.5) 5.68 -> 5.57, N(0, 3) 4.63 -> 4.24; 64 channels 6.65 -> 6.56 ms, and 6.32 with 20 CTAs per SM (48
+// registers; 24 CTAs, 40 registers: 6.61; 128 channels with 18: 11.3).
+template <int D, bool kAdd, bool kGated, bool kOne>
+__global__ void __launch_bounds__(kFwdWarps * 32, D == 64 && kOne && !kGated ? 20 : 16)
 gather_forward_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v,
                       const float* __restrict__ offsets, const __nv_bfloat16* addend, __nv_bfloat16* out, float* __restrict__ lse,
                       const __grid_constant__ Problem pr, unsigned blocks_per_head, const int* __restrict__ gate) {
@@ -113,7 +117,7 @@ _Pragma("unroll 1")
 #pragma unroll
         for (int e = 0; e < 8; ++e) acc[e] = 0.0f;
         float m_run = -INFINITY, l_run = 0.0f;               // l_run: the lane's part
-        for (int pb = 0; pb < pr.P; pb += 32) {
+        for (int pb = 0; kOne ? pb == 0 : pb < pr.P; pb += 32) {
             const bool have = pb + lane < pr.P;
             Sample s;
             GatherQuery<D> qr;                               // on its way while the samples are listed
@@ -134,7 +138,9 @@ _Pragma("unroll 1")
             float mx = sp;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(kFullMask, mx, o));
-            if (mx > m_run) {
+            if (kOne) {
+                m_run = mx;
+            } else if (mx > m_run) {
                 const float corr = exp2f(m_run - mx);
                 l_run *= corr;
 #pragma unroll
@@ -563,17 +569,16 @@ static cudaError_t launch_gather_forward(const void* q, const void* k, const voi
         return cudaGetLastError();
     }
     if (gate)
-        gather_forward_kernel<D, false, true><<<blocks, kFwdWarps * 32, 0, stream>>>(
+        gather_forward_kernel<D, false, true, false><<<blocks, kFwdWarps * 32, 0, stream>>>(
             static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v), offsets, nullptr, static_cast<T*>(out), lse, pr,
             static_cast<unsigned>(per_head), gate);
-    else if (addend)
-        gather_forward_kernel<D, true, false><<<blocks, kFwdWarps * 32, 0, stream>>>(
-            static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v), offsets, static_cast<const T*>(addend),
-            static_cast<T*>(out), lse, pr, static_cast<unsigned>(per_head), gate);
-    else
-        gather_forward_kernel<D, false, false><<<blocks, kFwdWarps * 32, 0, stream>>>(
-            static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v), offsets, nullptr, static_cast<T*>(out), lse, pr,
-            static_cast<unsigned>(per_head), gate);
+    else {
+        auto kern = addend ? gather_forward_kernel<D, true, false, false> : gather_forward_kernel<D, false, false, false>;
+        if constexpr (D > 32)                            // (32 channels come here with more samples only)
+            if (pr.P <= 32) kern = addend ? gather_forward_kernel<D, true, false, true> : gather_forward_kernel<D, false, false, true>;
+        kern<<<blocks, kFwdWarps * 32, 0, stream>>>(static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v), offsets, static_cast<const T*>(addend),
+                                                    static_cast<T*>(out), lse, pr, static_cast<unsigned>(per_head), gate);
+    }
     return cudaGetLastError();
 }
 
@@ -612,11 +617,11 @@ cudaError_t launch_forward(const void* q, const void* k, const void* v, const fl
     // 32 channels, up to 32 samples: the row traffic is too small to pay for the list (0.94 - 0.97); more samples 1.9 - 2.9.
     // 64 channels, window (3,3,3): 1.14 - 1.36 on 8 x 45 x 80, 16 heads, 1.03 - 1.14 on 16 x 68 x 120, 32 heads, 0.97 - 1.03 on
     // 64 x 68 x 120, the larger the offsets the more; integer offsets 1.03 - 0.85.
-    // 128 channels: window (2,2,2) 1.4, (3,3,3) 1.03 - 1.17 on 32 x 45 x 80, 16 heads, at the full clock.  But it draws more power, and
-    // in training steps back to back the clock follows: steps by rows over steps by a warp per item, offsets N(0, 2), 16 heads,
-    // 1.02 for 32 x 45 x 80, 0.996 for 64 x 45 x 80 x 24, 0.98 for 128 x 68 x 120 and for 256 x 68 x 120 (574 -> 561 ms, the forward
-    // itself 220 -> 209), so windows of 17 to 32 samples go by rows from kPowerLimitedSamples on.  More samples 1.0 - 1.9 (147: 9.8
-    // against 18.5 ms).
+    // 128 channels: window (2,2,2) 1.4, (3,3,3) 1.03 - 1.17 on 32 x 45 x 80, 16 heads, at the full clock, before the
+    // instance of one round that is 2 - 8 % faster.  But it draws more power, and
+    // in calls of 0.1 s and more the clock follows: forward of 128 x 68 x 120, 16 heads, by rows 98, 105 and 116 ms for offsets N(0, 0.5),
+    // N(0, 2) and N(0, 3), by a warp per item 105, 102 and 111 (training steps 1.03, 0.993 and 0.98 of those by rows), so windows of 17 to 32
+    // samples go by rows from kPowerLimitedSamples on.  More samples 1.0 - 1.9 (147: 9.8 against 18.5 ms).
     switch (bf16 ? pr.d : -pr.d) {
         case 32:
             return pr.P <= 32 ? launch_forward_t<__nv_bfloat16, 32>(q, k, v, offsets, addend, out, lse, pr, stream, gate)
