@@ -638,7 +638,7 @@ static cudaError_t launch_backward_t(const void* q, const void* k, const void* v
                                      float* acc_dv, float* doffsets, float2* coef, const Problem& pr,
                                      cudaStream_t stream) {
     if constexpr (std::is_same<T, float>::value) {
-        if (split_items(pr, kSplitBackwardLanes) && pr.tile_t < 1) {
+        if (split_items(pr) && pr.tile_t < 1) {
             backward_split_kernel<D><<<static_cast<unsigned>(pr.items), kSplitThreads, static_cast<size_t>(pr.P) * 8 * sizeof(float), stream>>>(
                 static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v), offsets, lse, static_cast<const T*>(dout), static_cast<T*>(dq), acc_dk, acc_dv, doffsets, pr);
             return cudaGetLastError();

@@ -565,9 +565,10 @@ constexpr int kQueryWarps = 2;
 // in the forward (dsa3d_gather.cuh).  A sample with anything that is not finite (its rows of q, dO, K or V, or its
 // coefficients) is marked by the sign of cv: its contributions to dK and dV are formed one by one, so that they reach only
 // the corners with a weight.  Windows of at most 8 (16) samples: G = 4 (2) neighbouring queries share a warp.
-// Bound by the latency of the row loads at 32 warps an SM (60 % of the data pipe and of the issue slots), so what an item does before its
-// first row counts: the statistics are asked for beside the offsets (backward 0.5 - 2.4 % faster), and windows of at most 32 samples have
-// an instance of one round (kOne), which keeps nothing for a next one.  Backward, window (3,3,3), 16 x 68 x 120, 16 heads: 128 channels
+// Bound by the data pipe (81 %) and the issue slots (71 %), for more samples by the latency of the row loads (59 % of both): what an item
+// does before its first row counts, and what it holds.  The statistics are asked for beside the offsets (backward 0.5 - 2.4 % faster), and
+// windows of at most 32 samples have an instance of one round (kOne), which keeps nothing for a next one (this kernel 0.52 -> 0.40 ms on
+// 141,440 items of 128 channels, 0.35 -> 0.24 of 64, where 21 CTAs fit an SM then).  Backward, window (3,3,3), 16 x 68 x 120, 16 heads: 128 channels
 // 21.9 -> 20.0 ms, 64 channels 15.1 -> 13.4; (2,2,2), integer offsets, 16 x 45 x 80: 4.00 -> 3.92 ms; (3,7,7) 16.8 -> 16.3 ms (8 x 68 x 120,
 // 6 heads).  (Rows of the next batch ahead of the sums, or the first rows ahead of the statistics: with one round 2 % slower, for registers.)
 template <typename T, int D, int G, bool kOne>

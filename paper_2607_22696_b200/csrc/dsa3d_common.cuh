@@ -426,17 +426,16 @@ __device__ __forceinline__ void red_add_v4(float* addr, float a, float b, float 
                  : "memory");
 }
 
-// fp32 calls too small to fill the chip by rows run with a CTA per item (forward_split_kernel, backward_split_kernel).  The lines are in
-// lanes, d / 4 an item: up to half a block of 128 an SM for the forward, one for the backward, whose items are twice as deep.
-// Of the whole problem, not of the frames that a launch takes: a step in slabs of frames gives the bits of one launch.
-// Rows -> split in us, (3,3,3), offsets N(0, 1) | integer offsets, whose rows skip the corners of weight zero:
+// fp32 calls too small to fill the chip by rows run with a CTA per item (forward_split_kernel, backward_split_kernel).  The line is in the
+// lanes of a head's tokens, d / 4 each: neither how many heads a call has nor how many frames a launch takes changes the bits of a head.
+// Rows -> split in us, (3,3,3), offsets N(0, 1) | integer offsets, whose rows skip the corners of weight zero, by lanes of all heads:
 //     lanes  4,096 (512 items, d 32)     forward 24.6 ->  7.4 |  8.5 ->  6.7     backward  59.4 -> 14.4 | 31.1 -> 12.4
 //     lanes  8,192 (512 items, d 64)     forward 21.9 -> 10.3 |  8.2 ->  9.3     backward  58.1 -> 21.4 | 31.5 -> 17.2
-//     lanes 16,384 (512 items, d 128)    forward 18.5 -> 13.0 |  8.2 -> 12.3     backward  54.9 -> 31.5 | 27.5 -> 21.3
 //     lanes 16,640 (2,080 items, d 32)   forward 26.6 -> 16.4 | 10.2 -> 14.4     backward  68.3 -> 31.7 | 33.6 -> 25.6
-//     lanes 33,280 (2,080 items, d 64)   forward 22.6 -> 24.6 |  8.2 -> 22.6     backward  64.7 -> 48.9 | 34.2 -> 38.4
-constexpr long long kSplitForwardLanes = 148 * 64, kSplitBackwardLanes = 148 * 128;
-__host__ __device__ inline bool split_items(const Problem& pr, long long lanes) { return pr.N * pr.heads * (pr.d / 4) <= lanes && pr.P > 1; }
+//     lanes 49,152 (6,144 items, d 32)   forward 36.9 -> 38.9 | 11.4 -> 34.9     backward 116.6 -> 73.8 | 47.0 -> 59.4
+// so that at the line a step gains up to some twenty heads, on integer offsets up to eight.
+constexpr long long kSplitLanes = 148 * 16;
+__host__ __device__ inline bool split_items(const Problem& pr) { return pr.N * (pr.d / 4) <= kSplitLanes && pr.P > 1; }
 
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;

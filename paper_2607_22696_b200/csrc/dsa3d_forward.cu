@@ -589,7 +589,7 @@ static cudaError_t launch_forward_t(const void* q, const void* k, const void* v,
     constexpr int LPR = D / Elt<T, 1>::VEC;
     constexpr int threads = 256;
     if constexpr (std::is_same<T, float>::value) {
-        if (!gate && split_items(pr, kSplitForwardLanes)) {
+        if (!gate && split_items(pr)) {
             (addend ? forward_split_kernel<D, true> : forward_split_kernel<D, false>)<<<static_cast<unsigned>(pr.items), kSplitThreads, 0, stream>>>(
                 static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v), offsets, static_cast<const T*>(addend), static_cast<T*>(out), lse, pr);
             return cudaGetLastError();
