@@ -29,6 +29,9 @@
 // through the rest of its work and drains its loads.
 #include <cuda_bf16.h>
 
+#include <cfloat>
+#include <cmath>
+
 #include "dsa3d_common.cuh"
 #include "dsa3d_kernels.h"
 #include "dsa3d_window_planes.cuh"
@@ -194,7 +197,9 @@ _Pragma("unroll 1")
             if (pl == lt + KT - 1) S::pair_barrier(pair);             // the scores are in place
         }
         // ---- softmax; the table then holds weights
-        float mx = -INFINITY, sum = 0.0f;
+        // the maximum starts at the lowest finite number: a part of a query whose logits are all minus infinity (masked keys) then has a
+        // sum of zero, where the difference of two infinities would make the whole query NaN
+        float mx = -FLT_MAX, sum = 0.0f;
         if constexpr (!BOUNDED) {
             constexpr int ROWS = (KT * KH + PARTS - 1) / PARTS;       // kernel rows (u, v) of the thread: every PARTS-th
             float sc[ROWS][KW];
@@ -290,7 +295,7 @@ _Pragma("unroll 1")
             }
             for (int i = me; i < KT * TABLE; i += PAIR) table[i] = split_weight(sums[i]);
         }
-        if (part == 0 && in_grid && !*abort_flag) lse[n * heads + m] = (mx + log2f(sum)) * kLn2;
+        if (part == 0 && in_grid && !*abort_flag) lse[n * heads + m] = sum > 0.0f ? (mx + log2f(sum)) * kLn2 : NAN;
         S::pair_barrier(pair);                                        // the weights are in place
         // ---- V planes: the output
         float acc[2][4][4];
