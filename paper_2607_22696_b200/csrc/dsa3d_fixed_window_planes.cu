@@ -90,7 +90,9 @@ template <int D, int KT, int KH, int KW> __device__ __forceinline__ void drain_p
         }
 }
 
-template <int D, int KT, int KH, int KW, bool BOUNDED>
+// kEdge: pairs whose x-rows both lie outside the grid do nothing but let the planes go by, and the tiles of a last, partial row of tiles
+// along t come behind all others, so that no CTA is left with a full tile more than the rest (see launch_planes).
+template <int D, int KT, int KH, int KW, bool BOUNDED, bool kEdge>
 __global__ void __launch_bounds__(PlaneShape<D, KT, KH, KW>::THREADS, 1)
 fixed_window_planes_kernel(const __nv_bfloat16* __restrict__ q, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                            __nv_bfloat16* __restrict__ out, float* __restrict__ lse, int T, int H, int W, int heads, int tiles_x, int tiles_y,
@@ -120,11 +122,12 @@ fixed_window_planes_kernel(const __nv_bfloat16* __restrict__ q, const __grid_con
     const int tiles_per_head = total / heads;                        // 32-bit throughout: the host checks the counts fit
     auto locate = [&](int ti, int& m, int& t0, int& y0, int& x0) {   // tile ti of this CTA
         const int item = static_cast<int>(blockIdx.x) + ti * static_cast<int>(gridDim.x);
-        m = item / tiles_per_head;
-        int tile = item - m * tiles_per_head;
+        int tile = item;
+        if (!(kEdge && D == 128)) { m = item / tiles_per_head; tile -= m * tiles_per_head; }
         x0 = (tile % tiles_x) * kPlTX; tile /= tiles_x;
-        y0 = (tile % tiles_y) * kPlTY;
-        t0 = (tile / tiles_y) * kPlTT;
+        y0 = (tile % tiles_y) * kPlTY; tile /= tiles_y;
+        if (kEdge && D == 128) { m = tile % heads; tile /= heads; }
+        t0 = tile * kPlTT;
     };
     // BOUNDED: an earlier kernel on the stream left 0 in *gate if every offset is finite and below 1 in size;
     // otherwise the general kernel behind this one takes the call
@@ -171,6 +174,14 @@ fixed_window_planes_kernel(const __nv_bfloat16* __restrict__ q, const __grid_con
     for (int ti = 0; ti < my_tiles; ++ti) {
         int m, t0, y0, x0;
         locate(ti, m, t0, y0, x0);
+        if (kEdge && (t0 + lt >= T || y0 + ly >= H)) {
+_Pragma("unroll 1")
+            for (int pl = 0; pl < 2 * RT; ++pl) {
+                wait(&s.bar_full[sl], parity, 14);
+                next_slot(ti, pl);
+            }
+            continue;
+        }
         const int qt = t0 + lt, qy = y0 + ly + qr, qxx = x0 + qx;
         const bool in_grid = qt < T && qy < H && qxx < W;
         const long long n = (static_cast<long long>(qt) * H + qy) * W + qxx;
@@ -332,6 +343,8 @@ bool make_plane_maps(const void* k, const void* v, const Problem& pr, int kh, in
     return encode_tensor_map_bf16(mk, k, 5, dims, strides, box, true) && encode_tensor_map_bf16(mv, v, 5, dims, strides, box, true);
 }
 
+// kEdge where a sixteenth or more of the pairs lies outside the grid: it costs four registers that 128 channels do not have (64 x 45 x 80, a
+// twenty-fourth outside: (3,5,5) 1.1 % and small offsets 0.6 % slower); 64 channels take it always.
 template <int D, int KT, int KH, int KW, bool BOUNDED>
 cudaError_t launch_planes(const void* q, const CUtensorMap& mk, const CUtensorMap& mv, void* out, float* lse,
                           const Problem& pr, int* flag, const float* offsets, const int* gate, cudaStream_t stream) {
@@ -339,7 +352,10 @@ cudaError_t launch_planes(const void* q, const CUtensorMap& mk, const CUtensorMa
     const int tiles_x = (pr.W + kPlTX - 1) / kPlTX, tiles_y = (pr.H + kPlTY - 1) / kPlTY,
               tiles_t = (pr.T + kPlTT - 1) / kPlTT;
     const size_t smem = sizeof(PlSmem<D, KT, KH, KW>) + 1024;
-    auto kern = fixed_window_planes_kernel<D, KT, KH, KW, BOUNDED>;
+    const long long pairs = static_cast<long long>(tiles_t) * kPlTT * tiles_y * (kPlTY / 2), live = static_cast<long long>(pr.T) * ((pr.H + 1) / 2);
+    auto kern = fixed_window_planes_kernel<D, KT, KH, KW, BOUNDED, true>;
+    if constexpr (D == 128)
+        if (16 * (pairs - live) < pairs) kern = fixed_window_planes_kernel<D, KT, KH, KW, BOUNDED, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
     const long long total = static_cast<long long>(tiles_x) * tiles_y * tiles_t * pr.heads;
