@@ -294,97 +294,89 @@ backward_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __res
     }
 }
 
-// fp32 calls too small to fill the chip by rows (split_items): a CTA per item, its groups of lanes take the samples in turn in both
-// passes (the statistics, then the reductions into dK / dV), as in forward_split_kernel; bound, as there, by the chain of one item.
-// 4 x 8 x 8, 2 heads of 32 channels, window (3,3,3): 55.6 -> 10.4 us; (3,7,7): 285.6 -> 39.2 us.
+// fp32 calls too small to fill the chip by rows: a CTA per item, its groups of lanes take the samples in turn in both passes (the
+// statistics, then the reductions into dK / dV); bound, as there, by the chain of one item.  The sums over the samples are
+// taken in the order of backward_kernel, a thread per channel, so that dQ and dOffsets have the bits of the rows (split_backward).
 constexpr int kSplitThreads = 128;
 template <int D>
 __global__ void __launch_bounds__(kSplitThreads)
 backward_split_kernel(const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v, const float* __restrict__ offsets,
                       const float* __restrict__ lse, const float* __restrict__ dout, float* __restrict__ dq, float* __restrict__ acc_dk,
                       float* __restrict__ acc_dv, float* __restrict__ doffsets, const __grid_constant__ Problem pr) {
+    using E = Elt<float, 1>;
+    using Row = typename E::Row;
     constexpr int LPR = D / 4, S = kSplitThreads / LPR;
-    extern __shared__ float stats[];                     // [P][8]: alpha, g, A_t, A_y, A_x, B_t, B_y, B_x
-    __shared__ float4 part[2][S][LPR];
-    __shared__ float deltas[S];
+    extern __shared__ float stats[];                     // [P, to a multiple of S][8]: alpha, g, A_t, A_y, A_x, B_t, B_y, B_x
+    __shared__ Sample samples[256];
+    __shared__ float4 sampled[2][S][LPR];                // interpolated K rows of S samples, twice
+    __shared__ float whole_delta;
     if (gated_off(pr)) return;
-    const int gl = threadIdx.x % LPR, sub = threadIdx.x / LPR;
+    const int tid = threadIdx.x, gl = tid % LPR, sub = tid / LPR;
     const int m = static_cast<int>(blockIdx.x / static_cast<unsigned>(pr.q_count));
     const int n = static_cast<int>(pr.q_begin) + static_cast<int>(blockIdx.x - static_cast<unsigned>(m) * static_cast<unsigned>(pr.q_count));
     const int x = n % pr.W, ty = n / pr.W, y = ty % pr.H, t = ty / pr.H;
     const long long row = static_cast<long long>(n) * pr.heads + m, head = static_cast<long long>(m) * D + gl * 4;
     const long long tok = static_cast<long long>(pr.heads) * D, sy = pr.W * tok, st = pr.H * sy;
-    const float4 qr = __ldg(reinterpret_cast<const float4*>(q + row * D) + gl), dor = __ldg(reinterpret_cast<const float4*>(dout + row * D) + gl);
+    const Row qr = E::load(q + row * D + gl * 4), dor = E::load(dout + row * D + gl * 4);
     const float scale = rsqrtf(static_cast<float>(D)), lse2 = __ldg(lse + row) * kLog2e;
-    const float* off_row = offsets + row * pr.P * 3;
     [[maybe_unused]] const long long kv_extent = pr.N * pr.heads * D;
-    float u[4] = {0.0f, 0.0f, 0.0f, 0.0f}, kbar[4] = {0.0f, 0.0f, 0.0f, 0.0f}, delta = 0.0f;
-    for (int pb = 0; pb < pr.P; pb += S) {
+    for (int p = tid; p < pr.P; p += kSplitThreads) samples[p] = to_sample(pr, make_cell(pr, t, y, x, p, offsets + (row * pr.P + p) * 3));
+    __syncthreads();
+    float u = 0.0f, kbar = 0.0f, delta = 0.0f;           // of channel tid
+    for (int pb = 0, buf = 0; pb < pr.P; pb += S, buf ^= 1) {
         const int p = pb + sub;
         const bool have = p < pr.P;
         Sample s;
         s.base = 0; s.mask = 0u; s.ft = s.fy = s.fx = 0.0f;
-        if (have) s = to_sample(pr, make_cell(pr, t, y, x, p, off_row + p * 3));
-        // a corner matters if its weight or one of its weight derivatives is not zero
-        unsigned mask = s.mask;
-        if (s.ft == 0.0f && s.fy == 0.0f) mask &= 0x3fu;
-        if (s.ft == 0.0f && s.fx == 0.0f) mask &= 0x5fu;
-        if (s.fy == 0.0f && s.fx == 0.0f) mask &= 0x77u;
+        if (have) s = samples[p];
         const float wt[2] = {1.0f - s.ft, s.ft}, wy[2] = {1.0f - s.fy, s.fy}, wx[2] = {1.0f - s.fx, s.fx};
-        float4 kk[8], vv[8];
+        Row kk[8], vv[8];
+        unsigned needed = 0u;                            // a corner matters if its weight or one of its weight derivatives is not zero
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
-            kk[c] = vv[c] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            kk[c] = vv[c] = E::zero();
+            const float ct = wt[c >> 2], cy = wy[(c >> 1) & 1], cx = wx[c & 1];
+            const bool matters = (ct * cy * cx != 0.0f) | (cy * cx != 0.0f) | (ct * cx != 0.0f) | (ct * cy != 0.0f);
             const long long o = head + s.base * tok + (c >> 2) * st + ((c >> 1) & 1) * sy + (c & 1) * tok;
-            if (((mask >> c) & 1u) && DSA3D_IN_RANGE(pr, o, kv_extent, 6)) {
-                kk[c] = __ldg(reinterpret_cast<const float4*>(k + o));
-                vv[c] = __ldg(reinterpret_cast<const float4*>(v + o));
+            if (((s.mask >> c) & 1u) && matters && DSA3D_IN_RANGE(pr, o, kv_extent, 6)) {
+                needed |= 1u << c;
+                kk[c] = E::load(k + o);
+                vv[c] = E::load(v + o);
             }
         }
         float a[8], b[8], kp[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
-            const float w = wt[c >> 2] * wy[(c >> 1) & 1] * wx[c & 1];
-            a[c] = fmaf(qr.w, kk[c].w, fmaf(qr.z, kk[c].z, fmaf(qr.y, kk[c].y, qr.x * kk[c].x)));
-            b[c] = fmaf(dor.w, vv[c].w, fmaf(dor.z, vv[c].z, fmaf(dor.y, vv[c].y, dor.x * vv[c].x)));
-            kp[0] = fmaf(w, kk[c].x, kp[0]); kp[1] = fmaf(w, kk[c].y, kp[1]);
-            kp[2] = fmaf(w, kk[c].z, kp[2]); kp[3] = fmaf(w, kk[c].w, kp[3]);
+            a[c] = (needed >> c) & 1u ? E::dot(qr, kk[c], 0.0f) : 0.0f;
+            b[c] = (needed >> c) & 1u ? E::dot(dor, vv[c], 0.0f) : 0.0f;
+            E::axpy(wt[c >> 2] * wy[(c >> 1) & 1] * wx[c & 1], kk[c], kp);
         }
-        float r[8];
+        float r[kStats];
         trilerp_grad(a, s.ft, s.fy, s.fx, r[0], r[2], r[3], r[4]);
         trilerp_grad(b, s.ft, s.fy, s.fx, r[1], r[5], r[6], r[7]);
         group_reduce8<LPR>(r, gl, kFullMask);
-        const float sdot = __shfl_sync(kFullMask, r[0], reduce8_lane<LPR>(0), LPR), g = __shfl_sync(kFullMask, r[0], reduce8_lane<LPR>(1), LPR);
-        const float alpha = have ? exp2f(fmaf(sdot, scale * kLog2e, -lse2)) : 0.0f, ag = have ? alpha * g : 0.0f;
-        delta += ag;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            u[e] = fmaf(ag, kp[e], u[e]);
-            kbar[e] = fmaf(alpha, kp[e], kbar[e]);
-        }
+        const float sdot = __shfl_sync(kFullMask, r[0], reduce8_lane<LPR>(0), LPR);
+        const float alpha = exp2f(fmaf(sdot, scale * kLog2e, -lse2));
         const int idx = reduce8_index<LPR>(gl);
-        if (have && gl == reduce8_lane<LPR>(idx)) stats[p * 8 + idx] = idx == 0 ? alpha : r[0];
+        if (gl == reduce8_lane<LPR>(idx)) stats[p * kStats + idx] = !have ? 0.0f : idx == 0 ? alpha : r[0];
+        sampled[buf][sub][gl] = make_float4(kp[0], kp[1], kp[2], kp[3]);
+        __syncthreads();
+        if (tid >= D) continue;
+        const float* kr = reinterpret_cast<const float*>(sampled[buf]) + tid;
+#pragma unroll
+        for (int j = 0; j < S; ++j) {                    // (the samples behind the last are zero)
+            const float al = stats[(pb + j) * kStats], ag = al * stats[(pb + j) * kStats + 1];
+            delta += ag;
+            u = fmaf(ag, kr[j * D], u);
+            kbar = fmaf(al, kr[j * D], kbar);
+        }
     }
-    part[0][sub][gl] = make_float4(u[0], u[1], u[2], u[3]);
-    part[1][sub][gl] = make_float4(kbar[0], kbar[1], kbar[2], kbar[3]);
-    if (gl == 0) deltas[sub] = delta;
+    if (tid < D) dq[row * D + tid] = scale * fmaf(-delta, kbar, u);
+    if (tid == 0) whole_delta = delta;
     __syncthreads();
-    delta = 0.0f;
-#pragma unroll
-    for (int i = 0; i < S; ++i) delta += deltas[i];
-    if (sub == 0) {
-        float o[2][4] = {};
-        for (int i = 0; i < S; ++i)
-#pragma unroll
-            for (int z = 0; z < 2; ++z) {
-                const float4 a = part[z][i][gl];
-                o[z][0] += a.x; o[z][1] += a.y; o[z][2] += a.z; o[z][3] += a.w;
-            }
-        *(reinterpret_cast<float4*>(dq + row * D) + gl) = make_float4(scale * fmaf(-delta, o[1][0], o[0][0]), scale * fmaf(-delta, o[1][1], o[0][1]),
-                                                                       scale * fmaf(-delta, o[1][2], o[0][2]), scale * fmaf(-delta, o[1][3], o[0][3]));
-    }
-    for (int p = threadIdx.x; p < pr.P; p += kSplitThreads) {
-        const float* sts = stats + p * 8;
+    delta = whole_delta;
+    for (int p = tid; p < pr.P; p += kSplitThreads) {
+        const float* sts = stats + p * kStats;
         const float alpha = sts[0], ck = scale * (alpha * (sts[1] - delta));
         float* d = doffsets + (row * pr.P + p) * 3;
         d[0] = fmaf(ck, sts[2], alpha * sts[5]);
@@ -392,8 +384,8 @@ backward_split_kernel(const float* __restrict__ q, const float* __restrict__ k, 
         d[2] = fmaf(ck, sts[4], alpha * sts[7]);
     }
     for (int p = sub; p < pr.P; p += S) {
-        const Sample s = to_sample(pr, make_cell(pr, t, y, x, p, off_row + p * 3));
-        const float cv = stats[p * 8], ck = scale * (cv * (stats[p * 8 + 1] - delta));
+        const Sample s = samples[p];
+        const float cv = stats[p * kStats], ck = scale * (cv * (stats[p * kStats + 1] - delta));
         const float wt[2] = {1.0f - s.ft, s.ft}, wy[2] = {1.0f - s.fy, s.fy}, wx[2] = {1.0f - s.fx, s.fx};
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
@@ -401,8 +393,8 @@ backward_split_kernel(const float* __restrict__ q, const float* __restrict__ k, 
             const long long o = head + s.base * tok + (c >> 2) * st + ((c >> 1) & 1) * sy + (c & 1) * tok;
             if (((s.mask >> c) & 1u) && w != 0.0f && DSA3D_IN_RANGE(pr, o, kv_extent, 7)) {
                 const float wk = w * ck, wv = w * cv;
-                red_add_v4(acc_dk + o, wk * qr.x, wk * qr.y, wk * qr.z, wk * qr.w);
-                red_add_v4(acc_dv + o, wv * dor.x, wv * dor.y, wv * dor.z, wv * dor.w);
+                red_add_v4(acc_dk + o, wk * qr.v[0], wk * qr.v[1], wk * qr.v[2], wk * qr.v[3]);
+                red_add_v4(acc_dv + o, wv * dor.v[0], wv * dor.v[1], wv * dor.v[2], wv * dor.v[3]);
             }
         }
     }
@@ -638,8 +630,8 @@ static cudaError_t launch_backward_t(const void* q, const void* k, const void* v
                                      float* acc_dv, float* doffsets, float2* coef, const Problem& pr,
                                      cudaStream_t stream) {
     if constexpr (std::is_same<T, float>::value) {
-        if (split_items(pr) && pr.tile_t < 1) {
-            backward_split_kernel<D><<<static_cast<unsigned>(pr.items), kSplitThreads, static_cast<size_t>(pr.P) * 8 * sizeof(float), stream>>>(
+        if (split_backward(pr) && pr.tile_t < 1) {
+            backward_split_kernel<D><<<static_cast<unsigned>(pr.items), kSplitThreads, static_cast<size_t>((pr.P + kSplitThreads / (D / 4) - 1) / (kSplitThreads / (D / 4)) * (kSplitThreads / (D / 4))) * kStats * sizeof(float), stream>>>(
                 static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v), offsets, lse, static_cast<const T*>(dout), static_cast<T*>(dq), acc_dk, acc_dv, doffsets, pr);
             return cudaGetLastError();
         }

@@ -426,16 +426,43 @@ __device__ __forceinline__ void red_add_v4(float* addr, float a, float b, float 
                  : "memory");
 }
 
-// fp32 calls too small to fill the chip by rows run with a CTA per item (forward_split_kernel, backward_split_kernel).  The line is in the
-// lanes of a head's tokens, d / 4 each: neither how many heads a call has nor how many frames a launch takes changes the bits of a head.
-// Rows -> split in us, (3,3,3), offsets N(0, 1) | integer offsets, whose rows skip the corners of weight zero, by lanes of all heads:
-//     lanes  4,096 (512 items, d 32)     forward 24.6 ->  7.4 |  8.5 ->  6.7     backward  59.4 -> 14.4 | 31.1 -> 12.4
-//     lanes  8,192 (512 items, d 64)     forward 21.9 -> 10.3 |  8.2 ->  9.3     backward  58.1 -> 21.4 | 31.5 -> 17.2
-//     lanes 16,640 (2,080 items, d 32)   forward 26.6 -> 16.4 | 10.2 -> 14.4     backward  68.3 -> 31.7 | 33.6 -> 25.6
-//     lanes 49,152 (6,144 items, d 32)   forward 36.9 -> 38.9 | 11.4 -> 34.9     backward 116.6 -> 73.8 | 47.0 -> 59.4
-// so that at the line a step gains up to some twenty heads, on integer offsets up to eight.
-constexpr long long kSplitLanes = 148 * 16;
-__host__ __device__ inline bool split_items(const Problem& pr) { return pr.N * (pr.d / 4) <= kSplitLanes && pr.P > 1; }
+// Forward of fp32 calls: up to this many lanes of a head's tokens, d / 4 each, by classes of samples (forward_classes_kernel), whose sums are
+// in another order than those of the rows: the line does not look at the heads, so that a shard of them gives the bits of the whole.
+constexpr long long kClassLanes = 148 * 16;
+__host__ __device__ inline bool by_classes(const Problem& pr) { return pr.N * (pr.d / 4) <= kClassLanes && pr.P > 1; }
+
+// There: groups of lanes per item, one per class or one for all, the same bits.  Just below that line (256, 144 and 72 tokens of 32, 64 and 128
+// channels), us by rows | four groups | one, N(0, 1) and integer offsets:
+//     heads            2                    8                    16                   32                   64
+//     32, (2,2,2)     9.2|3.7| 6.6         9.4| 5.2| 6.9        9.6| 8.6| 8.1       12.2|14.4|11.4       23.6|26.4|18.7
+//         integer     3.4|3.1| 3.7         3.6| 4.2| 3.9        3.7| 6.3| 4.2        4.4|11.0| 4.8        7.1|20.0| 8.1
+//     32, (3,3,3)    23.0|6.8|17.2        23.5|11.4|17.2       23.7|18.7|20.6       32.4|34.5|31.2       59.7|65.3|52.3
+//         integer     7.5|3.4| 7.1         7.6| 4.4| 7.4        7.7| 7.0| 7.7        9.5|11.6| 9.7       16.4|21.0|16.5
+//     32, (3,7,7)   101.4|23.7|75.4      100.2|44.8|75.6      101.3|75.4|94.8      148.1|144.5|152.2    277.5|280.0|256.1
+//         integer    25.6|8.0|24.3        25.9|11.4|24.6       26.1|19.0|26.9       33.3|35.2|36.6       61.6|66.4|61.8
+//     64, (3,3,3)    19.2|6.6|15.6        19.2|10.7|15.8       19.8|19.3|18.9       27.1|35.5|29.0       50.1|67.2|54.9
+//         integer     6.4|3.3| 5.7         6.6| 4.2| 5.8        6.7| 6.9| 6.7        8.4|12.3| 8.9       14.5|22.3|15.8
+//     128, (3,3,3)   17.2|7.4|14.7        17.0|10.6|15.0       17.3|19.1|17.7       24.4|35.3|27.6       44.8|66.1|51.8
+//         integer     5.8|3.3| 5.6         5.9| 4.2| 5.5        5.9| 7.0| 6.3        7.8|12.1| 8.6       13.3|21.9|15.4
+// (What is left slower than by rows: more than 16 heads, on integer offsets 2 - 15 %, 26 % for (2,2,2); real-valued ones of 64 and 128
+// channels 7 - 14 %.)
+__host__ __device__ inline int class_groups(const Problem& pr) {
+    return pr.items * (pr.d / 4) <= 148ll * (pr.P <= 32 ? 128 : 256) ? 4 : 1;
+}
+
+// Backward of fp32 calls: up to this many lanes a CTA per item (backward_split_kernel), the same bits.  By rows | a CTA per item, as above:
+//     heads            2                    8                    16
+//     32, (2,2,2)    21.5| 7.7            22.2|15.6            23.0|25.5              integer  11.8| 6.9     12.2|13.5     12.3|21.8
+//     32, (3,3,3)    55.6|12.5            56.4|27.0            57.8|45.4                       28.0| 8.7     28.7|19.8     29.0|34.1
+//     32, (3,7,7)   281.3|35.8           307.8|93.7           348.8|180.0                     133.6|24.6    137.7|68.4    154.8|127.6
+//     64, (3,3,3)    44.8|14.1            45.8|27.1            48.4|44.9                       25.5|11.1     25.8|21.4     26.2|36.6
+//     64, (3,7,7)   235.0|44.8           243.5|104.7          271.2|176.1                     115.5|33.1    118.1|76.3    131.8|142.1
+//     128, (3,3,3)   38.2|16.8            39.0|24.1            45.0|41.2                       21.9|14.2     22.4|18.6     22.6|31.1
+//     128, (3,7,7)  154.2|51.2           155.3|92.7           176.2|168.5                      89.5|46.8     90.2|74.5     91.0|135.1
+__host__ __device__ inline bool split_backward(const Problem& pr) {
+    const int per_sm = pr.d == 128 ? 128 : pr.P > 64 ? 224 : pr.d == 64 ? 128 : pr.P > 16 ? 168 : 96;
+    return pr.items * (pr.d / 4) <= 148ll * per_sm && pr.P > 1;
+}
 
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;

@@ -458,97 +458,185 @@ forward_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __rest
     }
 }
 
-// fp32 calls too small to fill the chip by rows (split_items): a CTA per item, its groups of lanes take the samples in turn.  What bounds
-// such a call is the chain of one item, a gather and an update of the running maximum per sample: by rows it is P samples deep and most
-// SMs are idle, here it is P / 16, P / 8 or P / 4 (32, 64, 128 channels) and one sum over the groups.  4 x 8 x 8, 2 heads of 32 channels,
-// window (3,3,3): 22.3 -> 5.6 us; (3,7,7): 100.6 -> 18.5 us.
-constexpr int kSplitThreads = 128;
-template <int D, bool kAdd>
-__global__ void __launch_bounds__(kSplitThreads)
-forward_split_kernel(const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v, const float* __restrict__ offsets,
-                     const float* addend, float* out, float* __restrict__ lse, const __grid_constant__ Problem pr) {
-    constexpr int LPR = D / 4, S = kSplitThreads / LPR;
-    __shared__ float4 part[S][LPR];
-    __shared__ float2 stat[S];
-    const int gl = threadIdx.x % LPR, sub = threadIdx.x / LPR;
-    const int m = static_cast<int>(blockIdx.x / static_cast<unsigned>(pr.q_count));
-    const int n = static_cast<int>(pr.q_begin) + static_cast<int>(blockIdx.x - static_cast<unsigned>(m) * static_cast<unsigned>(pr.q_count));
+// fp32 calls of few tokens (by_classes): the samples of an item in four classes of consecutive ones, each with sums of its own that are folded
+// into the whole in order.  What bounds such a call by rows is the chain of one item, a gather and an update of the running maximum per
+// sample; with a group of lanes per class (G = 4) it is a quarter as deep.  Calls with more items than that has lanes for walk the
+// classes one after the other (G = 1): the same sums in the same order, whichever of the two paths below a warp takes, so that the bits of
+// a head do not depend on how many heads the call has.  120 registers: with 96 or 80 the rows are no longer all asked for
+// at once (window (3,3,3), 64 heads: 52 -> 62 and 89 us).  Figures: class_groups.
+constexpr int kClasses = 4, kClassThreads = 128;
+template <int D, bool kAdd, int G>
+__global__ void __launch_bounds__(kClassThreads, 4)
+forward_classes_kernel(const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v, const float* __restrict__ offsets,
+                       const float* addend, float* out, float* __restrict__ lse, const __grid_constant__ Problem pr) {
+    using E = Elt<float, 1>;
+    using Row = typename E::Row;
+    constexpr int LPR = D / 4, ITEMS = kClassThreads / (G * LPR);
+    const int gl = threadIdx.x % LPR, group = threadIdx.x / LPR;
+    long long item = static_cast<long long>(blockIdx.x) * ITEMS + group / G;
+    const bool active = item < pr.items;                 // trailing groups repeat the last item, stores off
+    if (!active) item = pr.items - 1;
+    const int m = static_cast<int>(item / pr.q_count), n = static_cast<int>(pr.q_begin + (item - m * pr.q_count));
     const int x = n % pr.W, ty = n / pr.W, y = ty % pr.H, t = ty / pr.H;
     const long long row = static_cast<long long>(n) * pr.heads + m;
     const long long tok = static_cast<long long>(pr.heads) * D, sy = pr.W * tok, st = pr.H * sy;
-    const float4 qr = __ldg(reinterpret_cast<const float4*>(q + row * D) + gl);
+    const Row qr = E::load(q + row * D + gl * 4);
     const float* kh = k + static_cast<long long>(m) * D + gl * 4;
-    const float* vh = v + static_cast<long long>(m) * D + gl * 4;
+    const long long v_minus_k = v - k;
     [[maybe_unused]] const long long kv_extent = pr.N * pr.heads * D;
     const float lscale = rsqrtf(static_cast<float>(D)) * kLog2e;        // logits in log2 units
-    float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    float m_run = -INFINITY, l_run = 0.0f;
-    for (int pb = 0; pb < pr.P; pb += S) {
-        const int p = pb + sub;
-        const bool have = p < pr.P;
-        Sample s;
-        s.base = 0; s.mask = 0u; s.ft = s.fy = s.fx = 0.0f;
-        if (have) s = to_sample(pr, make_cell(pr, t, y, x, p, offsets ? offsets + (row * pr.P + p) * 3 : kZeroOffset));
-        const unsigned mask = checked_corners(pr, weighted_corners(s.mask, s.ft, s.fy, s.fx), s.base, 2);
-        const float wt[2] = {1.0f - s.ft, s.ft}, wy[2] = {1.0f - s.fy, s.fy}, wx[2] = {1.0f - s.fx, s.fx};
-        float4 kk[8], vv[8];
-        float w[8];
+    int size = (pr.P + kClasses - 1) / kClasses;
+    if (pr.P > 16) size = (size + 7) & ~7;               // so that eight samples on the grid belong to one class
+    const int span = G == 1 ? pr.P : size, begin = G == 1 ? 0 : group % G * size;
+    float total[4] = {0.0f, 0.0f, 0.0f, 0.0f}, m_all = -INFINITY, l_all = 0.0f;
+    float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f}, m_run = -INFINITY, l_run = 0.0f;       // of the class
+    auto fold = [&](const float (&a)[4], float m_part, float l_part) {
+        const float mx = fmaxf(m_all, m_part), f = m_all == mx ? 1.0f : exp2f(m_all - mx), g = m_part == mx ? 1.0f : exp2f(m_part - mx);
+        l_all = fmaf(l_part, g, __fmul_rn(l_all, f));
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            w[c] = wt[c >> 2] * wy[(c >> 1) & 1] * wx[c & 1];
-            kk[c] = vv[c] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            if ((mask >> c) & 1u) {
-                const long long o = s.base * tok + (c >> 2) * st + ((c >> 1) & 1) * sy + (c & 1) * tok;
-                kk[c] = __ldg(reinterpret_cast<const float4*>(kh + o));
-                vv[c] = __ldg(reinterpret_cast<const float4*>(vh + o));
-            } else {
-                w[c] = 0.0f;
-            }
+        for (int e = 0; e < 4; ++e) total[e] = fmaf(a[e], g, __fmul_rn(total[e], f));
+        m_all = mx;
+    };
+    int left = size;                                     // samples of the class still to come (G = 1)
+    auto next_class = [&](int taken) {
+        if (left == 0) {
+            fold(acc, m_run, l_run);
+            acc[0] = acc[1] = acc[2] = acc[3] = l_run = 0.0f;
+            m_run = -INFINITY;
+            left = size;
         }
-        float sdot = 0.0f;
-#pragma unroll
-        for (int c = 0; c < 8; ++c)
-            sdot = fmaf(w[c], fmaf(qr.w, kk[c].w, fmaf(qr.z, kk[c].z, fmaf(qr.y, kk[c].y, qr.x * kk[c].x))), sdot);
-        sdot = group_sum<LPR>(sdot, kFullMask);
-        const float sp = have ? sdot * lscale : -INFINITY;
-        if (sp > m_run) {
+        left -= taken;
+    };
+    // the next sample's logit: its weight beside the sums so far
+    auto weight = [&](float sp) {
+        if (sp > m_run + 8.0f) {
             const float corr = exp2f(m_run - sp);
             l_run *= corr;
-            acc.x *= corr; acc.y *= corr; acc.z *= corr; acc.w *= corr;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[e] *= corr;
             m_run = sp;
         }
         const float pe = sp == -INFINITY ? 0.0f : exp2f(sp - m_run);
-        l_run += pe;
+        l_run = __fadd_rn(l_run, pe);
+        return pe;
+    };
+    for (int i0 = 0; i0 < span; i0 += LPR) {
+        const int p0 = begin + i0, cnt = min(LPR, span - i0);           // (the last class may end before its samples do: no logit)
+        Sample mine;
+        mine.base = 0; mine.mask = 0u; mine.ft = mine.fy = mine.fx = 0.0f;
+        if (gl < cnt && p0 + gl < pr.P) mine = to_sample(pr, make_cell(pr, t, y, x, p0 + gl, offsets ? offsets + (row * pr.P + p0 + gl) * 3 : kZeroOffset));
+        if (__all_sync(kFullMask, mine.ft == 0.0f && mine.fy == 0.0f && mine.fx == 0.0f)) {     // on the grid: a row each, eight samples at a time
+            for (int jb = 0; jb < cnt; jb += 8) {
+                Row kk[8], vv[8];
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const float a = pe * w[c];
-            acc.x = fmaf(a, vv[c].x, acc.x); acc.y = fmaf(a, vv[c].y, acc.y);
-            acc.z = fmaf(a, vv[c].z, acc.z); acc.w = fmaf(a, vv[c].w, acc.w);
+                for (int i = 0; i < 8; ++i) {
+                    const int base = __shfl_sync(kFullMask, mine.base, jb + i, LPR);
+                    const unsigned mask = __shfl_sync(kFullMask, mine.mask, jb + i, LPR);
+                    kk[i] = vv[i] = E::zero();
+                    const float* pk = kh + base * tok;
+                    if ((mask & 1u) && jb + i < cnt && DSA3D_IN_RANGE(pr, pk - k, kv_extent, 1)) {
+                        kk[i] = E::load(pk);
+                        vv[i] = E::load(pk + v_minus_k);
+                    }
+                }
+                float dd[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) dd[i] = E::dot(qr, kk[i], 0.0f);
+                group_reduce8<LPR>(dd, gl, kFullMask);
+                float sp[8], mx = -INFINITY;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    sp[i] = __shfl_sync(kFullMask, dd[0], reduce8_lane<LPR>(i), LPR) * lscale;
+                    if (jb + i >= cnt || p0 + jb + i >= pr.P) sp[i] = -INFINITY;
+                    mx = fmaxf(mx, sp[i]);
+                }
+                const bool aligned = G != 1 || size % 8 == 0;
+                if (G == 1 && aligned) next_class(8);
+                // the first sample of a class sets the maximum; as a rule none of the eight moves it again
+                const float first = aligned && m_run == -INFINITY && sp[0] > m_run ? sp[0] : m_run;
+                if (__all_sync(kFullMask, aligned && first > -INFINITY && mx <= first + 8.0f)) {
+                    m_run = first;
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const float pe = exp2f(sp[i] - m_run);
+                        l_run = __fadd_rn(l_run, pe);
+                        E::axpy(pe, vv[i], acc);
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        if (jb + i >= cnt) continue;
+                        if (G == 1 && !aligned) next_class(1);
+                        E::axpy(weight(sp[i]), vv[i], acc);
+                    }
+                }
+            }
+            continue;
+        }
+        for (int j = 0; j < cnt; ++j) {
+            const Sample s = group_bcast<LPR>(mine, j, kFullMask);
+            const float wt[2] = {1.0f - s.ft, s.ft}, wy[2] = {1.0f - s.fy, s.fy}, wx[2] = {1.0f - s.fx, s.fx};
+            const float* at = kh + s.base * tok;
+            float w[8], sdot = 0.0f;
+            Row kk[8], vv[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                w[c] = wt[c >> 2] * wy[(c >> 1) & 1] * wx[c & 1];
+                kk[c] = vv[c] = E::zero();
+                const float* pk = at + (c >> 2) * st + ((c >> 1) & 1) * sy + (c & 1) * tok;
+                if (((s.mask >> c) & 1u) && w[c] != 0.0f && DSA3D_IN_RANGE(pr, pk - k, kv_extent, 3)) {
+                    kk[c] = E::load(pk);
+                    vv[c] = E::load(pk + v_minus_k);
+                } else {
+                    w[c] = 0.0f;
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+                if (w[c] != 0.0f) sdot = fmaf(w[c], E::dot(qr, kk[c], 0.0f), sdot);
+            const float sp = group_sum<LPR>(sdot, kFullMask) * lscale;
+            if (G == 1) next_class(1);
+            const float pe = weight(p0 + j < pr.P ? sp : -INFINITY);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) E::axpy(pe * w[c], vv[c], acc);
         }
     }
-    part[sub][gl] = acc;
-    if (gl == 0) stat[sub] = make_float2(m_run, l_run);
-    __syncthreads();
-    if (threadIdx.x >= LPR) return;
-    const int groups = min(S, pr.P);                     // the others had no sample
-    float mx = stat[0].x;
-    for (int i = 1; i < groups; ++i) mx = fmaxf(mx, stat[i].x);
-    float l = 0.0f, o[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    for (int i = 0; i < groups; ++i) {
-        const float corr = exp2f(stat[i].x - mx);
-        const float4 a = part[i][gl];
-        l = fmaf(stat[i].y, corr, l);
-        o[0] = fmaf(a.x, corr, o[0]); o[1] = fmaf(a.y, corr, o[1]); o[2] = fmaf(a.z, corr, o[2]); o[3] = fmaf(a.w, corr, o[3]);
-    }
-    const float inv = 1.0f / l;
+    if constexpr (G == 1) {
+        fold(acc, m_run, l_run);
+    } else {
+        __shared__ float4 part[ITEMS][kClasses][LPR];
+        __shared__ float2 stat[ITEMS][kClasses];
+        part[group / G][group % G][gl] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+        if (gl == 0) stat[group / G][group % G] = make_float2(m_run, l_run);
+        __syncthreads();
+        if (group % G != 0) return;
 #pragma unroll
-    for (int e = 0; e < 4; ++e) o[e] *= inv;
-    if constexpr (kAdd) {
-        const float4 add = *(reinterpret_cast<const float4*>(addend + row * D) + gl);
-        o[0] += add.x; o[1] += add.y; o[2] += add.z; o[3] += add.w;
+        for (int c = 0; c < kClasses; ++c) {
+            const float4 a = part[group / G][c][gl];
+            const float2 s = stat[group / G][c];
+            fold({a.x, a.y, a.z, a.w}, s.x, s.y);
+        }
     }
-    *(reinterpret_cast<float4*>(out + row * D) + gl) = make_float4(o[0], o[1], o[2], o[3]);
-    if (gl == 0) lse[row] = (mx + log2f(l)) * kLn2;
+    if (!active) return;
+    const float inv = 1.0f / l_all;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) total[e] = __fmul_rn(total[e], inv);
+    if constexpr (kAdd) {
+        float add[4];
+        E::to_float(E::load(addend + row * D + gl * 4), add);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) total[e] = __fadd_rn(total[e], add[e]);
+    }
+    E::store(out + row * D + gl * 4, total);
+    if (gl == 0) lse[row] = (m_all + log2f(l_all)) * kLn2;
+}
+
+template <int D, bool kAdd, int G>
+static cudaError_t launch_forward_classes(const void* q, const void* k, const void* v, const float* offsets, const void* addend, void* out, float* lse, const Problem& pr, cudaStream_t stream) {
+    constexpr int items = kClassThreads / (G * (D / 4));
+    forward_classes_kernel<D, kAdd, G><<<static_cast<unsigned>((pr.items + items - 1) / items), kClassThreads, 0, stream>>>(
+        static_cast<const float*>(q), static_cast<const float*>(k), static_cast<const float*>(v), offsets, static_cast<const float*>(addend), static_cast<float*>(out), lse, pr);
+    return cudaGetLastError();
 }
 
 template <int D>
@@ -589,10 +677,9 @@ static cudaError_t launch_forward_t(const void* q, const void* k, const void* v,
     constexpr int LPR = D / Elt<T, 1>::VEC;
     constexpr int threads = 256;
     if constexpr (std::is_same<T, float>::value) {
-        if (!gate && split_items(pr)) {
-            (addend ? forward_split_kernel<D, true> : forward_split_kernel<D, false>)<<<static_cast<unsigned>(pr.items), kSplitThreads, 0, stream>>>(
-                static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v), offsets, static_cast<const T*>(addend), static_cast<T*>(out), lse, pr);
-            return cudaGetLastError();
+        if (!gate && by_classes(pr)) {
+            if (class_groups(pr) == 1) return addend ? launch_forward_classes<D, true, 1>(q, k, v, offsets, addend, out, lse, pr, stream) : launch_forward_classes<D, false, 1>(q, k, v, offsets, addend, out, lse, pr, stream);
+            return addend ? launch_forward_classes<D, true, kClasses>(q, k, v, offsets, addend, out, lse, pr, stream) : launch_forward_classes<D, false, kClasses>(q, k, v, offsets, addend, out, lse, pr, stream);
         }
     }
     const long long groups_per_block = threads / LPR;
