@@ -674,22 +674,10 @@ int step_group_heads(const dsa3d::Problem& pr, size_t row_bytes) {
 int step_host_heads(const dsa3d::Problem& pr, int group, const void* q_h, const void* k_h, const void* v_h, const float* offsets_h, const void* dout_h,
                     const int window[3], void* out_h, float* lse_h, void* dq_h, void* dk_h, void* dv_h, float* doffsets_h, char* base, const Arena& a,
                     int dtype, HostStep* hs, cudaStream_t stream) {
-    cudaError_t e;
-#define DSA3D_TRY(call)                         \
-    do {                                        \
-        e = (call);                             \
-        if (e != cudaSuccess) return cuda_failed(e); \
-    } while (0)
     const bool bf16 = dtype == DSA3D_BF16;
-    const size_t elt = bf16 ? 2 : 4, N = static_cast<size_t>(pr.N);
-    // whatever pipelined steps may still have in flight comes first, and a later one shares no ordering per slab with this call
-    DSA3D_TRY(cudaStreamWaitEvent(stream, hs->out_done, 0));
-    DSA3D_TRY(cudaStreamWaitEvent(stream, hs->main_done, 0));
-    hs->last_arena = nullptr;
-    DSA3D_TRY(cudaEventRecord(hs->start, stream));
-    DSA3D_TRY(cudaStreamWaitEvent(hs->in, hs->start, 0));
-    DSA3D_TRY(cudaStreamWaitEvent(hs->out, hs->start, 0));
-    struct Group { int m0, heads; char *q, *k, *v, *dout, *out, *dq, *dk, *dv; float *offsets, *doffsets, *lse; };
+    const size_t elt = bf16 ? 2 : 4, N = static_cast<size_t>(pr.N), row = pr.d * elt, off = pr.P * 3 * sizeof(float);
+    // everything that can be refused comes before the first copy
+    struct Group { int m0, heads; char *q, *k, *v, *dout, *out, *dq, *dk, *dv; float *offsets, *doffsets, *lse; BackwardPlan plan; };
     Group groups[kMaxSlabs];
     int count = 0;
     size_t at = 0;                                       // the second pair of K and V buffers leaves room for the rounding
@@ -698,13 +686,20 @@ int step_host_heads(const dsa3d::Problem& pr, int group, const void* q_h, const 
         Group& g = groups[count++];
         g.m0 = m0;
         g.heads = pr.heads - m0 < group ? pr.heads - m0 : group;
-        const size_t items = N * g.heads, rows = items * pr.d * elt, offs = items * pr.P * 3 * sizeof(float);
-        for (char** p : {&g.q, &g.k, &g.v, &g.dout, &g.out, &g.dq, &g.dk, &g.dv}) *p = take(rows);
-        g.offsets = reinterpret_cast<float*>(take(offs));
-        g.doffsets = reinterpret_cast<float*>(take(offs));
+        const size_t items = N * g.heads;
+        for (char** p : {&g.q, &g.k, &g.v, &g.dout, &g.out, &g.dq, &g.dk, &g.dv}) *p = take(items * row);
+        g.offsets = reinterpret_cast<float*>(take(items * off));
+        g.doffsets = reinterpret_cast<float*>(take(items * off));
         g.lse = reinterpret_cast<float*>(take(items * sizeof(float)));
+        const int st = backward_plan(pr.T, pr.H, pr.W, g.heads, pr.d, window, dtype, true, g.dk, g.dv, a.ws_bytes ? base + a.workspace : nullptr, a.ws_bytes, g.plan);
+        if (st != DSA3D_OK) return st;
     }
     if (at > a.workspace) return DSA3D_ERR_WORKSPACE;
+#define DSA3D_TRY(call)                         \
+    do {                                        \
+        const cudaError_t e = (call);           \
+        if (e != cudaSuccess) return cuda_failed(e); \
+    } while (0)
     // a group's part of a host tensor of `head_bytes` per (token, head)
     auto up = [&](void* dst, const void* src, size_t head_bytes, const Group& g) {
         return cudaMemcpy2DAsync(dst, g.heads * head_bytes, static_cast<const char*>(src) + g.m0 * head_bytes, pr.heads * head_bytes, g.heads * head_bytes, N, cudaMemcpyHostToDevice, hs->in);
@@ -712,46 +707,61 @@ int step_host_heads(const dsa3d::Problem& pr, int group, const void* q_h, const 
     auto down = [&](void* dst, const void* src, size_t head_bytes, const Group& g) {
         return cudaMemcpy2DAsync(static_cast<char*>(dst) + g.m0 * head_bytes, pr.heads * head_bytes, src, g.heads * head_bytes, g.heads * head_bytes, N, cudaMemcpyDeviceToHost, hs->out);
     };
-    const size_t row = pr.d * elt, off = pr.P * 3 * sizeof(float);
-    for (int i = 0; i < count; ++i) {
-        const Group& g = groups[i];
-        DSA3D_TRY(up(g.k, k_h, row, g));
-        DSA3D_TRY(up(g.v, v_h, row, g));
-        DSA3D_TRY(up(g.q, q_h, row, g));
-        DSA3D_TRY(up(g.offsets, offsets_h, off, g));
-        DSA3D_TRY(cudaEventRecord(hs->q_ready[i], hs->in));
-        DSA3D_TRY(up(g.dout, dout_h, row, g));
-        DSA3D_TRY(cudaEventRecord(hs->dout_ready[i], hs->in));
-    }
-    for (int i = 0; i < count; ++i) {
-        const Group& g = groups[i];
-        BackwardPlan plan;
-        int st = backward_plan(pr.T, pr.H, pr.W, g.heads, pr.d, window, dtype, true, g.dk, g.dv, a.ws_bytes ? base + a.workspace : nullptr, a.ws_bytes, plan);
-        if (st != DSA3D_OK) return st;
-        DSA3D_TRY(cudaStreamWaitEvent(stream, hs->q_ready[i], 0));
-        st = forward_frames(plan.pr, g.q, g.k, g.v, g.offsets, g.out, g.lse, bf16, 0, pr.T, stream);
-        if (st != DSA3D_OK) return st;
-        DSA3D_TRY(cudaEventRecord(hs->fwd_done[i], stream));
-        DSA3D_TRY(cudaStreamWaitEvent(hs->out, hs->fwd_done[i], 0));
-        DSA3D_TRY(down(out_h, g.out, row, g));
-        DSA3D_TRY(down(lse_h, g.lse, sizeof(float), g));
-        DSA3D_TRY(cudaStreamWaitEvent(stream, hs->dout_ready[i], 0));
-        st = backward_frames(plan, g.q, g.k, g.v, g.offsets, g.lse, g.dout, g.dq, g.doffsets, 0, pr.T, true, stream, hs->gather_done[i]);
-        if (st != DSA3D_OK) return st;
-        st = backward_finish(plan, g.dk, g.dv, stream);
-        if (st != DSA3D_OK) return st;
-        DSA3D_TRY(cudaEventRecord(hs->slab_in_free[i], stream));
-        DSA3D_TRY(cudaStreamWaitEvent(hs->out, hs->gather_done[i], 0));
-        DSA3D_TRY(down(dq_h, g.dq, row, g));
-        DSA3D_TRY(down(doffsets_h, g.doffsets, off, g));
-        DSA3D_TRY(cudaStreamWaitEvent(hs->out, hs->slab_in_free[i], 0));
-        DSA3D_TRY(down(dk_h, g.dk, row, g));
-        DSA3D_TRY(down(dv_h, g.dv, row, g));
-    }
-    DSA3D_TRY(cudaEventRecord(hs->main_done, stream));
-    DSA3D_TRY(cudaEventRecord(hs->out_done, hs->out));
+    auto enqueue = [&]() -> int {
+        // whatever pipelined steps may still have in flight comes first, and a later one shares no ordering per slab with this call
+        DSA3D_TRY(cudaStreamWaitEvent(stream, hs->out_done, 0));
+        DSA3D_TRY(cudaStreamWaitEvent(stream, hs->main_done, 0));
+        hs->last_arena = nullptr;
+        DSA3D_TRY(cudaEventRecord(hs->start, stream));
+        DSA3D_TRY(cudaStreamWaitEvent(hs->in, hs->start, 0));
+        DSA3D_TRY(cudaStreamWaitEvent(hs->out, hs->start, 0));
+        for (int i = 0; i < count; ++i) {
+            const Group& g = groups[i];
+            DSA3D_TRY(up(g.k, k_h, row, g));
+            DSA3D_TRY(up(g.v, v_h, row, g));
+            DSA3D_TRY(up(g.q, q_h, row, g));
+            DSA3D_TRY(up(g.offsets, offsets_h, off, g));
+            DSA3D_TRY(cudaEventRecord(hs->q_ready[i], hs->in));
+            DSA3D_TRY(up(g.dout, dout_h, row, g));
+            DSA3D_TRY(cudaEventRecord(hs->dout_ready[i], hs->in));
+        }
+        for (int i = 0; i < count; ++i) {
+            const Group& g = groups[i];
+            DSA3D_TRY(cudaStreamWaitEvent(stream, hs->q_ready[i], 0));
+            int st = forward_frames(g.plan.pr, g.q, g.k, g.v, g.offsets, g.out, g.lse, bf16, 0, pr.T, stream);
+            if (st != DSA3D_OK) return st;
+            DSA3D_TRY(cudaEventRecord(hs->fwd_done[i], stream));
+            DSA3D_TRY(cudaStreamWaitEvent(hs->out, hs->fwd_done[i], 0));
+            DSA3D_TRY(down(out_h, g.out, row, g));
+            DSA3D_TRY(down(lse_h, g.lse, sizeof(float), g));
+            DSA3D_TRY(cudaStreamWaitEvent(stream, hs->dout_ready[i], 0));
+            st = backward_frames(g.plan, g.q, g.k, g.v, g.offsets, g.lse, g.dout, g.dq, g.doffsets, 0, pr.T, true, stream, hs->gather_done[i]);
+            if (st != DSA3D_OK) return st;
+            st = backward_finish(g.plan, g.dk, g.dv, stream);
+            if (st != DSA3D_OK) return st;
+            DSA3D_TRY(cudaEventRecord(hs->slab_in_free[i], stream));
+            DSA3D_TRY(cudaStreamWaitEvent(hs->out, hs->gather_done[i], 0));
+            DSA3D_TRY(down(dq_h, g.dq, row, g));
+            DSA3D_TRY(down(doffsets_h, g.doffsets, off, g));
+            DSA3D_TRY(cudaStreamWaitEvent(hs->out, hs->slab_in_free[i], 0));
+            DSA3D_TRY(down(dk_h, g.dk, row, g));
+            DSA3D_TRY(down(dv_h, g.dv, row, g));
+        }
+        DSA3D_TRY(cudaEventRecord(hs->main_done, stream));
+        DSA3D_TRY(cudaEventRecord(hs->out_done, hs->out));
+        return DSA3D_OK;
+    };
 #undef DSA3D_TRY
-    return DSA3D_OK;
+    const int st = enqueue();
+    if (st != DSA3D_OK) {
+        // the copies and kernels queued so far still run: `stream` and the next call come behind them, as behind a whole step
+        cudaEventRecord(hs->start, hs->in);
+        cudaStreamWaitEvent(hs->out, hs->start, 0);
+        cudaEventRecord(hs->main_done, stream);
+        cudaEventRecord(hs->out_done, hs->out);
+        cudaStreamWaitEvent(stream, hs->out_done, 0);
+    }
+    return st;
 }
 
 // One step enqueued on `stream_` and the two side streams.  ordered_start: uploads wait for the
