@@ -245,6 +245,12 @@ size_t dsa3d_backward_noalloc_max_elements(void);
 int dsa3d_test_backward_passes(int T, int H, int W, int heads, int d, const int window[3], int dtype,
                                size_t scratch_bytes, int* passes, size_t* largest);
 
+/*
+ * Test aid: the heads of a group of dsa3d_step_host for this problem in page-locked memory, 0 where the step goes by slabs of
+ * frames.  Host arithmetic only.
+ */
+int dsa3d_test_step_group_heads(int T, int H, int W, int heads, int d, const int window[3], int dtype, int* group);
+
 /* cudaError_t of the most recent failed address lookup of dsa3d_backward_noalloc on the
  * calling thread (0 if none). */
 int dsa3d_backward_noalloc_last_cuda_error(void);

@@ -84,6 +84,8 @@ def _declare(lib) -> None:
     lib.dsa3d_backward_noalloc_last_cuda_error.argtypes = []
     lib.dsa3d_test_backward_passes.restype = i
     lib.dsa3d_test_backward_passes.argtypes = [i, i, i, i, i, win, i, sz, ctypes.POINTER(i), ctypes.POINTER(sz)]
+    lib.dsa3d_test_step_group_heads.restype = i
+    lib.dsa3d_test_step_group_heads.argtypes = [i, i, i, i, i, win, i, ctypes.POINTER(i)]
     dptr = ctypes.POINTER(ctypes.c_double)
     lib.dsa3d_probe_gather.restype = i
     lib.dsa3d_probe_gather.argtypes = [p, sz, i, dptr, p]
@@ -351,6 +353,13 @@ def dsa3d_test_backward_passes(T, H, W, heads, d, window, dtype, scratch_bytes):
     _check(load().dsa3d_test_backward_passes(T, H, W, heads, d, _window(window), _DTYPES[dtype], scratch_bytes,
                                              ctypes.byref(passes), ctypes.byref(largest)))
     return passes.value, largest.value
+
+
+def dsa3d_test_step_group_heads(T, H, W, heads, d, window, dtype) -> int:
+    """Heads of a group of dsa3d_step_host in page-locked memory; 0: by slabs of frames."""
+    group = ctypes.c_int(0)
+    _check(load().dsa3d_test_step_group_heads(T, H, W, heads, d, _window(window), _DTYPES[dtype], ctypes.byref(group)))
+    return group.value
 
 
 def dsa3d_test_wait_timeout(polls: int, stream=None) -> None:

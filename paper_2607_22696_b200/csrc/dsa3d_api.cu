@@ -1105,6 +1105,14 @@ int dsa3d_test_backward_passes(int T, int H, int W, int heads, int d, const int 
     return rc;
 }
 
+int dsa3d_test_step_group_heads(int T, int H, int W, int heads, int d, const int window[3], int dtype, int* group) {
+    if (!group) return DSA3D_ERR_NULL_POINTER;
+    dsa3d::Problem pr;
+    const int rc = make_problem(T, H, W, heads, d, window, dtype, pr);
+    if (rc == DSA3D_OK) *group = step_group_heads(pr, arena_layout(pr, dtype).row_bytes);
+    return rc;
+}
+
 int dsa3d_debug_build(void) {
 #ifdef DSA3D_DEBUG
     return 1;
