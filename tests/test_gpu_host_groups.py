@@ -1,5 +1,5 @@
-"""dsa3d_step_host by groups of heads beside pipelined steps on the same arena, and from memory that is not all page-locked; against the
-device entry points."""
+"""dsa3d_step_host by groups of heads beside pipelined steps on the same arena, from memory that is not all page-locked, and with offsets
+too narrow for strided uploads; against the device entry points."""
 import pytest
 import torch
 
@@ -69,3 +69,19 @@ def test_memory_that_is_not_page_locked(pageable):
     binding.dsa3d_step_host(*host, *dims, window, *res, _arena(dims, window, BF16))
     torch.cuda.synchronize()
     _check(host, res, dims, window, f"pageable {pageable}")
+
+
+@pytest.mark.parametrize("dtype,dims", [(BF16, (3, 45, 80, 7, 128)), (F32, (2, 45, 80, 5, 128)), (F32, (2, 45, 80, 19, 32))])
+@pytest.mark.parametrize("window", [(1, 1, 1), (1, 1, 2), (1, 1, 3), (1, 2, 3)])
+def test_narrow_offsets(dtype, dims, window):
+    """12 bytes per sample and head: on both sides of 64 per token and group, the last group narrower than the others."""
+    assert binding.dsa3d_test_step_group_heads(*dims, window, dtype) > 0
+    host = [z.pin_memory() for z in small_problem(*dims, window, dtype, 1.0, 975)]
+    res = _results(host)
+    n = binding.dsa3d_step_host_arena_bytes(*dims, window, dtype)
+    arena = torch.full((n + 4096,), 0xA5, dtype=torch.uint8, device="cuda")
+    for _ in range(2):
+        binding.dsa3d_step_host(*host, *dims, window, *res, arena[:n])
+    torch.cuda.synchronize()
+    assert bool((arena[n:] == 0xA5).all())
+    _check(host, res, dims, window, f"window {window}")
