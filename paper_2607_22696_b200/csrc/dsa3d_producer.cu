@@ -1415,7 +1415,38 @@ convert_rows_bf16_kernel(const float* __restrict__ src, long long rows, int cols
     }
 }
 
-// Rows of a block of the two kernels above: 512, and fewer (a multiple of 64) where those would be less than three blocks per SM.  Blocks of 512
+// The same for short calls and any cols: a block owns 32 columns of half of the rows, a warp every 32nd row, and adds the warps' sums up in
+// order, so that the sums, of two blocks per column, are the same from call to call (a + b is b + a).  The padding columns of dst are
+// written as zeros.  Whole call by blocks of 512 rows, of 64 (rows_per_block), and so: 512 tokens, 1024 inputs, 1296 outputs 158, 61
+// and 55 us; 2048 tokens, 256 inputs, 162 outputs 62, 35 and 38 us.
+constexpr int kStripTokens = 2048;
+__global__ void __launch_bounds__(1024)
+convert_strip_bf16_kernel(const float* __restrict__ src, int rows, int cols, __nv_bfloat16* __restrict__ dst, long long ldd, float* __restrict__ colsum) {
+    __shared__ float sums[32][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = blockIdx.x * 32 + lane;
+    const int half = (rows + 1) / 2, end = blockIdx.y ? rows : half;
+    float sum = 0.0f;
+    for (int r0 = blockIdx.y * half + warp; r0 < end; r0 += 512) {      // sixteen rows asked for at once
+        float v[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = r0 + 32 * i < end && c < cols ? __ldg(src + static_cast<long long>(r0 + 32 * i) * cols + c) : 0.0f;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            sum += v[i];
+            if (r0 + 32 * i < end && c < ldd) dst[(r0 + 32 * i) * ldd + c] = __float2bfloat16_rn(v[i]);
+        }
+    }
+    if (!colsum) return;
+    sums[warp][lane] = sum;
+    __syncthreads();
+    if (warp > 0 || c >= cols) return;
+    float t = 0.0f;
+#pragma unroll
+    for (int w = 0; w < 32; ++w) t += sums[w][lane];
+    atomicAdd(colsum + c, t);
+}
+
+// Rows of a block of the two kernels above it: 512, and fewer (a multiple of 64) where those would be less than three blocks per SM.  Blocks of 512
 // rows leave a call of 24,960 tokens, 1296 outputs, a third of the SMs: conversion 210 -> 56 us with 64.  On 262,144 tokens 320 rows
 // were no faster than 512 (whole linear-layer backward 2.78 and 2.69 ms).
 int rows_per_block(long long rows) {
@@ -1698,7 +1729,11 @@ int dsa3d_offsets_linear_backward(const void* u, const void* w, const float* dof
         const long long ns = tokens - s0 < plan.slab ? tokens - s0 : plan.slab;
         const int rows = rows_per_block(ns);
         const unsigned row_blocks = static_cast<unsigned>((ns + rows - 1) / rows);
-        if (O % 4 == 0) {   // doffsets slab -> bf16 copy and column sums
+        if (tokens <= kStripTokens) {
+            const dim3 grid(static_cast<unsigned>((plan.ld_o + 31) / 32), tokens > 1 ? 2 : 1);
+            convert_strip_bf16_kernel<<<grid, 1024, 0, st>>>(doffsets, static_cast<int>(ns), O, g, plan.ld_o, dbias);
+            if ((e = cudaGetLastError()) != cudaSuccess) return cuda_failed(e);
+        } else if (O % 4 == 0) {   // doffsets slab -> bf16 copy and column sums
             int threads = ((O / 4 + 31) / 32) * 32;
             if (threads > 1024) threads = 1024;
             convert_rows_bf16_kernel<<<row_blocks, threads, 0, st>>>(doffsets + s0 * O, ns, O, g, plan.ld_o, dbias, rows);
