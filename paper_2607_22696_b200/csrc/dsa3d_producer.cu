@@ -1719,9 +1719,10 @@ int dsa3d_offsets_linear_backward(const void* u, const void* w, const float* dof
     if (dw && (e = cudaMemsetAsync(dw, 0, static_cast<size_t>(O) * C * sizeof(float), st)) != cudaSuccess) return cuda_failed(e);
     if (dbias && (e = cudaMemsetAsync(dbias, 0, static_cast<size_t>(O) * sizeof(float), st)) != cudaSuccess) return cuda_failed(e);
     if (du) {                                                        // w [O, C] -> w^T [C, O]
-        const dim3 grid((C + 63) / 64, static_cast<unsigned>((O + 63) / 64));
+        const int rows = (O + 63) / 64 <= 65535 ? 64 : 1024;         // a grid has at most 65,535 blocks along y
+        const dim3 grid((C + 63) / 64, static_cast<unsigned>((static_cast<long long>(O) + rows - 1) / rows));
         transpose_to_bf16_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(w), C, O, C, wt,
-                                                                      plan.ld_o, nullptr, 0, nullptr, 64);
+                                                                      plan.ld_o, nullptr, 0, nullptr, rows);
         if ((e = cudaGetLastError()) != cudaSuccess) return cuda_failed(e);
     }
     bool unsupported = false;
