@@ -485,6 +485,8 @@ forward_classes_kernel(const float* __restrict__ q, const float* __restrict__ k,
     const long long v_minus_k = v - k;
     [[maybe_unused]] const long long kv_extent = pr.N * pr.heads * D;
     const float lscale = rsqrtf(static_cast<float>(D)) * kLog2e;        // logits in log2 units
+    // with a q that is not finite a sample without a row has the logit 0 all the same: not by the products below that take eight at once
+    const bool finite = fabsf(qr.v[0] + qr.v[1] + qr.v[2] + qr.v[3]) < INFINITY;
     int size = (pr.P + kClasses - 1) / kClasses;
     if (pr.P > 16) size = (size + 7) & ~7;               // so that eight samples on the grid belong to one class
     const int span = G == 1 ? pr.P : size, begin = G == 1 ? 0 : group % G * size;
@@ -525,7 +527,7 @@ forward_classes_kernel(const float* __restrict__ q, const float* __restrict__ k,
         Sample mine;
         mine.base = 0; mine.mask = 0u; mine.ft = mine.fy = mine.fx = 0.0f;
         if (gl < cnt && p0 + gl < pr.P) mine = to_sample(pr, make_cell(pr, t, y, x, p0 + gl, offsets ? offsets + (row * pr.P + p0 + gl) * 3 : kZeroOffset));
-        if (__all_sync(kFullMask, mine.ft == 0.0f && mine.fy == 0.0f && mine.fx == 0.0f)) {     // on the grid: a row each, eight samples at a time
+        if (__all_sync(kFullMask, finite && mine.ft == 0.0f && mine.fy == 0.0f && mine.fx == 0.0f)) {     // on the grid: a row each, eight samples at a time
             for (int jb = 0; jb < cnt; jb += 8) {
                 Row kk[8], vv[8];
 #pragma unroll

@@ -59,3 +59,21 @@ def test_residual_of_small_calls(d, grid, heads):
     both, lse2 = torch.empty_like(out), torch.empty_like(lse)
     binding.dsa3d_forward_residual(q, k, v, off, add, *dims, window, both, lse2)
     assert torch.equal(both, out + add) and torch.equal(lse, lse2)      # one fp32 addition
+
+
+@pytest.mark.parametrize("d,grid", [(32, (4, 8, 8)), (64, (2, 8, 9)), (128, (2, 6, 6))])
+@pytest.mark.parametrize("heads", [1, 25])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_dead_samples_of_a_query_that_is_not_finite(d, grid, heads, bad):
+    """A sample without a corner inside the grid has the logit 0 whatever q holds: a query with no others has out = 0, lse = ln P, also
+    beside queries whose samples all lie on the grid."""
+    window, dims = (3, 3, 3), (*grid, heads, d)
+    q, k, v, off, _ = small_problem(*dims, window, F32, 1.3, 1030 + d)
+    off = off.round()
+    rows = torch.zeros(dims[:4], dtype=torch.bool)
+    rows.view(-1)[::3] = True
+    q[rows], off[rows] = bad, 1e6
+    out, lse = pu.gpu_forward(*(z.cuda() for z in (q, k, v, off)), dims, window)
+    out, lse = out.cpu(), lse.cpu()
+    assert float(out[rows].abs().max()) == 0.0 and float((lse[rows] - torch.tensor(27.0).log()).abs().max()) <= 1e-6
+    assert bool(torch.isfinite(out).all() and torch.isfinite(lse).all())
