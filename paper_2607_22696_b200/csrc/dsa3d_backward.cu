@@ -1,6 +1,6 @@
 // Backward of 3D Deformable Slide Attention: dQ, dK, dV and dOffsets, by rows.  The route of small fp32 calls and of
 // larger ones with integer offsets, and in bf16 of DSA3D_TILE and of a workspace too small for a pass of the cell-sorted
-// kernels (dsa3d_cells.cu), which serve the rest.
+// kernels (dsa3d_cells.cu), which serve the rest.  (The smallest fp32 calls: backward_split_kernel, the same sums.)
 //
 // Two kernels.
 //

@@ -17,7 +17,8 @@
 //   V planes   channels x positions x queries for head and remainder, a warp 64 channels of both x-rows.
 //
 // What bounds it, (3,7,7), 128 channels: chains of ldmatrix and products at 16 warps an SM, 340 clocks per query; the data pipe (ldmatrix,
-// table) is busy for 60 % of them, the tensor unit (63 products of two clocks) for 42 %.  A dense product of the tile's 128 queries with a
+// table) is busy for 60 % of them, the tensor unit for 42 % (66 products of 2.16 clocks; the first and the last region row are multiplied with both
+// x-rows although one of them does not reach it).  128 registers, 4 to 12 bytes spilled at 128 channels.  A dense product of the tile's 128 queries with a
 // plane (tcgen05) spends its time on moving every score plane from TMEM through shared memory into registers and on laying the weights out
 // among the plane's columns.  That kernel -> this one, 64 x 45 x 80, 16 heads of 128: (3,7,7) 4.94 -> 4.38 ms, (3,5,5) 3.39 -> 3.36 ms,
 // learned offsets 6.89 -> 6.69 ms; 16 x 45 x 80, 16 heads of 64: 1156 -> 869 us, 760 -> 693 us, 1494 -> 1425 us; 4 x 9 x 13, 2 heads of 64:

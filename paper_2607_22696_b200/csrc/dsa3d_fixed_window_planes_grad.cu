@@ -4,8 +4,8 @@
 // (ck = scale dS, cv = alpha: the two coefficients per sample that fixed_window_backward_query_kernel
 // leaves; the chain rule of the Formulation with every sample on a grid position).  For a tile of
 // 4 x 4 x 8 outputs each sum is  C . X_region  with C the coefficients placed at their region
-// positions (zero elsewhere) - the forward's P . V with other weights and other rows - and the region
-// (840 rows for (3,7,7)) is walked one plane (along t) at a time, exactly as the forward's second pass:
+// positions (zero elsewhere), and the region (840 rows for (3,7,7)) is walked one plane (along t) at a
+// time:
 //
 //   per (tile, head) three sweeps (dQ over K, dK over q, dV over dO), per sweep kt+3 planes:
 //     the plane's rows by TMA into a ring of buffers; every worker thread writes the coefficients of

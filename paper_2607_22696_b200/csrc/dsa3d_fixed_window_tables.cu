@@ -14,7 +14,7 @@
 // fixed_window_backward_query_kernel then takes its dot products from the table instead of
 // gathering K and V rows.
 //
-// Roles as in the plane-by-plane forward: 8 worker warps copy scores (the two warps that share a TMEM
+// Roles: 8 worker warps copy scores (the two warps that share a TMEM
 // quadrant split a plane's columns and the box's rows along y between them), one more warp holds the
 // thread that issues the TMA loads, two more one thread each that issues the MMAs of every other plane;
 // mbarriers order them, every wait is bounded, and a wait that runs out raises the library's timeout

@@ -88,7 +88,7 @@ __device__ __forceinline__ unsigned sm_neighbours(unsigned block, unsigned block
 // Bound by the L1 data pipe (87 % at 128 channels, 80 % at 64).  Windows of 17 to 32 samples have an instance of one round (kOne), which
 // keeps nothing for a next one: window (3,3,3), 16 x 68 x 120, 16 heads of 128, N(0, 1.5) 11.72 -> 10.92 ms, 16 x 45 x 80 integer offsets
 // 1.54 -> 1.26 ms, N(0, 0.5) 5.68 -> 5.57, N(0, 3) 4.63 -> 4.24; 64 channels 6.65 -> 6.56 ms, and 6.32 with 20 CTAs per SM (48
-// registers; 24 CTAs, 40 registers: 6.61; 128 channels with 18: 11.3).
+// registers; 24 CTAs, 40 registers: 6.61; 128 channels with 18: 11.3).  With several rounds 128 channels spill 100 bytes at 64 registers.
 template <int D, bool kAdd, bool kGated, bool kOne>
 __global__ void __launch_bounds__(kFwdWarps * 32, D == 64 && kOne && !kGated ? 20 : 16)
 gather_forward_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v,

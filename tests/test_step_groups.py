@@ -22,6 +22,9 @@ def library():
     (BF16, (4, 30, 52, 16, 64), 4),              # 512 bytes: rows of 1 KB make two groups
     (BF16, (2, 30, 52, 17, 128), 4),
     (BF16, (2, 4, 64, 256, 64), 32),             # eight groups at most, whatever their width
+    (BF16, (3, 30, 52, 16, 64), 4),
+    (F32, (2, 30, 52, 11, 64), 2),
+    (F32, (3, 30, 52, 9, 64), 2),
     (F32, (8, 45, 80, 8, 64), 2),
     (F32, (8, 45, 80, 4, 128), 1),
     (F32, (8, 45, 80, 3, 128), 0),
